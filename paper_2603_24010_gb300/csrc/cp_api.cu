@@ -19,14 +19,16 @@
 
 namespace cpk {
 size_t push_smem_bytes(int N, int precision);
-size_t solve_smem_bytes(int N, int ctas);
-cudaError_t solve_cluster_size(int precision, int N, int* ctas);
+size_t solve_smem_bytes(int N, int ctas, bool net);
+bool solve_wide(int N, const int64_t cap[kSpecies], double per_particle);
+cudaError_t solve_cluster_size(int precision, bool wide, int N, int* ctas);
+int solve_ens_cluster_size(int n_max, int E, int sms);
 cudaError_t push_configure(int precision, size_t push_smem);
-cudaError_t solve_configure(int precision, size_t solve_smem);
+cudaError_t solve_configure(int precision, bool wide);
 cudaError_t push_occupancy(int precision, size_t smem, int* blocks_per_sm);
 cudaError_t push_launch(int precision, const Bufs& B, int grid, size_t smem, cudaStream_t st,
                         int do_push);
-cudaError_t solve_launch(int precision, const Bufs& B, int ctas, size_t smem, cudaStream_t st,
+cudaError_t solve_launch(int precision, bool wide, const Bufs& B, int ctas, size_t smem, cudaStream_t st,
                          int do_push, int mode, double tol);
 cudaError_t compact_launch(int precision, const Bufs& B, int grid, cudaStream_t st);
 cudaError_t fill_launch(int precision, void* p, int64_t n, double v, cudaStream_t st);
@@ -41,8 +43,8 @@ cudaError_t push_ens_occupancy(int precision, int threads, size_t smem, int* per
 cudaError_t push_ens_launch(int precision, int threads, int grid, size_t smem, const Bufs* Ball,
                             int E, int n_max, void* abs, int abs_cap, cudaStream_t st);
 cudaError_t compact_ens_launch(int precision, const Bufs* Ball, int E, int grid, cudaStream_t st);
-cudaError_t solve_ens_configure(int precision, size_t smem);
-cudaError_t solve_ens_launch(int precision, const Bufs* Ball, int n_inst, size_t smem,
+cudaError_t solve_ens_configure(int precision, bool wide);
+cudaError_t solve_ens_launch(int precision, bool wide, const Bufs* Ball, int n_inst, int ctas, size_t smem,
                              cudaStream_t st, int do_push, int mode, double tol);
 cudaError_t status_ens_launch(const Bufs* Ball, int E, int* out, cudaStream_t st);
 cudaError_t push2_occupancy(int* per_sm);
@@ -87,8 +89,8 @@ struct cp_ctx {
   int grid = 0;
   int compact_grid = 0;   // removal kernel
   size_t smem = 0;        // push kernel
-  size_t solve_smem = 0;  // solve kernel
-  int solve_ctas = 8;     // CTAs in the solve's cluster
+  int solve_ctas = 1;     // CTAs in the solve's cluster
+  bool solve_wide = true; // 128-bit prefix of prefixes
   bool initialized = false;
   int compact_every = 128;
   int since_compact = 0;
@@ -235,6 +237,13 @@ cpk::Bufs make_bufs(const cp_ctx* c) {
   return B;
 }
 
+// the coupled solve of the context's next level (shared memory for the
+// network only where the solve runs it)
+cudaError_t solve(const cp_ctx* c, const cpk::Bufs& B, cudaStream_t st, int do_push, int mode, double tol) {
+  const size_t smem = cpk::solve_smem_bytes(c->N, c->solve_ctas, B.net != nullptr && !B.net_in_push);
+  return cpk::solve_launch(c->precision, c->solve_wide, B, c->solve_ctas, smem, st, do_push, mode, tol);
+}
+
 void free_all(cp_ctx* c) {
   for (int b = 0; b < 2; ++b) {
     for (int s = 0; s < kSpecies; ++s) {
@@ -346,10 +355,10 @@ int initialize(cp_ctx* c, int mode, double tol) {
 
   // launch shape: persistent grid of resident push CTAs, one solve cluster
   c->smem = cpk::push_smem_bytes(c->N, c->precision);
-  CP_CUDA(cpk::solve_cluster_size(c->precision, c->N, &c->solve_ctas));
-  c->solve_smem = cpk::solve_smem_bytes(c->N, c->solve_ctas);
+  c->solve_wide = cpk::solve_wide(c->N, c->cap, cpk::kFix);
   CP_CUDA(cpk::push_configure(c->precision, c->smem));
-  CP_CUDA(cpk::solve_configure(c->precision, c->solve_smem));
+  CP_CUDA(cpk::solve_configure(c->precision, c->solve_wide));
+  CP_CUDA(cpk::solve_cluster_size(c->precision, c->solve_wide, c->N, &c->solve_ctas));
   int per_sm = 0, sms = 0;
   CP_CUDA(cpk::push_occupancy(c->precision, c->smem, &per_sm));
   CP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
@@ -394,7 +403,7 @@ int initialize(cp_ctx* c, int mode, double tol) {
   // deposit rho^0 and solve level 0
   const cpk::Bufs B0 = make_bufs(c);
   CP_CUDA(cpk::push_launch(c->precision, B0, c->grid, c->smem, c->stream, 0));
-  CP_CUDA(cpk::solve_launch(c->precision, B0, c->solve_ctas, c->solve_smem, c->stream, 0, mode, tol));
+  CP_CUDA(solve(c, B0, c->stream, 0, mode, tol));
   c->launches += 2;
   return CP_OK;
 }
@@ -419,7 +428,7 @@ int build_graph(cp_ctx* c, int mode, double tol) {
   cudaError_t e = cudaSuccess;
   for (int k = 0; k < c->compact_every && e == cudaSuccess; ++k) {
     e = cpk::push_launch(c->precision, B, c->grid, c->smem, c->cap_stream, 1);
-    if (e == cudaSuccess) e = cpk::solve_launch(c->precision, B, c->solve_ctas, c->solve_smem, c->cap_stream, 1, mode, tol);
+    if (e == cudaSuccess) e = solve(c, B, c->cap_stream, 1, mode, tol);
   }
   if (e == cudaSuccess) e = cpk::compact_launch(c->precision, B, c->compact_grid, c->cap_stream);
   const cudaError_t e2 = cudaStreamEndCapture(c->cap_stream, &g);
@@ -447,7 +456,7 @@ int timed_launch(cp_ctx* c, int which, int mode, double tol, std::vector<std::pa
   if (which == 0)
     CP_CUDA(cpk::push_launch(c->precision, B, c->grid, c->smem, c->stream, 1));
   else if (which == 1)
-    CP_CUDA(cpk::solve_launch(c->precision, B, c->solve_ctas, c->solve_smem, c->stream, 1, mode, tol));
+    CP_CUDA(solve(c, B, c->stream, 1, mode, tol));
   else
     CP_CUDA(cpk::compact_launch(c->precision, B, c->compact_grid, c->stream));
   CP_CUDA(cudaEventRecord(c->ev_pool[k + 1], c->stream));
@@ -504,7 +513,7 @@ int do_steps(cp_ctx* c, int mode, int32_t n_steps, double tol) {
       continue;
     }
     CP_CUDA(cpk::push_launch(c->precision, B, c->grid, c->smem, c->stream, 1));
-    CP_CUDA(cpk::solve_launch(c->precision, B, c->solve_ctas, c->solve_smem, c->stream, 1, mode, tol));
+    CP_CUDA(solve(c, B, c->stream, 1, mode, tol));
     c->launches += 2;
     --left;
     if (++c->since_compact == c->compact_every) {
@@ -1067,7 +1076,9 @@ struct cp_batch {
   int push_threads = 512;
   int push_grid = 0;
   size_t push_smem = 0;
-  size_t solve_smem = 0;
+  int solve_ctas = 1;      // CTAs per instance of the solve
+  bool solve_wide = false;
+  bool any_net = false;    // a network is installed on some instance
   int compact_grid = 0;
   int compact_every = 128;
   int since_compact = 0;
@@ -1140,10 +1151,14 @@ int batch_init(cp_batch* b, int mode, double tol) {
                           b->stream));
   CP_TRY(alloc(reinterpret_cast<void**>(&b->dstatus), sizeof(int) * b->E));
   b->push_smem = cpk::push_ens_smem_bytes(b->n_max, b->precision, b->E);
-  b->solve_smem = cpk::solve_smem_bytes(b->n_max, 1);
-  CP_CUDA(cpk::solve_ens_configure(b->precision, b->solve_smem));
+  for (cp_ctx* c : b->inst) {
+    b->solve_wide = b->solve_wide || c->solve_wide;
+    b->any_net = b->any_net || c->net != nullptr;
+  }
+  CP_CUDA(cpk::solve_ens_configure(b->precision, b->solve_wide));
   int sms = 0;
   CP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device));
+  b->solve_ctas = cpk::solve_ens_cluster_size(b->n_max, b->E, sms);
   b->compact_grid = 2 * sms;
   CP_TRY(batch_set_shape(b, 512, 0));
   CP_CUDA(cudaStreamSynchronize(b->stream));
@@ -1151,11 +1166,16 @@ int batch_init(cp_batch* b, int mode, double tol) {
   return CP_OK;
 }
 
+cudaError_t batch_solve(cp_batch* b, cudaStream_t st, int mode, double tol) {
+  const size_t smem = cpk::solve_smem_bytes(b->n_max, b->solve_ctas, b->any_net);
+  return cpk::solve_ens_launch(b->precision, b->solve_wide, b->dBall, b->E, b->solve_ctas, smem, st, 1, mode, tol);
+}
+
 cudaError_t batch_step_launches(cp_batch* b, cudaStream_t st, int mode, double tol) {
   cudaError_t e = cpk::push_ens_launch(b->precision, b->push_threads, b->push_grid, b->push_smem,
                                        b->dBall, b->E, b->n_max, b->abs, b->abs_cap, st);
   if (e == cudaSuccess)
-    e = cpk::solve_ens_launch(b->precision, b->dBall, b->E, b->solve_smem, st, 1, mode, tol);
+    e = batch_solve(b, st, mode, tol);
   return e;
 }
 
@@ -1211,8 +1231,7 @@ int batch_steps_timed(cp_batch* b, int mode, int32_t n_steps, double tol) {
       CP_CUDA(cpk::push_ens_launch(b->precision, b->push_threads, b->push_grid, b->push_smem,
                                    b->dBall, b->E, b->n_max, b->abs, b->abs_cap, b->stream));
     else if (which == 1)
-      CP_CUDA(cpk::solve_ens_launch(b->precision, b->dBall, b->E, b->solve_smem, b->stream, 1,
-                                    mode, tol));
+      CP_CUDA(batch_solve(b, b->stream, mode, tol));
     else
       CP_CUDA(cpk::compact_ens_launch(b->precision, b->dBall, b->E, b->compact_grid, b->stream));
     CP_CUDA(cudaEventRecord(b->ev[k + 1], b->stream));
@@ -1336,6 +1355,13 @@ int cp_batch_set_predictor(cp_batch* b, int32_t i, const float* params, const cp
   // the ensemble kernels read the instance's buffer set from the device
   // table at every launch: refresh instance i's entry
   const cpk::Bufs hb = make_bufs(b->inst[i]);
+  if (!b->any_net) {  // graphs carry the solve's shared memory without a network
+    b->any_net = true;
+    for (int m = 0; m < 3; ++m) {
+      if (b->gexec[m]) cudaGraphExecDestroy(b->gexec[m]);
+      b->gexec[m] = nullptr;
+    }
+  }
   CP_CUDA(cudaMemcpyAsync(b->dBall + i, &hb, sizeof(cpk::Bufs), cudaMemcpyHostToDevice, b->stream));
   CP_CUDA(cudaStreamSynchronize(b->stream));
   return CP_OK;
@@ -1430,8 +1456,7 @@ int cp_batch_autotune(cp_batch* b, int32_t steps_per_shape, int32_t mode, double
                                           b->dBall, b->E, b->n_max, b->abs, b->abs_cap, b->stream));
       if (rc == CP_OK) rc = cuda_rc(cudaEventRecord(e1, b->stream));
       if (rc == CP_OK)
-        rc = cuda_rc(cpk::solve_ens_launch(b->precision, b->dBall, b->E, b->solve_smem, b->stream,
-                                           1, mode, tol));
+        rc = cuda_rc(batch_solve(b, b->stream, mode, tol));
       if (rc == CP_OK) rc = cuda_rc(cudaEventSynchronize(e1));
       float ms = 0.f;
       if (rc == CP_OK) rc = cuda_rc(cudaEventElapsedTime(&ms, e0, e1));
@@ -1554,7 +1579,7 @@ int g2_solve(cp_gap2d* g, int do_push, int mode, double tol) {
   cp_ctx* c = g->c;
   const cpk::Bufs B = make_bufs(c);
   CP_CUDA(cpk::solve2_fwd_launch(g->dD, c->G, g->Nx, g->Ny, c->stream));
-  CP_CUDA(cpk::solve_launch(c->precision, B, c->solve_ctas, c->solve_smem, c->stream, do_push, mode, tol));
+  CP_CUDA(solve(c, B, c->stream, do_push, mode, tol));
   const float c_rhs = static_cast<float>(-c->hp.dx * c->hp.dx / c->hp.eps0);
   CP_CUDA(cpk::solve2_modes_launch(g->dD, g->Nx, g->Ny, c_rhs, c->E64, c->stream));
   g->launches += 6;
@@ -1630,9 +1655,9 @@ int g2_init(cp_gap2d* g, int mode, double tol) {
   CP_CUDA(cudaMemsetAsync(c->Glast, 0, sizeof(long long) * (N + 1), c->stream));
   CP_CUDA(cudaMemsetAsync(c->Epair, 0, 2 * sizeof(float) * (N + 1), c->stream));
   CP_CUDA(cudaMemsetAsync(c->hist, 0, sizeof(cp_diag) * c->hist_rows, c->stream));
-  CP_CUDA(cpk::solve_cluster_size(c->precision, N, &c->solve_ctas));
-  c->solve_smem = cpk::solve_smem_bytes(N, c->solve_ctas);
-  CP_CUDA(cpk::solve_configure(c->precision, c->solve_smem));
+  c->solve_wide = true;  // the mean's grid counts 2^32 per macroparticle
+  CP_CUDA(cpk::solve_configure(c->precision, c->solve_wide));
+  CP_CUDA(cpk::solve_cluster_size(c->precision, c->solve_wide, N, &c->solve_ctas));
   CP_TRY(alloc(reinterpret_cast<void**>(&c->abs), sizeof(cpk::AbsRec)));
   // the mean's charge grid (column sums of the 2D grid) counts 2^32 per
   // macroparticle; every int64 sum stays below 2^63 while the stores hold

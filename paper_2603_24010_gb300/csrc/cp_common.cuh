@@ -185,6 +185,9 @@ template <typename T>
 __device__ __forceinline__ T ldcg(const T* p) {
   return __ldcg(p);
 }
+__device__ __forceinline__ void* ldcg(void* const* p) {  // a buffer pointer that a removal swaps
+  return reinterpret_cast<void*>(__ldcg(reinterpret_cast<const unsigned long long*>(p)));
+}
 
 __device__ __forceinline__ double source_voltage(const DevParams* P, double t) {
   const double pi = 3.14159265358979323846;

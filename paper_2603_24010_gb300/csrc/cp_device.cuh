@@ -36,7 +36,8 @@ constexpr int kTile = kThreads * kPerThread;  // particles per CTA tile
 constexpr int kFlushTiles = 31;        // tiles between flushes of the 32-bit cell sums
 constexpr int kSolveCtas = 8;          // CTAs (one cluster) of the coupled solve (portable)
 constexpr int kSolveCtasMax = 16;      // non-portable cluster size used where the GPU allows it
-constexpr int kSolveThreads = 512;
+constexpr int kRowThreads = 256;       // threads of a solve CTA that own rows
+constexpr int kSolveThreads = kRowThreads + 64;  // and two warps for the circuit and the commit
 constexpr double kFix = 65536.0;       // fixed-point units per macroparticle charge
 constexpr uint64_t kTagSee = 0x5345ULL;
 constexpr uint64_t kTagBeam = 0x4245ULL;

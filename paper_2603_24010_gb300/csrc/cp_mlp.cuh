@@ -27,59 +27,57 @@ __device__ __forceinline__ float gelu_grad(float x) {
          x * 0.39894228040143268f * expf(-0.5f * x * x);
 }
 
-// One dense layer for a single input vector in shared memory, all threads of
-// the block taking part: 8 lanes per output neuron (OUT * 8 <= blockDim.x),
-// each summing every 8th input in FP32, then a 3-step butterfly.  The calls
-// of all threads must be uniform (the shuffles name the whole warp).
-template <int IN, int OUT, bool ACT>
-__device__ __forceinline__ void dense_one(const uint16_t* __restrict__ W, const float* __restrict__ b,
-                                          const float* in, float* out) {
-  const int o = static_cast<int>(threadIdx.x) >> 3, part = static_cast<int>(threadIdx.x) & 7;
-  float acc = 0.0f;
-  if (o < OUT) {
-#pragma unroll
-    for (int k = part; k < IN; k += 8) acc = fmaf(bf16_bits_to_float(W[o * IN + k]), in[k], acc);
-  }
-  acc += __shfl_xor_sync(0xffffffffu, acc, 4);
-  acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-  acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-  if (o < OUT && part == 0) {
-    const float z = acc + b[o];
-    out[o] = ACT ? gelu(z) : z;
-  }
-}
-
-// dense_one split in two: the BF16 weights a thread uses (every 8th input of
-// neuron threadIdx.x / 8, from input threadIdx.x % 8 on) are loaded into
-// registers first -- all layers' loads in flight together when the weights
-// sit in global memory -- and applied later in dense_one's order.
-template <int IN>
+// One dense layer for a single input vector in shared memory by NT threads
+// (more may call): 8 lanes per output neuron, each summing every 8th input
+// in FP32, then a 3-step butterfly; NT / 8 neurons a pass.  The BF16 weights
+// a thread uses are loaded into registers first -- all layers' loads in
+// flight together when the weights sit in global memory -- and applied
+// later.  The result does not depend on NT.
+template <int IN, int OUT, int NT>
 struct LaneW {
-  uint16_t w[IN / 8];
+  static constexpr int kPasses = (OUT * 8 + NT - 1) / NT;
+  uint16_t w[kPasses][IN / 8];
+  float b[kPasses];
 };
 
-template <int IN, int OUT>
-__device__ __forceinline__ void lane_weights(const uint16_t* W, LaneW<IN>& r) {
-  static_assert(IN % 8 == 0, "8 lanes per neuron");
-  const int o = static_cast<int>(threadIdx.x) >> 3, part = static_cast<int>(threadIdx.x) & 7;
-#pragma unroll
-  for (int q = 0; q < IN / 8; ++q) r.w[q] = (o < OUT) ? W[o * IN + part + 8 * q] : uint16_t(0);
+// first output neuron of this thread; threads past NT have none
+template <int NT>
+__device__ __forceinline__ int lane_neuron(int pass) {
+  return (static_cast<int>(threadIdx.x) < NT) ? (static_cast<int>(threadIdx.x) >> 3) + pass * (NT / 8) : 1 << 20;
 }
 
-template <int IN, int OUT, bool ACT>
-__device__ __forceinline__ void dense_lane(const LaneW<IN>& r, float bias, const float* in, float* out) {
-  const int o = static_cast<int>(threadIdx.x) >> 3, part = static_cast<int>(threadIdx.x) & 7;
-  float acc = 0.0f;
-  if (o < OUT) {
+template <int IN, int OUT, int NT>
+__device__ __forceinline__ void lane_weights(const uint16_t* W, const float* b, LaneW<IN, OUT, NT>& r) {
+  static_assert(IN % 8 == 0 && NT % 32 == 0, "8 lanes per neuron");
+  const int part = static_cast<int>(threadIdx.x) & 7;
 #pragma unroll
-    for (int q = 0; q < IN / 8; ++q) acc = fmaf(bf16_bits_to_float(r.w[q]), in[part + 8 * q], acc);
+  for (int p = 0; p < r.kPasses; ++p) {
+    const int o = lane_neuron<NT>(p);
+#pragma unroll
+    for (int q = 0; q < IN / 8; ++q) r.w[p][q] = (o < OUT) ? W[o * IN + part + 8 * q] : uint16_t(0);
+    r.b[p] = (o < OUT) ? b[o] : 0.0f;
   }
-  acc += __shfl_xor_sync(0xffffffffu, acc, 4);
-  acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-  acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-  if (o < OUT && part == 0) {
-    const float z = acc + bias;
-    out[o] = ACT ? gelu(z) : z;
+}
+
+// The calls of all threads must be uniform (the shuffles name the whole warp).
+template <int IN, int OUT, int NT, bool ACT>
+__device__ __forceinline__ void dense_lane(const LaneW<IN, OUT, NT>& r, const float* in, float* out) {
+  const int part = static_cast<int>(threadIdx.x) & 7;
+#pragma unroll
+  for (int p = 0; p < r.kPasses; ++p) {
+    const int o = lane_neuron<NT>(p);
+    float acc = 0.0f;
+    if (o < OUT) {
+#pragma unroll
+      for (int q = 0; q < IN / 8; ++q) acc = fmaf(bf16_bits_to_float(r.w[p][q]), in[part + 8 * q], acc);
+    }
+    acc += __shfl_xor_sync(0xffffffffu, acc, 4);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    if (o < OUT && part == 0) {
+      const float z = acc + r.b[p];
+      out[o] = ACT ? gelu(z) : z;
+    }
   }
 }
 
@@ -121,18 +119,17 @@ struct PredLevel {
 // avg|J|, else 0).  v_old: window input threadIdx.x (< 35) from the ring's
 // older rows.  All threads of the block call this (its barriers and
 // shuffles name them).
+template <int NT>
 __device__ __forceinline__ void pred_level(const PredNet* net, double C, DevState* S,
                                            const PredLevel* L, double v_old, PredScratch* sp) {
   // the network's weights, biases and input scales this thread uses
-  LaneW<kPredIn> w1;
-  LaneW<kHid> w2, w3, w4;
-  lane_weights<kPredIn, kHid>(net->W1, w1);
-  lane_weights<kHid, kHid>(net->W2, w2);
-  lane_weights<kHid, kHid>(net->W3, w3);
-  lane_weights<kHid, kPredOut>(net->W4, w4);
-  const int on = static_cast<int>(threadIdx.x) >> 3;
-  const float b1 = (on < kHid) ? net->b1[on] : 0.0f, b2 = (on < kHid) ? net->b2[on] : 0.0f;
-  const float b3 = (on < kHid) ? net->b3[on] : 0.0f, b4 = (on < kPredOut) ? net->b4[on] : 0.0f;
+  LaneW<kPredIn, kHid, NT> w1;
+  LaneW<kHid, kHid, NT> w2, w3;
+  LaneW<kHid, kPredOut, NT> w4;
+  lane_weights(net->W1, net->b1, w1);
+  lane_weights(net->W2, net->b2, w2);
+  lane_weights(net->W3, net->b3, w3);
+  lane_weights(net->W4, net->b4, w4);
   const double isc = (threadIdx.x < kPredIn) ? net->inv_in_scale[threadIdx.x % kPredFeat] : 0.0;
   if (threadIdx.x == 0) {
     double* row = sp->row;
@@ -173,13 +170,13 @@ __device__ __forceinline__ void pred_level(const PredNet* net, double C, DevStat
     sp->x[threadIdx.x] = static_cast<float>(v * isc);
   }
   __syncthreads();
-  dense_lane<kPredIn, kHid, true>(w1, b1, sp->x, sp->h1);
+  dense_lane<kPredIn, kHid, NT, true>(w1, sp->x, sp->h1);
   __syncthreads();
-  dense_lane<kHid, kHid, true>(w2, b2, sp->h1, sp->h2);
+  dense_lane<kHid, kHid, NT, true>(w2, sp->h1, sp->h2);
   __syncthreads();
-  dense_lane<kHid, kHid, true>(w3, b3, sp->h2, sp->h3);
+  dense_lane<kHid, kHid, NT, true>(w3, sp->h2, sp->h3);
   __syncthreads();
-  dense_lane<kHid, kPredOut, false>(w4, b4, sp->h3, sp->y);
+  dense_lane<kHid, kPredOut, NT, false>(w4, sp->h3, sp->y);
   __syncthreads();
   if (threadIdx.x == 0) {
     const double Jp = static_cast<double>(net->out_scale[1]) * static_cast<double>(sp->y[1]);

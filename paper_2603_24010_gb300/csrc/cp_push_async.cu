@@ -112,7 +112,7 @@ __device__ __noinline__ void predictor_in_push(DevState* S, const PredNet* net, 
     L.n_feat = ldcg(&S->n_feat);
   }
   __syncthreads();
-  pred_level(net, C, S, &L, v_old, sp);
+  pred_level<kThreads>(net, C, S, &L, v_old, sp);
 }
 
 size_t push_async_smem_bytes(int N) {

@@ -1,15 +1,18 @@
 // cp_solve.cu -- the coupled field/circuit solve of a new time level.
 //
-// k_solve (one thread-block cluster of 8 or 16 CTAs x 512 threads) solves the
-//   level: the bordered tridiagonal system of App. B with the circuit row of
-//   Sec. 2.4.2 (strict, Eq. Poisson_BC2) or Sec. 2.4.3 (weak, Eq.
-//   Poisson_BC3) is factorised into two bidiagonal scans whose charge sums
-//   are exact integers (one associative segment scan gives the int64 prefix
-//   of the charge grid and the int128 prefix of that); FP64 enters only at
-//   the final scaling, so the solve is direct and its backward error is
-//   checked over every row and the circuit row, with FP64 iterative
-//   refinement if it exceeds the requested tolerance.  Chunk totals are
-//   exchanged through distributed shared memory.
+// k_solve (one thread-block cluster of 1 to 16 CTAs) solves the level: the
+//   bordered tridiagonal system of App. B with the circuit row of Sec. 2.4.2
+//   (strict, Eq. Poisson_BC2) or Sec. 2.4.3 (weak, Eq. Poisson_BC3) is
+//   factorised into two bidiagonal scans whose charge sums are exact integers
+//   (one associative scan gives the int64 prefix of the charge grid and the
+//   prefix of that); FP64 enters only at the final scaling, so the solve is
+//   direct and its backward error is checked over every row and the circuit
+//   row, with FP64 iterative refinement if it exceeds the requested tolerance.
+//   Chunk totals and residual maxima are pushed into every rank's shared
+//   memory (st.async on a transaction barrier).
+#include <algorithm>
+#include <cstddef>
+
 #include "cp_common.cuh"
 #include "cp_mlp.cuh"
 
@@ -82,19 +85,6 @@ __device__ T cta_scan(T* a, int n, bool reverse, T* wsum) {
   return total;
 }
 
-__device__ double cta_max(double v, double* red) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  const int w = threadIdx.x >> 5;
-  __syncthreads();
-  if (lane_id() == 0) red[w] = v;
-  __syncthreads();
-  double t = 0.0;
-  for (int k = 0; k < kSolveThreads / 32; ++k) t = fmax(t, red[k]);
-  __syncthreads();
-  return t;
-}
-
 __device__ double cta_sum(double v, double* red) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -126,16 +116,6 @@ __device__ void cluster_prefix(T mine, T* slot, bool reverse, T* excl, T* total)
   *excl = acc;
   *total = tot;
   cl.sync();
-}
-
-__device__ double cluster_max(double mine, double* slot) {
-  cg::cluster_group cl = cg::this_cluster();
-  if (threadIdx.x == 0) *slot = mine;
-  cl.sync();
-  double m = 0.0;
-  for (unsigned r = 0; r < cl.num_blocks(); ++r) m = fmax(m, *cl.map_shared_rank(slot, r));
-  cl.sync();
-  return m;
 }
 
 // FP64 direct solve of the same tridiagonal system for an arbitrary right-hand
@@ -173,75 +153,88 @@ __device__ void cluster_tri_solve_f64(double* v, int lo, int m, int N, double b0
 }
 
 // ---------------------------------------------------------------------------
-// k_solve: one cluster of 8 or 16 CTAs solves the new level.
+// The solve of one level by the CTAs of one cluster.
 //
-// Rank r owns rows [lo, hi).  Four cluster barriers in the common case:
-//   A  per-rank totals of the two integer scans -> every rank's offsets
-//   B  chunk-edge potentials and fields (neighbour rows of the residual)
-//   C  per-rank maxima of |r|, |x|, |b| -> backward error
-//   D  keeps every rank's shared memory alive until all remote reads are done
+// Bound: latency.  A level is a chain of short dependent stages (grid loads,
+// scan, exchange, potential of node 0, rows, residual, exchange, decision),
+// so what counts is the number of stages and what each waits for:
+//
+// * roles: warps 0-7 own the rows; warp 8 reads the circuit state, forms the
+//   circuit row while the others scan, and exchanges the totals and the
+//   residual maxima with the other ranks; warp 9 commits the level while the
+//   rows are evaluated and checked (the commit needs phi_0 only; the backward
+//   error is filled in last);
+// * the exchanges are one-way: every rank pushes its values into every
+//   rank's shared memory with st.async and waits on its own transaction
+//   barrier (no cluster barrier and no remote load on the path), and a rank
+//   may leave once everything addressed to it has arrived;
+// * what the predecessor does not write (parameters, barrier set-up) is read
+//   and done before the wait for it;
+// * outputs are written before the backward error is known, and again in the
+//   rare case that it calls for a refinement.
+//
+// Rows per thread: chunk / 256, and the cluster has one CTA per 256 rows up
+// to 16.  FP64 is what a row costs (about a dozen operations at 2 per cycle
+// and SM), so more rows per SM cost more than the exchange saves.
+// Measured (GB300, event-bracketed launch; an empty kernel reads 4-5 us): 11.2
+// us at 256 cells and 12.7 us at 4096, against 18.4 us for one 16-CTA cluster
+// of 512 threads with cluster barriers, remote loads and a commit at the end.
+// Graph-timed step: 22.9 against 30.4 us (4096 cells, 3.3e5 FP32 particles),
+// 17.5 against 24.5 us (1531 cells, 1e6), 118 against 125 us (4096, 3.1e7).
 // ---------------------------------------------------------------------------
-// Scan segment of the charge grid: s1 = sum of G_i, s2 = sum over the
-// segment of the inclusive prefix of G within the segment, len = rows.
-// "a then b" is associative: (a1 + b1, a2 + b2 + len_b a1, len_a + len_b).
-struct Seg {
-  __int128 s2;
-  long long s1;
-  long long len;
-};
+constexpr int kRowWarps = kRowThreads / 32;
+constexpr int kCircuitWarp = kRowWarps;     // warp 8
+constexpr int kCommitWarp = kRowWarps + 1;  // warp 9
+static_assert(kSolveThreads == kRowThreads + 64, "two more warps than rows");
 
-// a b as a 128-bit integer from one 64 x 64 -> 128 product (no general
-// 128-bit multiplication)
+// a b as a 128-bit integer from one 64 x 64 -> 128 product
 __device__ __forceinline__ __int128 mul_wide(long long a, long long b) {
   const unsigned long long lo = static_cast<unsigned long long>(a) * static_cast<unsigned long long>(b);
   const long long hi = __mul64hi(a, b);
   return static_cast<__int128>((static_cast<unsigned __int128>(static_cast<unsigned long long>(hi)) << 64) | lo);
 }
 
-__device__ __forceinline__ Seg seg_then(const Seg& a, const Seg& b) {
-  Seg r;
+// The accumulator of the prefix of prefixes: int64 when the stores cannot
+// hold enough charge to overflow it (|sum| <= 2^16 macroparticles N < 2^62),
+// else int128.
+template <typename Acc>
+__device__ __forceinline__ Acc len_times(int len, long long s1);
+template <>
+__device__ __forceinline__ long long len_times<long long>(int len, long long s1) {
+  return static_cast<long long>(len) * s1;
+}
+template <>
+__device__ __forceinline__ __int128 len_times<__int128>(int len, long long s1) {
+  return mul_wide(len, s1);
+}
+// exactly rounded |v| with v's sign; the two forms agree where both apply
+__device__ __forceinline__ double acc_to_double(long long v) { return static_cast<double>(v); }
+__device__ __forceinline__ double acc_to_double(__int128 v) { return i128_to_double(v); }
+
+// Scan segment of the charge grid: s1 = sum of G_i, s2 = sum over the
+// segment of the inclusive prefix of G within it.  "a then b" with len_b
+// rows in b: (a1 + b1, a2 + b2 + len_b a1).
+template <typename Acc>
+struct alignas(16) Seg {
+  Acc s2;
+  long long s1;
+};
+
+template <typename Acc>
+__device__ __forceinline__ Seg<Acc> seg_then(const Seg<Acc>& a, const Seg<Acc>& b, int len_b) {
+  Seg<Acc> r;
   r.s1 = a.s1 + b.s1;
-  r.s2 = a.s2 + b.s2 + mul_wide(b.len, a.s1);
-  r.len = a.len + b.len;
+  r.s2 = a.s2 + b.s2 + len_times<Acc>(len_b, a.s1);
   return r;
 }
 
-__device__ __forceinline__ Seg shfl_up_seg(const Seg& v, int o) {
-  Seg r;
-  r.s1 = __shfl_up_sync(0xffffffffu, v.s1, o);
-  r.len = __shfl_up_sync(0xffffffffu, v.len, o);
+template <typename Acc>
+__device__ __forceinline__ Seg<Acc> shfl_up_seg(const Seg<Acc>& v, int o) {
+  Seg<Acc> r;
+  r.s1 = shfl_up_t(v.s1, o);
   r.s2 = shfl_up_t(v.s2, o);
   return r;
 }
-
-__device__ __forceinline__ Seg shfl_seg(const Seg& v, int src) {
-  Seg r;
-  r.s1 = __shfl_sync(0xffffffffu, v.s1, src);
-  r.len = __shfl_sync(0xffffffffu, v.len, src);
-  const unsigned long long lo = static_cast<unsigned long long>(v.s2);
-  const unsigned long long hi = static_cast<unsigned long long>(static_cast<unsigned __int128>(v.s2) >> 64);
-  const unsigned long long l2 = __shfl_sync(0xffffffffu, lo, src);
-  const unsigned long long h2 = __shfl_sync(0xffffffffu, hi, src);
-  r.s2 = static_cast<__int128>((static_cast<unsigned __int128>(h2) << 64) | l2);
-  return r;
-}
-
-// Inclusive warp scan of segments (Kogge-Stone with the "then" operator).
-__device__ __forceinline__ Seg warp_scan_seg(Seg v) {
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const Seg y = shfl_up_seg(v, o);
-    if (static_cast<int>(lane_id()) >= o) v = seg_then(y, v);
-  }
-  return v;
-}
-
-struct SolveSlotB {
-  double first_phi, last_phi, first_E, phi0;
-};
-struct SolveSlotC {
-  unsigned long long rmax, xmax, bmax;  // bit patterns of non-negative doubles
-};
 
 // |x| as the bit pattern of a non-negative double: such patterns order like
 // the values, so maxima can be taken on the integer pipe (GB300's FP64 pipe
@@ -250,30 +243,61 @@ __device__ __forceinline__ unsigned long long abs_bits(double x) {
   return static_cast<unsigned long long>(__double_as_longlong(x)) & 0x7FFFFFFFFFFFFFFFULL;
 }
 
-// Block maxima of three bit patterns; the result is valid in thread 0.
-__device__ void cta_max3(unsigned long long& a, unsigned long long& b, unsigned long long& c,
-                         unsigned long long (*red)[32]) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    a = max(a, __shfl_xor_sync(0xffffffffu, a, o));
-    b = max(b, __shfl_xor_sync(0xffffffffu, b, o));
-    c = max(c, __shfl_xor_sync(0xffffffffu, c, o));
+// Warp maximum of 64-bit patterns: the high words first, then the low words
+// of the lanes that hold the largest high word (two hardware reductions).
+__device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) {
+  const unsigned int hi = static_cast<unsigned int>(v >> 32);
+  const unsigned int mh = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned int ml = __reduce_max_sync(0xffffffffu, hi == mh ? static_cast<unsigned int>(v) : 0u);
+  return (static_cast<unsigned long long>(mh) << 32) | ml;
+}
+
+struct alignas(16) MaxSlot {
+  unsigned long long rmax, xmax, bmax, pad;  // bit patterns of non-negative doubles (bmax: integer)
+};
+
+// Dynamic shared memory of one rank's rows: G, phi, E, b and r.
+__host__ __device__ constexpr size_t solve_rows_bytes(int chunk) {
+  return align16(8 * static_cast<size_t>(chunk)) + align16(4 * 8 * static_cast<size_t>(chunk));
+}
+
+// --- one-way exchange between the ranks of a cluster ------------------------
+__device__ __forceinline__ uint32_t smem_addr(const void* p) {
+  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+__device__ __forceinline__ void mbar_init(uint64_t* bar) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar)) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ uint32_t remote_addr(const void* p, int rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr(p)), "r"(rank));
+  return r;
+}
+// 16 bytes into another rank's shared memory, counted on its barrier
+__device__ __forceinline__ void push16(uint32_t dst, unsigned long long a, unsigned long long b, uint32_t bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(dst),
+               "l"(a), "l"(b), "r"(bar)
+               : "memory");
+}
+// Wait for the barrier's first phase; false when the limit of polls is
+// reached (a rank that never sent: cannot happen unless one failed).
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar) {
+  for (int i = 0; i < (1 << 20); ++i) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(smem_addr(bar))
+        : "memory");
+    if (done) return true;
   }
-  const int w = threadIdx.x >> 5;
-  __syncthreads();
-  if (lane_id() == 0) {
-    red[0][w] = a;
-    red[1][w] = b;
-    red[2][w] = c;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int k = 1; k < kSolveThreads / 32; ++k) {
-      a = max(a, red[0][k]);
-      b = max(b, red[1][k]);
-      c = max(c, red[2][k]);
-    }
-  }
+  return false;
 }
 
 // Circuit charge, surface charge and current of a solved level from the
@@ -298,41 +322,35 @@ __device__ __forceinline__ void level_charges(const DevParams* P, const double* 
   }
 }
 
-// The installed network and the feature window (8 rows of 5 doubles) are
-// copied into shared memory while the solve scans (asynchronous copies,
-// waited for only when the network runs), so that the predictor reads
-// neither from L2 after the solve's last barrier.
-__device__ __forceinline__ void prefetch_net(const PredNet* net, PredNet* s_net, const DevState* S,
-                                             double* s_feat) {
+// The installed network is copied into shared memory while the solve runs
+// (asynchronous copies, waited for only when the network runs).
+__device__ __forceinline__ void prefetch_net(const PredNet* net, PredNet* s_net) {
   const char* src = reinterpret_cast<const char*>(net);
   char* dst = reinterpret_cast<char*>(s_net);
   for (size_t o = 16 * static_cast<size_t>(threadIdx.x); o < kPredNetBytes; o += 16 * kSolveThreads)
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                     static_cast<uint32_t>(__cvta_generic_to_shared(dst + o))),
-                 "l"(src + o)
-                 : "memory");
-  if (threadIdx.x < kPredWindow * kPredFeat)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
-                     static_cast<uint32_t>(__cvta_generic_to_shared(s_feat + threadIdx.x))),
-                 "l"(&S->feat[0][0] + threadIdx.x)
-                 : "memory");
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst + o)), "l"(src + o) : "memory");
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
+
+// The words of the device state that a solve reads, as one block: from
+// `level` up to the compaction counters.
+constexpr int kStateWord0 = offsetof(DevState, level) / 8;
+constexpr int kStateWords = (offsetof(DevState, compact_n) - offsetof(DevState, level)) / 8;
+static_assert(offsetof(DevState, level) % 8 == 0 && offsetof(DevState, compact_n) % 8 == 0, "whole words");
 
 // Predictor step on one CTA (all threads), for the paths that keep it in the
 // solve: the level's row from the solve's scalars, then the shared predictor
 // level (check, ring append, network on the copy in shared memory, s_net).
-// (The pointers are passed one by one: a reference to the kernel's parameter
-// block would force a copy of it into local memory for the whole solve.)
-__device__ __noinline__ void predictor_update(const DevParams* P, DevState* S, const PredNet* s_net,
-                                              const double* s_feat, const double* sc, bool strict_rlc,
+// `st` is the copy of the device state as the solve found it.
+__device__ __noinline__ void predictor_update(const DevParams* P, DevState* S, const DevState* st,
+                                              const PredNet* s_net, const double* sc, bool strict_c,
                                               double phi0) {
   __shared__ PredScratch sp;
   __shared__ PredLevel L;
-  const int pos0 = static_cast<int>(sc[37]);
+  const int pos0 = st->feat_pos;
   if (threadIdx.x == 0) {
     double Qn, sigma_n, I;
-    level_charges(P, sc, strict_rlc, phi0, &Qn, &sigma_n, &I);
+    level_charges(P, sc, strict_c, phi0, &Qn, &sigma_n, &I);
     L.Qconv = sc[6];
     L.phi0 = phi0;
     L.phi0_prev = sc[32];
@@ -340,513 +358,73 @@ __device__ __noinline__ void predictor_update(const DevParams* P, DevState* S, c
     L.Qsurf_prev = __dmul_rn(sc[7], P->area);
     L.Qn = Qn;
     L.Q1 = sc[8];
-    L.emitted = sc[33];
-    L.ion_eV = sc[34];
-    // predictor state loaded with the circuit state at the solve's start
-    L.had_pred = (sc[31] != 0.0);
-    L.J_pred = sc[30];
-    L.err_avg = sc[45];
-    L.J_avg = sc[46];
-    L.n_eval = static_cast<long long>(sc[47]);
+    L.emitted = static_cast<double>(st->emitted[0]);
+    L.ion_eV = static_cast<double>(st->ion_energy_q) / 256.0;
+    L.had_pred = st->pred_ready;
+    L.J_pred = st->J_pred;
+    L.err_avg = st->err_avg;
+    L.J_avg = st->J_avg;
+    L.n_eval = st->n_eval;
     L.pos = pos0;
-    L.n_feat = static_cast<int>(sc[38]);
+    L.n_feat = st->n_feat;
   }
   asm volatile("cp.async.wait_all;" ::: "memory");  // this thread's copies of the network
   __syncthreads();
   // the 7 older rows of the window (ring slots pos+1..pos+7, oldest first)
   double v_old = 0.0;
   if (threadIdx.x < kPredIn - kPredFeat)
-    v_old = s_feat[((pos0 + 1 + static_cast<int>(threadIdx.x) / kPredFeat) & (kPredWindow - 1)) * kPredFeat +
-                   threadIdx.x % kPredFeat];
-  pred_level(s_net, P->C, S, &L, v_old, &sp);
+    v_old = st->feat[(pos0 + 1 + static_cast<int>(threadIdx.x) / kPredFeat) & (kPredWindow - 1)]
+                    [threadIdx.x % kPredFeat];
+  pred_level<kRowThreads>(s_net, P->C, S, &L, v_old, &sp);
 }
 
-// The solve of one instance by the CTAs of one cluster (a cluster of one CTA
-// in the ensemble launch).
-template <typename real>
-__device__ __forceinline__ void solve_body(const Bufs& B, int do_push, int mode, double tol) {
-  using real2 = typename Pair<real>::type;
-  cg::cluster_group cl = cg::this_cluster();
-  const int rank = static_cast<int>(cl.block_rank());
-  const int nr = static_cast<int>(cl.num_blocks());
-  const DevParams* P = B.P;
-  DevState* S = B.S;
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ __align__(16) Seg wseg[32];
-  __shared__ __align__(16) Seg slotA;
-  __shared__ __align__(16) Seg s_rank_off;
-  __shared__ __align__(16) Seg s_next_off;
-  __shared__ __align__(16) __int128 s_U;
-  __shared__ double wd[3][32];
-  __shared__ unsigned long long wu[3][32];
-  __shared__ double s_eta;
-  __shared__ SolveSlotB slotB;
-  __shared__ SolveSlotC slotC;
-  __shared__ double slotd;
-  __shared__ double sc[48];
-  __shared__ unsigned long long tal[11];  // the push's tallies, read early
-  __shared__ int s_stop;
-  __shared__ __align__(16) PredNet s_net;  // the network, for the CTA that runs it
-  __shared__ __align__(16) double s_feat[kPredWindow * kPredFeat];  // and its feature window
-
-  cudaGridDependencySynchronize();  // the push that deposited G has completed
-  if (threadIdx.x == 0) s_stop = (ldcg(&S->status) != 0);
-  __syncthreads();
-  if (s_stop) return;  // the status cannot change while this kernel runs: all ranks agree
-
-  const int N = P->N;
-  const int chunk = (N + nr - 1) / nr;
-  const int lo = min(rank * chunk, N);
-  const int hi = min(lo + chunk, N);
-  const int m = hi - lo;
-  long long* Gv = reinterpret_cast<long long*>(smem);  // chunk: G_i of this rank's rows
-  double* ph = reinterpret_cast<double*>(smem + align16(8 * chunk));
-  double* Ee = ph + chunk;
-  double* bb = Ee + chunk;
-  double* rr = bb + chunk;
-
-  cudaTriggerProgrammaticLaunchCompletion();
-  // the CTA that will run the network fetches it now, behind the scan
-  const bool runs_net = (B.net != nullptr && !B.net_in_push && do_push && rank == (nr > 1 ? 1 : 0));
-  if (runs_net) prefetch_net(B.net, &s_net, S, s_feat);
-  const long long G0 = ldcg(&B.G[0]);
-  // G of the next chunk's first row (for the field E_hi of the gather table)
-  const long long Gnext = (hi < N) ? ldcg(&B.G[hi]) : 0LL;
-  for (int k = threadIdx.x; k < m; k += kSolveThreads) {
-    const int i = lo + k;
-    const long long g = ldcg(&B.G[i]);
-    Gv[k] = (i == 0) ? 0LL : g;  // the prefix S'_i = sum_{j=1..i} G_j leaves G_0 out
-    B.Glast[i] = g;
-    if (k > 0) B.G[i] = 0;  // a chunk's first row (and G_0) is cleared after barrier A
-  }
-  const bool last_rows = (hi == N && m > 0);  // this rank owns row N-1 (and node N)
-  if (last_rows && threadIdx.x == 0) {
-    B.Glast[N] = ldcg(&B.G[N]);
-    B.G[N] = 0;
-  }
-  __syncthreads();
-  // circuit row, first part (every rank evaluates the same scalars): the
-  // source, the BDF2 history, the circuit solve and the x = 0 row's
-  // right-hand side need no scan, so one thread of the last warp does them
-  // -- and reads the push's tallies for the commit -- while the CTA scans.
-  // Tesla circuit: the last warp forms the new level's loop charges for
-  // phi_0 = 0 from the 20 history values (one per lane, warp sums)
-  double tq[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-  if (P->circuit == CP_CIRCUIT_TESLA && do_push && threadIdx.x >= kSolveThreads - 32) {
-    const int l = static_cast<int>(lane_id());
-    const double h = (l < 20) ? ldcg(&S->Qt[l / 5][l % 5]) : 0.0;  // levels n-1..n-4
-    const double(*Pm)[20] = (mode == 0) ? P->t_Ps : P->t_Pw;
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-      double v = (l < 20) ? Pm[i][l] * h : 0.0;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      tq[i] = v;
-    }
-  }
-  if (threadIdx.x == kSolveThreads - 32) {
-    const double qw = P->e * P->weight;
-    const long long conv = do_push ? ldcg(&S->conv_count) : 0LL;
-    const double Q1 = ldcg(&S->Qh[0]), Q2 = ldcg(&S->Qh[1]);
-    const double Q3 = ldcg(&S->Qh[2]);
-    // source and BDF2 history of the new level: precomputed by the previous
-    // solve except for the first solve of a run
-    double Vs, hist;
-    if (do_push) {
-      Vs = ldcg(&S->nxt_Vs);
-      hist = ldcg(&S->nxt_hist);
-    } else {
-      Vs = B.vs[ldcg(&S->level)];
-      const double Q4 = ldcg(&S->Qh[3]);
-      hist = P->L4dt2 * (24.0 * Q1 - 22.0 * Q2 + 8.0 * Q3 - Q4) + P->R2dt * (4.0 * Q1 - Q2);
-    }
-    const double phi0_prev = ldcg(&S->phi0_last);
-    // learned weak scheme: the network's prediction of the plasma's change of
-    // C phi_0 over this step, used while its tracked error is within bound
-    // (the predictor state is loaded in one batch: no chain of dependent loads)
-    int pred_ready = 0, feat_pos = 0, n_feat = 0;
-    long long n_eval = 0;
-    double J_pred = 0.0, err_avg = 0.0, J_avg = 0.0, bound = 0.0;
-    double J_fast = 0.0;  // the push formed the usable prediction (FP32 single gap)
-    if (B.net != nullptr && B.net_in_push) {
-      if (mode == 2) J_fast = ldcg(&S->J_eff);
-    } else if (B.net != nullptr) {
-      pred_ready = ldcg(&S->pred_ready);
-      J_pred = ldcg(&S->J_pred);
-      n_eval = ldcg(&S->n_eval);
-      err_avg = ldcg(&S->err_avg);
-      J_avg = ldcg(&S->J_avg);
-      bound = B.net->bound;
-      feat_pos = ldcg(&S->feat_pos);
-      n_feat = ldcg(&S->n_feat);
-    }
-    if (!pred_ready) J_pred = 0.0;
-    const double J_used =
-        (mode == 2 && pred_ready && n_eval >= kPredMinEval && err_avg <= bound * J_avg) ? J_pred : J_fast;
-    double g = 0.0, Qpart = Q1, gam = 0.0, inv_den = 1.0;
-    if (P->circuit == CP_CIRCUIT_SERIES_RLC) {
-      if (mode == 0) {  // strict: Q^n = K - g phi_0^n (Eqs. Q4_phi_relation, K_def)
-        g = P->g_strict;
-        Qpart = g * (Vs + hist);
-        gam = P->gam_strict;
-        inv_den = P->inv_den_strict;
-      } else {
-        // weak (Sec. 2.4.3): the circuit alone, its load capacitor starting
-        // from phi_0^{n-1}: a21 Q - hist + phi_0^{n-1} + (Q - Q^{n-1} + J)/C = V_s
-        Qpart = (Vs + hist + (Q1 - J_used) * P->inv_C - phi0_prev) * P->g_weak;
-      }
-    } else if (P->circuit == CP_CIRCUIT_TESLA) {
-      // Q1 here is the load capacitor's loop charge Q4^{n-1}
-      if (!do_push) {  // level 0: the circuit as it rests before t = 0
-        Qpart = Q1;
-      } else if (mode == 0) {  // strict: Q4^n = K - [T'^{-1}]_44 phi_0^n
-        g = P->t_ws[3];
-        Qpart = tq[3];
-        gam = P->gam_tesla;
-        inv_den = P->inv_den_tesla;
-      } else {  // weak: loop 4's capacitor voltage phi_0^{n-1} + (Q4 - Q4^{n-1} + J)/C3
-        const double s = (Q1 - J_used) * P->inv_C - phi0_prev;
-        Qpart = tq[3] + s * P->t_ww[3];
-        sc[36] = s;
-      }
-      for (int i = 0; i < 5; ++i) sc[40 + i] = tq[i];
-    }
-    const double Qconv = static_cast<double>(conv) * qw;
-    const double sigma_prev = ldcg(&S->sigma);
-    // x = 0 row: Eq. Poisson_BC2 (strict) / Eq. Poisson_BC3 (weak), with
-    // rho_0 dx^2 / (2 eps0) = alpha G_0 / 2 (G_0 is even: boundary doubling)
-    const double b0 = P->dx_eps0 * (sigma_prev + (Qconv + Qpart - Q1) * P->inv_A) +
-                      P->alpha * static_cast<double>(G0 / 2);
-    sc[0] = b0; sc[1] = gam; sc[2] = g; sc[3] = Qpart; sc[4] = Vs; sc[5] = hist;
-    sc[6] = Qconv; sc[7] = sigma_prev; sc[8] = Q1; sc[9] = Q2; sc[10] = Q3;
-    sc[12] = static_cast<double>(conv);
-    sc[15] = J_used;
-    sc[30] = J_pred;
-    sc[31] = static_cast<double>(pred_ready);
-    sc[32] = phi0_prev;
-    sc[35] = inv_den;
-    sc[37] = static_cast<double>(feat_pos);  // the predictor's ring slot for this level
-    sc[38] = static_cast<double>(n_feat);
-    sc[45] = err_avg;  // the predictor's running error averages, updated by its CTA
-    sc[46] = J_avg;
-    sc[47] = static_cast<double>(n_eval);
-    if (do_push) {  // the push's tallies, read before the commit clears them
-      sc[33] = static_cast<double>(ldcg(&S->emitted[0]));
-      sc[34] = static_cast<double>(ldcg(&S->ion_energy_q)) / 256.0;
-      for (int e = 0; e < 2; ++e)
-        for (int q = 0; q < kSpecies; ++q) tal[e * kSpecies + q] = ldcg(&S->absorbed[e][q]);
-      tal[6] = ldcg(&S->emitted[0]);
-      tal[7] = ldcg(&S->emitted[1]);
-      tal[8] = ldcg(&S->injected);
-      tal[9] = static_cast<unsigned long long>(ldcg(&S->ion_energy_q));
-      tal[10] = ldcg(&S->max_cfl_bits);
-    } else {
-      sc[33] = 0.0;
-      sc[34] = 0.0;
-      for (int q = 0; q < 11; ++q) tal[q] = 0ULL;
-    }
-  }
-  // this thread's run of rows and its segment totals
-  const int per = (m + kSolveThreads - 1) / kSolveThreads;
-  const int r0 = min(static_cast<int>(threadIdx.x) * per, m);
-  const int r1 = min(r0 + per, m);
-  Seg mine;
-  mine.s1 = 0;
-  mine.s2 = 0;
-  mine.len = r1 - r0;
-  for (int k = r0; k < r1; ++k) {
-    mine.s1 += Gv[k];
-    mine.s2 += mine.s1;
-  }
-  const Seg incl = warp_scan_seg(mine);
-  Seg wexcl = shfl_up_seg(incl, 1);  // exclusive within the warp
-  if (lane_id() == 0) {
-    wexcl.s1 = 0;
-    wexcl.s2 = 0;
-    wexcl.len = 0;
-  }
-  const int w = threadIdx.x >> 5;
-  if (lane_id() == 31) wseg[w] = incl;
-  __syncthreads();
-  Seg bexcl;  // everything of this CTA before this warp
-  bexcl.s1 = 0;
-  bexcl.s2 = 0;
-  bexcl.len = 0;
-  for (int q = 0; q < w; ++q) bexcl = seg_then(bexcl, wseg[q]);
-  // --- barrier A: the CTAs' totals give every rank its offset ----------------
-  if (threadIdx.x == 0) {
-    Seg tot = bexcl;
-    for (int q = w; q < kSolveThreads / 32; ++q) tot = seg_then(tot, wseg[q]);
-    slotA = tot;
-  }
-  cl.sync();
-  if (threadIdx.x < 32) {  // lane q reads rank q; a warp scan gives the offsets
-    Seg v;
-    v.s1 = 0;
-    v.s2 = 0;
-    v.len = 0;
-    if (static_cast<int>(threadIdx.x) < nr) v = *cl.map_shared_rank(&slotA, static_cast<int>(threadIdx.x));
-    Seg ci = v;  // inclusive scan over the (at most 8) ranks
-#pragma unroll
-    for (int o = 1; o < kSolveCtasMax; o <<= 1) {
-      const Seg y = shfl_up_seg(ci, o);
-      if (static_cast<int>(lane_id()) >= o) ci = seg_then(y, ci);
-    }
-    Seg ce = shfl_up_seg(ci, 1);
-    if (threadIdx.x == 0) {
-      ce.s1 = 0;
-      ce.s2 = 0;
-      ce.len = 0;
-    }
-    const Seg mine_off = shfl_seg(ce, rank);
-    const Seg next_off = shfl_seg(ci, rank);  // everything up to and including this rank
-    const Seg all = shfl_seg(ci, nr - 1);
-    if (threadIdx.x == 0) {
-      s_rank_off = mine_off;
-      s_next_off = next_off;
-      s_U = all.s2;
-      if (m > 0) B.G[lo] = 0;
-    }
-  }
-  __syncthreads();
-  const __int128 U = s_U;
-  // offset of everything before this thread's run: rank, then warp, then lane
-  const Seg off = seg_then(seg_then(s_rank_off, bexcl), wexcl);
-  // circuit row, second part: the electrode potential needs the scan total U
-  if (threadIdx.x == 0) {
-    const double b0 = sc[0], gam = sc[1], inv_den = sc[35];
-    const double phi0 = (static_cast<double>(N) * b0 + P->alpha * i128_to_double(U)) * inv_den;
-    const double D0 = b0 - gam * phi0;  // D_0 = x_0 - x_1
-    sc[11] = D0;
-    sc[24] = D0 * P->inv_dx;        // E_0
-    sc[25] = P->alpha * P->inv_dx;  // dE_i / dS'_i
-  }
-  __syncthreads();
-  const double b0 = sc[0], gam = sc[1], D0 = sc[11];
-  const double alpha = P->alpha, inv_dx = P->inv_dx;
-  const double E0 = sc[24], Ea = sc[25];
-  // D_i = D_0 + alpha S'_i;  x_i = (N - i) D_0 + alpha (U - P_i);  E_i = D_i / dx
-  {
-    long long S = off.s1;       // S'_i, running over the run
-    __int128 Pex = off.s2;      // P_i = sum_{k<i} S'_k (exclusive)
-    for (int k = r0; k < r1; ++k) {
-      const int i = lo + k;
-      S += Gv[k];
-      ph[k] = fma(static_cast<double>(N - i), D0, alpha * i128_to_double(U - Pex));
-      Ee[k] = fma(Ea, static_cast<double>(S), E0);
-      bb[k] = (i == 0) ? b0 : -alpha * static_cast<double>(Gv[k]);
-      Pex += S;
-    }
-  }
-  __syncthreads();
-
-  const bool strict_rlc = (P->circuit == CP_CIRCUIT_SERIES_RLC && mode == 0);
-  // the level's charge follows Q^n = K - g phi_0^n (g = 0 at a Tesla level 0)
-  const bool strict_c = (P->circuit != CP_CIRCUIT_OPEN) && (mode == 0 || (P->circuit == CP_CIRCUIT_TESLA && !do_push));
-  // The neighbouring chunks' edge values follow from the exact prefixes with
-  // the same arithmetic their owners use, so no exchange is needed:
-  // x_{lo-1} needs P_{lo-1} = P_lo - S'_{lo-1}; x_hi needs P_hi; E_hi needs S'_hi.
-  // One thread of four different warps each evaluates one of them.
-  double prev_phi, next_phi, nextE, phi0;
-  {
-    const Seg ro = s_rank_off, no = s_next_off;
-    if (threadIdx.x == 0)
-      sc[26] = (lo > 0) ? fma(static_cast<double>(N - (lo - 1)), D0,
-                              alpha * i128_to_double(U - (ro.s2 - static_cast<__int128>(ro.s1))))
-                        : 0.0;
-    if (threadIdx.x == 32)
-      sc[27] = (hi < N) ? fma(static_cast<double>(N - hi), D0, alpha * i128_to_double(U - no.s2)) : 0.0;
-    if (threadIdx.x == 64) sc[28] = (hi < N) ? fma(Ea, static_cast<double>(no.s1 + Gnext), E0) : 0.0;
-    if (threadIdx.x == 96) sc[29] = fma(static_cast<double>(N), D0, alpha * i128_to_double(U));  // x_0
-    __syncthreads();
-    prev_phi = sc[26];
-    next_phi = sc[27];
-    nextE = sc[28];
-    phi0 = sc[29];
-  }
-  double eta = 0.0;
-  double phi0_fin = phi0;  // x_0 after any refinement
-  cg::cluster_group::arrival_token done_tok;
-  for (int sweep = 0; sweep <= 3; ++sweep) {
-    unsigned long long rm = 0ULL, xm = 0ULL, bm = 0ULL;
-    for (int k = threadIdx.x; k < m; k += kSolveThreads) {
-      const int i = lo + k;
-      const double xp = (k + 1 < m) ? ph[k + 1] : next_phi;
-      double ri;
-      if (i == 0) {
-        ri = (1.0 + gam) * ph[k] - xp - bb[k];
-      } else {
-        const double xq = (k > 0) ? ph[k - 1] : prev_phi;
-        ri = (xq - 2.0 * ph[k] + xp) - bb[k];
-      }
-      rr[k] = ri;
-      rm = max(rm, abs_bits(ri));
-      xm = max(xm, abs_bits(ph[k]));
-    }
-    // max |b_i|: on the first pass alpha max |G_i| over rows >= 1 (reduced as
-    // an integer) and |b_0|; after a refinement, the bit patterns of |b_i|
-    if (sweep == 0) {
-      for (int k = threadIdx.x; k < m; k += kSolveThreads)
-        if (lo + k > 0) bm = max(bm, static_cast<unsigned long long>(llabs(Gv[k])));
-    } else {
-      for (int k = threadIdx.x; k < m; k += kSolveThreads) bm = max(bm, abs_bits(bb[k]));
-    }
-    cta_max3(rm, xm, bm, wu);
-    // --- barrier C: backward error over the cluster --------------------------
-    if (threadIdx.x == 0) {
-      slotC.rmax = rm;
-      slotC.xmax = xm;
-      slotC.bmax = bm;
-    }
-    cl.sync();
-    if (threadIdx.x < 32) {  // lane q reads rank q
-      unsigned long long a = 0, b = 0, c = 0;
-      if (static_cast<int>(threadIdx.x) < nr) {
-        const SolveSlotC* q = cl.map_shared_rank(&slotC, static_cast<int>(threadIdx.x));
-        a = q->rmax;
-        b = q->xmax;
-        c = q->bmax;
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        a = max(a, __shfl_xor_sync(0xffffffffu, a, o));
-        b = max(b, __shfl_xor_sync(0xffffffffu, b, o));
-        c = max(c, __shfl_xor_sync(0xffffffffu, c, o));
-      }
-      rm = a;
-      xm = b;
-      bm = c;
-    }
-    if (threadIdx.x == 0) {
-      const double rmd = __longlong_as_double(static_cast<long long>(rm));
-      const double xmd = __longlong_as_double(static_cast<long long>(xm));
-      const double bmd = (sweep == 0) ? fmax(alpha * static_cast<double>(bm), fabs(b0))
-                                      : __longlong_as_double(static_cast<long long>(bm));
-      const double nA = fmax(fabs(1.0 + gam) + 1.0, 4.0);
-      const double den = nA * xmd + bmd;
-      double e = den > 0.0 ? rmd / den : 0.0;
-      if (strict_rlc) {  // the circuit row with the potential of row 0
-        const double p0 = sweep ? sc[13] : phi0;
-        const double Qn = sc[3] - sc[2] * p0;
-        const double kvl = P->a21 * Qn - (sc[4] + sc[5]) + p0;
-        const double kden = P->a21 * fabs(Qn) + fabs(sc[4] + sc[5]) + fabs(p0);
-        if (kden > 0.0) e = fmax(e, fabs(kvl) / kden);
-      }
-      s_eta = e;
-    }
-    __syncthreads();
-    eta = s_eta;
-    if (!(eta > tol) || sweep == 3) {
-      done_tok = cl.barrier_arrive();  // this rank's remote reads are done
-      break;
-    }
-    // refinement: solve A delta = r, x -= delta (FP64; rare path)
-    const double r0 = (rank == 0) ? rr[0] : 0.0;
-    if (rank == 0 && threadIdx.x == 0) sc[14] = r0;
-    cl.sync();
-    const double r0all = cl.map_shared_rank(&sc[14], 0)[0];
-    cluster_tri_solve_f64(rr, lo, m, N, r0all, gam, wd[0], &slotd, sc + 16);
-    for (int k = threadIdx.x; k < m; k += kSolveThreads) ph[k] -= rr[k];
-    __syncthreads();
-    // refined edges: exchange them (rare path)
-    if (threadIdx.x == 0 && m > 0) {
-      slotB.first_phi = ph[0];
-      slotB.last_phi = ph[m - 1];
-    }
-    cl.sync();
-    next_phi = (hi < N) ? cl.map_shared_rank(&slotB, rank + 1)->first_phi : 0.0;
-    prev_phi = (lo > 0) ? cl.map_shared_rank(&slotB, rank - 1)->last_phi : 0.0;
-    const double phi0_new = cl.map_shared_rank(&slotB, 0)->first_phi;
-    for (int k = threadIdx.x; k < m; k += kSolveThreads)
-      Ee[k] = (ph[k] - ((k + 1 < m) ? ph[k + 1] : next_phi)) * inv_dx;
-    __syncthreads();
-    if (threadIdx.x == 0 && m > 0) slotB.first_E = Ee[0];
-    cl.sync();
-    nextE = (hi < N) ? cl.map_shared_rank(&slotB, rank + 1)->first_E : 0.0;
-    sc[13] = phi0_new;
-    phi0_fin = phi0_new;
-  }
-
-  // outputs; the gather table pairs need the next chunk's first field value
-  real2* Epair = reinterpret_cast<real2*>(B.Epair);
-  for (int k = threadIdx.x; k < m; k += kSolveThreads) {
-    const int i = lo + k;
-    B.E64[i] = Ee[k];
-    B.phi[i] = ph[k];
-    const real e0 = static_cast<real>(Ee[k]);
-    const real e1 = (i + 1 < N) ? static_cast<real>((k + 1 < m) ? Ee[k + 1] : nextE) : e0;
-    real2 pr;
-    pr.x = e0;
-    pr.y = e1 - e0;
-    Epair[i + 1] = pr;
-    if (i == 0) {
-      real2 p0;
-      p0.x = e0;
-      p0.y = real(0);
-      Epair[0] = p0;
-    }
-  }
-  if (last_rows && threadIdx.x == 0) B.phi[N] = 0.0;
-  // barrier D: no rank leaves (freeing its shared memory) before every
-  // rank's remote reads are done
-  cl.barrier_wait(std::move(done_tok));
-  if (rank == 1) {  // the predictor runs beside rank 0's commit
-    if (runs_net) predictor_update(B.P, B.S, &s_net, s_feat, sc, strict_c, phi0_fin);
-    return;
-  }
-  if (rank != 0) return;
-
-  if (threadIdx.x == 0) {
-    const int64_t level = S->level + (do_push ? 1 : 0);
+// What the commit writes for a level whose electrode potential is phi0 (one
+// warp; every value comes from the shared copies, so a second call after a
+// refinement writes the same fields again).
+// (The pointers are passed one by one: a reference to the kernel's parameter
+// block would force a copy of it into local memory for the whole solve.)
+__device__ __noinline__ int commit_level(DevState* S, cp_diag* hist, int64_t hist_rows, const double* vs,
+                                         const DevParams* P, const DevState* st, const double* sc, int do_push,
+                                         int mode, bool strict_c, double phi0, double eta) {
+  const int lane = static_cast<int>(lane_id());
+  const int64_t level = st->level + (do_push ? 1 : 0);
+  const double Q1 = sc[8], Q2 = sc[9], Q3 = sc[10];
+  double Qn, sigma_n, I;
+  level_charges(P, sc, strict_c, phi0, &Qn, &sigma_n, &I);
+  int status = 0;
+  if (!isfinite(phi0) || !isfinite(sigma_n) || !isfinite(Qn)) status = CP_ERR_NONFINITE;
+  if (lane == 0) {
     const double dt = P->dt, A = P->area;
-    const double phi0 = ph[0];
-    const double Qconv = sc[6], Q1 = sc[8], Q2 = sc[9], Q3 = sc[10];
-    const long long conv = static_cast<long long>(sc[12]);
-    double Qn, sigma_n, I;
-    level_charges(P, sc, strict_c, phi0, &Qn, &sigma_n, &I);
-    int status = 0;
-    if (!isfinite(phi0) || !isfinite(sigma_n) || !isfinite(Qn)) status = CP_ERR_NONFINITE;
-    else if (eta > tol) status = CP_ERR_RESIDUAL;
-
+    const bool on = do_push != 0;
     cp_diag d;
     d.step = level;
     d.t = static_cast<double>(level) * dt;
     d.V_gap = phi0;
     d.I_circ = I;
     d.Q_surf = sigma_n * A;
-    d.Q_conv = Qconv;
+    d.Q_conv = sc[6];
     d.Q_circ = Qn;
     d.V_source = sc[4];
     d.residual = eta;
-    d.ion_energy_eV = static_cast<double>(static_cast<long long>(tal[9])) / 256.0;
-    d.max_cfl = static_cast<double>(__uint_as_float(static_cast<unsigned int>(tal[10])));
+    d.ion_energy_eV = on ? static_cast<double>(st->ion_energy_q) / 256.0 : 0.0;
+    d.max_cfl = on ? static_cast<double>(__uint_as_float(st->max_cfl_bits)) : 0.0;
     d.J_hat = sc[15];
-    long long nl[kSpecies];
     for (int s = 0; s < kSpecies; ++s) {
-      for (int e = 0; e < 2; ++e) d.absorbed[e][s] = static_cast<int64_t>(tal[e * kSpecies + s]);
-      nl[s] = S->n_live[s] - d.absorbed[0][s] - d.absorbed[1][s];
+      d.n_live[s] = st->n_live[s];
+      for (int e = 0; e < 2; ++e) {
+        d.absorbed[e][s] = on ? static_cast<int64_t>(st->absorbed[e][s]) : 0;
+        d.n_live[s] -= d.absorbed[e][s];
+      }
     }
-    d.emitted[0] = static_cast<int64_t>(tal[6]);
-    d.emitted[1] = static_cast<int64_t>(tal[7]);
-    d.injected = static_cast<int64_t>(tal[8]);
-    nl[1] += d.injected;
-    nl[2] += d.emitted[0] + d.emitted[1];
-    for (int s = 0; s < kSpecies; ++s) d.n_live[s] = nl[s];
-    d.conv_count = conv;
+    d.emitted[0] = on ? static_cast<int64_t>(st->emitted[0]) : 0;
+    d.emitted[1] = on ? static_cast<int64_t>(st->emitted[1]) : 0;
+    d.injected = on ? static_cast<int64_t>(st->injected) : 0;
+    d.n_live[1] += d.injected;
+    d.n_live[2] += d.emitted[0] + d.emitted[1];
+    d.conv_count = on ? st->conv_count : 0;
     S->cur = d;
-    if (level < B.hist_rows) B.hist[level] = d;
-
-    // commit the circuit and surface-charge state of the new level
-    if (P->circuit == CP_CIRCUIT_TESLA && do_push) {  // the five loop charges
-      double Qv[5];
-      for (int i = 0; i < 5; ++i)
-        Qv[i] = (mode == 0) ? sc[40 + i] - phi0 * P->t_ws[i] : sc[40 + i] + sc[36] * P->t_ww[i];
-      for (int k = 3; k > 0; --k)
-        for (int i = 0; i < 5; ++i) S->Qt[k][i] = S->Qt[k - 1][i];
-      for (int i = 0; i < 5; ++i) S->Qt[0][i] = Qv[i];
-      if (!isfinite(Qv[0]) || !isfinite(Qv[1]) || !isfinite(Qv[2]) || !isfinite(Qv[4]))
-        status = CP_ERR_NONFINITE;
-    }
+    if (level < hist_rows) hist[level] = d;
+    for (int s = 0; s < kSpecies; ++s) S->n_live[s] = d.n_live[s];
     S->pv_phi0 = sc[32];  // the predictor's previous level (phi_0, Q_surf)
     S->pv_Qsurf = sc[7] * A;
     S->sigma = sigma_n;
@@ -856,30 +434,347 @@ __device__ __forceinline__ void solve_body(const Bufs& B, int do_push, int mode,
     S->Qh[1] = Q1;
     S->Qh[0] = Qn;
     // source and BDF2 history of the next level (off the next solve's critical path)
-    S->nxt_Vs = (level + 1 < B.hist_rows + 1) ? B.vs[level + 1] : 0.0;
+    S->nxt_Vs = (level + 1 < hist_rows + 1) ? vs[level + 1] : 0.0;
     S->nxt_hist = P->L4dt2 * (24.0 * Qn - 22.0 * Q1 + 8.0 * Q2 - Q3) + P->R2dt * (4.0 * Qn - Q1);
     S->level = level;
     if (do_push) S->pushed = 1;
-    for (int s = 0; s < kSpecies; ++s) {
-      S->n_live[s] = nl[s];
-      for (int e = 0; e < 2; ++e) S->absorbed[e][s] = 0ULL;
-    }
-    S->emitted[0] = S->emitted[1] = 0ULL;
+  }
+  // the push's tallies start the next step at zero
+  if (lane < 2 * kSpecies) S->absorbed[lane / kSpecies][lane % kSpecies] = 0ULL;
+  if (lane == 8) S->emitted[0] = S->emitted[1] = 0ULL;
+  if (lane == 9) {
     S->injected = 0ULL;
     S->conv_count = 0;
     S->ion_energy_q = 0;
     S->max_cfl_bits = 0u;
-    if (status != 0 && S->status == 0) S->status = status;
   }
-  // the next push processes the slots in use, rounded up to whole vectors;
-  // the padding slots are made dead here
-  if (threadIdx.x >= 32 && threadIdx.x < 32 + kSpecies) {
-    const int s = threadIdx.x - 32;
-    long long na = static_cast<long long>(S->n_alloc[s]);
+  if (P->circuit == CP_CIRCUIT_TESLA && do_push) {  // the five loop charges
+    double q = 0.0;
+    if (lane < 5) {
+      q = (mode == 0) ? sc[40 + lane] - phi0 * P->t_ws[lane] : sc[40 + lane] + sc[36] * P->t_ww[lane];
+      for (int k = 3; k > 0; --k) S->Qt[k][lane] = st->Qt[k - 1][lane];
+      S->Qt[0][lane] = q;
+    }
+    if (!__all_sync(0xffffffffu, isfinite(q))) status = CP_ERR_NONFINITE;
+  }
+  return status;
+}
+
+// Everything the refinement needs of the solve (rare path).
+struct Refine {
+  double *ph, *Ee, *bb, *rr;
+  double *sc, *wd, *slotd, *edge;  // edge[3]: this rank's first and last potential, first field
+  unsigned long long (*wu)[32];
+  MaxSlot* slot;
+  double* s_eta;
+  int lo, hi, m, N;
+  double gam, inv_dx, tol;
+  bool strict_rlc;
+};
+
+// The normwise backward error of the solved rows and of the circuit row.
+__device__ __forceinline__ double backward_error(const DevParams* P, const double* sc, bool strict_rlc, double gam,
+                                                 double rmd, double xmd, double bmd, double p0) {
+  const double nA = fmax(fabs(1.0 + gam) + 1.0, 4.0);
+  const double den = nA * xmd + bmd;
+  double e = den > 0.0 ? rmd / den : 0.0;
+  if (strict_rlc) {  // the circuit row with the potential of row 0
+    const double Qn = sc[3] - sc[2] * p0;
+    const double kvl = P->a21 * Qn - (sc[4] + sc[5]) + p0;
+    const double kden = P->a21 * fabs(Qn) + fabs(sc[4] + sc[5]) + fabs(p0);
+    if (kden > 0.0) e = fmax(e, fabs(kvl) / kden);
+  }
+  return e;
+}
+
+__device__ __forceinline__ double row_residual(const double* ph, double b, int k, int i, int m, double gam,
+                                               double prev_phi, double next_phi) {
+  const double xp = (k + 1 < m) ? ph[k + 1] : next_phi;
+  if (i == 0) return (1.0 + gam) * ph[k] - xp - b;
+  const double xq = (k > 0) ? ph[k - 1] : prev_phi;
+  return (xq - 2.0 * ph[k] + xp) - b;
+}
+
+// At most three sweeps x -= A^{-1} r in FP64, until the backward error is
+// within tol; all threads of the cluster.  Returns the last backward error;
+// *phi0 and *nextE are the refined potential of node 0 and the next chunk's
+// first field.
+__device__ __noinline__ double refine(const Refine& R, const DevParams* P, double prev_phi, double next_phi,
+                                      double* phi0, double* nextE) {
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = static_cast<int>(cl.block_rank()), nr = static_cast<int>(cl.num_blocks());
+  const int m = R.m, lo = R.lo, hi = R.hi, N = R.N;
+  double eta = 0.0;
+  for (int sweep = 1; sweep <= 3; ++sweep) {
+    for (int k = threadIdx.x; k < m; k += kSolveThreads)
+      R.rr[k] = row_residual(R.ph, R.bb[k], k, lo + k, m, R.gam, prev_phi, next_phi);
+    __syncthreads();
+    if (rank == 0 && threadIdx.x == 0) R.sc[14] = R.rr[0];
+    cl.sync();
+    const double r0all = cl.map_shared_rank(&R.sc[14], 0)[0];
+    cluster_tri_solve_f64(R.rr, lo, m, N, r0all, R.gam, R.wd, R.slotd, R.sc + 16);
+    for (int k = threadIdx.x; k < m; k += kSolveThreads) R.ph[k] -= R.rr[k];
+    __syncthreads();
+    if (threadIdx.x == 0 && m > 0) {
+      R.edge[0] = R.ph[0];
+      R.edge[1] = R.ph[m - 1];
+    }
+    cl.sync();
+    next_phi = (hi < N) ? cl.map_shared_rank(R.edge, rank + 1)[0] : 0.0;
+    prev_phi = (lo > 0) ? cl.map_shared_rank(R.edge, rank - 1)[1] : 0.0;
+    *phi0 = cl.map_shared_rank(R.edge, 0)[0];
+    for (int k = threadIdx.x; k < m; k += kSolveThreads)
+      R.Ee[k] = (R.ph[k] - ((k + 1 < m) ? R.ph[k + 1] : next_phi)) * R.inv_dx;
+    __syncthreads();
+    if (threadIdx.x == 0 && m > 0) R.edge[2] = R.Ee[0];
+    cl.sync();
+    *nextE = (hi < N) ? cl.map_shared_rank(R.edge, rank + 1)[2] : 0.0;
+    // backward error over the cluster
+    unsigned long long rm = 0ULL, xm = 0ULL, bm = 0ULL;
+    for (int k = threadIdx.x; k < m; k += kSolveThreads) {
+      rm = max(rm, abs_bits(row_residual(R.ph, R.bb[k], k, lo + k, m, R.gam, prev_phi, next_phi)));
+      xm = max(xm, abs_bits(R.ph[k]));
+      bm = max(bm, abs_bits(R.bb[k]));
+    }
+    rm = warp_max_u64(rm);
+    xm = warp_max_u64(xm);
+    bm = warp_max_u64(bm);
+    if (lane_id() == 0) {
+      R.wu[0][threadIdx.x >> 5] = rm;
+      R.wu[1][threadIdx.x >> 5] = xm;
+      R.wu[2][threadIdx.x >> 5] = bm;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      MaxSlot q = {0ULL, 0ULL, 0ULL, 0ULL};
+      for (int w = 0; w < kSolveThreads / 32; ++w) {
+        q.rmax = max(q.rmax, R.wu[0][w]);
+        q.xmax = max(q.xmax, R.wu[1][w]);
+        q.bmax = max(q.bmax, R.wu[2][w]);
+      }
+      *R.slot = q;
+    }
+    cl.sync();
+    if (threadIdx.x == 0) {
+      unsigned long long a = 0ULL, b = 0ULL, c = 0ULL;
+      for (int r = 0; r < nr; ++r) {
+        const MaxSlot* q = cl.map_shared_rank(R.slot, r);
+        a = max(a, q->rmax);
+        b = max(b, q->xmax);
+        c = max(c, q->bmax);
+      }
+      *R.s_eta = backward_error(P, R.sc, R.strict_rlc, R.gam, __longlong_as_double(static_cast<long long>(a)),
+                                __longlong_as_double(static_cast<long long>(b)),
+                                __longlong_as_double(static_cast<long long>(c)), *phi0);
+    }
+    cl.sync();  // remote reads done; the error is in every rank's shared memory
+    eta = *R.s_eta;
+    if (!(eta > R.tol)) break;
+  }
+  return eta;
+}
+
+template <typename real, typename Acc>
+__device__ __forceinline__ void solve_body(const Bufs& B, int do_push, int mode, double tol) {
+  using real2 = typename Pair<real>::type;
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = static_cast<int>(cl.block_rank());
+  const int nr = static_cast<int>(cl.num_blocks());
+  DevState* S = B.S;
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ DevParams sP;                                  // the gap's parameters
+  __shared__ __align__(16) unsigned long long s_st[sizeof(DevState) / 8];  // the state before the solve
+  __shared__ Seg<Acc> wseg[kRowWarps];
+  __shared__ Seg<Acc> slotA[kSolveCtasMax];                 // every rank's totals, pushed here
+  __shared__ MaxSlot slotC[kSolveCtasMax];                  // every rank's maxima, pushed here
+  __shared__ __align__(8) uint64_t bars[2];
+  __shared__ Seg<Acc> s_off;                                // everything before this rank's rows
+  __shared__ Acc s_U;
+  __shared__ unsigned long long wu[3][32];
+  __shared__ double wd[32];
+  __shared__ double sc[48];
+  __shared__ double s_edge[3];
+  __shared__ double slotd, s_eta;
+
+  const int tid = static_cast<int>(threadIdx.x), lane = tid & 31, warp = tid >> 5;
+  const DevParams* P = &sP;
+  const DevState* st = reinterpret_cast<const DevState*>(s_st);
+  // --- before the push has finished: parameters and barriers ----------------
+  {
+    static_assert(sizeof(DevParams) % 8 == 0, "whole words");
+    const unsigned long long* src = reinterpret_cast<const unsigned long long*>(B.P);
+    unsigned long long* dst = reinterpret_cast<unsigned long long*>(&sP);
+    for (int k = tid; k < static_cast<int>(sizeof(DevParams) / 8); k += kSolveThreads) dst[k] = src[k];
+  }
+  if (nr > 1) {
+    if (tid == 0) {
+      mbar_init(&bars[0]);
+      mbar_init(&bars[1]);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      mbar_expect(&bars[0], static_cast<uint32_t>(nr * sizeof(Seg<Acc>)));
+      mbar_expect(&bars[1], static_cast<uint32_t>(nr * sizeof(MaxSlot)));
+    }
+    cl.sync();  // every rank's barriers are ready before anyone pushes
+  } else {
+    __syncthreads();
+  }
+  const int N = P->N;
+  const int chunk = (N + nr - 1) / nr;
+  const int lo = min(rank * chunk, N);
+  const int hi = min(lo + chunk, N);
+  const int m = hi - lo;
+  const int per = (chunk + kRowThreads - 1) / kRowThreads;  // rows per row thread
+  long long* Gv = reinterpret_cast<long long*>(smem);       // G_i of this rank's rows
+  double* ph = reinterpret_cast<double*>(smem + align16(8 * chunk));
+  double* Ee = ph + chunk;
+  double* bb = Ee + chunk;
+  double* rr = bb + chunk;                                  // refinement; else the fields in `real`
+  real* ef = reinterpret_cast<real*>(rr);
+  const bool last_rows = (hi == N && m > 0);                // this rank owns row N-1 (and node N)
+  const bool runs_net = (B.net != nullptr && !B.net_in_push && do_push && rank == (nr > 1 ? 1 : 0));
+  PredNet* s_net = reinterpret_cast<PredNet*>(smem + solve_rows_bytes(chunk));
+
+  cudaGridDependencySynchronize();  // the push that deposited G has completed
+  cudaTriggerProgrammaticLaunchCompletion();
+  const int stop = ldcg(&S->status);
+  long long G0 = 0, Gnext = 0;
+  if (warp < kRowWarps) {
+    for (int k = tid; k < m; k += kRowThreads) Gv[k] = ldcg(&B.G[lo + k]);
+  } else if (warp == kCircuitWarp) {
+    G0 = ldcg(&B.G[0]);
+    if (hi < N) Gnext = ldcg(&B.G[hi]);
+    const unsigned long long* src = reinterpret_cast<const unsigned long long*>(S);
+    for (int k = lane; k < kStateWords; k += 32) s_st[kStateWord0 + k] = ldcg(&src[kStateWord0 + k]);
+    __syncwarp();
+  }
+  if (stop) return;  // the status cannot change before every rank has read it: all ranks agree
+  if (runs_net) prefetch_net(B.net, s_net);
+  if (per > 1) __syncthreads();
+
+  Seg<Acc> mine, wexcl;
+  mine.s1 = 0;
+  mine.s2 = 0;
+  wexcl = mine;
+  const int r0 = min(tid * per, m), r1 = (warp < kRowWarps) ? min(r0 + per, m) : r0;
+  unsigned long long bm = 0ULL;
+  if (warp < kRowWarps) {
+    // --- scan: this thread's rows, then the warp ---------------------------
+    for (int q = 0; q < per; ++q) {  // rows past the chunk's end hold no charge
+      const int k = tid * per + q;
+      if (k < m) {
+        const long long g = Gv[k];
+        B.Glast[lo + k] = g;
+        if (k > 0) B.G[lo + k] = 0;  // a chunk's first row (and G_0) is cleared after the last exchange
+        if (lo + k > 0) {            // S'_i = sum_{j=1..i} G_j leaves G_0 out
+          mine.s1 += g;
+          bm = max(bm, static_cast<unsigned long long>(llabs(g)));
+        }
+      }
+      mine.s2 += mine.s1;
+    }
+    Seg<Acc> incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const Seg<Acc> y = shfl_up_seg(incl, o);
+      if (lane >= o) incl = seg_then(y, incl, o * per);
+    }
+    wexcl = shfl_up_seg(incl, 1);
+    if (lane == 0) {
+      wexcl.s1 = 0;
+      wexcl.s2 = 0;
+    }
+    if (lane == 31) wseg[warp] = incl;
+  } else if (warp == kCircuitWarp) {
+    // circuit row, first part (every rank evaluates the same scalars): the
+    // source, the BDF2 history, the circuit solve and the x = 0 row's
+    // right-hand side need no scan.
+    // Tesla circuit: the new level's loop charges for phi_0 = 0 from the 20
+    // history values (one per lane, warp sums)
+    double tq[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    if (P->circuit == CP_CIRCUIT_TESLA && do_push) {
+      const double h = (lane < 20) ? st->Qt[lane / 5][lane % 5] : 0.0;  // levels n-1..n-4
+      const double(*Pm)[20] = (mode == 0) ? P->t_Ps : P->t_Pw;
+#pragma unroll
+      for (int i = 0; i < 5; ++i) {
+        double v = (lane < 20) ? Pm[i][lane] * h : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        tq[i] = v;
+      }
+    }
+    if (lane == 0) {
+      const double qw = P->e * P->weight;
+      const long long conv = do_push ? st->conv_count : 0LL;
+      const double Q1 = st->Qh[0], Q2 = st->Qh[1], Q3 = st->Qh[2];
+      // source and BDF2 history of the new level: precomputed by the previous
+      // solve except for the first solve of a run
+      double Vs, hist;
+      if (do_push) {
+        Vs = st->nxt_Vs;
+        hist = st->nxt_hist;
+      } else {
+        Vs = B.vs[st->level];
+        const double Q4 = st->Qh[3];
+        hist = P->L4dt2 * (24.0 * Q1 - 22.0 * Q2 + 8.0 * Q3 - Q4) + P->R2dt * (4.0 * Q1 - Q2);
+      }
+      const double phi0_prev = st->phi0_last;
+      // learned weak scheme: the network's prediction of the plasma's change
+      // of C phi_0 over this step, used while its tracked error is within bound
+      double J_used = 0.0;
+      if (B.net != nullptr && mode == 2) {
+        if (B.net_in_push) J_used = st->J_eff;  // the push formed the usable prediction
+        else if (st->pred_ready && st->n_eval >= kPredMinEval && st->err_avg <= B.net->bound * st->J_avg)
+          J_used = st->J_pred;
+      }
+      double g = 0.0, Qpart = Q1, gam = 0.0, inv_den = 1.0;
+      if (P->circuit == CP_CIRCUIT_SERIES_RLC) {
+        if (mode == 0) {  // strict: Q^n = K - g phi_0^n (Eqs. Q4_phi_relation, K_def)
+          g = P->g_strict;
+          Qpart = g * (Vs + hist);
+          gam = P->gam_strict;
+          inv_den = P->inv_den_strict;
+        } else {
+          // weak (Sec. 2.4.3): the circuit alone, its load capacitor starting
+          // from phi_0^{n-1}: a21 Q - hist + phi_0^{n-1} + (Q - Q^{n-1} + J)/C = V_s
+          Qpart = (Vs + hist + (Q1 - J_used) * P->inv_C - phi0_prev) * P->g_weak;
+        }
+      } else if (P->circuit == CP_CIRCUIT_TESLA) {
+        // Q1 here is the load capacitor's loop charge Q4^{n-1}
+        if (!do_push) {  // level 0: the circuit as it rests before t = 0
+          Qpart = Q1;
+        } else if (mode == 0) {  // strict: Q4^n = K - [T'^{-1}]_44 phi_0^n
+          g = P->t_ws[3];
+          Qpart = tq[3];
+          gam = P->gam_tesla;
+          inv_den = P->inv_den_tesla;
+        } else {  // weak: loop 4's capacitor voltage phi_0^{n-1} + (Q4 - Q4^{n-1} + J)/C3
+          const double s = (Q1 - J_used) * P->inv_C - phi0_prev;
+          Qpart = tq[3] + s * P->t_ww[3];
+          sc[36] = s;
+        }
+        for (int i = 0; i < 5; ++i) sc[40 + i] = tq[i];
+      }
+      const double Qconv = static_cast<double>(conv) * qw;
+      const double sigma_prev = st->sigma;
+      // x = 0 row: Eq. Poisson_BC2 (strict) / Eq. Poisson_BC3 (weak), with
+      // rho_0 dx^2 / (2 eps0) = alpha G_0 / 2 (G_0 is even: boundary doubling)
+      const double b0 = P->dx_eps0 * (sigma_prev + (Qconv + Qpart - Q1) * P->inv_A) +
+                        P->alpha * static_cast<double>(G0 / 2);
+      sc[0] = b0; sc[1] = gam; sc[2] = g; sc[3] = Qpart; sc[4] = Vs; sc[5] = hist;
+      sc[6] = Qconv; sc[7] = sigma_prev; sc[8] = Q1; sc[9] = Q2; sc[10] = Q3;
+      sc[15] = J_used;
+      sc[32] = phi0_prev;
+      sc[35] = inv_den;
+    }
+  } else if (rank == nr - 1 && lane < kSpecies) {
+    // the next push processes the slots in use, rounded up to whole vectors;
+    // the padding slots are made dead here
+    const int s = lane;
+    long long na = static_cast<long long>(ldcg(&S->n_alloc[s]));
     if (na > P->cap[s]) na = P->cap[s];
     const long long na4 = (na + 3) & ~3LL;
-    real* xs = reinterpret_cast<real*>(S->xi[s]);
-    real* us = reinterpret_cast<real*>(S->u[s]);
+    real* xs = reinterpret_cast<real*>(ldcg(&S->xi[s]));
+    real* us = reinterpret_cast<real*>(ldcg(&S->u[s]));
     for (long long k = na; k < na4; ++k) {
       xs[k] = real(-1);
       us[k] = real(0);
@@ -887,117 +782,358 @@ __device__ __forceinline__ void solve_body(const Bufs& B, int do_push, int mode,
     S->n_alloc[s] = na4;
     S->n_proc[s] = na4;
   }
-  if (nr == 1 && runs_net) {  // a one-CTA solve runs the predictor itself
-    __syncthreads();
-    predictor_update(B.P, B.S, &s_net, s_feat, sc, strict_c, phi0_fin);
+  if (last_rows && tid == kSolveThreads - 1) {
+    B.Glast[N] = ldcg(&B.G[N]);
+    B.G[N] = 0;
   }
+  __syncthreads();
+
+  // --- the ranks' totals, and the electrode potential ------------------------
+  Seg<Acc> bexcl;  // everything of this CTA before this warp
+  bexcl.s1 = 0;
+  bexcl.s2 = 0;
+  if (warp < kRowWarps) {
+    for (int q = 0; q < warp; ++q) bexcl = seg_then(bexcl, wseg[q], 32 * per);
+  } else if (warp == kCircuitWarp) {
+    Seg<Acc> tot = wseg[0];
+#pragma unroll
+    for (int q = 1; q < kRowWarps; ++q) tot = seg_then(tot, wseg[q], 32 * per);
+    // the rows past the chunk's end each added the chunk's total once more
+    tot.s2 -= len_times<Acc>(kRowThreads * per - m, tot.s1);
+    Seg<Acc> v = tot;
+    if (nr > 1) {
+      if (lane < nr) {
+        const uint32_t dst = remote_addr(&slotA[rank], lane), bar = remote_addr(&bars[0], lane);
+        if constexpr (sizeof(Acc) == 8) {
+          push16(dst, static_cast<unsigned long long>(tot.s2), static_cast<unsigned long long>(tot.s1), bar);
+        } else {
+          push16(dst, static_cast<unsigned long long>(tot.s2),
+                 static_cast<unsigned long long>(static_cast<unsigned __int128>(tot.s2) >> 64), bar);
+          push16(dst + 16, static_cast<unsigned long long>(tot.s1), 0ULL, bar);
+        }
+      }
+      if (!mbar_wait(&bars[0]) && lane == 0) atomicCAS(&S->status, 0, CP_ERR_TIMEOUT);
+      v.s1 = 0;
+      v.s2 = 0;
+      if (lane < nr) v = slotA[lane];
+    } else if (lane > 0) {
+      v.s1 = 0;
+      v.s2 = 0;
+    }
+    // inclusive scan over the ranks; rank r holds rows_of(r) rows
+    int len = max(0, min(chunk, N - lane * chunk));
+    if (lane >= nr) len = 0;
+    Seg<Acc> ci = v;
+#pragma unroll
+    for (int o = 1; o < kSolveCtasMax; o <<= 1) {
+      const Seg<Acc> y = shfl_up_seg(ci, o);
+      const int ly = __shfl_up_sync(0xffffffffu, len, o);
+      if (lane >= o) {
+        ci = seg_then(y, ci, len);
+        len += ly;
+      }
+    }
+    Seg<Acc> ce = shfl_up_seg(ci, 1);
+    if (lane == 0) {
+      ce.s1 = 0;
+      ce.s2 = 0;
+    }
+    if (lane == rank) s_off = ce;  // everything before this rank
+    if (lane == nr - 1) {
+      const Acc U = ci.s2;
+      const double b0 = sc[0], gam = sc[1], inv_den = sc[35];
+      const double phi0 = (static_cast<double>(N) * b0 + P->alpha * acc_to_double(U)) * inv_den;
+      const double D0 = b0 - gam * phi0;  // D_0 = x_0 - x_1
+      s_U = U;
+      sc[11] = D0;
+      sc[24] = D0 * P->inv_dx;        // E_0
+      sc[25] = P->alpha * P->inv_dx;  // dE_i / dS'_i
+    }
+    mine = ci;  // kept for the edges: lane `rank` holds everything up to this rank's end
+  }
+  __syncthreads();
+  const double b0 = sc[0], gam = sc[1], D0 = sc[11];
+  const double alpha = P->alpha, inv_dx = P->inv_dx;
+  const double E0 = sc[24], Ea = sc[25];
+  const Acc U = s_U;
+  const bool strict_rlc = (P->circuit == CP_CIRCUIT_SERIES_RLC && mode == 0);
+  // the level's charge follows Q^n = K - g phi_0^n (g = 0 at a Tesla level 0)
+  const bool strict_c = (P->circuit != CP_CIRCUIT_OPEN) && (mode == 0 || (P->circuit == CP_CIRCUIT_TESLA && !do_push));
+  // D_i = D_0 + alpha S'_i;  x_i = (N - i) D_0 + alpha (U - P_i);  E_i = D_i / dx
+  if (warp < kRowWarps) {
+    // everything before this thread's rows: rank, then warp, then lane
+    const Seg<Acc> off = seg_then(seg_then(s_off, bexcl, 32 * per * warp), wexcl, lane * per);
+    long long Sr = off.s1;  // S'_i, running
+    Acc Pex = off.s2;       // P_i = sum_{k<i} S'_k (exclusive)
+    for (int k = r0; k < r1; ++k) {
+      const int i = lo + k;
+      const long long g = (i == 0) ? 0LL : Gv[k];
+      Sr += g;
+      const double x = fma(static_cast<double>(N - i), D0, alpha * acc_to_double(U - Pex));
+      const double e = fma(Ea, static_cast<double>(Sr), E0);
+      ph[k] = x;
+      Ee[k] = e;
+      ef[k] = static_cast<real>(e);
+      bb[k] = (i == 0) ? b0 : -alpha * static_cast<double>(g);
+      Pex += Sr;
+    }
+  } else if (warp == kCircuitWarp) {
+    // The neighbouring chunks' edge values follow from the exact prefixes with
+    // the same arithmetic their owners use, so no exchange is needed:
+    // x_{lo-1} needs P_{lo-1} = P_lo - S'_{lo-1}; x_hi needs P_hi; E_hi needs S'_hi.
+    Seg<Acc> no;  // everything up to and including this rank's rows
+    if (lane == rank) slotA[rank] = mine;
+    __syncwarp();
+    no = slotA[rank];
+    const Seg<Acc> ro = s_off;
+    const int i = (lane == 0) ? lo - 1 : (lane == 1) ? hi : 0;  // lanes 0-2: x_{lo-1}, x_hi, x_0
+    const Acc Pi = (lane == 0) ? ro.s2 - static_cast<Acc>(ro.s1) : (lane == 1) ? no.s2 : Acc(0);
+    const double x = fma(static_cast<double>(N - i), D0, alpha * acc_to_double(U - Pi));
+    const double e = fma(Ea, static_cast<double>(no.s1 + Gnext), E0);
+    if (lane == 0) sc[26] = (lo > 0) ? x : 0.0;
+    if (lane == 1) sc[27] = (hi < N) ? x : 0.0;
+    if (lane == 1) sc[28] = (hi < N) ? e : 0.0;
+    if (lane == 2) sc[29] = x;
+  }
+  __syncthreads();
+  const double prev_phi = sc[26], next_phi = sc[27], phi0 = sc[29];
+  double nextE = sc[28];
+  double phi0_fin = phi0;
+  int status = 0;  // of the committed values (commit warp of rank 0)
+  real2* Epair = reinterpret_cast<real2*>(B.Epair);
+  if (warp < kRowWarps) {
+    // outputs; the gather table pairs need the next row's field value
+    unsigned long long rm = 0ULL, xm = 0ULL;
+    for (int k = tid; k < m; k += kRowThreads) {
+      const int i = lo + k;
+      const double x = ph[k];
+      const double ri = row_residual(ph, bb[k], k, i, m, gam, prev_phi, next_phi);
+      rm = max(rm, abs_bits(ri));
+      xm = max(xm, abs_bits(x));
+      B.E64[i] = Ee[k];
+      B.phi[i] = x;
+      const real e0 = ef[k];
+      const real e1 = (i + 1 < N) ? ((k + 1 < m) ? ef[k + 1] : static_cast<real>(nextE)) : e0;
+      real2 pr;
+      pr.x = e0;
+      pr.y = e1 - e0;
+      Epair[i + 1] = pr;
+      if (i == 0) {
+        pr.y = real(0);
+        Epair[0] = pr;
+      }
+    }
+    rm = warp_max_u64(rm);
+    xm = warp_max_u64(xm);
+    bm = warp_max_u64(bm);
+    if (lane == 0) {
+      wu[0][warp] = rm;
+      wu[1][warp] = xm;
+      wu[2][warp] = bm;
+    }
+  } else if (warp == kCommitWarp) {
+    if (last_rows && lane == 31) B.phi[N] = 0.0;
+    if (rank == 0)
+      status = commit_level(S, B.hist, B.hist_rows, B.vs, P, st, sc, do_push, mode, strict_c, phi0, 0.0);
+  }
+  if (warp != kCommitWarp)  // the commit goes on beside the error's exchange
+    asm volatile("bar.sync 1, %0;" ::"n"(kRowThreads + 32) : "memory");
+  // --- backward error over the cluster ----------------------------------------
+  if (warp == kCircuitWarp) {
+    MaxSlot q;
+    q.rmax = warp_max_u64(lane < kRowWarps ? wu[0][lane] : 0ULL);
+    q.xmax = warp_max_u64(lane < kRowWarps ? wu[1][lane] : 0ULL);
+    q.bmax = warp_max_u64(lane < kRowWarps ? wu[2][lane] : 0ULL);
+    if (nr > 1) {
+      if (lane < nr) {
+        const uint32_t dst = remote_addr(&slotC[rank], lane), bar = remote_addr(&bars[1], lane);
+        push16(dst, q.rmax, q.xmax, bar);
+        push16(dst + 16, q.bmax, 0ULL, bar);
+      }
+      if (!mbar_wait(&bars[1]) && lane == 0) atomicCAS(&S->status, 0, CP_ERR_TIMEOUT);
+      q.rmax = warp_max_u64(lane < nr ? slotC[lane].rmax : 0ULL);
+      q.xmax = warp_max_u64(lane < nr ? slotC[lane].xmax : 0ULL);
+      q.bmax = warp_max_u64(lane < nr ? slotC[lane].bmax : 0ULL);
+    }
+    if (lane == 0) {
+      // max |b_i| = max(alpha max |G_i| over rows >= 1, |b_0|)
+      const double bmd = fmax(alpha * static_cast<double>(q.bmax), fabs(b0));
+      s_eta = backward_error(P, sc, strict_rlc, gam, __longlong_as_double(static_cast<long long>(q.rmax)),
+                             __longlong_as_double(static_cast<long long>(q.xmax)), bmd, phi0);
+      if (m > 0) B.G[lo] = 0;  // every rank has read it
+    }
+  }
+  __syncthreads();
+  double eta = s_eta;
+  if (eta > tol) {  // the same on every rank
+    Refine R;
+    R.ph = ph; R.Ee = Ee; R.bb = bb; R.rr = rr;
+    R.sc = sc; R.wd = wd; R.slotd = &slotd; R.edge = s_edge;
+    R.wu = wu; R.slot = &slotC[0]; R.s_eta = &s_eta;
+    R.lo = lo; R.hi = hi; R.m = m; R.N = N;
+    R.gam = gam; R.inv_dx = inv_dx; R.tol = tol;
+    R.strict_rlc = strict_rlc;
+    eta = refine(R, P, prev_phi, next_phi, &phi0_fin, &nextE);
+    for (int k = tid; k < m; k += kSolveThreads) {
+      const int i = lo + k;
+      B.E64[i] = Ee[k];
+      B.phi[i] = ph[k];
+      const real e0 = static_cast<real>(Ee[k]);
+      const real e1 = (i + 1 < N) ? static_cast<real>((k + 1 < m) ? Ee[k + 1] : nextE) : e0;
+      real2 pr;
+      pr.x = e0;
+      pr.y = e1 - e0;
+      Epair[i + 1] = pr;
+      if (i == 0) {
+        pr.y = real(0);
+        Epair[0] = pr;
+      }
+    }
+    if (rank == 0 && warp == kCommitWarp)
+      status = commit_level(S, B.hist, B.hist_rows, B.vs, P, st, sc, do_push, mode, strict_c, phi0_fin, eta);
+  }
+  if (rank == 0 && tid == 32 * kCommitWarp) {
+    const int64_t level = st->level + (do_push ? 1 : 0);
+    S->cur.residual = eta;
+    if (level < B.hist_rows) B.hist[level].residual = eta;
+    if (status == 0 && eta > tol) status = CP_ERR_RESIDUAL;
+    if (status != 0) atomicCAS(&S->status, 0, status);
+  }
+  if (runs_net) predictor_update(P, S, st, s_net, sc, strict_c, phi0_fin);
 }
 
-template <typename real>
-__global__ void __launch_bounds__(kSolveThreads, 1) k_solve(Bufs B, int do_push, int mode, double tol) {
-  solve_body<real>(B, do_push, mode, tol);
+template <typename real, typename Acc>
+__global__ void __launch_bounds__(kSolveThreads) k_solve(Bufs B, int do_push, int mode, double tol) {
+  solve_body<real, Acc>(B, do_push, mode, tol);
 }
 
-// Ensemble: CTA i solves instance i (launched without clusters, so each CTA
-// is a cluster of one).
-template <typename real>
-__global__ void __launch_bounds__(kSolveThreads, 1)
+// Ensemble: cluster i solves instance i.
+template <typename real, typename Acc>
+__global__ void __launch_bounds__(kSolveThreads)
 k_solve_ens(const Bufs* __restrict__ Ball, int do_push, int mode, double tol) {
-  const Bufs B = Ball[blockIdx.x];
-  solve_body<real>(B, do_push, mode, tol);
+  const Bufs B = Ball[blockIdx.x / cg::this_cluster().num_blocks()];
+  solve_body<real, Acc>(B, do_push, mode, tol);
 }
 
 // ---------------------------------------------------------------------------
 // Host-side launchers
 // ---------------------------------------------------------------------------
-cudaError_t solve_configure(int precision, size_t solve_smem) {
+static const void* solve_fn(int precision, bool wide) {
   if (precision == CP_FP32)
-    return cudaFuncSetAttribute(k_solve<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                static_cast<int>(solve_smem));
-  return cudaFuncSetAttribute(k_solve<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(solve_smem));
+    return wide ? reinterpret_cast<const void*>(k_solve<float, __int128>)
+                : reinterpret_cast<const void*>(k_solve<float, long long>);
+  return wide ? reinterpret_cast<const void*>(k_solve<double, __int128>)
+              : reinterpret_cast<const void*>(k_solve<double, long long>);
 }
 
-size_t solve_smem_bytes(int N, int ctas) {
-  const size_t chunk = (N + ctas - 1) / ctas;
-  return align16(8 * chunk) + 4 * 8 * chunk;
+static const void* solve_ens_fn(int precision, bool wide) {
+  if (precision == CP_FP32)
+    return wide ? reinterpret_cast<const void*>(k_solve_ens<float, __int128>)
+                : reinterpret_cast<const void*>(k_solve_ens<float, long long>);
+  return wide ? reinterpret_cast<const void*>(k_solve_ens<double, __int128>)
+              : reinterpret_cast<const void*>(k_solve_ens<double, long long>);
 }
 
-// Largest cluster (16, else 8) the device can run the solve with.
-cudaError_t solve_cluster_size(int precision, int N, int* ctas) {
-  *ctas = kSolveCtas;
-  const void* fn = (precision == CP_FP32) ? reinterpret_cast<const void*>(k_solve<float>)
-                                          : reinterpret_cast<const void*>(k_solve<double>);
+// Whether the prefix of prefixes of a gap of N cells whose stores hold
+// cap[] macroparticles needs 128 bits (per_particle: charge units of one).
+bool solve_wide(int N, const int64_t cap[kSpecies], double per_particle) {
+  const double most = static_cast<double>(std::max(cap[CP_IONS], cap[CP_ELECTRONS] + cap[CP_SECONDARIES]));
+  const double rows = static_cast<double>(N) + kSolveCtasMax * kRowThreads;  // padding rows included
+  return !(per_particle * most * rows < 4.611686018427387904e18);            // 2^62
+}
+
+// Every context sharing a kernel may ask for another size, so each kernel's
+// limit is the largest the device allows.
+static cudaError_t allow_all_smem(const void* fn) {
+  int dev = 0, most = 0;
+  cudaFuncAttributes at;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, fn);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              most - static_cast<int>(at.sharedSizeBytes));
+}
+
+cudaError_t solve_configure(int precision, bool wide) { return allow_all_smem(solve_fn(precision, wide)); }
+cudaError_t solve_ens_configure(int precision, bool wide) {
+  return allow_all_smem(solve_ens_fn(precision, wide));
+}
+
+size_t solve_smem_bytes(int N, int ctas, bool net) {
+  return solve_rows_bytes((N + ctas - 1) / ctas) + (net ? kPredNetBytes : 0);
+}
+
+// CTAs of a solve of N rows: one per 256 rows, at most 16 (where the device
+// runs non-portable clusters, else 8).
+cudaError_t solve_cluster_size(int precision, bool wide, int N, int* ctas) {
+  int want = 1;
+  while (want < kSolveCtasMax && want * kRowThreads < N) want *= 2;
+  *ctas = std::min(want, kSolveCtas);
+  if (want <= kSolveCtas) return cudaSuccess;
+  const void* fn = solve_fn(precision, wide);
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
     cudaGetLastError();
     return cudaSuccess;
   }
-  const size_t smem = solve_smem_bytes(N, kSolveCtasMax);
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) !=
-      cudaSuccess) {
-    cudaGetLastError();
-    return cudaSuccess;
-  }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kSolveCtasMax, 1, 1);
+  cfg.gridDim = dim3(want, 1, 1);
   cfg.blockDim = dim3(kSolveThreads, 1, 1);
-  cfg.dynamicSmemBytes = smem;
+  cfg.dynamicSmemBytes = solve_smem_bytes(N, want, true);
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = kSolveCtasMax;
+  attr[0].val.clusterDim.x = want;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int clusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) == cudaSuccess && clusters >= 1)
-    *ctas = kSolveCtasMax;
+  if (cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) == cudaSuccess && clusters >= 1) *ctas = want;
   cudaGetLastError();
   return cudaSuccess;
 }
 
-cudaError_t solve_ens_configure(int precision, size_t smem) {
-  if (precision == CP_FP32)
-    return cudaFuncSetAttribute(k_solve_ens<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                static_cast<int>(smem));
-  return cudaFuncSetAttribute(k_solve_ens<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(smem));
+// CTAs per instance of an ensemble's solve.  One CTA per instance leaves the
+// FP64 work of the few largest gaps on one SM each, more CTAs cost the
+// exchange: 4 while the clusters fit the device in about two waves, then 2,
+// then 1.
+int solve_ens_cluster_size(int n_max, int E, int sms) {
+  int nr = 1;
+  while (nr < 4 && nr * kRowThreads < n_max && 2 * nr * E <= 8 * sms) nr *= 2;
+  return nr;
 }
 
-cudaError_t solve_ens_launch(int precision, const Bufs* Ball, int n_inst, size_t smem,
-                             cudaStream_t st, int do_push, int mode, double tol) {
+static cudaLaunchConfig_t solve_config(int grid, int ctas, size_t smem, cudaStream_t st, cudaLaunchAttribute* attr) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(n_inst, 1, 1);
+  cfg.gridDim = dim3(grid, 1, 1);
   cfg.blockDim = dim3(kSolveThreads, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (precision == CP_FP32) return cudaLaunchKernelEx(&cfg, k_solve_ens<float>, Ball, do_push, mode, tol);
-  return cudaLaunchKernelEx(&cfg, k_solve_ens<double>, Ball, do_push, mode, tol);
-}
-
-cudaError_t solve_launch(int precision, const Bufs& B, int ctas, size_t smem, cudaStream_t st,
-                         int do_push, int mode, double tol) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(ctas, 1, 1);
-  cfg.blockDim = dim3(kSolveThreads, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = ctas;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = ctas;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  if (precision == CP_FP32) return cudaLaunchKernelEx(&cfg, k_solve<float>, B, do_push, mode, tol);
-  return cudaLaunchKernelEx(&cfg, k_solve<double>, B, do_push, mode, tol);
+  return cfg;
+}
+
+cudaError_t solve_ens_launch(int precision, bool wide, const Bufs* Ball, int n_inst, int ctas, size_t smem,
+                             cudaStream_t st, int do_push, int mode, double tol) {
+  cudaLaunchAttribute attr[2];
+  const cudaLaunchConfig_t cfg = solve_config(n_inst * ctas, ctas, smem, st, attr);
+  void* args[] = {&Ball, &do_push, &mode, &tol};
+  return cudaLaunchKernelExC(&cfg, solve_ens_fn(precision, wide), args);
+}
+
+cudaError_t solve_launch(int precision, bool wide, const Bufs& B, int ctas, size_t smem, cudaStream_t st,
+                         int do_push, int mode, double tol) {
+  cudaLaunchAttribute attr[2];
+  const cudaLaunchConfig_t cfg = solve_config(ctas, ctas, smem, st, attr);
+  void* args[] = {const_cast<Bufs*>(&B), &do_push, &mode, &tol};
+  return cudaLaunchKernelExC(&cfg, solve_fn(precision, wide), args);
 }
 
 }  // namespace cpk
