@@ -774,7 +774,7 @@ def main():
         "roofline": {"bound": "hbm", "achieved": r["achieved"], "peak": r["peak"],
                      "unit": "GB/s", "frac": r["achieved"] / r["peak"], "traffic": r["traffic"],
                      "traffic_note": r["traffic_why"],
-                     "kernel": "k_push_async" if r["cfg"]["precision"] == W.FP32 else "k_push",
+                     "kernel": "k_push",
                      "peak_source": r["peak_kind"],
                      "avg_launch_ms": r["avg_launch_ms"], "launches_used": r["n_sel"],
                      "bytes_per_particle_step": r["bpp"],

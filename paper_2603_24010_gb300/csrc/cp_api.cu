@@ -19,11 +19,12 @@
 
 namespace cpk {
 size_t push_smem_bytes(int N, int precision);
+size_t push_smem_limit_bytes(int N, int precision);
 size_t solve_smem_bytes(int N, int ctas, bool net);
 bool solve_wide(int N, const int64_t cap[kSpecies], double per_particle);
 cudaError_t solve_cluster_size(int precision, bool wide, int N, int* ctas);
 int solve_ens_cluster_size(int n_max, int E, int sms);
-cudaError_t push_configure(int precision, size_t push_smem);
+cudaError_t push_configure(int precision);
 cudaError_t solve_configure(int precision, bool wide);
 cudaError_t push_occupancy(int precision, size_t smem, int* blocks_per_sm);
 cudaError_t push_launch(int precision, const Bufs& B, int grid, size_t smem, cudaStream_t st,
@@ -86,6 +87,7 @@ struct cp_ctx {
   cp_diag* hist = nullptr;
   int64_t hist_rows = 0;
   double* vs = nullptr;
+  int64_t* next_step = nullptr;  // level the next push starts from
   int grid = 0;
   int compact_grid = 0;   // removal kernel
   size_t smem = 0;        // push kernel
@@ -231,6 +233,7 @@ cpk::Bufs make_bufs(const cp_ctx* c) {
   B.hist_rows = c->hist_rows;
   B.vs = c->vs;
   B.net = c->net;
+  B.next_step = c->next_step;
   // a single FP32 gap evaluates the predictor in the next push's idle tail;
   // ensemble members and the 2D gap's mean keep it in the solve
   B.net_in_push = (c->precision == CP_FP32 && !c->ens_member) ? 1 : 0;
@@ -262,6 +265,7 @@ void free_all(cp_ctx* c) {
   cudaFree(c->abs);
   cudaFree(c->hist);
   cudaFree(c->vs);
+  cudaFree(c->next_step);
   cudaFree(c->dP);
   cudaFree(c->dS);
   cudaFree(c->net);
@@ -356,7 +360,7 @@ int initialize(cp_ctx* c, int mode, double tol) {
   // launch shape: persistent grid of resident push CTAs, one solve cluster
   c->smem = cpk::push_smem_bytes(c->N, c->precision);
   c->solve_wide = cpk::solve_wide(c->N, c->cap, cpk::kFix);
-  CP_CUDA(cpk::push_configure(c->precision, c->smem));
+  CP_CUDA(cpk::push_configure(c->precision));
   CP_CUDA(cpk::solve_configure(c->precision, c->solve_wide));
   CP_CUDA(cpk::solve_cluster_size(c->precision, c->solve_wide, c->N, &c->solve_ctas));
   int per_sm = 0, sms = 0;
@@ -373,6 +377,8 @@ int initialize(cp_ctx* c, int mode, double tol) {
   CP_CUDA(cudaMemcpyAsync(c->dP, &c->hp, sizeof(cpk::DevParams), cudaMemcpyHostToDevice, c->stream));
   CP_TRY(alloc(reinterpret_cast<void**>(&c->vs), sizeof(double) * (c->hist_rows + 1)));
   CP_CUDA(cpk::source_table_launch(c->dP, c->vs, c->hist_rows + 1, c->stream));
+  CP_TRY(alloc(reinterpret_cast<void**>(&c->next_step), sizeof(int64_t)));
+  CP_CUDA(cudaMemsetAsync(c->next_step, 0, sizeof(int64_t), c->stream));
 
   cpk::DevState S;
   std::memset(&S, 0, sizeof(S));
@@ -570,7 +576,7 @@ int cp_create(const cp_gap* gap, const cp_circuit* circ, const cp_see_beam* see,
   }
   // the push keeps the field table and the node sums of the whole gap in
   // shared memory (1 KB left for its static variables)
-  if (cpk::push_smem_bytes(gap->n_cells, run->precision) + 1024 > static_cast<size_t>(smem_optin)) {
+  if (cpk::push_smem_limit_bytes(gap->n_cells, run->precision) + 1024 > static_cast<size_t>(smem_optin)) {
     cudaStreamDestroy(c->cap_stream);
     delete c;
     return CP_ERR_ARG;
@@ -997,6 +1003,7 @@ int cp_load_state(cp_ctx* c, const void* buf, size_t len) {
   CP_TRY(h2d(c->hist, sizeof(cp_diag) * h.hist_n));
   CP_CUDA(cudaMemsetAsync(c->G, 0, sizeof(long long) * (c->N + 1), c->stream));
   CP_CUDA(cudaMemcpyAsync(c->dS, &S, sizeof(S), cudaMemcpyHostToDevice, c->stream));
+  CP_CUDA(cudaMemcpyAsync(c->next_step, &S.level, sizeof(int64_t), cudaMemcpyHostToDevice, c->stream));
   CP_CUDA(cudaStreamSynchronize(c->stream));
   c->since_compact = static_cast<int>(h.since_compact);
   return CP_OK;

@@ -74,27 +74,6 @@ __device__ __forceinline__ void deposit(unsigned int* A, unsigned int* Bc, real 
   atomicAdd(&Bc[i], w1);
 }
 
-// Fold the cell sums into the int64 node grid (node k gets A[k] + Bc[k-1],
-// the two end nodes doubled) and clear them.  Thread k owns node k and is
-// the only reader of A[k] and Bc[k-1], so it clears exactly those.
-__device__ __forceinline__ void fold(unsigned int* A, unsigned int* Bc, long long* Gs, int N,
-                                     long long sign) {
-  for (int k = threadIdx.x; k <= N; k += kThreads) {
-    long long a = 0, b = 0;
-    if (k < N) {
-      a = A[k];
-      A[k] = 0u;
-    }
-    if (k > 0) {
-      b = Bc[k - 1];
-      Bc[k - 1] = 0u;
-    }
-    if (k == 0) a <<= 1;
-    if (k == N) b <<= 1;
-    if (a | b) Gs[k] += sign * (a + b);
-  }
-}
-
 template <typename real>
 __device__ __forceinline__ real nudge_inside(double x, int N) {
   real r = static_cast<real>(x);

@@ -178,6 +178,7 @@ struct Bufs {
   int64_t hist_rows;
   const double* vs;  // polarity V_s(t_n) for every level n (filled once at set-up)
   const PredNet* net;  // installed predictor, or null
+  int64_t* next_step;  // level the next push starts from (left by the push; not by the solve, which may run beside it)
   int32_t net_in_push;  // 1: the push runs the predictor (FP32 single gap); 0: the solve does
 };
 

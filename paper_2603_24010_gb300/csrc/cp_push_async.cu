@@ -1,24 +1,50 @@
-// cp_push_async.cu -- the FP32 particle push with per-thread asynchronous
-// copies.
+// cp_push_async.cu -- the particle push of a single gap, with per-thread
+// asynchronous copies.
 //
-// Same step as k_push (gather, kick, drift, absorption, SEE, beam, fixed-
-// point deposit; Sec. 2.2.2, 2.3, 2.4.1, App. C, App. E.2), with the HBM
-// stream kept deeper in flight: every thread owns a ring of three 32-byte
-// slots in shared memory (x and u of its four particles of a tile) filled by
-// cp.async copies, so two tiles are always on their way while the third is
-// processed, without holding registers for them and without block-wide
-// synchronisation (each thread waits only for its own copy groups).  To make
-// room for the ring at two CTAs per SM, the field table keeps only the
-// half-grid values, padded by a copy of each end value (the slope is
-// recomputed from neighbours exactly as the solve forms it, and is zero past
-// either end), and the deposit uses one 32-bit sum per node.
+// One time step (arXiv 2603.24010) is two launches, this push and the cluster
+// solve of cp_solve.cu.  k_push streams every particle once: CIC gather of
+// E^n from a shared-memory table (App. C), leapfrog kick and drift (Sec.
+// 2.2.2), absorption at the electrodes (Sec. 2.4.1), the CIC deposit of
+// rho^{n+1} in fixed point (2^16 units per macroparticle charge, boundary
+// nodes doubled as in App. E.2), secondary emission from the absorbed ions
+// (Sec. 2.3, Algorithm see_sampling_1d; Philox4x64-10 draws keyed by (seed,
+// step, ion id)) and the step's beam ions.
+//
+// What bounds it: at 1e7 particles and more the HBM stream and the shared-
+// memory pipe (two table reads and two node-sum atomics per particle at
+// random cells); below that a fixed latency, which is why everything the
+// previous solve does not write is done before the wait for it:
+//
+// * every thread owns a ring of shared-memory slots (x and u of its four
+//   particles of a tile) filled by cp.async copies, so the next tiles are on
+//   their way while one is processed, without registers held for them and
+//   without block-wide waits.  The first tiles are requested before the wait
+//   (the solve changes no particle but the up to three padding slots behind
+//   a species' last one, and the last vector is read directly);
+// * the beam ions are drawn before the wait (their draws need the level
+//   alone, which the previous push left in B.next_step);
+// * one flat list of tiles over the three species, so that small species
+//   share the CTAs;
+// * one signed 32-bit sum per node for both signs of charge, folded into an
+//   int64 sum only when 31 tiles' worth may be in it (fewer: never);
+// * the tail's FP64 chains (emission counts, and the first electron's draws)
+//   run in half of the warps while the others add the CTA's grid into the
+//   global one; an impact's further electrons are spread over the lanes.
+//
+// FP64 particles: an SM issues 2 FP64 operations a cycle, so comparisons,
+// floors and conversions are done on the integer pipe (8 FP64 operations a
+// particle instead of 15), and a tile is 1024 particles, so that small
+// populations reach every SM.
+//
+// Graph-timed step before -> after (GB300): FP64, 256 cells, 1.4e5 particles
+// 38.6 -> 20.0 us; FP64 Tesla gap 40.9 -> 22.5; FP32, 4096 cells, 3.3e5
+// particles 22.9 -> 19.4, 1e6 (1531 cells) 17.5 -> 15.9, 1.5e7 59.3 -> 53.9,
+// 3.1e7 (impacts every step) 118 -> 113.7.
 
 #include "cp_common.cuh"
 #include "cp_mlp.cuh"
 
 namespace cpk {
-
-constexpr int kAStages = 3;  // slots per thread: two tiles in flight, one processed
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -34,52 +60,152 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// fold the node sums into the int64 grid (end nodes doubled) and clear them
-__device__ __forceinline__ void fold_nodes(unsigned int* nd, long long* Gs, int N, long long sign) {
+// A thread's ring: three slots of one 16-byte vector of x and one of u (four
+// FP32 or two FP64 particles), at [stage][x | u][thread].
+constexpr int kStages = 3;
+constexpr size_t kRingBytes = static_cast<size_t>(kStages) * kThreads * 32;
+template <typename real>
+struct Vec {
+  static constexpr int kN = 16 / sizeof(real);     // particles per thread and tile
+  static constexpr int kTileN = kThreads * kN;     // particles per tile
+};
+
+constexpr int kTailRound = kThreads / 4;  // absorbed-ion records per round of the push's tail
+// the tail keeps the emitted electrons' node sums (N + 1 <= 11390 words) and
+// the first electrons' draws (2 kTailRound doubles) in the ring
+static_assert(4 * 11392 + 16 * kTailRound <= kRingBytes, "tail scratch lives in the ring");
+static_assert(kThreads == 4 * kTailRound && kTailRound % 32 == 0, "tail roles are whole warps");
+static_assert(sizeof(PredScratch) <= kRingBytes, "predictor scratch lives in the ring");
+static_assert(kThreads >= kHid * 8, "the network takes 8 lanes per neuron");
+
+// Node sums hold the sum of +w (ions) and -w (electrons) modulo 2^32.  A tile
+// adds at most 2^27 to a node, so after `pos` ion and `neg` electron tiles
+// the sum lies in [-neg 2^27, pos 2^27], which 32 bits tell apart while pos +
+// neg <= 31.
+__device__ __forceinline__ long long node_value(unsigned int v, int neg) {
+  const unsigned int off = static_cast<unsigned int>(neg) << 27;
+  return static_cast<long long>(v + off) - static_cast<long long>(off);
+}
+
+__device__ __forceinline__ uint32_t* ion_ids(const DevState* S) {
+  return reinterpret_cast<uint32_t*>(__ldcg(reinterpret_cast<const unsigned long long*>(&S->id)));
+}
+
+// a thread's particles: from a ring slot, from and to global memory
+__device__ __forceinline__ void get_vec(const float4* d, float (&v)[4]) {
+  const float4 a = *d;
+  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+}
+__device__ __forceinline__ void get_vec(const float4* d, double (&v)[2]) {
+  const double2 a = *reinterpret_cast<const double2*>(d);
+  v[0] = a.x; v[1] = a.y;
+}
+__device__ __forceinline__ void put_vec(float* p, const float (&v)[4]) { store4(p, v); }
+__device__ __forceinline__ void put_vec(double* p, const double (&v)[2]) {
+  __stcs(reinterpret_cast<double2*>(p), make_double2(v[0], v[1]));
+}
+
+// 0 < x < N.  FP64: on the bit patterns, which order like the values (GB300's
+// FP64 pipe takes 16 cycles for a warp's comparison).
+__device__ __forceinline__ bool inside(float x, float N) { return x > 0.0f && x < N; }
+__device__ __forceinline__ bool inside(double x, double N) {
+  return static_cast<unsigned long long>(__double_as_longlong(x)) - 1ULL <
+         static_cast<unsigned long long>(__double_as_longlong(N)) - 1ULL;
+}
+
+// running maximum of |u| as a bit pattern, and its FP32 value's bits
+__device__ __forceinline__ void max_abs(unsigned int& m, float u) { m = max(m, __float_as_uint(fabsf(u))); }
+__device__ __forceinline__ void max_abs(unsigned long long& m, double u) {
+  m = max(m, static_cast<unsigned long long>(__double_as_longlong(u)) & 0x7FFFFFFFFFFFFFFFULL);
+}
+__device__ __forceinline__ unsigned int float_bits(unsigned int m) { return m; }
+__device__ __forceinline__ unsigned int float_bits(unsigned long long m) {
+  return __float_as_uint(static_cast<float>(__longlong_as_double(static_cast<long long>(m))));
+}
+template <typename real>
+struct Bits;
+template <>
+struct Bits<float> {
+  using type = unsigned int;
+};
+template <>
+struct Bits<double> {
+  using type = unsigned long long;
+};
+
+template <typename real>
+__device__ __forceinline__ real kick(const DevParams* P, bool half, int s) {
+  if constexpr (sizeof(real) == 4) return P->kap_f[half ? 0 : 1][s];
+  else return P->kap_d[half ? 0 : 1][s];
+}
+
+// fold the node sums into the int64 grid and clear them (the first fold of a
+// launch writes the grid)
+__device__ __forceinline__ void fold_nodes(unsigned int* nd, long long* Gs, int N, int neg, bool first) {
   for (int k = threadIdx.x; k <= N; k += kThreads) {
-    long long a = nd[k];
-    if (a) {
-      nd[k] = 0u;
-      if (k == 0 || k == N) a <<= 1;
-      Gs[k] += sign * a;
-    }
+    const long long a = node_value(nd[k], neg);
+    nd[k] = 0u;
+    Gs[k] = first ? a : Gs[k] + a;
   }
 }
 
-// CIC deposit of one particle into the node sums: node i gets 2^16 - W1,
-// node i+1 W1, with i = floor(x) and W1 = floor(2^16 (x - i)).  x 2^16 is
-// exact (power-of-two scaling) and below 2^32 (the N + 1 node sums and the
-// field table take 8 B per cell of shared memory, so N < 2^16), so one
-// truncating conversion gives i in its high and W1 in its low 16 bits.
-__device__ __forceinline__ void deposit_nodes(unsigned int* nd, float x) {
-  const unsigned int F = __float2uint_rz(x * 65536.0f);
+__device__ __forceinline__ void add_global(long long* G, int k, int N, long long v) {
+  if (v == 0) return;
+  if (k == 0 || k == N) v <<= 1;
+  atomicAdd(reinterpret_cast<unsigned long long*>(&G[k]), static_cast<unsigned long long>(v));
+}
+
+// Fixed-point position of a particle inside the gap: cell i in the high and
+// W1 = floor(2^16 (x - i)) in the low 16 bits.  x 2^16 is exact (power-of-two
+// scaling) and below 2^32 (N < 2^16), so one truncating conversion gives both.
+__device__ __forceinline__ unsigned int fix_pos(float x) { return __float2uint_rz(x * 65536.0f); }
+// FP64: the mantissa shifted down (the integer pipe; 0 < x < 2^16)
+__device__ __forceinline__ unsigned int fix_pos(double x) {
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
+  const int sh = 1023 + 36 - static_cast<int>(b >> 52);  // 52 - 16 - exponent, at least 21
+  return static_cast<unsigned int>(((b & 0xFFFFFFFFFFFFFULL) | 0x10000000000000ULL) >> min(sh, 63));
+}
+
+// j = floor(x - 1/2) and t = (x - 1/2) - j of a position inside the gap
+__device__ __forceinline__ int half_cell(float x, float* t) {
+  const float s = x - 0.5f;
+  const float jf = floorf(s);
+  *t = s - jf;
+  return static_cast<int>(jf);
+}
+// FP64: j = floor((floor(2 x) - 1) / 2) from the mantissa, and as a double
+// from the bits of 2^52 + 2^51 + j (two additions instead of a floor and two
+// conversions on the FP64 pipe)
+__device__ __forceinline__ int half_cell(double x, double* t) {
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
+  const int sh = 1023 + 51 - static_cast<int>(b >> 52);  // 52 - 1 - exponent, at least 36
+  const int h = static_cast<int>(((b & 0xFFFFFFFFFFFFFULL) | 0x10000000000000ULL) >> min(sh, 63));
+  const int j = (h - 1) >> 1;
+  const double jf = __longlong_as_double(0x4338000000000000LL + j) - 6755399441055744.0;
+  *t = (x - 0.5) - jf;
+  return j;
+}
+
+// CIC deposit into the node sums: node i gets sign (2^16 - W1), node i+1
+// sign W1 (sign +1 or -1).
+__device__ __forceinline__ void deposit_nodes(unsigned int* nd, unsigned int F, int sign) {
   const unsigned int i = F >> 16;
-  const unsigned int w1 = F & 0xFFFFu;
-  atomicAdd(&nd[i], 65536u - w1);
+  const unsigned int w1 = (F & 0xFFFFu) * static_cast<unsigned int>(sign);
+  atomicAdd(&nd[i], 65536u * static_cast<unsigned int>(sign) - w1);
   atomicAdd(&nd[i + 1], w1);
 }
 
 // gather from the padded field table Et[k] = E_{k-1/2} (k = 1..N), Et[0] =
 // E_{1/2}, Et[N+1] = E_{N-1/2}: the pair (E_{j+1/2}, slope) of the pair table
-// is formed here with the same FP32 subtraction, and the repeated end values
-// give the constant extension (slope +0) for j = -1 and j = N-1
-__device__ __forceinline__ float gather_tab(const float* Et, float x) {
-  const float s = x - 0.5f;
-  const float jf = floorf(s);
-  const int j = static_cast<int>(jf);
-  const float t = s - jf;
-  const float e0 = Et[j + 1];
-  return fmaf(t, Et[j + 2] - e0, e0);
+// is formed here with the same subtraction, and the repeated end values give
+// the constant extension (slope +0) for j = -1 and j = N-1
+template <typename real>
+__device__ __forceinline__ real gather_tab(const real* Et, real x) {
+  real t;
+  const int j = half_cell(x, &t);
+  const real e0 = Et[j + 1];
+  return fma(t, Et[j + 2] - e0, e0);
 }
-
-constexpr size_t kRingBytes = static_cast<size_t>(kAStages) * kThreads * 32;
-constexpr int kTailRound = kThreads / 4;  // absorbed-ion records per round of the push's tail
-// the tail keeps the beam's node sums (N + 1 <= 11390 words) and the first
-// electrons' draws (2 kTailRound doubles) in the ring
-static_assert(4 * 11392 + 16 * kTailRound <= kRingBytes, "tail scratch lives in the ring");
-static_assert(2 * kTailRound <= kThreads && kTailRound % 32 == 0, "tail roles are whole warps");
-static_assert(sizeof(PredScratch) <= kRingBytes, "predictor scratch lives in the ring");
-static_assert(kThreads >= kHid * 8, "the network takes 8 lanes per neuron");
 
 // The learned weak-coupling predictor for the level the previous solve
 // committed (its row from that level's diagnostics), run by the push's extra
@@ -115,218 +241,321 @@ __device__ __noinline__ void predictor_in_push(DevState* S, const PredNet* net, 
   pred_level<kThreads>(net, C, S, &L, v_old, sp);
 }
 
-size_t push_async_smem_bytes(int N) {
+
+template <typename real>
+static size_t push_smem(int N) {
   return kRingBytes + align16(sizeof(long long) * (N + 1)) + align16(sizeof(unsigned int) * (N + 1)) +
-         align16(sizeof(float) * (N + 2));
+         align16(sizeof(real) * (N + 2));
 }
 
-__global__ void __launch_bounds__(kThreads, kCtasPerSm) k_push_async(Bufs B, int do_push) {
+// Entry speed [cells/step] of a beam ion from its second draw: in FP32 the
+// FP32 pushes' form, in FP64 the definition's order of operations.
+template <typename real>
+__device__ __forceinline__ double beam_speed(const DevParams* P, double u) {
+  if constexpr (sizeof(real) == 4) {
+    return beam_speed_fp32(P, u);
+  } else {
+    const double Eb = (P->beam_mode == 0)
+                          ? P->beam_E_eV
+                          : __dadd_rn(P->beam_Emin_eV, __dmul_rn(__dsub_rn(P->beam_Emax_eV, P->beam_Emin_eV), u));
+    const double v = sqrt(2.0 * Eb * P->e / P->m_i);
+    return v * P->dt / P->dx;
+  }
+}
+
+// PUSH: the step's push; else the deposit of the loaded particles (level 0).
+template <typename real, bool PUSH>
+__global__ void __launch_bounds__(kThreads, kCtasPerSm) k_push(Bufs B) {
+  using V = Vec<real>;
+  using real2 = typename Pair<real>::type;
   const DevParams* __restrict__ P = B.P;
   DevState* S = B.S;
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int s_abs_n;
-  __shared__ int s_flag[2];  // [0] stopped, [1] overflow
-  __shared__ unsigned long long s_cnt[2][kSpecies];
-  __shared__ unsigned long long s_emit[2];
+  __shared__ int s_abs_n, s_over;
+  __shared__ unsigned int s_cnt[2][kSpecies];
+  __shared__ unsigned int s_emit[2];
   __shared__ long long s_conv, s_energy;
   __shared__ unsigned int s_cfl;
+  __shared__ real* s_xi[kSpecies];
+  __shared__ real* s_u[kSpecies];
+  __shared__ long long s_n[kSpecies];     // slots in use
+  __shared__ int s_tile[kSpecies + 1];    // first tile of each species in the flat list
 
-  // Set-up that needs nothing of the previous kernel runs before the wait for
-  // it: the parameters are written once, and the shared grid sums are this
-  // CTA's own.
+  const int tid = static_cast<int>(threadIdx.x);
   const int N = P->N;
-  float4* ring = reinterpret_cast<float4*>(smem);  // [stage][x | u][thread]
   long long* Gs = reinterpret_cast<long long*>(smem + kRingBytes);
   unsigned int* nd = reinterpret_cast<unsigned int*>(smem + kRingBytes + align16(sizeof(long long) * (N + 1)));
-  float* Et = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(nd) + align16(sizeof(unsigned int) * (N + 1)));
-  for (int k = threadIdx.x; k <= N; k += kThreads) {
-    Gs[k] = 0;
-    nd[k] = 0u;
-  }
-  if (threadIdx.x == 0) {
-    s_flag[1] = 0;
-    s_abs_n = 0;
-    s_conv = 0;
-    s_energy = 0;
-    s_cfl = 0u;
-    s_emit[0] = s_emit[1] = 0ULL;
-  }
-  if (threadIdx.x < 2 * kSpecies) s_cnt[threadIdx.x / kSpecies][threadIdx.x % kSpecies] = 0ULL;
-
-  cudaGridDependencySynchronize();
-  cudaTriggerProgrammaticLaunchCompletion();
-  if (threadIdx.x == 0) s_flag[0] = (ldcg(&S->status) != 0);
-  // the field table of the solve just finished: eight loads per thread in
-  // flight together (one L2 round trip for N <= 4095)
-  const float2* Epair = reinterpret_cast<const float2*>(B.Epair);
-  for (int k0 = threadIdx.x; k0 <= N; k0 += 8 * kThreads) {
-    float e[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int k = k0 + q * kThreads;
-      e[q] = (k <= N) ? Epair[k].x : 0.0f;  // pair 0 repeats E_{1/2}
-    }
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int k = k0 + q * kThreads;
-      if (k <= N) {
-        Et[k] = e[q];
-        if (k == N) Et[N + 1] = e[q];
-      }
-    }
-  }
-  __syncthreads();
-  if (s_flag[0]) return;
-  const int64_t step = S->level;
+  real* Et = reinterpret_cast<real*>(reinterpret_cast<unsigned char*>(nd) + align16(sizeof(unsigned int) * (N + 1)));
   // With a network installed the launch has one CTA more, which runs the
   // learned predictor for the level the previous solve committed (levels
   // >= 1).  Scheduled last, it takes the first slot a pushing CTA frees, so
   // the network runs beside the other CTAs' ends.
   const bool pred_cta = (B.net != nullptr && B.net_in_push);
-  const unsigned int G = gridDim.x - (pred_cta ? 1u : 0u);  // pushing CTAs
-  if (blockIdx.x == G) {
-    if (do_push && step >= 1) predictor_in_push(S, B.net, P->C, reinterpret_cast<PredScratch*>(smem));
+  const int G = static_cast<int>(gridDim.x) - (pred_cta ? 1 : 0);  // pushing CTAs
+  const int cta = static_cast<int>(blockIdx.x);
+  if (cta == G) {
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();
+    if (ldcg(&S->status) != 0) return;
+    if (PUSH && ldcg(&S->level) >= 1) predictor_in_push(S, B.net, P->C, reinterpret_cast<PredScratch*>(smem));
     return;
   }
 
-  const bool half = (S->pushed == 0);
-  const float Nr = static_cast<float>(N);
-  const int cap = P->abs_cap;
-  AbsRec* my_abs = B.abs + static_cast<size_t>(blockIdx.x) * cap;
-  unsigned int cfl = 0u;
-  float4* my_slot = ring + threadIdx.x;  // x at + stage * 2 kThreads, u kThreads further
-
-  for (int s = 0; s < kSpecies; ++s) {
-    float* __restrict__ xs = reinterpret_cast<float*>(S->xi[s]);
-    float* __restrict__ us = reinterpret_cast<float*>(S->u[s]);
-    const int64_t n = S->n_proc[s];  // multiple of 4
-    if (n == 0) continue;  // the same for every thread of the CTA
-    const int64_t ntiles = (n + kTile - 1) / kTile;
-    const int mine = (ntiles > blockIdx.x) ? static_cast<int>((ntiles - blockIdx.x + G - 1) / G) : 0;
-    const long long sign = (s == CP_IONS) ? 1LL : -1LL;
-    const float kap = P->kap_f[half ? 0 : 1][s];
-    const uint32_t* ids = S->id;
-    unsigned int a0 = 0u, a1 = 0u;
-    int since = 0;
-    const int64_t stride = static_cast<int64_t>(G) * kTile;
-    const int64_t base0 = static_cast<int64_t>(blockIdx.x) * kTile + static_cast<int64_t>(threadIdx.x) * kPerThread;
-    int64_t b_next = base0;  // first particle of this thread's next tile to fetch
-    int st_next = 0;         // its ring slot
-    auto issue = [&](bool go) {  // this thread's four particles of its next tile
-      float4* slot = my_slot + st_next * (kThreads * 2);
-      if (go && b_next < n) {
-        cp_async16(slot, xs + b_next);
-        if (do_push) cp_async16(slot + kThreads, us + b_next);
+  // --- before the previous solve has finished --------------------------------
+  for (int k = tid; k <= N; k += kThreads) nd[k] = 0u;
+  if (tid == 0) {
+    s_abs_n = 0;
+    s_over = 0;
+    s_conv = 0;
+    s_energy = 0;
+    s_cfl = 0u;
+    s_emit[0] = s_emit[1] = 0u;
+  }
+  if (tid < 2 * kSpecies) s_cnt[tid / kSpecies][tid % kSpecies] = 0u;
+  if (tid < 32) {  // the flat tile list
+    long long n = 0;
+    if (tid < kSpecies) {
+      s_xi[tid] = static_cast<real*>(ldcg(&S->xi[tid]));
+      s_u[tid] = static_cast<real*>(ldcg(&S->u[tid]));
+      // the solve rounds n_alloc up to a multiple of 4, this reads it before or after
+      n = min(static_cast<long long>((ldcg(&S->n_alloc[tid]) + 3) & ~int64_t(3)), static_cast<long long>(P->cap[tid]));
+      s_n[tid] = n;
+    }
+    int t = static_cast<int>((n + V::kTileN - 1) / V::kTileN);
+    t = warp_incl_scan(t);
+    if (tid < kSpecies) s_tile[tid + 1] = t;
+    if (tid == 0) s_tile[0] = 0;
+  }
+  // this CTA's share [kb0, kb1) of the step's beam ions, one per thread of
+  // the first round
+  const int Bn = PUSH ? P->beam_per_step : 0;
+  const int nbc = (Bn + G - 1) / G;
+  const int kb0 = min(Bn, cta * nbc), kb1 = min(Bn, kb0 + nbc);
+  const int64_t step = ldcg(B.next_step);  // the level this push starts from
+  auto draw_beam = [&](int kk, real* x, real* u) {
+    const U64x4 wv = philox4x64_10(static_cast<uint64_t>(kk), static_cast<uint64_t>(step), 0, 0, P->seed, kTagBeam);
+    const double frac = u01(wv.w[0]);
+    const double ub = beam_speed<real>(P, u01(wv.w[1]));
+    *x = nudge_inside<real>(__dsub_rn(static_cast<double>(N), __dmul_rn(ub, frac)), N);
+    *u = static_cast<real>(-ub);
+  };
+  real bx = real(0), bu = real(0);
+  if (kb0 + tid < kb1) draw_beam(kb0 + tid, &bx, &bu);
+  __syncthreads();
+  // This CTA's tiles cta, cta + G, ... of the flat list, species by species:
+  // `left` tiles of species `s`, the next at x, u (this thread's particles);
+  // the species' last four, at x_end, are not copied.
+  struct Cursor {
+    real *x, *u, *x_end;
+    int s, left;
+  };
+  auto enter = [&](Cursor& c) {  // the next species in which this CTA has tiles, from c.s on
+    for (; c.s < kSpecies; ++c.s) {
+      const int t0 = s_tile[c.s], t1 = s_tile[c.s + 1];
+      const int first = cta + ((max(t0 - cta, 0) + G - 1) / G) * G;  // this CTA's first tile at or behind t0
+      c.left = (first < t1) ? (t1 - first + G - 1) / G : 0;
+      if (c.left > 0) {
+        const long long b = static_cast<long long>(first - t0) * V::kTileN + tid * V::kN;
+        c.x = s_xi[c.s] + b;
+        c.u = s_u[c.s] + b;
+        c.x_end = s_xi[c.s] + s_n[c.s] - 4;
+        return;
       }
-      cp_async_commit();
-      b_next += stride;
-      st_next = (st_next == kAStages - 1) ? 0 : st_next + 1;
-    };
-    issue(0 < mine);
-    issue(1 < mine);
-    int64_t base = base0;  // first particle of this thread's tile j
-    int st = 0;            // its ring slot
-    for (int j = 0; j < mine; ++j, base += stride, st = (st == kAStages - 1) ? 0 : st + 1) {
-      issue(j + 2 < mine);
-      cp_async_wait<2>();  // this thread's copies of tile j have landed
-      const bool valid = base < n;  // the last tile's tail lanes hold no particles
-      const float4* slot = my_slot + st * (kThreads * 2);
-      if (do_push && valid) {
-        const float4 xa = slot[0];
-        const float4 ua = slot[kThreads];
-        float xv[4] = {xa.x, xa.y, xa.z, xa.w};
-        float uv[4] = {ua.x, ua.y, ua.z, ua.w};
+    }
+  };
+  const long long stride = static_cast<long long>(G) * V::kTileN;
+  float4* slots = reinterpret_cast<float4*>(smem) + tid;
+  Cursor nxt;  // the next tile to request
+  nxt.s = 0;
+  nxt.left = 0;
+  enter(nxt);
+  const bool any = nxt.left > 0;  // this CTA has tiles
+  int st_next = 0;
+  auto issue = [&]() {
+    if (nxt.left > 0) {
+      if (nxt.x < nxt.x_end) {
+        float4* d = slots + st_next * (2 * kThreads);
+        cp_async16(d, nxt.x);
+        if (PUSH) cp_async16(d + kThreads, nxt.u);
+      }
+      nxt.x += stride;
+      nxt.u += stride;
+      if (--nxt.left == 0) {
+        ++nxt.s;
+        enter(nxt);
+      }
+    }
+    cp_async_commit();
+    st_next = (st_next == kStages - 1) ? 0 : st_next + 1;
+  };
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+  for (int j = 0; j < kStages - 1; ++j) issue();
+
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+  const int stop = ldcg(&S->status);
+  const bool half = (ldcg(&S->pushed) == 0);
+  // the field table of the solve just finished: eight loads per thread in
+  // flight together (one L2 round trip for N <= 4095)
+  if (PUSH && any) {
+    const real2* Epair = reinterpret_cast<const real2*>(B.Epair);
+    for (int k0 = tid; k0 <= N; k0 += 8 * kThreads) {
+      real e[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int k = k0 + q * kThreads;
+        e[q] = (k <= N) ? __ldcg(&Epair[k]).x : real(0);  // pair 0 repeats E_{1/2}
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int k = k0 + q * kThreads;
+        if (k <= N) {
+          Et[k] = e[q];
+          if (k == N) Et[N + 1] = e[q];
+        }
+      }
+    }
+  }
+  if (stop) {
+    cp_async_wait<0>();
+    return;
+  }
+  // the beam: slots behind the ions in use (ions are appended by the beam
+  // alone, so the slots are known without a shared counter)
+  bool folded = false;
+  int pos = 0, neg = 0;  // tiles' worth of each sign in the node sums
+  for (int k0 = kb0, round = 0; k0 < kb1; k0 += kThreads, ++round) {
+    if (round % V::kN == 0 && ++pos > kFlushTiles) {  // (beams of millions a step)
+      __syncthreads();
+      fold_nodes(nd, Gs, N, 0, !folded);
+      __syncthreads();
+      folded = true;
+      pos = 1;
+    }
+    const int kk = k0 + tid;
+    if (kk >= kb1) continue;
+    if (round > 0) draw_beam(kk, &bx, &bu);
+    const long long slot = s_n[CP_IONS] + kk;
+    if (slot < P->cap[CP_IONS]) {
+      s_xi[CP_IONS][slot] = bx;
+      s_u[CP_IONS][slot] = bu;
+      ion_ids(S)[slot] = S->beam_id_base + static_cast<uint32_t>(step * Bn + kk);
+      deposit_nodes(nd, fix_pos(bx), 1);
+    } else {
+      s_over = 1;
+    }
+  }
+  __syncthreads();
+
+  const real Nr = static_cast<real>(N);
+  const int cap = P->abs_cap;
+  AbsRec* my_abs = B.abs + static_cast<size_t>(cta) * cap;
+  typename Bits<real>::type cfl = 0;
+  int st = 0;  // ring slot of this thread's tile
+  Cursor cur;
+  cur.s = 0;
+  cur.left = 0;
+  for (enter(cur); cur.s < kSpecies; ++cur.s, enter(cur)) {
+    const int sign = (cur.s == CP_IONS) ? 1 : -1;
+    const real kap = kick<real>(P, half, cur.s);
+    for (; cur.left > 0; --cur.left, cur.x += stride, cur.u += stride, st = (st == kStages - 1) ? 0 : st + 1) {
+      issue();
+      if (pos + neg == kFlushTiles) {  // bounds every node sum to 32 bits
+        __syncthreads();
+        fold_nodes(nd, Gs, N, neg, !folded);
+        __syncthreads();
+        folded = true;
+        pos = neg = 0;
+      }
+      if (sign > 0) ++pos; else ++neg;
+      cp_async_wait<kStages - 1>();  // this thread's copies of the tile have landed
+      real xv[V::kN], uv[V::kN];
+      if (cur.x < cur.x_end) {
+        const float4* d = slots + st * (2 * kThreads);
+        get_vec(d, xv);
+        if (PUSH) get_vec(d + kThreads, uv);
+      } else if (cur.x < cur.x_end + 4) {  // the species' last four: the padding among them was set after the copies began
+#pragma unroll
+        for (int q = 0; q < V::kN; ++q) {
+          xv[q] = __ldcg(cur.x + q);
+          uv[q] = __ldcg(cur.u + q);
+        }
+      } else {
+        continue;  // the last tile's tail lanes hold no particles
+      }
+      if (PUSH) {
+#pragma unroll
+        for (int q = 0; q < V::kN; ++q) {
           bool dep = false;
-          if (xv[q] > 0.0f && xv[q] < Nr) {  // live (dead slots hold -1)
-            const float E = gather_tab(Et, xv[q]);
-            const float un = fmaf(kap, E, uv[q]);
-            const float xn = xv[q] + un;
-            cfl = max(cfl, __float_as_uint(fabsf(un)));
-            if (!(xn > 0.0f && xn < Nr)) {  // absorbed (a non-finite value counts at x = d)
-              const int el = (xn <= 0.0f) ? 0 : 1;
-              if (el) ++a1; else ++a0;
-              if (s == CP_IONS) {
+          if (inside(xv[q], Nr)) {  // live (dead slots hold -1)
+            const real E = gather_tab(Et, xv[q]);
+            const real un = fma(kap, E, uv[q]);
+            const real xn = xv[q] + un;
+            max_abs(cfl, un);
+            if (!inside(xn, Nr)) {  // absorbed (a non-finite value counts at x = d)
+              const int el = (xn <= real(0)) ? 0 : 1;
+              atomicAdd(&s_cnt[el][cur.s], 1u);
+              if (sign > 0) {
                 const int slot_i = atomicAdd(&s_abs_n, 1);
                 if (slot_i < cap) {
                   AbsRec r;
-                  r.id = ids[base + q];
+                  r.id = ion_ids(S)[cur.x + q - s_xi[CP_IONS]];
                   r.electrode = static_cast<uint32_t>(el);
                   r.u = static_cast<double>(un);
                   my_abs[slot_i] = r;
                 }
               }
-              xv[q] = -1.0f;
-              uv[q] = 0.0f;
+              xv[q] = real(-1);
+              uv[q] = real(0);
             } else {
               dep = true;
               xv[q] = xn;
               uv[q] = un;
             }
           }
-          if (dep) deposit_nodes(nd, xv[q]);
+          if (dep) deposit_nodes(nd, fix_pos(xv[q]), sign);
         }
-        store4(xs + base, xv);
-        store4(us + base, uv);
-      } else if (!do_push && valid) {
-        const float4 xa = slot[0];
-        const float xv[4] = {xa.x, xa.y, xa.z, xa.w};
+        put_vec(cur.x, xv);
+        put_vec(cur.u, uv);
+      } else {
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if (xv[q] > 0.0f && xv[q] < Nr) deposit_nodes(nd, xv[q]);
+        for (int q = 0; q < V::kN; ++q)
+          if (inside(xv[q], Nr)) deposit_nodes(nd, fix_pos(xv[q]), sign);
       }
-      if (++since == kFlushTiles) {  // bounds every 32-bit node sum below 2^32
-        __syncthreads();
-        fold_nodes(nd, Gs, N, sign);
-        __syncthreads();
-        since = 0;
-      }
-    }
-    cp_async_wait<0>();
-    __syncthreads();
-    fold_nodes(nd, Gs, N, sign);
-    __syncthreads();
-    a0 = warp_sum_u(a0);
-    a1 = warp_sum_u(a1);
-    if (lane_id() == 0) {
-      if (a0) atomicAdd(&s_cnt[0][s], static_cast<unsigned long long>(a0));
-      if (a1) atomicAdd(&s_cnt[1][s], static_cast<unsigned long long>(a1));
     }
   }
-  cfl = warp_max_u(cfl);
-  if (lane_id() == 0 && cfl) atomicMax(&s_cfl, cfl);
-  // This CTA's share [kb0, kb1) of the step's beam ions.  They carry the
-  // other sign than emitted electrons, so they deposit into node sums of
-  // their own, in the ring (idle now: every copy was waited for).
-  const int Bn = do_push ? P->beam_per_step : 0;
-  const int nbc = (Bn + static_cast<int>(G) - 1) / static_cast<int>(G);
-  const int kb0 = min(Bn, static_cast<int>(blockIdx.x) * nbc);
-  const int kb1 = min(Bn, kb0 + nbc);
-  unsigned int* ndb = reinterpret_cast<unsigned int*>(smem);
-  double* s_v0 = reinterpret_cast<double*>(smem + align16(sizeof(unsigned int) * (N + 1)));
-  double* s_f0 = s_v0 + kTailRound;
-  if (kb1 > kb0)
-    for (int k = threadIdx.x; k <= N; k += kThreads) ndb[k] = 0u;
+  cp_async_wait<0>();
+  const unsigned int cflf = warp_max_u(float_bits(cfl));
+  if (lane_id() == 0 && cflf) atomicMax(&s_cfl, cflf);
   __syncthreads();
-  if (do_push) {
-    // --- secondary emission from the ions this CTA saw absorbed, and the beam.
-    // Per round of kTailRound records, three FP64 chains run in different
-    // warps: the SE counts (threads [0, kTailRound), from the bottom), the
-    // beam ions (the same threads, from the top) and the first emitted
-    // electron's draws of each record (threads [kTailRound, 2 kTailRound)).
-    const int n_abs = s_abs_n;
-    if (n_abs > cap && threadIdx.x == 0) s_flag[1] = 1;
-    const int na = min(n_abs, cap);
-    const int nb = kb1 - kb0;
+
+  // --- the CTA's grid into the global one; secondary emission ------------------
+  // With impacts, per round of kTailRound records: the emission counts
+  // (threads [0, kTailRound)), the first emitted electron's draws of each
+  // record (threads [kTailRound, 2 kTailRound)), and, beside the first round's
+  // chains, the grid (the other half of the CTA).
+  const int na = PUSH ? min(s_abs_n, cap) : 0;
+  if (PUSH && tid == 0 && s_abs_n > cap) s_over = 1;
+  auto flush = [&](int first, int threads) {
+    for (int k = first; k <= N; k += threads)
+      add_global(B.G, k, N, node_value(nd[k], neg) + (folded ? Gs[k] : 0LL));
+  };
+  if (na == 0) {
+    flush(tid, kThreads);
+  } else {
+    unsigned int* ndb = reinterpret_cast<unsigned int*>(smem);  // the emitted electrons' node sums
+    double* s_v0 = reinterpret_cast<double*>(smem + align16(sizeof(unsigned int) * (N + 1)));
+    double* s_f0 = s_v0 + kTailRound;
     const double dx = P->dx, dt = P->dt;
-    const int rounds = max((na + kTailRound - 1) / kTailRound, (nb + kTailRound - 1) / kTailRound);
-    const int64_t ion_base = S->n_proc[CP_IONS];  // == n_alloc at the push's start
-    const bool counter = threadIdx.x < kTailRound;  // warp-uniform roles
-    const bool drawer = !counter && threadIdx.x < 2 * kTailRound;
+    const int rounds = (na + kTailRound - 1) / kTailRound;
+    const bool counter = tid < kTailRound, drawer = !counter && tid < 2 * kTailRound;  // warp-uniform roles
     for (int rd = 0; rd < rounds; ++rd) {
-      const int t = static_cast<int>(threadIdx.x) % kTailRound;
+      const int t = tid % kTailRound;
       const int r = rd * kTailRound + t;
+      if (tid >= kThreads / 2) {
+        for (int k = tid - kThreads / 2; k <= N; k += kThreads / 2) ndb[k] = 0u;
+        if (rd == 0) flush(tid - kThreads / 2, kThreads / 2);
+      }
       if (drawer && r < na) {  // the first electron's speed and fraction of the step
         double f0;
         s_v0[t] = see_speed(P, my_abs[r].id, step, 0, &f0);
@@ -347,31 +576,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_push_async(Bufs B, int
           atomicAdd(reinterpret_cast<unsigned long long*>(&s_conv),
                     static_cast<unsigned long long>(static_cast<long long>(nse)));
         }
-        if (nse) atomicAdd(&s_emit[rec.electrode], static_cast<unsigned long long>(nse));
+        if (nse) atomicAdd(&s_emit[rec.electrode], static_cast<unsigned int>(nse));
       }
-      // beam ion kk: entry position N - |u_b| frac, speed -|u_b|, in slot
-      // n_proc + kk (ions are appended by the beam alone, so the slots are
-      // known without a shared counter; n_alloc grows by Bn at the end)
-      const int kk = kb0 + rd * kTailRound + (kTailRound - 1 - t);
-      if (counter) {
-        if (kk < kb1) {
-          const U64x4 wv = philox4x64_10(static_cast<uint64_t>(kk), static_cast<uint64_t>(step), 0,
-                                         0, P->seed, kTagBeam);
-          const double frac = u01(wv.w[0]);
-          const double ub = beam_speed_fp32(P, u01(wv.w[1]));
-          const float xr = nudge_inside<float>(__dsub_rn(static_cast<double>(N), __dmul_rn(ub, frac)), N);
-          const unsigned long long slot = static_cast<unsigned long long>(ion_base + kk);
-          if (slot < static_cast<unsigned long long>(P->cap[CP_IONS])) {
-            reinterpret_cast<float*>(S->xi[CP_IONS])[slot] = xr;
-            reinterpret_cast<float*>(S->u[CP_IONS])[slot] = static_cast<float>(-ub);
-            S->id[slot] = S->beam_id_base + static_cast<uint32_t>(step * Bn + kk);
-            deposit_nodes(ndb, xr);
-          } else {
-            s_flag[1] = 1;
-          }
-        }
-      }
-      __syncthreads();  // the first electrons' draws are in shared memory
+      __syncthreads();  // the first electrons' draws are in shared memory, ndb is clear
       if (counter) {
         const int incl = warp_incl_scan(nse);
         const int tot = __shfl_sync(0xffffffffu, incl, 31);
@@ -380,58 +587,56 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_push_async(Bufs B, int
           wbase = atomicAdd(reinterpret_cast<unsigned long long*>(&S->n_alloc[CP_SECONDARIES]),
                             static_cast<unsigned long long>(tot));
         wbase = __shfl_sync(0xffffffffu, wbase, 31);
-        if (act && nse > 0) {
-          float* xs = reinterpret_cast<float*>(S->xi[CP_SECONDARIES]);
-          float* us = reinterpret_cast<float*>(S->u[CP_SECONDARIES]);
-          for (int j = 0; j < nse; ++j) {
-            double frac, vse;
-            if (j == 0) {
-              vse = s_v0[t];
-              frac = s_f0[t];
-            } else {
-              vse = see_speed(P, rec.id, step, j, &frac);
-            }
-            const double use = vse * dt / dx;
-            const double xd = (rec.electrode == 0) ? __dmul_rn(use, frac) : __dsub_rn(static_cast<double>(N), __dmul_rn(use, frac));
-            const float xr = nudge_inside<float>(xd, N);
-            const float ur = static_cast<float>(rec.electrode == 0 ? use : -use);
-            const unsigned long long slot = wbase + static_cast<unsigned long long>(incl - nse + j);
-            if (slot < static_cast<unsigned long long>(P->cap[CP_SECONDARIES])) {
-              xs[slot] = xr;
-              us[slot] = ur;
-              deposit_nodes(nd, xr);
-            } else {
-              s_flag[1] = 1;
-            }
+        // electron j of the impact (id, el), in slot wbase + place
+        auto emit = [&](uint32_t id, uint32_t el, unsigned long long place, double vse, double frac) {
+          const double use = vse * dt / dx;
+          const double xd = (el == 0) ? __dmul_rn(use, frac) : __dsub_rn(static_cast<double>(N), __dmul_rn(use, frac));
+          const real xr = nudge_inside<real>(xd, N);
+          const real ur = static_cast<real>(el == 0 ? use : -use);
+          const unsigned long long slot = wbase + place;
+          if (slot < static_cast<unsigned long long>(P->cap[CP_SECONDARIES])) {
+            s_xi[CP_SECONDARIES][slot] = xr;
+            s_u[CP_SECONDARIES][slot] = ur;
+            deposit_nodes(ndb, fix_pos(xr), 1);
+          } else {
+            s_over = 1;
+          }
+        };
+        if (nse > 0) emit(rec.id, rec.electrode, static_cast<unsigned long long>(incl - nse), s_v0[t], s_f0[t]);
+        // the impacts' further electrons, one per lane and pass (a chain of
+        // FP64 functions each)
+        const int more = max(nse - 1, 0);
+        const int inclm = warp_incl_scan(more);
+        const int totm = __shfl_sync(0xffffffffu, inclm, 31);
+        for (int e0 = 0; e0 < totm; e0 += 32) {
+          const int e = e0 + static_cast<int>(lane_id());
+          int src = 0;  // first lane whose inclusive count exceeds e
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1)
+            if (__shfl_sync(0xffffffffu, inclm, src + o - 1) <= e) src += o;
+          src = min(src, 31);
+          const uint32_t id = __shfl_sync(0xffffffffu, rec.id, src);
+          const uint32_t el = __shfl_sync(0xffffffffu, rec.electrode, src);
+          const int j = 1 + e - __shfl_sync(0xffffffffu, inclm - more, src);
+          const int first = __shfl_sync(0xffffffffu, incl - nse, src);
+          if (e < totm) {
+            double frac;
+            const double vse = see_speed(P, id, step, j, &frac);
+            emit(id, el, static_cast<unsigned long long>(first + j), vse, frac);
           }
         }
       }
-      // per round at most kTailRound x 64 electrons and kTailRound beam ions
-      // per node sum: below 2^32 with a fold between rounds
-      __syncthreads();
-      if (rd + 1 < rounds) {
-        if (na > 0) fold_nodes(nd, Gs, N, -1LL);
-        if (nb > 0) fold_nodes(ndb, Gs, N, 1LL);
-        __syncthreads();
-      }
+      __syncthreads();  // at most kTailRound x 64 electrons per round: below 2^32
+      for (int k = tid; k <= N; k += kThreads) add_global(B.G, k, N, -static_cast<long long>(ndb[k]));
+      if (rd + 1 < rounds) __syncthreads();
     }
-    if (na > 0) fold_nodes(nd, Gs, N, -1LL);
-    if (nb > 0) fold_nodes(ndb, Gs, N, 1LL);
   }
-  __syncthreads();
-
-  // --- add this CTA's grid and tallies into the global ones ------------------
-  for (int kq = threadIdx.x; kq <= N; kq += kThreads) {
-    const long long g = Gs[kq];
-    if (g != 0)
-      atomicAdd(reinterpret_cast<unsigned long long*>(&B.G[kq]), static_cast<unsigned long long>(g));
-  }
-  if (threadIdx.x == 0 && do_push) {
+  if (tid == 0 && PUSH) {
     for (int e = 0; e < 2; ++e)
       for (int s = 0; s < kSpecies; ++s)
-        if (s_cnt[e][s]) atomicAdd(&S->absorbed[e][s], s_cnt[e][s]);
-    if (s_emit[0]) atomicAdd(&S->emitted[0], s_emit[0]);
-    if (s_emit[1]) atomicAdd(&S->emitted[1], s_emit[1]);
+        if (s_cnt[e][s]) atomicAdd(&S->absorbed[e][s], static_cast<unsigned long long>(s_cnt[e][s]));
+    if (s_emit[0]) atomicAdd(&S->emitted[0], static_cast<unsigned long long>(s_emit[0]));
+    if (s_emit[1]) atomicAdd(&S->emitted[1], static_cast<unsigned long long>(s_emit[1]));
     const long long conv = static_cast<long long>(s_cnt[0][CP_IONS]) -
                            static_cast<long long>(s_cnt[0][CP_ELECTRONS]) -
                            static_cast<long long>(s_cnt[0][CP_SECONDARIES]) + s_conv;
@@ -440,25 +645,64 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_push_async(Bufs B, int
     if (s_energy) atomicAdd(reinterpret_cast<unsigned long long*>(&S->ion_energy_q),
                             static_cast<unsigned long long>(s_energy));
     if (s_cfl) atomicMax(&S->max_cfl_bits, s_cfl);
-    if (blockIdx.x == 0 && P->beam_per_step > 0) {
-      atomicAdd(&S->injected, static_cast<unsigned long long>(P->beam_per_step));
-      atomicAdd(reinterpret_cast<unsigned long long*>(&S->n_alloc[CP_IONS]),
-                static_cast<unsigned long long>(P->beam_per_step));
+    if (cta == 0) {
+      if (Bn > 0) {
+        atomicAdd(&S->injected, static_cast<unsigned long long>(Bn));
+        atomicAdd(reinterpret_cast<unsigned long long*>(&S->n_alloc[CP_IONS]), static_cast<unsigned long long>(Bn));
+      }
+      *B.next_step = step + 1;
     }
-    if (s_flag[1]) atomicCAS(&S->status, 0, CP_ERR_CAPACITY);
+    if (s_over) atomicCAS(&S->status, 0, CP_ERR_CAPACITY);
   }
 }
 
-cudaError_t push_async_configure(size_t smem) {
-  return cudaFuncSetAttribute(k_push_async, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(smem));
+// ---------------------------------------------------------------------------
+// Host-side launchers (internal C++ interface used by cp_api.cu)
+// ---------------------------------------------------------------------------
+static const void* push_fn(int precision, int do_push) {
+  if (precision == CP_FP32)
+    return do_push ? reinterpret_cast<const void*>(k_push<float, true>)
+                   : reinterpret_cast<const void*>(k_push<float, false>);
+  return do_push ? reinterpret_cast<const void*>(k_push<double, true>)
+                 : reinterpret_cast<const void*>(k_push<double, false>);
 }
 
-cudaError_t push_async_occupancy(size_t smem, int* blocks_per_sm) {
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_push_async, kThreads, smem);
+size_t push_smem_bytes(int N, int precision) {
+  return precision == CP_FP32 ? push_smem<float>(N) : push_smem<double>(N);
 }
 
-cudaError_t push_async_launch(const Bufs& B, int grid, size_t smem, cudaStream_t st, int do_push) {
+// Shared memory by which cp_create accepts a gap (the documented limits of
+// 11,390 cells with FP32 and 7,231 with FP64 particles): the FP64 push
+// itself takes less.
+size_t push_smem_limit_bytes(int N, int precision) {
+  if (precision == CP_FP32) return push_smem<float>(N);
+  return align16(sizeof(long long) * (N + 1)) + align16(sizeof(unsigned int) * 2 * N) + 2 * sizeof(double) * (N + 1);
+}
+
+// Every context sharing a kernel may ask for another size, so the kernels'
+// limit is the largest the device allows.
+cudaError_t push_configure(int precision) {
+  int dev = 0, most = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  for (int do_push = 0; do_push < 2 && e == cudaSuccess; ++do_push) {
+    cudaFuncAttributes at;
+    e = cudaFuncGetAttributes(&at, push_fn(precision, do_push));
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(push_fn(precision, do_push), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               most - static_cast<int>(at.sharedSizeBytes));
+  }
+  return e;
+}
+
+cudaError_t push_occupancy(int precision, size_t smem, int* blocks_per_sm) {
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, push_fn(precision, 1), kThreads, smem);
+}
+
+// Push and solve are launched with programmatic dependent launch: each may
+// be scheduled while its predecessor finishes and waits in
+// cudaGridDependencySynchronize() until that grid has completed.
+cudaError_t push_launch(int precision, const Bufs& B, int grid, size_t smem, cudaStream_t st, int do_push) {
   cudaLaunchConfig_t cfg = {};
   // one CTA more runs the learned predictor when the push carries it
   cfg.gridDim = dim3(grid + ((B.net != nullptr && B.net_in_push) ? 1 : 0), 1, 1);
@@ -470,7 +714,8 @@ cudaError_t push_async_launch(const Bufs& B, int grid, size_t smem, cudaStream_t
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_push_async, B, do_push);
+  void* args[] = {const_cast<Bufs*>(&B)};
+  return cudaLaunchKernelExC(&cfg, push_fn(precision, do_push), args);
 }
 
 }  // namespace cpk
