@@ -52,9 +52,10 @@ cudaError_t push2_occupancy(int* per_sm);
 cudaError_t push2_launch(const DevParams* P, DevState* S, void* D, const void* D_host, void* abs,
                          int abs_cap, int grid, cudaStream_t st);
 cudaError_t sort2_launch(DevState* S, void* D, int T, int s, int sms, cudaStream_t st);
-cudaError_t solve2_fwd_launch(void* D, long long* G1, int Nx, int Ny, cudaStream_t st);
-cudaError_t solve2_modes_launch(void* D, int Nx, int Ny, float c_rhs, const double* E64,
-                                cudaStream_t st);
+cudaError_t solve2_configure();
+cudaError_t solve2_fwd_launch(const void* D_host, long long* G1, int Nx, int Ny, cudaStream_t st);
+cudaError_t solve2_modes_launch(const void* D_host, int Nx, int Ny, float c_rhs, cudaStream_t st);
+cudaError_t solve2_fields_launch(const void* D_host, int Nx, int Ny, const double* E64, cudaStream_t st);
 cudaError_t deposit2_level0_launch(DevState* S, const void* D, int sms, cudaStream_t st);
 cudaError_t tables2_launch(void* D, int Ny, double r2, cudaStream_t st);
 cudaError_t samples_launch(const DevParams* P, const cp_diag* hist, int64_t first, int64_t n,
@@ -1553,6 +1554,8 @@ struct cp_gap2d {
   double t_ms[3] = {0.0, 0.0, 0.0};  // push, solve (all kernels), sort
   int64_t t_n[3] = {0, 0, 0};
   std::vector<cudaEvent_t> ev;
+  cudaStream_t side = nullptr;           // captured beside the main stream: the mean's solve
+  cudaEvent_t fork = nullptr, join = nullptr;
 };
 
 namespace {
@@ -1568,6 +1571,9 @@ void g2_free(cp_gap2d* g) {
   g->owned.clear();
   for (cudaEvent_t e : g->ev) cudaEventDestroy(e);
   g->ev.clear();
+  if (g->side) cudaStreamDestroy(g->side);
+  if (g->fork) cudaEventDestroy(g->fork);
+  if (g->join) cudaEventDestroy(g->join);
   if (g->c) {
     // the 1D context's particle pointers are this object's: forget them first
     cp_ctx* c = g->c;
@@ -1581,22 +1587,72 @@ void g2_free(cp_gap2d* g) {
 }
 
 // Kernels of one step after the push: row sums + spectra, the 1D coupled
-// solve of the mean, the transverse modes and the fields.
-int g2_solve(cp_gap2d* g, int do_push, int mode, double tol) {
+// solve of the mean beside the transverse modes (on the side stream while a
+// graph is captured), and the fields.
+int g2_solve(cp_gap2d* g, cudaStream_t st, bool fork, int do_push, int mode, double tol) {
   cp_ctx* c = g->c;
   const cpk::Bufs B = make_bufs(c);
-  CP_CUDA(cpk::solve2_fwd_launch(g->dD, c->G, g->Nx, g->Ny, c->stream));
-  CP_CUDA(solve(c, B, c->stream, do_push, mode, tol));
+  CP_CUDA(cpk::solve2_fwd_launch(&g->hd, c->G, g->Nx, g->Ny, st));
+  if (fork) {
+    CP_CUDA(cudaEventRecord(g->fork, st));
+    CP_CUDA(cudaStreamWaitEvent(g->side, g->fork, 0));
+  }
+  CP_CUDA(solve(c, B, fork ? g->side : st, do_push, mode, tol));
+  if (fork) CP_CUDA(cudaEventRecord(g->join, g->side));
   const float c_rhs = static_cast<float>(-c->hp.dx * c->hp.dx / c->hp.eps0);
-  CP_CUDA(cpk::solve2_modes_launch(g->dD, g->Nx, g->Ny, c_rhs, c->E64, c->stream));
-  g->launches += 6;
+  CP_CUDA(cpk::solve2_modes_launch(&g->hd, g->Nx, g->Ny, c_rhs, st));
+  if (fork) CP_CUDA(cudaStreamWaitEvent(st, g->join, 0));
+  CP_CUDA(cpk::solve2_fields_launch(&g->hd, g->Nx, g->Ny, c->E64, st));
+  g->launches += 4;
   return CP_OK;
 }
 
-int g2_sort(cp_gap2d* g) {
+int g2_sort(cp_gap2d* g, cudaStream_t st) {
   cp_ctx* c = g->c;
-  for (int s = 0; s < kSpecies; ++s) CP_CUDA(cpk::sort2_launch(c->dS, g->dD, g->T, s, g->sms, c->stream));
+  for (int s = 0; s < kSpecies; ++s) CP_CUDA(cpk::sort2_launch(c->dS, g->dD, g->T, s, g->sms, st));
   g->launches += 6 * kSpecies;
+  return CP_OK;
+}
+
+int g2_push(cp_gap2d* g, cudaStream_t st) {
+  cp_ctx* c = g->c;
+  CP_CUDA(cpk::push2_launch(c->dP, c->dS, g->dD, &g->hd, g->abs, g->abs_cap, g->grid, st));
+  g->launches += 1;
+  return CP_OK;
+}
+
+// Capture sort_every steps and the re-sort that follows them.
+int g2_build_graph(cp_gap2d* g, int mode, double tol) {
+  cp_ctx* c = g->c;
+  if (c->gexec[mode] && c->gtol[mode] == tol) return CP_OK;
+  if (c->gexec[mode]) {
+    cudaGraphExecDestroy(c->gexec[mode]);
+    c->gexec[mode] = nullptr;
+  }
+  if (!g->side) {
+    CP_CUDA(cudaStreamCreateWithFlags(&g->side, cudaStreamNonBlocking));
+    CP_CUDA(cudaEventCreateWithFlags(&g->fork, cudaEventDisableTiming));
+    CP_CUDA(cudaEventCreateWithFlags(&g->join, cudaEventDisableTiming));
+  }
+  const int64_t launches = g->launches;
+  cudaGraph_t gr = nullptr;
+  CP_CUDA(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
+  int rc = CP_OK;
+  for (int k = 0; k < g->sort_every && rc == CP_OK; ++k) {
+    rc = g2_push(g, c->cap_stream);
+    if (rc == CP_OK) rc = g2_solve(g, c->cap_stream, true, 1, mode, tol);
+  }
+  if (rc == CP_OK) rc = g2_sort(g, c->cap_stream);
+  const cudaError_t e = cudaStreamEndCapture(c->cap_stream, &gr);
+  g->launches = launches;
+  if (rc != CP_OK || e != cudaSuccess) {
+    if (gr) cudaGraphDestroy(gr);
+    return CP_ERR_CUDA;
+  }
+  const cudaError_t e2 = cudaGraphInstantiate(&c->gexec[mode], gr, 0);
+  cudaGraphDestroy(gr);
+  CP_CUDA(e2);
+  c->gtol[mode] = tol;
   return CP_OK;
 }
 
@@ -1750,6 +1806,7 @@ int g2_init(cp_gap2d* g, int mode, double tol) {
   D.use_win = (Ny >= cpk::kW2) ? 1 : 0;
   for (int s = 0; s < kSpecies; ++s) {
     D.n_sorted[s] = 0;
+    D.chunk[s] = cpk::kPass2;
     D.cap[s] = c->cap[s];
   }
   CP_TRY(g2_alloc(g, reinterpret_cast<void**>(&g->dD), sizeof(cpk::Dev2D)));
@@ -1773,11 +1830,12 @@ int g2_init(cp_gap2d* g, int mode, double tol) {
   }
   c->initialized = true;
   g->initialized = true;
+  CP_CUDA(cpk::solve2_configure());
   // level 0: sort, deposit, solve
-  CP_TRY(g2_sort(g));
+  CP_TRY(g2_sort(g, c->stream));
   g->since_sort = 0;
   CP_CUDA(cpk::deposit2_level0_launch(c->dS, g->dD, g->sms, c->stream));
-  CP_TRY(g2_solve(g, 0, mode, tol));
+  CP_TRY(g2_solve(g, c->stream, false, 0, mode, tol));
   return CP_OK;
 }
 
@@ -1809,21 +1867,28 @@ int g2_steps(cp_gap2d* g, int mode, int32_t n_steps, double tol) {
     CP_CUDA(cudaEventRecord(g->ev[k + 1], c->stream));
     return CP_OK;
   };
-  for (int k = 0; k < n_steps; ++k) {
+  for (int k = 0; k < n_steps;) {
     if (g->since_sort == g->sort_every) {  // periodic re-sort (also drops absorbed slots)
       if (g->timing) CP_TRY(g2_timed(g, 2, &rec));
-      CP_TRY(g2_sort(g));
+      CP_TRY(g2_sort(g, c->stream));
       if (g->timing) CP_TRY(mark_end());
       g->since_sort = 0;
     }
+    if (!g->timing && g->since_sort == 0 && n_steps - k >= g->sort_every) {
+      CP_TRY(g2_build_graph(g, mode, tol));
+      CP_CUDA(cudaGraphLaunch(c->gexec[mode], c->stream));
+      g->launches += 5 * g->sort_every + 6 * kSpecies;
+      k += g->sort_every;
+      continue;
+    }
     if (g->timing) CP_TRY(g2_timed(g, 0, &rec));
-    CP_CUDA(cpk::push2_launch(c->dP, c->dS, g->dD, &g->hd, g->abs, g->abs_cap, g->grid, c->stream));
-    g->launches += 1;
+    CP_TRY(g2_push(g, c->stream));
     if (g->timing) CP_TRY(mark_end());
     if (g->timing) CP_TRY(g2_timed(g, 1, &rec));
-    CP_TRY(g2_solve(g, 1, mode, tol));
+    CP_TRY(g2_solve(g, c->stream, false, 1, mode, tol));
     if (g->timing) CP_TRY(mark_end());
     g->since_sort += 1;
+    ++k;
   }
   if (g->timing) {
     CP_CUDA(cudaStreamSynchronize(c->stream));

@@ -19,13 +19,14 @@
 // * Solve: each row of the grid is summed exactly (the int64 column sums are
 //   the 1D coupled problem of Sec. 2.4.2/2.4.3, solved by the 1D cluster
 //   solve, circuit and history included) and Fourier-transformed in y
-//   (radix-2 FFT in shared memory, FP32); every transverse mode k != 0
-//   solves its tridiagonal system in x with phi = 0 on both electrodes
-//   (Thomas, one thread per mode); the inverse transform and the 1D field
+//   (FFT, FP32); every transverse mode k != 0 solves its tridiagonal system
+//   in x with phi = 0 on both electrodes (Thomas as two scans, one warp per
+//   mode, beside the mean's solve); the inverse transform and the 1D field
 //   give E_x = E_0(x) + dE_x and E_y on the staggered grid.
 #include <cuda_runtime.h>
 
 #include <algorithm>
+
 
 #include "cp_common.cuh"
 #include "cp_gap2d.cuh"
@@ -76,6 +77,21 @@ __device__ __forceinline__ Stencil2 stencil2(const Dev2D& D, float x, float y) {
   st.jj1 = wrapi(st.jj + 1, D.Ny);
   st.vy = sy - syf;
   return st;
+}
+
+// floor(x) of |x| < 2^22 as the bits of 1.5 2^23 + floor(x), one addition
+// rounded down: the integer is bits - kFloorBits and the value r - kFloorMagic
+// (no floor or conversion instruction: those issue at a quarter rate)
+constexpr float kFloorMagic = 12582912.0f;
+constexpr int kFloorBits = 0x4B400000;
+__device__ __forceinline__ int floor_split(float x, float* frac) {
+  const float r = __fadd_rd(x, kFloorMagic);
+  *frac = x - (r - kFloorMagic);
+  return __float_as_int(r) - kFloorBits;
+}
+// floor(f 2^16) of a fraction f in [0, 1), from the mantissa of 2^23 + f 2^16
+__device__ __forceinline__ unsigned int frac16(float f) {
+  return __float_as_uint(__fmaf_rd(f, 65536.0f, 8388608.0f)) & 0xFFFFu;
 }
 
 __device__ __forceinline__ float bilin(float f00, float f10, float f01, float f11, float a, float b) {
@@ -156,34 +172,145 @@ __device__ __forceinline__ void deposit2_global(const Dev2D& D, float x, float y
 // ---------------------------------------------------------------------------
 // k2_push
 // ---------------------------------------------------------------------------
+// Field and deposit window of one CTA.  The field window holds each node's
+// value and that of the next node in y (one 8-byte load per stencil column).
+// The deposit window, by cell (indexed like its lower corner node): the
+// particle count n, the sums x, y of the per-axis weights wx1, wy1 and the
+// high bits and low 16 bits of the sum of wx1 wy1 (< 2^32 each).  The four
+// corner weights of a particle are linear in these (A = 2^16):
+// w00 = A^2 - A wx1 - A wy1 + wx1 wy1, w10 = A wx1 - wx1 wy1,
+// w01 = A wy1 - wx1 wy1, w11 = wx1 wy1; the flush forms each node's exact
+// int64 sum from its four cells.  An item of at most 32768 particles keeps
+// every 32-bit sum below 2^31.
+constexpr int kWin2 = kW2 * kW2;
+__device__ __forceinline__ void get2(const float* p, float (&v)[2]) {
+  const float2 t = __ldcs(reinterpret_cast<const float2*>(p));
+  v[0] = t.x; v[1] = t.y;
+}
+__device__ __forceinline__ void put2(float* p, const float (&v)[2]) {
+  __stcs(reinterpret_cast<float2*>(p), make_float2(v[0], v[1]));
+}
+struct Window2 {
+  float2 Ex[kWin2], Ey[kWin2];
+  unsigned int n[kWin2], x[kWin2], y[kWin2], hi[kWin2], lo[kWin2];
+};
+
+__device__ __forceinline__ void deposit_window(Window2& W, int d, unsigned int wx1, unsigned int wy1) {
+  const unsigned int xy = wx1 * wy1;  // < 2^32
+  atomicAdd(&W.n[d], 1u);
+  atomicAdd(&W.x[d], wx1);
+  atomicAdd(&W.y[d], wy1);
+  atomicAdd(&W.hi[d], xy >> 16);
+  atomicAdd(&W.lo[d], xy & 0xFFFFu);
+}
+
+// The work item in hand and the CTA's tallies.
+struct Item2 {
+  float *xs, *us, *ys, *ws;
+  const uint32_t* ids;
+  AbsRec2* abs;
+  float kx, ky;
+  int s, ox, oy, win, abs_cap;
+  int abs_n, over;
+  unsigned int cfl;
+  unsigned int cnt[2][kSpecies];
+};
+
+// The general path of one live particle (slot p, values before the step):
+// gather and deposit in the window where the stencils fit, else in global
+// memory; absorption.  Out of line: few particles take it, and inlined it
+// costs the others registers.
+__device__ __noinline__ void push_general(const Dev2D& D, Item2& T, Window2& W, long long p, float x, float y, float u,
+                                          float w) {
+  const int Ny = D.Ny, ox = T.ox, oy = T.oy;
+  const bool win = T.win != 0;
+  const Stencil2 st = stencil2(D, x, y);
+  float ex, ey;
+  // window origins of the two 2x2 stencils (the window is contiguous in y, so
+  // the corners sit at +1 row / +1 column of their origin)
+  const int le = win_rel(st.i, st.j, ox, oy, Ny), lf = win_rel(st.a, st.jj, ox, oy, Ny);
+  if (win && le >= 0 && lf >= 0) {
+    const int e00 = le, e10 = le + (st.i1 - st.i) * kW2;
+    const int f00 = lf, f10 = lf + kW2;
+    const float2 cx0 = W.Ex[e00], cx1 = W.Ex[e10], cy0 = W.Ey[f00], cy1 = W.Ey[f10];
+    ex = bilin(cx0.x, cx1.x, cx0.y, cx1.y, st.t, st.v);
+    ey = bilin(cy0.x, cy1.x, cy0.y, cy1.y, st.fx, st.vy);
+  } else {
+    const float* Ex = D.Ex;
+    const float* Ey = D.Ey;
+    const long long ri = static_cast<long long>(st.i) * Ny, ri1 = static_cast<long long>(st.i1) * Ny;
+    const long long ra = static_cast<long long>(st.a) * Ny, ra1 = static_cast<long long>(st.a1) * Ny;
+    ex = bilin(__ldg(&Ex[ri + st.j]), __ldg(&Ex[ri1 + st.j]), __ldg(&Ex[ri + st.j1]), __ldg(&Ex[ri1 + st.j1]), st.t,
+               st.v);
+    ey = bilin(__ldg(&Ey[ra + st.jj]), __ldg(&Ey[ra1 + st.jj]), __ldg(&Ey[ra + st.jj1]), __ldg(&Ey[ra1 + st.jj1]),
+               st.fx, st.vy);
+  }
+  const float un = fmaf(T.kx, ex, u);
+  const float wn = fmaf(T.ky, ey, w);
+  const float xn = x + un;
+  float yn = y + wn;
+  if (yn < 0.0f) yn += D.Nyf;
+  if (yn >= D.Nyf) yn -= D.Nyf;
+  if (!(yn >= 0.0f && yn < D.Nyf)) {  // more than one period in a step (or not finite)
+    yn -= D.Nyf * floorf(yn / D.Nyf);
+    if (!(yn >= 0.0f && yn < D.Nyf)) yn = 0.0f;
+  }
+  atomicMax(&T.cfl, __float_as_uint(fmaxf(fabsf(un), fabsf(wn))));
+  if (!(xn > 0.0f && xn < D.Nxf)) {  // absorbed
+    const int el = (xn <= 0.0f) ? 0 : 1;
+    atomicAdd(&T.cnt[el][T.s], 1u);
+    if (T.s == CP_IONS) {
+      const int slot = atomicAdd(&T.abs_n, 1);
+      if (slot < T.abs_cap) {
+        AbsRec2 r;
+        r.id = T.ids[p];
+        r.el = static_cast<uint32_t>(el);
+        r.u = un;
+        r.w = wn;
+        r.eta = yn;
+        r.pad = 0.0f;
+        T.abs[slot] = r;
+      } else {
+        T.over = 1;
+      }
+    }
+    T.xs[p] = -1.0f;
+    T.us[p] = 0.0f;
+    T.ys[p] = 0.0f;
+    T.ws[p] = 0.0f;
+    return;
+  }
+  T.xs[p] = xn;
+  T.us[p] = un;
+  T.ys[p] = yn;
+  T.ws[p] = wn;
+  int i, j;
+  unsigned int wx1, wy1;
+  cell_weights(xn, yn, &i, &j, &wx1, &wy1);
+  const int d00 = win ? win_rel(i, j, ox, oy, Ny) : -1;
+  if (d00 >= 0) deposit_window(W, d00, wx1, wy1);
+  else deposit2_global(D, xn, yn, T.s == CP_IONS ? 1LL : -1LL);
+}
+
+// What bounds it: instruction issue and, for grids whose tiles hold few
+// particles, the staging and flush of each item's window.  Floors come from
+// one addition rounded down instead of floor and conversion instructions (a
+// quarter of the issue rate), window indices from masks, range checks are two
+// compares, two particles per thread are processed while the next two are on
+// their way, and what few particles need is out of line.  Push at 1024 x 1024
+// cells, 2e7 particles: 226 -> 176 us; at 96 x 128, 3e5: 42.4 -> 21.8 us
+// (items sized by the store, the beam's draws as items of their own).
 __global__ void __launch_bounds__(kThreads2, 2)
 k2_push(const DevParams* __restrict__ P, DevState* S, const Dev2D* __restrict__ Dp,
         const __grid_constant__ Dev2D Dc, int* __restrict__ item_ctr, AbsRec2* __restrict__ abs_all,
         int abs_cap) {
-  // field window: each node holds its value and that of the next node in y
-  // (one 8-byte load per stencil column)
-  __shared__ float2 Exw[kW2 * kW2];
-  __shared__ float2 Eyw[kW2 * kW2];
-  // Deposit window, by cell (indexed like its lower corner node): the
-  // particle count n, the sums sx, sy of the per-axis weights wx1, wy1 and
-  // the high bits and low 16 bits of the sum sxy of wx1 wy1 (< 2^32 each).
-  // The four corner weights of a particle are linear in these (A = 2^16):
-  // w00 = A^2 - A wx1 - A wy1 + wx1 wy1, w10 = A wx1 - wx1 wy1,
-  // w01 = A wy1 - wx1 wy1, w11 = wx1 wy1; the flush forms each node's exact
-  // int64 sum from its four cells.  An item of at most 32768 particles keeps
-  // every 32-bit sum below 2^31.
-  extern __shared__ unsigned int cwin[];
-  unsigned int* Cn = cwin;
-  unsigned int* Cx = cwin + kW2 * kW2;
-  unsigned int* Cy = cwin + 2 * kW2 * kW2;
-  unsigned int* Ch = cwin + 3 * kW2 * kW2;
-  unsigned int* Cl = cwin + 4 * kW2 * kW2;
+  extern __shared__ __align__(16) unsigned char smem2[];
+  Window2& W = *reinterpret_cast<Window2*>(smem2);
+  __shared__ Item2 T;
   __shared__ int s_items[2 * kSpecies + 1];  // item offsets: sorted / tail per species
-  __shared__ int s_abs_n, s_stop, s_over;
-  __shared__ unsigned long long s_cnt[2][kSpecies];
+  __shared__ int s_stop;
   __shared__ unsigned long long s_emit[2];
   __shared__ long long s_conv, s_energy;
-  __shared__ unsigned int s_cfl;
 
   cudaGridDependencySynchronize();
   cudaTriggerProgrammaticLaunchCompletion();
@@ -191,46 +318,83 @@ k2_push(const DevParams* __restrict__ P, DevState* S, const Dev2D* __restrict__ 
   // swaps the y, w buffers and sets n_sorted on the device, so those are read
   // from the device copy
   const Dev2D& D = Dc;
+  // beam ions per work item: about two items per CTA, whole warps
+  const int nbeam = min(kThreads2, (P->beam_per_step / (2 * static_cast<int>(gridDim.x)) + 32) & ~31);
   if (threadIdx.x == 0) {
     s_stop = (ldcg(&S->status) != 0);
-    s_abs_n = 0;
-    s_over = 0;
+    T.abs_n = 0;
+    T.over = 0;
+    T.cfl = 0u;
+    T.abs = abs_all + static_cast<size_t>(blockIdx.x) * abs_cap;
+    T.abs_cap = abs_cap;
+    T.ids = S->id;
     s_conv = 0;
     s_energy = 0;
-    s_cfl = 0u;
     s_emit[0] = s_emit[1] = 0ULL;
-    int acc = 0;
+    int acc = (P->beam_per_step + nbeam - 1) / nbeam;  // the beam's items come first
     for (int s = 0; s < kSpecies; ++s) {
       s_items[2 * s] = acc;
       acc += D.wi_off[s * (D.T + 1) + D.T];
       s_items[2 * s + 1] = acc;
       const long long tail = S->n_proc[s] - Dp->n_sorted[s];
-      acc += static_cast<int>((tail + kChunk2 - 1) / kChunk2);
+      acc += static_cast<int>((tail + kPass2 - 1) / kPass2);
     }
     s_items[2 * kSpecies] = acc;
   }
-  if (threadIdx.x < 2 * kSpecies) s_cnt[threadIdx.x / kSpecies][threadIdx.x % kSpecies] = 0ULL;
+  if (threadIdx.x < 2 * kSpecies) T.cnt[threadIdx.x / kSpecies][threadIdx.x % kSpecies] = 0u;
   __syncthreads();
   if (s_stop) return;
   const bool half = (S->pushed == 0);
   const int64_t step = S->level;
   const int Ny = D.Ny;
-  AbsRec2* my_abs = abs_all + static_cast<size_t>(blockIdx.x) * abs_cap;
   unsigned int cfl = 0u;
-  unsigned int a_cnt[2][kSpecies] = {{0u, 0u, 0u}, {0u, 0u, 0u}};
 
   const int n_items = s_items[2 * kSpecies];
   // Work items are taken from a queue (one atomic ticket per item): items
   // differ in size (whole and partial tiles, the unsorted tails), and a
   // fixed round-robin deal left CTAs idle while others finished theirs.
   // The last CTA out resets the queue for the next launch.
-  __shared__ int s_item;
-  for (;;) {
-    __syncthreads();  // every thread has read the previous ticket
-    if (threadIdx.x == 0) s_item = atomicAdd(&item_ctr[0], 1);
-    __syncthreads();
-    const int item = s_item;
+  __shared__ int s_item[2];
+  if (threadIdx.x == 0) s_item[0] = atomicAdd(&item_ctr[0], 1);
+  for (int turn = 0;; turn ^= 1) {
+    __syncthreads();  // the ticket is there, and every thread has read the one before it
+    const int item = s_item[turn];
     if (item >= n_items) break;
+    if (threadIdx.x == 0) s_item[turn ^ 1] = atomicAdd(&item_ctr[0], 1);  // the next item's, in its shadow
+    if (item < s_items[0]) {
+      // Beam ions entering at x = d with a Gaussian transverse profile, one
+      // per thread.  Their draws are FP64 chains (2 operations a cycle and SM,
+      // about 5 us), so they are items of their own, spread over the CTAs.
+      // Their slots lie behind the ions in use: the beam alone appends ions.
+      const int Bn = P->beam_per_step, k = item * nbeam + static_cast<int>(threadIdx.x);
+      if (static_cast<int>(threadIdx.x) < nbeam && k < Bn) {
+        const double pi = 3.14159265358979323846;
+        const U64x4 wv = philox4x64_10(static_cast<uint64_t>(k), static_cast<uint64_t>(step), 0, 0, P->seed, kTagBeam);
+        const double frac = u01(wv.w[0]);
+        const double Eb = (P->beam_mode == 0)
+                              ? P->beam_E_eV
+                              : __dadd_rn(P->beam_Emin_eV, __dmul_rn(__dsub_rn(P->beam_Emax_eV, P->beam_Emin_eV), u01(wv.w[1])));
+        const double ub = sqrt(2.0 * Eb * P->e / P->m_i) * P->dt / P->dx;
+        const double z = sqrt(-2.0 * log(u01(wv.w[2]))) * cos(2.0 * pi * u01(wv.w[3]));
+        double yc = D.beam_yc + D.beam_sigma * z;
+        yc -= static_cast<double>(Ny) * floor(yc / static_cast<double>(Ny));
+        float yr = static_cast<float>(yc);
+        if (!(yr < D.Nyf)) yr = 0.0f;
+        const float xr = nudge_inside<float>(__dsub_rn(static_cast<double>(D.Nx), __dmul_rn(ub, frac)), D.Nx);
+        const long long slot = S->n_proc[CP_IONS] + k;
+        if (slot < P->cap[CP_IONS]) {
+          static_cast<float*>(S->xi[CP_IONS])[slot] = xr;
+          static_cast<float*>(S->u[CP_IONS])[slot] = static_cast<float>(-ub);
+          static_cast<float*>(Dp->y[CP_IONS])[slot] = yr;
+          static_cast<float*>(Dp->w[CP_IONS])[slot] = 0.0f;
+          S->id[slot] = S->beam_id_base + static_cast<uint32_t>(step * Bn + k);
+          deposit2_global(D, xr, yr, 1LL);
+        } else {
+          T.over = 1;
+        }
+      }
+      continue;
+    }
     int s = 0;
     while (item >= s_items[2 * s + 2]) ++s;
     const bool tail = item >= s_items[2 * s + 1];
@@ -248,175 +412,135 @@ k2_push(const DevParams* __restrict__ P, DevState* S, const Dev2D* __restrict__ 
       }
       const int t = lo;
       const int* ts = D.tile_start + s * (D.T + 1);
-      p0 = ts[t] + static_cast<long long>(k - wo[t]) * kChunk2;
-      p1 = min(static_cast<long long>(ts[t + 1]), p0 + kChunk2);
+      const int chunk = Dp->chunk[s];
+      p0 = ts[t] + static_cast<long long>(k - wo[t]) * chunk;
+      p1 = min(static_cast<long long>(ts[t + 1]), p0 + chunk);
       ox = (t / D.nty) * kT2 - kH2 - 1;
       oy = (t % D.nty) * kT2 - kH2 - 1;
       win = D.use_win != 0;
-      // stage the field window; zero the deposit window
-      for (int q = threadIdx.x; win && q < kW2 * kW2; q += kThreads2) {
-        const int lx = q / kW2, ly = q % kW2;
-        const int gx = ox + lx;
-        const int gy = wrapi(oy + ly, Ny);  // one wrap: Ny >= the window edge
-        const int gy1 = wrapi(gy + 1, Ny);
+      // stage the field window, all of a thread's loads in flight; zero the
+      // deposit window
+      constexpr int kNodes = (kW2 * kW2 + kThreads2 - 1) / kThreads2;
+      float e[kNodes][4];
+#pragma unroll
+      for (int c = 0; c < kNodes; ++c) {
+        const int q = threadIdx.x + c * kThreads2;
+        const int gx = ox + q / kW2;
+        const int gy = (oy + q % kW2) & (Ny - 1), gy1 = (gy + 1) & (Ny - 1);
         const long long r = static_cast<long long>(gx) * Ny;
-        Exw[q] = (gx >= 0 && gx < D.Nx) ? make_float2(D.Ex[r + gy], D.Ex[r + gy1]) : make_float2(0.0f, 0.0f);
-        Eyw[q] = (gx >= 0 && gx <= D.Nx) ? make_float2(D.Ey[r + gy], D.Ey[r + gy1]) : make_float2(0.0f, 0.0f);
-        Cn[q] = Cx[q] = Cy[q] = Ch[q] = Cl[q] = 0u;
+        const bool ix = win && q < kW2 * kW2 && gx >= 0 && gx < D.Nx, iy = win && q < kW2 * kW2 && gx >= 0 && gx <= D.Nx;
+        e[c][0] = ix ? __ldcg(&D.Ex[r + gy]) : 0.0f;
+        e[c][1] = ix ? __ldcg(&D.Ex[r + gy1]) : 0.0f;
+        e[c][2] = iy ? __ldcg(&D.Ey[r + gy]) : 0.0f;
+        e[c][3] = iy ? __ldcg(&D.Ey[r + gy1]) : 0.0f;
       }
-      __syncthreads();
+#pragma unroll
+      for (int c = 0; c < kNodes; ++c) {
+        const int q = threadIdx.x + c * kThreads2;
+        if (q < kW2 * kW2) {
+          W.Ex[q] = make_float2(e[c][0], e[c][1]);
+          W.Ey[q] = make_float2(e[c][2], e[c][3]);
+          W.n[q] = W.x[q] = W.y[q] = W.hi[q] = W.lo[q] = 0u;
+        }
+      }
     } else {
       const int k = item - s_items[2 * s + 1];
-      p0 = Dp->n_sorted[s] + static_cast<long long>(k) * kChunk2;
-      p1 = min(static_cast<long long>(S->n_proc[s]), p0 + kChunk2);
+      p0 = Dp->n_sorted[s] + static_cast<long long>(k) * kPass2;
+      p1 = min(static_cast<long long>(S->n_proc[s]), p0 + kPass2);
     }
     float* xs = reinterpret_cast<float*>(S->xi[s]);
     float* us = reinterpret_cast<float*>(S->u[s]);
     float* ys = reinterpret_cast<float*>(Dp->y[s]);
     float* ws = reinterpret_cast<float*>(Dp->w[s]);
-    const uint32_t* ids = S->id;
     const float kx = D.kx[half ? 0 : 1][s], ky = D.ky[half ? 0 : 1][s];
-    const long long sign = (s == CP_IONS) ? 1LL : -1LL;
-    for (long long b0 = p0; b0 < p1; b0 += kThreads2 * 4) {
-      const long long base = b0 + static_cast<long long>(threadIdx.x) * 4;
-      if (base < p1) {
-        float xv[4], uv[4], yv[4], wv[4];
-        load4(xs + base, xv);
-        load4(us + base, uv);
-        load4(ys + base, yv);
-        load4(ws + base, wv);
-        // Fast path, without divergent branches: a live particle whose
-        // stencils lie in the window, that stays inside the gap and whose
-        // deposit lands in the window (the common case).  Every other live
-        // particle is flagged and takes the general path below, on its
-        // unchanged values, with the same arithmetic.
-        unsigned int slow = 0u;
+    // half-grid columns (window coordinates) of the fast path: both of a
+    // stencil's columns inside the gap and the window
+    const int ymask = Ny - 1;
+    const int lo_h = max(0, -ox);
+    const int hi_h = min(D.Nx - 2 - ox, kW2 - 3);
+    if (hi_h < lo_h) win = false;  // (no cell of the tile has one)
+    const unsigned int n_h = static_cast<unsigned int>(hi_h - lo_h);
+    if (threadIdx.x == 0) {
+      T.xs = xs; T.us = us; T.ys = ys; T.ws = ws;
+      T.kx = kx; T.ky = ky;
+      T.s = s; T.ox = ox; T.oy = oy; T.win = win;
+    }
+    __syncthreads();
+    // the next pass's particles are requested before this pass's are processed
+    const long long base0 = p0 + static_cast<long long>(threadIdx.x) * kPer2;
+    constexpr long long kStep = kThreads2 * kPer2;
+    float nx[kPer2], nu[kPer2], ny[kPer2], nw[kPer2];
+    auto fetch = [&](long long b) {
+      get2(xs + b, nx);
+      get2(us + b, nu);
+      get2(ys + b, ny);
+      get2(ws + b, nw);
+    };
+    if (base0 < p1) fetch(base0);
+    for (long long base = base0; base < p1; base += kStep) {
+      float xv[kPer2], uv[kPer2], yv[kPer2], wv[kPer2];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float x = xv[q];
-          const bool alive = (x > 0.0f && x < D.Nxf);
-          const float xa = alive ? x : 1.0f, ya = alive ? yv[q] : 0.0f;  // defined indices for dead slots
-          const Stencil2 st = stencil2(D, xa, ya);
-          const int le = win_rel(st.i, st.j, ox, oy, Ny), lf = win_rel(st.a, st.jj, ox, oy, Ny);
-          const bool gw = win && alive && le >= 0 && lf >= 0;
-          const int e00 = gw ? le : 0, e10 = gw ? le + (st.i1 - st.i) * kW2 : 0;
-          const int f00 = gw ? lf : 0, f10 = f00 + kW2;
-          const float2 cx0 = Exw[e00], cx1 = Exw[e10], cy0 = Eyw[f00], cy1 = Eyw[f10];
-          const float ex = bilin(cx0.x, cx1.x, cx0.y, cx1.y, st.t, st.v);
-          const float ey = bilin(cy0.x, cy1.x, cy0.y, cy1.y, st.fx, st.vy);
-          const float un = fmaf(kx, ex, uv[q]);
-          const float wn = fmaf(ky, ey, wv[q]);
-          const float xn = x + un;
-          float yn = yv[q] + wn;
-          if (yn < 0.0f) yn += D.Nyf;
-          if (yn >= D.Nyf) yn -= D.Nyf;
-          const bool inside = (xn > 0.0f && xn < D.Nxf) && (yn >= 0.0f && yn < D.Nyf);
-          int i, j;
-          unsigned int wx1, wy1;
-          cell_weights(inside ? xn : 1.0f, inside ? yn : 0.0f, &i, &j, &wx1, &wy1);
-          const int d00 = win ? win_rel(i, j, ox, oy, Ny) : -1;
-          const bool good = gw && inside && d00 >= 0;
-          if (good) {
-            const unsigned int xy = wx1 * wy1;  // < 2^32
-            atomicAdd(&Cn[d00], 1u);
-            if (wx1) atomicAdd(&Cx[d00], wx1);
-            if (wy1) atomicAdd(&Cy[d00], wy1);
-            if (xy >> 16) atomicAdd(&Ch[d00], xy >> 16);
-            if (xy & 0xFFFFu) atomicAdd(&Cl[d00], xy & 0xFFFFu);
-            cfl = max(cfl, __float_as_uint(fmaxf(fabsf(un), fabsf(wn))));
-            xv[q] = xn;
-            uv[q] = un;
-            yv[q] = yn;
-            wv[q] = wn;
-          } else if (alive) {
-            slow |= 1u << q;
-          }
+      for (int q = 0; q < kPer2; ++q) {
+        xv[q] = nx[q];
+        uv[q] = nu[q];
+        yv[q] = ny[q];
+        wv[q] = nw[q];
+      }
+      if (base + kStep < p1) fetch(base + kStep);
+      // Fast path, without divergent branches: a live particle whose
+      // stencils lie in the window and off the electrodes' half cells, that
+      // stays inside the gap and whose deposit lands in the window (the
+      // common case).  Every other live particle is flagged and takes the
+      // general path below, on its unchanged values, with the same
+      // arithmetic.
+      unsigned int slow = 0u;
+#pragma unroll
+      for (int q = 0; q < kPer2; ++q) {
+        const float x = xv[q], y = yv[q];
+        const bool alive = (x > 0.0f && x < D.Nxf);
+        if (!win) {
+          if (alive) slow |= 1u << q;
+          continue;
         }
-        if (slow) {  // the general path
-  #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            if (!((slow >> q) & 1u)) continue;
-            const float x = xv[q];
-            const Stencil2 st = stencil2(D, x, yv[q]);
-            float ex, ey;
-            // window origins of the two 2x2 stencils (the window is contiguous in
-            // y, so the corners sit at +1 row / +1 column of their origin)
-            const int le = win_rel(st.i, st.j, ox, oy, Ny), lf = win_rel(st.a, st.jj, ox, oy, Ny);
-            if (win && le >= 0 && lf >= 0) {
-              const int e00 = le, e10 = le + (st.i1 - st.i) * kW2;
-              const int f00 = lf, f10 = lf + kW2;
-              const float2 cx0 = Exw[e00], cx1 = Exw[e10], cy0 = Eyw[f00], cy1 = Eyw[f10];
-              ex = bilin(cx0.x, cx1.x, cx0.y, cx1.y, st.t, st.v);
-              ey = bilin(cy0.x, cy1.x, cy0.y, cy1.y, st.fx, st.vy);
-            } else {
-              const float* Ex = D.Ex;
-              const float* Ey = D.Ey;
-              const long long ri = static_cast<long long>(st.i) * Ny, ri1 = static_cast<long long>(st.i1) * Ny;
-              const long long ra = static_cast<long long>(st.a) * Ny, ra1 = static_cast<long long>(st.a1) * Ny;
-              ex = bilin(__ldg(&Ex[ri + st.j]), __ldg(&Ex[ri1 + st.j]), __ldg(&Ex[ri + st.j1]),
-                         __ldg(&Ex[ri1 + st.j1]), st.t, st.v);
-              ey = bilin(__ldg(&Ey[ra + st.jj]), __ldg(&Ey[ra1 + st.jj]), __ldg(&Ey[ra + st.jj1]),
-                         __ldg(&Ey[ra1 + st.jj1]), st.fx, st.vy);
-            }
-            const float un = fmaf(kx, ex, uv[q]);
-            const float wn = fmaf(ky, ey, wv[q]);
-            const float xn = x + un;
-            float yn = yv[q] + wn;
-            if (yn < 0.0f) yn += D.Nyf;
-            if (yn >= D.Nyf) yn -= D.Nyf;
-            if (!(yn >= 0.0f && yn < D.Nyf)) {  // more than one period in a step (or not finite)
-              yn -= D.Nyf * floorf(yn / D.Nyf);
-              if (!(yn >= 0.0f && yn < D.Nyf)) yn = 0.0f;
-            }
-            cfl = max(cfl, __float_as_uint(fmaxf(fabsf(un), fabsf(wn))));
-            if (!(xn > 0.0f && xn < D.Nxf)) {  // absorbed
-              const int el = (xn <= 0.0f) ? 0 : 1;
-              ++a_cnt[el][s];
-              if (s == CP_IONS) {
-                const int slot = atomicAdd(&s_abs_n, 1);
-                if (slot < abs_cap) {
-                  AbsRec2 r;
-                  r.id = ids[base + q];
-                  r.el = static_cast<uint32_t>(el);
-                  r.u = un;
-                  r.w = wn;
-                  r.eta = yn;
-                  r.pad = 0.0f;
-                  my_abs[slot] = r;
-                } else {
-                  s_over = 1;
-                }
-              }
-              xv[q] = -1.0f;
-              uv[q] = 0.0f;
-              yv[q] = 0.0f;
-              wv[q] = 0.0f;
-              continue;
-            }
-            xv[q] = xn;
-            uv[q] = un;
-            yv[q] = yn;
-            wv[q] = wn;
-            int i, j;
-            unsigned int wx1, wy1;
-            cell_weights(xn, yn, &i, &j, &wx1, &wy1);
-            const int d00 = win ? win_rel(i, j, ox, oy, Ny) : -1;
-            if (d00 >= 0) {
-              const unsigned int xy = wx1 * wy1;  // < 2^32
-              atomicAdd(&Cn[d00], 1u);
-              if (wx1) atomicAdd(&Cx[d00], wx1);
-              if (wy1) atomicAdd(&Cy[d00], wy1);
-              if (xy >> 16) atomicAdd(&Ch[d00], xy >> 16);
-              if (xy & 0xFFFFu) atomicAdd(&Cl[d00], xy & 0xFFFFu);
-            } else {
-              deposit2_global(D, xn, yn, sign);
-            }
-          }
+        float fx, fy, tx, ty;  // fractions on the nodes and on the half grid
+        const int i = floor_split(x, &fx) - ox, ih = floor_split(x - 0.5f, &tx) - ox;
+        const int j = (floor_split(y, &fy) - oy) & ymask, jh = (floor_split(y - 0.5f, &ty) - oy) & ymask;
+        // ih in [lo_h, lo_h + n_h] puts i = ih or ih + 1 into the window too, and
+        // jh <= kW2 - 3 does so for j = jh or jh + 1
+        const bool gw = alive && static_cast<unsigned>(ih - lo_h) <= n_h && jh <= kW2 - 3;
+        const int e0 = gw ? ih * kW2 + j : 0, f0 = gw ? i * kW2 + jh : 0;
+        const float2 cx0 = W.Ex[e0], cx1 = W.Ex[e0 + kW2], cy0 = W.Ey[f0], cy1 = W.Ey[f0 + kW2];
+        const float ex = bilin(cx0.x, cx1.x, cx0.y, cx1.y, tx, fy);
+        const float ey = bilin(cy0.x, cy1.x, cy0.y, cy1.y, fx, ty);
+        const float un = fmaf(kx, ex, uv[q]);
+        const float wn = fmaf(ky, ey, wv[q]);
+        const float xn = x + un;
+        float yn = y + wn;
+        if (yn < 0.0f) yn += D.Nyf;
+        if (yn >= D.Nyf) yn -= D.Nyf;
+        const bool inside = (xn > 0.0f && xn < D.Nxf) && (yn >= 0.0f && yn < D.Nyf);
+        const int di = floor_split(xn, &fx) - ox;
+        const int dj = (floor_split(yn, &fy) - oy) & ymask;
+        const bool good = gw && inside && static_cast<unsigned>(di) <= kW2 - 2 && dj <= kW2 - 2;
+        if (good) {
+          deposit_window(W, di * kW2 + dj, frac16(fx), frac16(fy));
+          cfl = max(cfl, __float_as_uint(fmaxf(fabsf(un), fabsf(wn))));
+          xv[q] = xn;
+          uv[q] = un;
+          yv[q] = yn;
+          wv[q] = wn;
+        } else if (alive) {
+          slow |= 1u << q;
         }
-        store4(xs + base, xv);
-        store4(us + base, uv);
-        store4(ys + base, yv);
-        store4(ws + base, wv);
+      }
+      put2(xs + base, xv);
+      put2(us + base, uv);
+      put2(ys + base, yv);
+      put2(ws + base, wv);
+      if (slow) {  // rewrites the flagged particles' slots
+#pragma unroll
+        for (int q = 0; q < kPer2; ++q)
+          if ((slow >> q) & 1u) push_general(D, T, W, base + q, xv[q], yv[q], uv[q], wv[q]);
       }
     }
     if (win) {  // flush the deposit window into the int64 grid
@@ -424,18 +548,18 @@ k2_push(const DevParams* __restrict__ P, DevState* S, const Dev2D* __restrict__ 
       for (int q = threadIdx.x; q < kW2 * kW2; q += kThreads2) {
         const int p = q / kW2, r = q % kW2;
         constexpr long long A = 65536;
-        auto sxy = [&](int c) { return (static_cast<long long>(Ch[c]) << 16) + static_cast<long long>(Cl[c]); };
+        auto sxy = [&](int c) { return (static_cast<long long>(W.hi[c]) << 16) + static_cast<long long>(W.lo[c]); };
         // w00 of cell (p, r), w10 of (p-1, r), w01 of (p, r-1), w11 of (p-1, r-1)
-        long long v = A * A * static_cast<long long>(Cn[q]) - A * static_cast<long long>(Cx[q]) -
-                      A * static_cast<long long>(Cy[q]) + sxy(q);
-        if (p > 0) v += A * static_cast<long long>(Cx[q - kW2]) - sxy(q - kW2);
-        if (r > 0) v += A * static_cast<long long>(Cy[q - 1]) - sxy(q - 1);
+        long long v = A * A * static_cast<long long>(W.n[q]) - A * static_cast<long long>(W.x[q]) -
+                      A * static_cast<long long>(W.y[q]) + sxy(q);
+        if (p > 0) v += A * static_cast<long long>(W.x[q - kW2]) - sxy(q - kW2);
+        if (r > 0) v += A * static_cast<long long>(W.y[q - 1]) - sxy(q - 1);
         if (p > 0 && r > 0) v += sxy(q - kW2 - 1);
         if (v == 0) continue;
         const int gx = ox + q / kW2;
         const int gy = wrapi(oy + q % kW2, Ny);
         const long long dbl = (gx == 0 || gx == D.Nx) ? 2 : 1;
-        atomic_add_i64(&D.G2[static_cast<long long>(gx) * Ny + gy], sign * dbl * static_cast<long long>(v));
+        atomic_add_i64(&D.G2[static_cast<long long>(gx) * Ny + gy], s == CP_IONS ? dbl * v : -dbl * v);
       }
       __syncthreads();
     }
@@ -448,21 +572,15 @@ k2_push(const DevParams* __restrict__ P, DevState* S, const Dev2D* __restrict__ 
       __threadfence();
     }
   }
-  // tallies of the absorbed particles
-  for (int e = 0; e < 2; ++e)
-    for (int s = 0; s < kSpecies; ++s) {
-      const unsigned int v = warp_sum_u(a_cnt[e][s]);
-      if (lane_id() == 0 && v) atomicAdd(&s_cnt[e][s], static_cast<unsigned long long>(v));
-    }
   cfl = warp_max_u(cfl);
-  if (lane_id() == 0 && cfl) atomicMax(&s_cfl, cfl);
+  if (lane_id() == 0 && cfl) atomicMax(&T.cfl, cfl);
   __syncthreads();
 
   // --- secondary emission from the ions this CTA saw absorbed ---------------
-  const int na = min(s_abs_n, abs_cap);
+  const int na = min(T.abs_n, abs_cap);
   const double dx = P->dx, dt = P->dt, dy = D.dy;
   for (int r = threadIdx.x; r < na; r += kThreads2) {
-    const AbsRec2 rec = my_abs[r];
+    const AbsRec2 rec = T.abs[r];
     const double vx = static_cast<double>(rec.u) * dx / dt;
     const double vy = static_cast<double>(rec.w) * dy / dt;
     const double Eev = 0.5 * P->m_i * (vx * vx + vy * vy) / P->e;
@@ -496,73 +614,30 @@ k2_push(const DevParams* __restrict__ P, DevState* S, const Dev2D* __restrict__ 
         ws[slot] = 0.0f;
         deposit2_global(D, xr, rec.eta, -1LL);
       } else {
-        s_over = 1;
+        T.over = 1;
       }
     }
   }
 
-  // --- beam ions entering at x = d with a Gaussian transverse profile --------
-  const int Bn = P->beam_per_step;
-  if (Bn > 0) {
-    float* xs = reinterpret_cast<float*>(S->xi[CP_IONS]);
-    float* us = reinterpret_cast<float*>(S->u[CP_IONS]);
-    float* ys = reinterpret_cast<float*>(Dp->y[CP_IONS]);
-    float* ws = reinterpret_cast<float*>(Dp->w[CP_IONS]);
-    uint32_t* idw = S->id;
-    const uint32_t id0 = S->beam_id_base;
-    const double pi = 3.14159265358979323846;
-    for (int k0 = blockIdx.x * kThreads2; k0 < Bn; k0 += gridDim.x * kThreads2) {
-      const int k = k0 + threadIdx.x;
-      const bool act = k < Bn;
-      const unsigned ball = __ballot_sync(0xffffffffu, act);
-      unsigned long long wbase = 0ULL;
-      if (lane_id() == 0 && ball)
-        wbase = atomicAdd(reinterpret_cast<unsigned long long*>(&S->n_alloc[CP_IONS]),
-                          static_cast<unsigned long long>(__popc(ball)));
-      wbase = __shfl_sync(0xffffffffu, wbase, 0);
-      if (!act) continue;
-      const U64x4 wv = philox4x64_10(static_cast<uint64_t>(k), static_cast<uint64_t>(step), 0, 0,
-                                     P->seed, kTagBeam);
-      const double frac = u01(wv.w[0]);
-      const double Eb = (P->beam_mode == 0)
-                            ? P->beam_E_eV
-                            : __dadd_rn(P->beam_Emin_eV, __dmul_rn(__dsub_rn(P->beam_Emax_eV, P->beam_Emin_eV), u01(wv.w[1])));
-      const double ub = sqrt(2.0 * Eb * P->e / P->m_i) * dt / dx;
-      const double z = sqrt(-2.0 * log(u01(wv.w[2]))) * cos(2.0 * pi * u01(wv.w[3]));
-      double yc = D.beam_yc + D.beam_sigma * z;
-      yc -= static_cast<double>(Ny) * floor(yc / static_cast<double>(Ny));
-      float yr = static_cast<float>(yc);
-      if (!(yr < D.Nyf)) yr = 0.0f;
-      const float xr = nudge_inside<float>(__dsub_rn(static_cast<double>(D.Nx), __dmul_rn(ub, frac)), D.Nx);
-      const unsigned long long slot =
-          wbase + static_cast<unsigned long long>(__popc(ball & ((1u << lane_id()) - 1u)));
-      if (slot < static_cast<unsigned long long>(P->cap[CP_IONS])) {
-        xs[slot] = xr;
-        us[slot] = static_cast<float>(-ub);
-        ys[slot] = yr;
-        ws[slot] = 0.0f;
-        idw[slot] = id0 + static_cast<uint32_t>(step * Bn + k);
-        deposit2_global(D, xr, yr, 1LL);
-      } else {
-        s_over = 1;
-      }
-    }
-  }
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int e = 0; e < 2; ++e)
       for (int s = 0; s < kSpecies; ++s)
-        if (s_cnt[e][s]) atomicAdd(&S->absorbed[e][s], s_cnt[e][s]);
+        if (T.cnt[e][s]) atomicAdd(&S->absorbed[e][s], static_cast<unsigned long long>(T.cnt[e][s]));
     if (s_emit[0]) atomicAdd(&S->emitted[0], s_emit[0]);
     if (s_emit[1]) atomicAdd(&S->emitted[1], s_emit[1]);
-    const long long conv = static_cast<long long>(s_cnt[0][CP_IONS]) -
-                           static_cast<long long>(s_cnt[0][CP_ELECTRONS]) -
-                           static_cast<long long>(s_cnt[0][CP_SECONDARIES]) + s_conv;
+    const long long conv = static_cast<long long>(T.cnt[0][CP_IONS]) -
+                           static_cast<long long>(T.cnt[0][CP_ELECTRONS]) -
+                           static_cast<long long>(T.cnt[0][CP_SECONDARIES]) + s_conv;
     if (conv) atomic_add_i64(&S->conv_count, conv);
     if (s_energy) atomic_add_i64(&S->ion_energy_q, s_energy);
-    if (s_cfl) atomicMax(&S->max_cfl_bits, s_cfl);
-    if (blockIdx.x == 0 && Bn > 0) atomicAdd(&S->injected, static_cast<unsigned long long>(Bn));
-    if (s_over || s_abs_n > abs_cap) atomicCAS(&S->status, 0, CP_ERR_CAPACITY);
+    if (T.cfl) atomicMax(&S->max_cfl_bits, T.cfl);
+    if (blockIdx.x == 0 && P->beam_per_step > 0) {
+      atomicAdd(&S->injected, static_cast<unsigned long long>(P->beam_per_step));
+      atomicAdd(reinterpret_cast<unsigned long long*>(&S->n_alloc[CP_IONS]),
+                static_cast<unsigned long long>(P->beam_per_step));
+    }
+    if (T.over) atomicCAS(&S->status, 0, CP_ERR_CAPACITY);
   }
 }
 
@@ -645,13 +720,18 @@ __global__ void k2_scan(DevState* S, Dev2D* Dp, int s, int G) {
   int* cnt = D.tile_cnt + s * T;
   int* ts = D.tile_start + s * (T + 1);
   int* wo = D.wi_off + s * (T + 1);
-  (void)G;
+  // Particles per work item: about two items for each of the push's G CTAs, so
+  // that small stores reach every SM, in whole passes of a CTA; at most
+  // kChunk2 (the deposit window's 32-bit sums).
+  const long long want = (S->n_proc[s] / (2 * G) + kPass2 - 1) / kPass2;
+  const int chunk = kPass2 * static_cast<int>(max(1LL, min(want, static_cast<long long>(kChunk2 / kPass2))));
+  if (threadIdx.x == 0) D.chunk[s] = chunk;
   const int per = (T + blockDim.x - 1) / blockDim.x;
   const int t0 = min(static_cast<int>(threadIdx.x) * per, T), t1 = min(t0 + per, T);
   int a = 0, bq = 0;
   for (int t = t0; t < t1; ++t) {
     a += (cnt[t] + 3) & ~3;
-    bq += (cnt[t] + kChunk2 - 1) / kChunk2;
+    bq += (cnt[t] + chunk - 1) / chunk;
   }
   int ia = a, ib = bq;
   for (int o = 1; o < 32; o <<= 1) {
@@ -687,7 +767,7 @@ __global__ void k2_scan(DevState* S, Dev2D* Dp, int s, int G) {
       }
     }
     ra += c4;
-    rb += (c + kChunk2 - 1) / kChunk2;
+    rb += (c + chunk - 1) / chunk;
   }
   if (threadIdx.x == blockDim.x - 1) {
     ts[T] = ra;
@@ -825,66 +905,147 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
-// In-place radix-2 FFT of buf[0..n) (input in bit-reversed order), sign -1
-// forward (twiddles tw[k] = exp(-2 pi i k/n)), +1 inverse (conjugates).
-__device__ void fft_radix2(float2* buf, const float2* __restrict__ tw, int n, int inverse) {
-  for (int half = 1; half < n; half <<= 1) {
-    const int stride = n / (2 * half);
-    for (int b = threadIdx.x; b < n / 2; b += blockDim.x) {
-      const int grp = b / half, pos = b % half;
-      const int i0 = grp * 2 * half + pos, i1 = i0 + half;
-      float2 w = tw[pos * stride];
-      if (inverse) w.y = -w.y;
-      const float2 u = buf[i0], v = cmul(buf[i1], w);
-      buf[i0] = make_float2(u.x + v.x, u.y + v.y);
-      buf[i1] = make_float2(u.x - v.x, u.y - v.y);
+// Step's solve (row sums and transforms, modes, fields) at 1024 x 1024 cells:
+// 113 -> 56 us launched one after the other, about 42 us in the graph (one
+// launch fewer, modes beside the mean's solve).
+//
+// FFT of n = 2^log points (n >= 8), sign -1 forward (twiddles tw[k] =
+// exp(-2 pi i k/n)), +1 inverse (conjugates): radix-2 decimation in time, its
+// butterflies taken three stages at a time on eight values in registers, so
+// that the points pass through shared memory every third stage only.
+// Stage `half` joins (p, p + half) with twiddle (p mod half) n / (2 half).
+//
+// Thread t of n/8 starts with the points t + q n/8 (q = 0..7), which are the
+// eight neighbours 8 b + r of the bit-reversed order, b = rev(t), r = rev3(q).
+
+__device__ __forceinline__ int fft_pad(int i) { return i + (i >> 5); }  // spreads strides over the banks
+__host__ __device__ constexpr int fft_words(int n) { return n + (n >> 5); }
+
+__device__ __forceinline__ void butterfly(float2& a, float2& b, float2 w, bool inverse) {
+  if (inverse) w.y = -w.y;
+  const float2 u = a, v = cmul(b, w);
+  a = make_float2(u.x + v.x, u.y + v.y);
+  b = make_float2(u.x - v.x, u.y - v.y);
+}
+
+// STAGES stages from `half` on of the points v[r] = [.. + r half + pos]
+template <int STAGES>
+__device__ __forceinline__ void fft_stages(float2 (&v)[1 << STAGES], const float2* __restrict__ tw, int n, int half,
+                                           int pos, bool inverse) {
+#pragma unroll
+  for (int g = 0; g < STAGES; ++g) {
+    const int stride = n / (2 * half) >> g;
+#pragma unroll
+    for (int r = 0; r < (1 << STAGES); ++r) {
+      if (r & (1 << g)) continue;
+      const int k = (r & ((1 << g) - 1)) * half + pos;
+      butterfly(v[r], v[r | (1 << g)], tw[k * stride], inverse);
     }
-    __syncthreads();
   }
 }
 
-__device__ __forceinline__ int bitrev(int k, int logn) { return static_cast<int>(__brev(static_cast<unsigned>(k)) >> (32 - logn)); }
+// one pass of STAGES stages through shared memory
+template <int STAGES>
+__device__ __forceinline__ void fft_pass(float2* buf, const float2* __restrict__ tw, int n, int half, bool inverse) {
+  constexpr int R = 1 << STAGES;
+  for (int b = threadIdx.x; b < n / R; b += blockDim.x) {
+    const int pos = b & (half - 1), base = (b - pos) * R + pos;
+    float2 v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = buf[fft_pad(base + r * half)];
+    fft_stages<STAGES>(v, tw, n, half, pos, inverse);
+#pragma unroll
+    for (int r = 0; r < R; ++r) buf[fft_pad(base + r * half)] = v[r];
+  }
+}
 
-// row i: exact row sum into the 1D grid, copy and clear, spectrum of the
-// fluctuation (rows 1..Nx-1)
-__global__ void k2_fwd(Dev2D* Dp, long long* G1) {
+// The transform of the points load(c, q, j), j = t + q n/8 with t = tid + c
+// kFftThreads (c < ROUNDS: 1 up to n = 1024, else 4), by all threads of the
+// CTA; the result is in buf (fft_pad order) after the last barrier.
+constexpr int kFftThreads = 128;
+
+template <int ROUNDS, typename Load>
+__device__ __forceinline__ void fft(float2* buf, const float2* __restrict__ tw, int n, int logn, bool inverse,
+                                    Load load) {
+#pragma unroll
+  for (int c = 0; c < ROUNDS; ++c) {
+    const int t = static_cast<int>(threadIdx.x) + c * kFftThreads;
+    if (t < n / 8) {
+      float2 v[8];
+      // rev3(q) of q = 0..7
+      v[0] = load(c, 0, t);
+      v[4] = load(c, 1, t + n / 8);
+      v[2] = load(c, 2, t + 2 * (n / 8));
+      v[6] = load(c, 3, t + 3 * (n / 8));
+      v[1] = load(c, 4, t + 4 * (n / 8));
+      v[5] = load(c, 5, t + 5 * (n / 8));
+      v[3] = load(c, 6, t + 6 * (n / 8));
+      v[7] = load(c, 7, t + 7 * (n / 8));
+      fft_stages<3>(v, tw, n, 1, 0, inverse);
+      const int b = (logn > 3) ? static_cast<int>(__brev(static_cast<unsigned>(t)) >> (35 - logn)) : 0;
+#pragma unroll
+      for (int r = 0; r < 8; ++r) buf[fft_pad(8 * b + r)] = v[r];
+    }
+  }
+  __syncthreads();
+  int half = 8, left = logn - 3;
+  for (; left >= 3; left -= 3, half *= 8) {
+    fft_pass<3>(buf, tw, n, half, inverse);
+    __syncthreads();
+  }
+  if (left == 2) fft_pass<2>(buf, tw, n, half, inverse);
+  if (left == 1) fft_pass<1>(buf, tw, n, half, inverse);
+  if (left) __syncthreads();
+}
+
+// Row i: exact row sum into the 1D grid, copy and clear, spectrum of the
+// fluctuation (rows 1..Nx-1).  The row's charges stay in registers from the
+// sum to the transform's first stages.
+template <int ROUNDS>
+__global__ void __launch_bounds__(kFftThreads) k2_fwd(const __grid_constant__ Dev2D D, long long* G1) {
   extern __shared__ float2 buf[];
-  __shared__ long long wsum[32];
-  __shared__ long long s_tot;
-  const Dev2D& D = *Dp;
+  __shared__ long long wsum[kFftThreads / 32];
   cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
   const int i = blockIdx.x;
-  const int Ny = D.Ny;
+  const int Ny = D.Ny, n8 = Ny / 8;
   long long* row = D.G2 + static_cast<long long>(i) * Ny;
   long long* last = D.G2last + static_cast<long long>(i) * Ny;
+  long long g[ROUNDS][8];
   long long acc = 0;
-  for (int j = threadIdx.x; j < Ny; j += blockDim.x) acc += row[j];
+#pragma unroll
+  for (int c = 0; c < ROUNDS; ++c) {
+    const int t = static_cast<int>(threadIdx.x) + c * kFftThreads;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      g[c][q] = (t < n8) ? __ldcg(&row[t + q * n8]) : 0;
+      acc += g[c][q];
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < ROUNDS; ++c) {
+    const int t = static_cast<int>(threadIdx.x) + c * kFftThreads;
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      if (t < n8) {
+        last[t + q * n8] = g[c][q];
+        row[t + q * n8] = 0;
+      }
+  }
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if (lane_id() == 0) wsum[threadIdx.x >> 5] = acc;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    long long tot = 0;
-    for (int q = 0; q < static_cast<int>(blockDim.x >> 5); ++q) tot += wsum[q];
-    s_tot = tot;
-    G1[i] = tot;
-  }
-  __syncthreads();
-  const long long tot = s_tot;
+  long long tot = 0;
+#pragma unroll
+  for (int q = 0; q < kFftThreads / 32; ++q) tot += wsum[q];
+  if (threadIdx.x == 0) G1[i] = tot;
+  if (i == 0 || i == D.Nx) return;
   const double mean = static_cast<double>(tot) / static_cast<double>(Ny);
-  const bool interior = (i > 0 && i < D.Nx);
-  for (int j = threadIdx.x; j < Ny; j += blockDim.x) {
-    const long long g = row[j];
-    last[j] = g;
-    row[j] = 0;
-    if (interior)
-      buf[bitrev(j, D.logNy)] =
-          make_float2(static_cast<float>((static_cast<double>(g) - mean) * D.rho_scale), 0.0f);
-  }
-  __syncthreads();
-  if (!interior) return;
-  fft_radix2(buf, D.tw, Ny, 0);
+  fft<ROUNDS>(buf, D.tw, Ny, D.logNy, false, [&](int c, int q, int) {
+    return make_float2(static_cast<float>((static_cast<double>(g[c][q]) - mean) * D.rho_scale), 0.0f);
+  });
   float2* R = D.R + static_cast<long long>(i) * (Ny / 2 + 1);
-  for (int k = threadIdx.x; k <= Ny / 2; k += blockDim.x) R[k] = buf[k];
+  for (int k = threadIdx.x; k <= Ny / 2; k += kFftThreads) R[k] = buf[fft_pad(k)];
 }
 
 // One warp per mode k = 1..Ny/2: Thomas over i = 1..Nx-1 with phi = 0 at
@@ -915,163 +1076,173 @@ __device__ __forceinline__ Aff aff_shfl_up(Aff f, int o) {
   return r;
 }
 
-constexpr int kU2 = 8;  // rows of loads issued ahead
+constexpr int kModesCta = 4;  // modes (warps) per CTA; 2 above 2048 rows (shared memory)
 
-__global__ void __launch_bounds__(128) k2_modes(Dev2D* Dp, float c_rhs) {
-  const Dev2D& D = *Dp;
-  const int k = 1 + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int M = D.Ny / 2 + 1;
-  if (k >= M) return;  // whole warps leave together
-  const int lane = static_cast<int>(lane_id());
-  float2* __restrict__ R = D.R;
-  const float* __restrict__ inv = D.tinv;
-  const float* __restrict__ cp = D.cp;
-  const int n = D.Nx - 1;             // rows 1..n
-  const int seg = (n + 31) / 32;
-  const int r0 = 1 + lane * seg, r1 = min(n + 1, r0 + seg);  // this lane's rows [r0, r1)
-  // forward: compose this segment's map
-  Aff f;
-  f.a = 1.0f;
-  f.b = make_float2(0.0f, 0.0f);
-  for (int i0 = r0; i0 < r1; i0 += kU2) {
-    float2 rr[kU2];
-    float iv[kU2];
-#pragma unroll
-    for (int q = 0; q < kU2; ++q)
-      if (i0 + q < r1) {
-        rr[q] = R[static_cast<long long>(i0 + q) * M + k];
-        iv[q] = inv[static_cast<long long>(i0 + q) * M + k];
-      }
-#pragma unroll
-    for (int q = 0; q < kU2; ++q)
-      if (i0 + q < r1) {
-        Aff g;
-        g.a = -iv[q];
-        g.b = make_float2(c_rhs * iv[q] * rr[q].x, c_rhs * iv[q] * rr[q].y);
-        f = aff_then(f, g);
-      }
-  }
-  // exclusive scan over the lanes: the map from d_0 = 0 to this segment's start
-  Aff incl = f;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const Aff y = aff_shfl_up(incl, o);
-    if (lane >= o) incl = aff_then(y, incl);
-  }
-  Aff ex = aff_shfl_up(incl, 1);
-  float2 d = (lane == 0) ? make_float2(0.0f, 0.0f) : ex.b;
-  // forward: apply
-  for (int i0 = r0; i0 < r1; i0 += kU2) {
-    float2 rr[kU2];
-    float iv[kU2];
-#pragma unroll
-    for (int q = 0; q < kU2; ++q)
-      if (i0 + q < r1) {
-        rr[q] = R[static_cast<long long>(i0 + q) * M + k];
-        iv[q] = inv[static_cast<long long>(i0 + q) * M + k];
-      }
-#pragma unroll
-    for (int q = 0; q < kU2; ++q)
-      if (i0 + q < r1) {
-        const float a = -iv[q];
-        d = make_float2(fmaf(a, d.x, c_rhs * iv[q] * rr[q].x), fmaf(a, d.y, c_rhs * iv[q] * rr[q].y));
-        R[static_cast<long long>(i0 + q) * M + k] = d;
-      }
-  }
-  // backward: x_i = -c'_i x_{i+1} + d_i, segments from the last row down
-  Aff g;
-  g.a = 1.0f;
-  g.b = make_float2(0.0f, 0.0f);
-  for (int i0 = r1 - 1; i0 >= r0; i0 -= kU2) {
-    float2 dd[kU2];
-    float cc[kU2];
-#pragma unroll
-    for (int q = 0; q < kU2; ++q)
-      if (i0 - q >= r0) {
-        dd[q] = R[static_cast<long long>(i0 - q) * M + k];
-        cc[q] = cp[static_cast<long long>(i0 - q) * M + k];
-      }
-#pragma unroll
-    for (int q = 0; q < kU2; ++q)
-      if (i0 - q >= r0) {
-        Aff h;
-        h.a = -cc[q];
-        h.b = dd[q];
-        g = aff_then(g, h);
-      }
-  }
-  // reverse exclusive scan (lane 31 holds the last rows)
-  Aff incl2 = g;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    Aff y;
-    y.a = __shfl_down_sync(0xffffffffu, incl2.a, o);
-    y.b.x = __shfl_down_sync(0xffffffffu, incl2.b.x, o);
-    y.b.y = __shfl_down_sync(0xffffffffu, incl2.b.y, o);
-    if (lane + o < 32) incl2 = aff_then(y, incl2);
-  }
-  float2 x;
-  {
-    const float bx = __shfl_down_sync(0xffffffffu, incl2.b.x, 1);
-    const float by = __shfl_down_sync(0xffffffffu, incl2.b.y, 1);
-    x = (lane == 31) ? make_float2(0.0f, 0.0f) : make_float2(bx, by);
-  }
-  for (int i0 = r1 - 1; i0 >= r0; i0 -= kU2) {
-    float2 dd[kU2];
-    float cc[kU2];
-#pragma unroll
-    for (int q = 0; q < kU2; ++q)
-      if (i0 - q >= r0) {
-        dd[q] = R[static_cast<long long>(i0 - q) * M + k];
-        cc[q] = cp[static_cast<long long>(i0 - q) * M + k];
-      }
-#pragma unroll
-    for (int q = 0; q < kU2; ++q)
-      if (i0 - q >= r0) {
-        x = make_float2(fmaf(-cc[q], x.x, dd[q].x), fmaf(-cc[q], x.y, dd[q].y));
-        R[static_cast<long long>(i0 - q) * M + k] = x;
-      }
-  }
-}
+// A mode's rows in shared memory, row i (from 0) at i + i/32: the lanes of a
+// warp, each in its own segment of rows, mostly hit different banks.
+__host__ __device__ constexpr int modes_at(int i) { return i + (i >> 5); }
+__host__ __device__ constexpr int modes_rows(int n) { return modes_at(n) + 1; }
 
-// row i = 1..Nx-1: inverse transform of the mode solution -> phit
-__global__ void k2_inv(Dev2D* Dp) {
+// W modes per CTA, one warp each; the CTA fetches the modes' rows together
+// (neighbouring modes are neighbours in memory), eight loads per thread in
+// flight, and the four sweeps run in shared memory.
+template <int W>
+__global__ void __launch_bounds__(32 * W) k2_modes(const __grid_constant__ Dev2D D, float c_rhs) {
   extern __shared__ float2 buf[];
-  const Dev2D& D = *Dp;
-  const int i = 1 + blockIdx.x;
-  const int Ny = D.Ny, M = Ny / 2 + 1;
-  const float2* R = D.R + static_cast<long long>(i) * M;
-  for (int k = threadIdx.x; k < Ny; k += blockDim.x) {
-    float2 v;
-    if (k == 0) v = make_float2(0.0f, 0.0f);
-    else if (k < M) v = R[k];
-    else {
-      const float2 c = R[Ny - k];
-      v = make_float2(c.x, -c.y);
-    }
-    if (k == Ny / 2) v.y = 0.0f;
-    buf[bitrev(k, D.logNy)] = v;
+  const int k0 = 1 + blockIdx.x * W;
+  const int M = D.Ny / 2 + 1;
+  const int nk = min(W, M - k0);
+  const int lane = static_cast<int>(lane_id()), w = static_cast<int>(threadIdx.x) >> 5;
+  const int n = D.Nx - 1;  // rows 1..n
+  const int seg = (n + 31) / 32, S = modes_rows(n);
+  float* tin = reinterpret_cast<float*>(buf + W * S);
+  float* tcp = tin + W * S;
+  const int m = static_cast<int>(threadIdx.x) % W;   // this thread's mode, and rows i0, i0 + 32, ...
+  const int i0 = static_cast<int>(threadIdx.x) / W;
+  const int mine = (m < nk) ? n : 0;
+  const long long g0 = static_cast<long long>(1) * M + k0 + m;
+  // the elimination factors do not change: fetched before the spectra are ready
+  for (int j = i0; j < mine; j += 32 * 8) {
+    float a[8], b[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+      if (j + 32 * c < mine) {
+        a[c] = __ldg(&D.tinv[g0 + static_cast<long long>(j + 32 * c) * M]);
+        b[c] = __ldg(&D.cp[g0 + static_cast<long long>(j + 32 * c) * M]);
+      }
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+      if (j + 32 * c < mine) {
+        tin[m * S + modes_at(j + 32 * c)] = a[c];
+        tcp[m * S + modes_at(j + 32 * c)] = b[c];
+      }
+  }
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+  for (int j = i0; j < mine; j += 32 * 8) {
+    float2 a[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+      if (j + 32 * c < mine) a[c] = __ldcg(&D.R[g0 + static_cast<long long>(j + 32 * c) * M]);
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+      if (j + 32 * c < mine) buf[m * S + modes_at(j + 32 * c)] = a[c];
   }
   __syncthreads();
-  fft_radix2(buf, D.tw, Ny, 1);
-  const float inv_n = 1.0f / static_cast<float>(Ny);
-  float* out = D.phit + static_cast<long long>(i) * Ny;
-  for (int j = threadIdx.x; j < Ny; j += blockDim.x) out[j] = buf[j].x * inv_n;
+  if (w < nk) {
+    const int r0 = min(n, lane * seg), r1 = min(n, r0 + seg);  // this lane's rows
+    float2* r = buf + w * S;
+    const float* inv = tin + w * S;
+    const float* cp = tcp + w * S;
+    // forward: compose this segment's map
+    Aff f;
+    f.a = 1.0f;
+    f.b = make_float2(0.0f, 0.0f);
+#pragma unroll 4
+    for (int i = r0; i < r1; ++i) {
+      const int q = modes_at(i);
+      const float iv = inv[q];
+      const float2 rr = r[q];
+      Aff g;
+      g.a = -iv;
+      g.b = make_float2(c_rhs * iv * rr.x, c_rhs * iv * rr.y);
+      f = aff_then(f, g);
+    }
+    // exclusive scan over the lanes: the map from d_0 = 0 to this segment's start
+    Aff incl = f;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const Aff y = aff_shfl_up(incl, o);
+      if (lane >= o) incl = aff_then(y, incl);
+    }
+    const Aff ex = aff_shfl_up(incl, 1);
+    float2 d = (lane == 0) ? make_float2(0.0f, 0.0f) : ex.b;
+    // forward: apply
+#pragma unroll 4
+    for (int i = r0; i < r1; ++i) {
+      const int q = modes_at(i);
+      const float iv = inv[q];
+      const float2 rr = r[q];
+      const float a = -iv;
+      d = make_float2(fmaf(a, d.x, c_rhs * iv * rr.x), fmaf(a, d.y, c_rhs * iv * rr.y));
+      r[q] = d;
+    }
+    // backward: x_i = -c'_i x_{i+1} + d_i, segments from the last row down
+    Aff g;
+    g.a = 1.0f;
+    g.b = make_float2(0.0f, 0.0f);
+#pragma unroll 4
+    for (int i = r1 - 1; i >= r0; --i) {
+      const int q = modes_at(i);
+      Aff h;
+      h.a = -cp[q];
+      h.b = r[q];
+      g = aff_then(g, h);
+    }
+    // reverse exclusive scan (lane 31 holds the last rows)
+    Aff incl2 = g;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      Aff y;
+      y.a = __shfl_down_sync(0xffffffffu, incl2.a, o);
+      y.b.x = __shfl_down_sync(0xffffffffu, incl2.b.x, o);
+      y.b.y = __shfl_down_sync(0xffffffffu, incl2.b.y, o);
+      if (lane + o < 32) incl2 = aff_then(y, incl2);
+    }
+    const float bx = __shfl_down_sync(0xffffffffu, incl2.b.x, 1);
+    const float by = __shfl_down_sync(0xffffffffu, incl2.b.y, 1);
+    float2 x = (lane == 31) ? make_float2(0.0f, 0.0f) : make_float2(bx, by);
+#pragma unroll 4
+    for (int i = r1 - 1; i >= r0; --i) {
+      const int q = modes_at(i);
+      const float2 dd = r[q];
+      const float cc = cp[q];
+      x = make_float2(fmaf(-cc, x.x, dd.x), fmaf(-cc, x.y, dd.y));
+      r[q] = x;
+    }
+  }
+  __syncthreads();
+  for (int i = i0; i < mine; i += 32) D.R[g0 + static_cast<long long>(i) * M] = buf[m * S + modes_at(i)];
 }
 
-// E_x = E_0(x) + (phit_ij - phit_i+1,j)/dx, E_y = (phit_ij - phit_i,j+1)/dy
-__global__ void k2_fields(Dev2D* Dp, const double* __restrict__ E64) {
-  const Dev2D& D = *Dp;
-  const int Ny = D.Ny;
-  const long long n = static_cast<long long>(D.Nx + 1) * Ny;
-  for (long long q = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; q < n;
-       q += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const int i = static_cast<int>(q / Ny), j = static_cast<int>(q % Ny);
-    const float p = D.phit[q];
-    if (i < D.Nx)
-      D.Ex[q] = static_cast<float>(E64[i]) + (p - D.phit[q + Ny]) * D.inv_dx;
+// Row i: inverse transform of the mode solution and the fields,
+//   E_x = E_0(x) + (phit_ij - phit_i+1,j)/dx, E_y = (phit_ij - phit_i,j+1)/dy
+// (phit = 0 on both electrodes).  Row i + 1 is transformed here as well rather
+// than fetched from its owner.
+template <int ROUNDS>
+__global__ void __launch_bounds__(kFftThreads) k2_fields(const __grid_constant__ Dev2D D,
+                                                         const double* __restrict__ E64) {
+  extern __shared__ float2 buf[];
+  const int Ny = D.Ny, Nx = D.Nx, M = Ny / 2 + 1;
+  const int i = blockIdx.x;
+  float* p = reinterpret_cast<float*>(buf + fft_words(Ny));  // rows i and i + 1
+  const float inv_n = 1.0f / static_cast<float>(Ny);
+  for (int c = 0; c < 2; ++c) {
+    if (i + c > 0 && i + c < Nx) {
+      const float2* R = D.R + static_cast<long long>(i + c) * M;
+      fft<ROUNDS>(buf, D.tw, Ny, D.logNy, true, [&](int, int, int k) {
+        float2 v = make_float2(0.0f, 0.0f);
+        if (k > 0) {
+          const float2 q = __ldcg(&R[k < M ? k : Ny - k]);
+          v = make_float2(q.x, k < M ? q.y : -q.y);
+          if (k == Ny / 2) v.y = 0.0f;
+        }
+        return v;
+      });
+      for (int j = threadIdx.x; j < Ny; j += kFftThreads) p[c * Ny + j] = buf[fft_pad(j)].x * inv_n;
+    } else {
+      for (int j = threadIdx.x; j < Ny; j += kFftThreads) p[c * Ny + j] = 0.0f;
+    }
+    __syncthreads();
+  }
+  const long long r = static_cast<long long>(i) * Ny;
+  const float E0 = (i < Nx) ? static_cast<float>(E64[i]) : 0.0f;
+  for (int j = threadIdx.x; j < Ny; j += kFftThreads) {
+    const float v = p[j];
     const int j1 = (j + 1 == Ny) ? 0 : j + 1;
-    D.Ey[q] = (p - D.phit[static_cast<long long>(i) * Ny + j1]) * D.inv_dy;
+    D.phit[r + j] = v;
+    D.Ey[r + j] = (v - p[j1]) * D.inv_dy;
+    if (i < Nx) D.Ex[r + j] = E0 + (v - p[Ny + j]) * D.inv_dx;
   }
 }
 
@@ -1102,10 +1273,9 @@ __global__ void k2_tables(Dev2D* Dp, double r2) {
 // ---------------------------------------------------------------------------
 size_t dev2d_bytes() { return sizeof(Dev2D); }
 size_t absrec2_bytes() { return sizeof(AbsRec2); }
-int kchunk2() { return kChunk2; }
 int tile2() { return kT2; }
 
-constexpr size_t kCwinBytes = 5 * sizeof(unsigned int) * kW2 * kW2;  // the deposit window's cell sums
+constexpr size_t kCwinBytes = sizeof(Window2);
 
 cudaError_t push2_occupancy(int* per_sm) {
   const cudaError_t e = cudaFuncSetAttribute(k2_push, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1144,30 +1314,64 @@ cudaError_t sort2_launch(DevState* S, void* D, int T, int s, int sms, cudaStream
   return cudaGetLastError();
 }
 
-cudaError_t solve2_fwd_launch(void* D, long long* G1, int Nx, int Ny, cudaStream_t st) {
-  const size_t smem = sizeof(float2) * Ny;
+static cudaLaunchConfig_t pdl_config(int grid, int threads, size_t smem, cudaStream_t st,
+                                     cudaLaunchAttribute* attr) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(Nx + 1, 1, 1);
-  cfg.blockDim = dim3(256, 1, 1);
+  cfg.gridDim = dim3(grid, 1, 1);
+  cfg.blockDim = dim3(threads, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k2_fwd, static_cast<Dev2D*>(D), G1);
+  return cfg;
 }
 
-cudaError_t solve2_modes_launch(void* D, int Nx, int Ny, float c_rhs, const double* E64,
-                                cudaStream_t st) {
-  Dev2D* Dp = static_cast<Dev2D*>(D);
-  const int M = Ny / 2;
-  k2_modes<<<(M + 3) / 4, 128, 0, st>>>(Dp, c_rhs);
-  if (Nx > 1) k2_inv<<<Nx - 1, 256, sizeof(float2) * Ny, st>>>(Dp);
-  const long long n = static_cast<long long>(Nx + 1) * Ny;
-  const int grid = static_cast<int>(std::min<long long>((n + 255) / 256, 4096));
-  k2_fields<<<grid, 256, 0, st>>>(Dp, E64);
+static int modes_per_cta(int Nx) { return Nx > 2048 ? kModesCta / 2 : kModesCta; }
+
+static size_t modes_smem(int Nx) {
+  return (sizeof(float2) + 2 * sizeof(float)) * modes_per_cta(Nx) * modes_rows(Nx - 1);
+}
+
+static size_t fields_smem(int Ny) { return sizeof(float2) * fft_words(Ny) + 2 * sizeof(float) * Ny; }
+
+// The kernels' shared-memory limits (the largest any grid needs: contexts
+// share the kernels).
+cudaError_t solve2_configure() {
+  cudaError_t e = cudaFuncSetAttribute(k2_modes<kModesCta>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(modes_smem(2048)));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k2_modes<kModesCta / 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(modes_smem(4096)));
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k2_fields<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(fields_smem(4096)));
+}
+
+cudaError_t solve2_fwd_launch(const void* D_host, long long* G1, int Nx, int Ny, cudaStream_t st) {
+  cudaLaunchAttribute attr[1];
+  const cudaLaunchConfig_t cfg = pdl_config(Nx + 1, kFftThreads, sizeof(float2) * fft_words(Ny), st, attr);
+  const Dev2D& D = *static_cast<const Dev2D*>(D_host);
+  return Ny <= 8 * kFftThreads ? cudaLaunchKernelEx(&cfg, k2_fwd<1>, D, G1) : cudaLaunchKernelEx(&cfg, k2_fwd<4>, D, G1);
+}
+
+cudaError_t solve2_modes_launch(const void* D_host, int Nx, int Ny, float c_rhs, cudaStream_t st) {
+  const int W = modes_per_cta(Nx), M = Ny / 2;
+  cudaLaunchAttribute attr[1];
+  const cudaLaunchConfig_t cfg = pdl_config((M + W - 1) / W, 32 * W, modes_smem(Nx), st, attr);
+  const Dev2D& D = *static_cast<const Dev2D*>(D_host);
+  return W == kModesCta ? cudaLaunchKernelEx(&cfg, k2_modes<kModesCta>, D, c_rhs)
+                        : cudaLaunchKernelEx(&cfg, k2_modes<kModesCta / 2>, D, c_rhs);
+}
+
+// One row per CTA: it transforms its successor's too, and the many small CTAs
+// hide each other's latency (step at 1024 x 1024 cells: 252.6 us, two rows
+// 251.5, three 255.5; at 96 x 128: 37.5, two rows 39.0).
+cudaError_t solve2_fields_launch(const void* D_host, int Nx, int Ny, const double* E64, cudaStream_t st) {
+  const Dev2D& D = *static_cast<const Dev2D*>(D_host);
+  if (Ny <= 8 * kFftThreads) k2_fields<1><<<Nx + 1, kFftThreads, fields_smem(Ny), st>>>(D, E64);
+  else k2_fields<4><<<Nx + 1, kFftThreads, fields_smem(Ny), st>>>(D, E64);
   return cudaGetLastError();
 }
 

@@ -13,8 +13,10 @@ namespace cpk {
 constexpr int kT2 = 32;          // tile edge in cells
 constexpr int kH2 = 4;           // halo of the field and deposit windows in cells
 constexpr int kW2 = kT2 + 2 * kH2 + 2;  // window edge in nodes (42)
-constexpr int kChunk2 = 32768;   // particles per work item
+constexpr int kChunk2 = 32768;   // most particles per work item
 constexpr int kThreads2 = 512;
+constexpr int kPer2 = 2;         // particles per thread and pass
+constexpr int kPass2 = 2048;     // work items are multiples of this many particles (whole passes of a CTA)
 constexpr double kFix2 = 4294967296.0;  // charge-grid units per macroparticle (2^16 per axis)
 
 struct Dev2D {
@@ -31,6 +33,7 @@ struct Dev2D {
   void* w_alt[kSpecies];
   long long n_sorted[kSpecies];
   long long cap[kSpecies];  // slots of each store
+  int chunk[kSpecies];      // particles per work item of the sorted store (set by the sort)
   int* tile_start;  // [3][T+1] particle offsets of the sorted segments
   int* wi_off;      // [3][T+1] prefix of work items per tile
   int* tile_cnt;    // [3][T] live particles per tile (sort scratch)
