@@ -51,7 +51,7 @@ cudaError_t status_ens_launch(const Bufs* Ball, int E, int* out, cudaStream_t st
 cudaError_t push2_occupancy(int* per_sm);
 cudaError_t push2_launch(const DevParams* P, DevState* S, void* D, const void* D_host, void* abs,
                          int abs_cap, int grid, cudaStream_t st);
-cudaError_t sort2_launch(DevState* S, void* D, int T, int s, int sms, cudaStream_t st);
+cudaError_t sort2_launch(DevState* S, void* D, int T, int sms, cudaStream_t st);
 cudaError_t solve2_configure();
 cudaError_t solve2_fwd_launch(const void* D_host, long long* G1, int Nx, int Ny, cudaStream_t st);
 cudaError_t solve2_modes_launch(const void* D_host, int Nx, int Ny, float c_rhs, cudaStream_t st);
@@ -1609,8 +1609,8 @@ int g2_solve(cp_gap2d* g, cudaStream_t st, bool fork, int do_push, int mode, dou
 
 int g2_sort(cp_gap2d* g, cudaStream_t st) {
   cp_ctx* c = g->c;
-  for (int s = 0; s < kSpecies; ++s) CP_CUDA(cpk::sort2_launch(c->dS, g->dD, g->T, s, g->sms, st));
-  g->launches += 6 * kSpecies;
+  CP_CUDA(cpk::sort2_launch(c->dS, g->dD, g->T, g->sms, st));
+  g->launches += 5;
   return CP_OK;
 }
 
@@ -1758,7 +1758,6 @@ int g2_init(cp_gap2d* g, int mode, double tol) {
   CP_TRY(g2_alloc(g, &p, sizeof(int) * 3 * (T + 1))); D.tile_start = static_cast<int*>(p);
   CP_TRY(g2_alloc(g, &p, sizeof(int) * 3 * (T + 1))); D.wi_off = static_cast<int*>(p);
   CP_TRY(g2_alloc(g, &p, sizeof(int) * 3 * T)); D.tile_cnt = static_cast<int*>(p);
-  CP_TRY(g2_alloc(g, &p, sizeof(int) * 3 * T)); D.tile_cur = static_cast<int*>(p);
   CP_TRY(g2_alloc(g, &p, sizeof(float) * Nx * Ny)); D.Ex = static_cast<float*>(p);
   CP_TRY(g2_alloc(g, &p, sizeof(float) * nodes)); D.Ey = static_cast<float*>(p);
   CP_TRY(g2_alloc(g, &p, sizeof(long long) * nodes)); D.G2 = static_cast<long long*>(p);
@@ -1769,8 +1768,9 @@ int g2_init(cp_gap2d* g, int mode, double tol) {
   CP_TRY(g2_alloc(g, &p, sizeof(float) * nodes)); D.phit = static_cast<float*>(p);
   CP_TRY(g2_alloc(g, &p, sizeof(float) * M)); D.kappa = static_cast<float*>(p);
   CP_TRY(g2_alloc(g, &p, sizeof(float2) * (Ny / 2))); D.tw = static_cast<float2*>(p);
-  for (int* q : {D.tile_start, D.wi_off}) CP_CUDA(cudaMemsetAsync(q, 0, sizeof(int) * 3 * (T + 1), c->stream));
-  for (int* q : {D.tile_cnt, D.tile_cur}) CP_CUDA(cudaMemsetAsync(q, 0, sizeof(int) * 3 * T, c->stream));
+  CP_CUDA(cudaMemsetAsync(D.tile_start, 0, sizeof(int) * 3 * (T + 1), c->stream));
+  CP_CUDA(cudaMemsetAsync(D.wi_off, 0, sizeof(int) * 3 * (T + 1), c->stream));
+  CP_CUDA(cudaMemsetAsync(D.tile_cnt, 0, sizeof(int) * 3 * T, c->stream));
   CP_CUDA(cudaMemsetAsync(D.G2, 0, sizeof(long long) * nodes, c->stream));
   CP_CUDA(cudaMemsetAsync(D.G2last, 0, sizeof(long long) * nodes, c->stream));
   CP_CUDA(cudaMemsetAsync(D.phit, 0, sizeof(float) * nodes, c->stream));
@@ -1814,7 +1814,7 @@ int g2_init(cp_gap2d* g, int mode, double tol) {
   CP_CUDA(cpk::tables2_launch(g->dD, Ny, (D.dx / D.dy) * (D.dx / D.dy), c->stream));
   int per_sm = 0;
   CP_CUDA(cudaDeviceGetAttribute(&g->sms, cudaDevAttrMultiProcessorCount, c->device));
-  CP_TRY(g2_alloc(g, &p, sizeof(int) * 2 * g->sms * T));
+  CP_TRY(g2_alloc(g, &p, sizeof(int) * 2 * g->sms * T * kSpecies));
   D.bhist = static_cast<int*>(p);
   CP_CUDA(cudaMemcpyAsync(&g->dD->bhist, &D.bhist, sizeof(int*), cudaMemcpyHostToDevice, c->stream));
   CP_CUDA(cpk::push2_occupancy(&per_sm));
@@ -1877,7 +1877,7 @@ int g2_steps(cp_gap2d* g, int mode, int32_t n_steps, double tol) {
     if (!g->timing && g->since_sort == 0 && n_steps - k >= g->sort_every) {
       CP_TRY(g2_build_graph(g, mode, tol));
       CP_CUDA(cudaGraphLaunch(c->gexec[mode], c->stream));
-      g->launches += 5 * g->sort_every + 6 * kSpecies;
+      g->launches += 5 * g->sort_every + 5;
       k += g->sort_every;
       continue;
     }

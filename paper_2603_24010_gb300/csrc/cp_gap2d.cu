@@ -673,8 +673,19 @@ __device__ __forceinline__ void block_range(long long n, long long* b0, long lon
   *b1 = n * (blockIdx.x + 1) / gridDim.x;
 }
 
-__global__ void k2_hist(const DevState* S, Dev2D* Dp, int s) {
+// exclusive prefix of v over the block's threads (blockDim a multiple of 32)
+__device__ __forceinline__ int block_excl_scan(int v, int* wsum) {
+  const int incl = warp_incl_scan(v);
+  if (lane_id() == 31) wsum[threadIdx.x >> 5] = incl;
+  __syncthreads();
+  int base = 0;
+  for (int q = 0; q < static_cast<int>(threadIdx.x >> 5); ++q) base += wsum[q];
+  return base + incl - v;
+}
+
+__global__ void k2_hist(const DevState* S, Dev2D* Dp) {
   extern __shared__ int hist[];
+  const int s = blockIdx.y;
   const Dev2D& D = *Dp;
   for (int t = threadIdx.x; t < D.T; t += blockDim.x) hist[t] = 0;
   __syncthreads();
@@ -708,57 +719,27 @@ __global__ void k2_hist(const DevState* S, Dev2D* Dp, int s) {
   }
   __syncthreads();
   const int G = gridDim.x;  // layout [tile][block]: each tile's counts contiguous
-  for (int t = threadIdx.x; t < D.T; t += blockDim.x) D.bhist[static_cast<long long>(t) * G + blockIdx.x] = hist[t];
+  for (int t = threadIdx.x; t < D.T; t += blockDim.x) D.bhist[(static_cast<long long>(s) * D.T + t) * G + blockIdx.x] = hist[t];
 }
 
-// one block: tile totals and per-block offsets, tile segment starts (padded
-// to 4), work-item prefix, dead padding in the destination, block bases
-__global__ void k2_scan(DevState* S, Dev2D* Dp, int s, int G) {
+// one block per species: tile segment starts (padded to 4) and the dead
+// padding in the destination
+__global__ void k2_scan(DevState* S, Dev2D* Dp) {
   Dev2D& D = *Dp;
-  __shared__ int wsum[32], wsum2[32];
-  const int T = D.T;
-  int* cnt = D.tile_cnt + s * T;
+  __shared__ int wsum[32];
+  const int s = blockIdx.x, T = D.T;
+  const int* cnt = D.tile_cnt + s * T;
   int* ts = D.tile_start + s * (T + 1);
-  int* wo = D.wi_off + s * (T + 1);
-  // Particles per work item: about two items for each of the push's G CTAs, so
-  // that small stores reach every SM, in whole passes of a CTA; at most
-  // kChunk2 (the deposit window's 32-bit sums).
-  const long long want = (S->n_proc[s] / (2 * G) + kPass2 - 1) / kPass2;
-  const int chunk = kPass2 * static_cast<int>(max(1LL, min(want, static_cast<long long>(kChunk2 / kPass2))));
-  if (threadIdx.x == 0) D.chunk[s] = chunk;
   const int per = (T + blockDim.x - 1) / blockDim.x;
   const int t0 = min(static_cast<int>(threadIdx.x) * per, T), t1 = min(t0 + per, T);
-  int a = 0, bq = 0;
-  for (int t = t0; t < t1; ++t) {
-    a += (cnt[t] + 3) & ~3;
-    bq += (cnt[t] + chunk - 1) / chunk;
-  }
-  int ia = a, ib = bq;
-  for (int o = 1; o < 32; o <<= 1) {
-    const int ya = __shfl_up_sync(0xffffffffu, ia, o), yb = __shfl_up_sync(0xffffffffu, ib, o);
-    if (static_cast<int>(lane_id()) >= o) {
-      ia += ya;
-      ib += yb;
-    }
-  }
-  const int w = threadIdx.x >> 5;
-  if (lane_id() == 31) {
-    wsum[w] = ia;
-    wsum2[w] = ib;
-  }
-  __syncthreads();
-  int ba = 0, bb = 0;
-  for (int q = 0; q < w; ++q) {
-    ba += wsum[q];
-    bb += wsum2[q];
-  }
-  int ra = ba + ia - a, rb = bb + ib - bq;
+  int a = 0;
+  for (int t = t0; t < t1; ++t) a += (cnt[t] + 3) & ~3;
+  int ra = block_excl_scan(a, wsum);
   float* xd = reinterpret_cast<float*>(S->xi_alt[s]);
   float* ud = reinterpret_cast<float*>(S->u_alt[s]);
   const long long cap = D.cap[s];
   for (int t = t0; t < t1; ++t) {
     ts[t] = ra;
-    wo[t] = rb;
     const int c = cnt[t], c4 = (c + 3) & ~3;
     for (int k = c; k < c4; ++k) {  // dead padding slots
       if (ra + k < cap) {
@@ -767,59 +748,36 @@ __global__ void k2_scan(DevState* S, Dev2D* Dp, int s, int G) {
       }
     }
     ra += c4;
-    rb += (c + chunk - 1) / chunk;
   }
-  if (threadIdx.x == blockDim.x - 1) {
-    ts[T] = ra;
-    wo[T] = rb;
-  }
+  if (threadIdx.x == blockDim.x - 1) ts[T] = ra;
 }
 
 // one block per tile: exclusive scan of the per-block counts over the blocks
 // (each block's offset within the tile) and the tile's total
-__global__ void k2_tilescan(Dev2D* Dp, int s, int G) {
+__global__ void k2_tilescan(Dev2D* Dp, int G) {
   Dev2D& D = *Dp;
   __shared__ int wsum[32];
-  const int t = blockIdx.x, T = D.T;
+  const int t = blockIdx.x, s = blockIdx.y, T = D.T;
   const int per = (G + blockDim.x - 1) / blockDim.x;
   const int b0 = min(static_cast<int>(threadIdx.x) * per, G), b1 = min(b0 + per, G);
-  int* col = D.bhist + static_cast<long long>(t) * G;
+  int* col = D.bhist + (static_cast<long long>(s) * T + t) * G;
   int loc = 0;
   for (int b = b0; b < b1; ++b) loc += col[b];
-  int incl = loc;
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (static_cast<int>(lane_id()) >= o) incl += y;
-  }
-  const int w = threadIdx.x >> 5;
-  if (lane_id() == 31) wsum[w] = incl;
-  __syncthreads();
-  int base = 0;
-  for (int q = 0; q < w; ++q) base += wsum[q];
-  int run = base + incl - loc;
+  int run = block_excl_scan(loc, wsum);
   for (int b = b0; b < b1; ++b) {
     const int c = col[b];
     col[b] = run;
     run += c;
   }
-  if (threadIdx.x == blockDim.x - 1) D.tile_cnt[s * T + t] = base + incl;
+  if (threadIdx.x == blockDim.x - 1) D.tile_cnt[s * T + t] = run;
 }
 
-// block bases: tile start + the block's offset within the tile
-__global__ void k2_bases(Dev2D* Dp, int s, int G) {
-  Dev2D& D = *Dp;
-  const long long n = static_cast<long long>(G) * D.T;
-  const int* ts = D.tile_start + s * (D.T + 1);
-  for (long long q = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; q < n;
-       q += static_cast<long long>(gridDim.x) * blockDim.x)
-    D.bhist[q] += ts[q / G];
-}
-
-__global__ void __launch_bounds__(512, 2) k2_scatter(const DevState* S, Dev2D* Dp, int s) {
+__global__ void __launch_bounds__(512, 2) k2_scatter(const DevState* S, Dev2D* Dp) {
   extern __shared__ int cur[];
   const Dev2D& D = *Dp;
-  for (int t = threadIdx.x; t < D.T; t += blockDim.x)
-    cur[t] = D.bhist[static_cast<long long>(t) * gridDim.x + blockIdx.x];
+  const int s = blockIdx.y;
+  for (int t = threadIdx.x; t < D.T; t += blockDim.x)  // this block's first slot in each tile
+    cur[t] = D.tile_start[s * (D.T + 1) + t] + D.bhist[(static_cast<long long>(s) * D.T + t) * gridDim.x + blockIdx.x];
   __syncthreads();
   const float* xs = reinterpret_cast<const float*>(S->xi[s]);
   const float* us = reinterpret_cast<const float*>(S->u[s]);
@@ -865,7 +823,7 @@ __global__ void __launch_bounds__(512, 2) k2_scatter(const DevState* S, Dev2D* D
       base = __shfl_sync(0xffffffffu, base, rs);
       if (t < 0) continue;
       const long long o = static_cast<long long>(base) + (static_cast<int>(lane_id()) - rs);
-      if (o >= D.cap[s]) continue;  // the sorted store would not fit (reported by k2_swap)
+      if (o >= D.cap[s]) continue;  // the sorted store would not fit (reported by k2_finish)
       xd[o] = x[c];
       ud[o] = u[c];
       yd[o] = y[c];
@@ -875,9 +833,31 @@ __global__ void __launch_bounds__(512, 2) k2_scatter(const DevState* S, Dev2D* D
   }
 }
 
-// swap the sorted buffers in; one thread
-__global__ void k2_swap(DevState* S, Dev2D* Dp, int s) {
+// One block per species: the push's work items and the sorted buffers swapped
+// in.  An item holds at most `chunk` particles of one tile: about two items
+// for each of the push's G CTAs, so that small stores reach every SM, in
+// whole passes of a CTA, and at most kChunk2 (the deposit window's sums).
+__global__ void k2_finish(DevState* S, Dev2D* Dp, int G) {
   Dev2D& D = *Dp;
+  __shared__ int wsum[32];
+  const int s = blockIdx.x, T = D.T;
+  const int* cnt = D.tile_cnt + s * T;
+  int* wo = D.wi_off + s * (T + 1);
+  const long long n = D.tile_start[s * (T + 1) + T];
+  const long long want = (n / (2 * G) + kPass2 - 1) / kPass2;
+  const int chunk = kPass2 * static_cast<int>(max(1LL, min(want, static_cast<long long>(kChunk2 / kPass2))));
+  const int per = (T + blockDim.x - 1) / blockDim.x;
+  const int t0 = min(static_cast<int>(threadIdx.x) * per, T), t1 = min(t0 + per, T);
+  int a = 0;
+  for (int t = t0; t < t1; ++t) a += (cnt[t] + chunk - 1) / chunk;
+  int run = block_excl_scan(a, wsum);
+  for (int t = t0; t < t1; ++t) {
+    wo[t] = run;
+    run += (cnt[t] + chunk - 1) / chunk;
+  }
+  if (threadIdx.x == blockDim.x - 1) wo[T] = run;
+  if (threadIdx.x != 0) return;
+  D.chunk[s] = chunk;
   void* t;
   t = S->xi[s]; S->xi[s] = S->xi_alt[s]; S->xi_alt[s] = t;
   t = S->u[s]; S->u[s] = S->u_alt[s]; S->u_alt[s] = t;
@@ -888,14 +868,14 @@ __global__ void k2_swap(DevState* S, Dev2D* Dp, int s) {
     S->id = S->id_alt;
     S->id_alt = ti;
   }
-  long long n = D.tile_start[s * (D.T + 1) + D.T];
-  if (n > D.cap[s]) {
-    n = D.cap[s] & ~3LL;
+  long long m = D.tile_start[s * (T + 1) + T];
+  if (m > D.cap[s]) {
+    m = D.cap[s] & ~3LL;
     atomicCAS(&S->status, 0, CP_ERR_CAPACITY);
   }
-  D.n_sorted[s] = n;
-  S->n_alloc[s] = n;
-  S->n_proc[s] = n;
+  D.n_sorted[s] = m;
+  S->n_alloc[s] = m;
+  S->n_proc[s] = m;
 }
 
 // ---------------------------------------------------------------------------
@@ -1301,16 +1281,15 @@ cudaError_t push2_launch(const DevParams* P, DevState* S, void* D, const void* D
                             static_cast<AbsRec2*>(abs), abs_cap);
 }
 
-cudaError_t sort2_launch(DevState* S, void* D, int T, int s, int sms, cudaStream_t st) {
+cudaError_t sort2_launch(DevState* S, void* D, int T, int sms, cudaStream_t st) {
   Dev2D* Dp = static_cast<Dev2D*>(D);
   const size_t hs = sizeof(int) * T;
   const int G = 2 * sms;  // must match the blocks the per-block histograms were sized for
-  k2_hist<<<G, 512, hs, st>>>(S, Dp, s);
-  k2_tilescan<<<T, 128, 0, st>>>(Dp, s, G);
-  k2_scan<<<1, 1024, 0, st>>>(S, Dp, s, G);
-  k2_bases<<<std::min(4096, (G * T + 255) / 256), 256, 0, st>>>(Dp, s, G);
-  k2_scatter<<<G, 512, hs, st>>>(S, Dp, s);
-  k2_swap<<<1, 1, 0, st>>>(S, Dp, s);
+  k2_hist<<<dim3(G, kSpecies), 512, hs, st>>>(S, Dp);
+  k2_tilescan<<<dim3(T, kSpecies), 128, 0, st>>>(Dp, G);
+  k2_scan<<<kSpecies, 1024, 0, st>>>(S, Dp);
+  k2_scatter<<<dim3(G, kSpecies), 512, hs, st>>>(S, Dp);
+  k2_finish<<<kSpecies, 1024, 0, st>>>(S, Dp, G);
   return cudaGetLastError();
 }
 
@@ -1339,6 +1318,10 @@ static size_t fields_smem(int Ny) { return sizeof(float2) * fft_words(Ny) + 2 * 
 // The kernels' shared-memory limits (the largest any grid needs: contexts
 // share the kernels).
 cudaError_t solve2_configure() {
+  const int most = static_cast<int>(sizeof(int)) * (4096 / kT2) * (4096 / kT2);  // the sort's tile counters
+  cudaError_t es = cudaFuncSetAttribute(k2_hist, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (es == cudaSuccess) es = cudaFuncSetAttribute(k2_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (es != cudaSuccess) return es;
   cudaError_t e = cudaFuncSetAttribute(k2_modes<kModesCta>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(modes_smem(2048)));
   if (e == cudaSuccess)

@@ -37,7 +37,6 @@ struct Dev2D {
   int* tile_start;  // [3][T+1] particle offsets of the sorted segments
   int* wi_off;      // [3][T+1] prefix of work items per tile
   int* tile_cnt;    // [3][T] live particles per tile (sort scratch)
-  int* tile_cur;    // [3][T] scatter cursors
   float* Ex;        // [Nx][Ny]   E_x at (i+1/2, j)
   float* Ey;        // [Nx+1][Ny] E_y at (i, j+1/2)
   long long* G2;    // [Nx+1][Ny] charge being deposited
@@ -45,7 +44,7 @@ struct Dev2D {
   float2* R;        // [Nx+1][Ny/2+1] transverse spectra
   float* cp;        // [Nx+1][Ny/2+1] Thomas factors c'_i of each mode
   float* tinv;      // [Nx+1][Ny/2+1] Thomas factors 1/(b - c'_{i-1}) of each mode
-  int* bhist;       // [sort blocks][T] per-block tile counts, then bases
+  int* bhist;       // [3][T][sort blocks] per-block tile counts, then offsets within the tile
   float* phit;      // [Nx+1][Ny] potential of the k != 0 modes
   float* kappa;     // [Ny/2+1] (dx/dy)^2 (2 - 2 cos 2 pi k/Ny)
   float2* tw;       // [Ny/2] exp(-2 pi i k/Ny)
