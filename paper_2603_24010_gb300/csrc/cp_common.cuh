@@ -47,6 +47,21 @@ __device__ __forceinline__ void store4(double* p, const double (&v)[4]) {
   __stcs(reinterpret_cast<double2*>(p) + 1, make_double2(v[2], v[3]));
 }
 
+// floor(x) of |x| < 2^22 as the bits of 1.5 2^23 + floor(x), one addition
+// rounded down: the integer is bits - kFloorBits and the value r - kFloorMagic
+// (no floor or conversion instruction: those issue at a quarter rate)
+constexpr float kFloorMagic = 12582912.0f;
+constexpr int kFloorBits = 0x4B400000;
+__device__ __forceinline__ int floor_split(float x, float* frac) {
+  const float r = __fadd_rd(x, kFloorMagic);
+  *frac = x - (r - kFloorMagic);
+  return __float_as_int(r) - kFloorBits;
+}
+// floor(f 2^16) of a fraction f in [0, 1), from the mantissa of 2^23 + f 2^16
+__device__ __forceinline__ unsigned int frac16(float f) {
+  return __float_as_uint(__fmaf_rd(f, 65536.0f, 8388608.0f)) & 0xFFFFu;
+}
+
 // floor(f 2^16) of a fraction f in [0, 1): exact power-of-two scaling, truncation
 __device__ __forceinline__ unsigned int frac_to_fix(float f) { return __float2uint_rz(f * 65536.0f); }
 __device__ __forceinline__ unsigned int frac_to_fix(double f) { return __double2uint_rz(f * 65536.0); }
@@ -83,12 +98,26 @@ __device__ __forceinline__ real nudge_inside(double x, int N) {
   return r;
 }
 
+// a / b correctly rounded, for a divisor used many times: r = 1 / b rounded.
+// Two residual corrections of a r (Markstein 1990: with r the rounded
+// reciprocal and q within one ulp of the quotient, q + r (a - q b) rounds to
+// a / b); infinities and NaN go through the product.
+__device__ __forceinline__ double div_by(double a, double b, double r) {
+  const double q0 = __dmul_rn(a, r);
+  const double q1 = __fma_rn(__fma_rn(-q0, b, a), r, q0);
+  const double q2 = __fma_rn(__fma_rn(-q1, b, a), r, q1);
+  return isfinite(q0) ? q2 : q0;
+}
+
+__device__ __forceinline__ double over_E_ref(const DevParams* P, double E) { return __ddiv_rn(E, P->E_ref_eV); }
+
 // Mean yield and count of one impact, in FP64 with every operation rounded
 // as written (no contraction), so a given velocity decides the same count
 // as any IEEE binary64 evaluation in the same order.
-__device__ __forceinline__ int see_count(const DevParams* P, double Eev, uint64_t id, int64_t step) {
-  double g = __dmul_rn(__dmul_rn(P->see_scale, P->gamma_coef),
-                       __dsqrt_rn(__ddiv_rn(Eev, P->E_ref_eV)));
+// (Params: DevParams or a copy of the fields used here.)
+template <typename Params>
+__device__ __forceinline__ int see_count(const Params* P, double Eev, uint64_t id, int64_t step) {
+  double g = __dmul_rn(__dmul_rn(P->see_scale, P->gamma_coef), __dsqrt_rn(over_E_ref(P, Eev)));
   if (g > P->gamma_max) g = P->gamma_max;
   if (!(g > 0.0)) g = 0.0;
   const U64x4 w = philox4x64_10(id, static_cast<uint64_t>(step), 0, 0, P->seed, kTagSee);
@@ -113,8 +142,8 @@ __device__ __forceinline__ int see_count(const DevParams* P, double Eev, uint64_
 // it has flown (draws 0, 1: Box-Muller normal z; draw 2: the fraction) of
 // counter (id, step, 1 + j): |z| sqrt(e T_emit / m_e) (half-Maxwellian), or
 // the lognormal law of Algorithm see_sampling_1d, E = exp(mu + sigma z) eV.
-__device__ __forceinline__ double see_speed(const DevParams* P, uint64_t id, int64_t step, int j,
-                                            double* frac) {
+template <typename Params>
+__device__ __forceinline__ double see_speed(const Params* P, uint64_t id, int64_t step, int j, double* frac) {
   const double pi = 3.14159265358979323846;
   const U64x4 wv = philox4x64_10(id, static_cast<uint64_t>(step), static_cast<uint64_t>(1 + j), 0,
                                  P->seed, kTagSee);

@@ -79,21 +79,6 @@ __device__ __forceinline__ Stencil2 stencil2(const Dev2D& D, float x, float y) {
   return st;
 }
 
-// floor(x) of |x| < 2^22 as the bits of 1.5 2^23 + floor(x), one addition
-// rounded down: the integer is bits - kFloorBits and the value r - kFloorMagic
-// (no floor or conversion instruction: those issue at a quarter rate)
-constexpr float kFloorMagic = 12582912.0f;
-constexpr int kFloorBits = 0x4B400000;
-__device__ __forceinline__ int floor_split(float x, float* frac) {
-  const float r = __fadd_rd(x, kFloorMagic);
-  *frac = x - (r - kFloorMagic);
-  return __float_as_int(r) - kFloorBits;
-}
-// floor(f 2^16) of a fraction f in [0, 1), from the mantissa of 2^23 + f 2^16
-__device__ __forceinline__ unsigned int frac16(float f) {
-  return __float_as_uint(__fmaf_rd(f, 65536.0f, 8388608.0f)) & 0xFFFFu;
-}
-
 __device__ __forceinline__ float bilin(float f00, float f10, float f01, float f11, float a, float b) {
   return (1.0f - b) * ((1.0f - a) * f00 + a * f10) + b * ((1.0f - a) * f01 + a * f11);
 }
