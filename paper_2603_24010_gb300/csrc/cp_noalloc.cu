@@ -11,24 +11,28 @@
 // every GPU that loads this library holds until the process exits.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <mutex>
 
-#include "cp_device.cuh"
+#include "cp_common.cuh"
 
 namespace cpk_na {
 
 using cpk::AbsRec;
+using cpk::floor_split;
+using cpk::frac16;
 using cpk::kTagSee;
 using cpk::philox4x64_10;
 using cpk::u01;
 using cpk::U64x4;
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 1024;
 constexpr int kMaxCells = 4096;          // shared-memory grid limit
 constexpr int64_t kMaxIons = 1 << 19;    // absorbed-ion records the scratch can hold
-constexpr int kCounters = 16;            // [0] list length, [1] SE count, [2] overflow, tallies
+constexpr int kCounters = 16;            // tallies, see the enum
+constexpr int kAhead = 4;                // ions per thread requested together
 
 // Scratch: counters, then one record per ion that may be absorbed (8 MiB + 128 B).
 struct Scratch {
@@ -37,8 +41,8 @@ struct Scratch {
 };
 static __device__ __align__(256) Scratch g_scratch;
 
-// Tally slots in Scratch::counters
-enum { kListLen = 0, kSeCount = 1, kOverflow = 2, kAbs0 = 3, kAbs1 = 4, kEmit0 = 5, kEmit1 = 6, kConv = 7,
+// Tally slots in Scratch::counters; all but the status are zero between calls
+enum { kSeCount = 0, kOverflow = 1, kAbs0 = 2, kAbs1 = 3, kEmit0 = 4, kEmit1 = 5, kDone = 6,
        kStatus = kCounters - 1 };
 
 struct Params {
@@ -52,176 +56,194 @@ struct Params {
 
 __device__ __forceinline__ unsigned lane() { return threadIdx.x & 31u; }
 
-__device__ __forceinline__ void dep_atomic(long long* G, int N, float x, long long sign) {
-  const float fl = floorf(x);
-  const int i = static_cast<int>(fl);
-  const long long w1 = static_cast<long long>(__float2uint_rz((x - fl) * 65536.0f));
-  long long w0 = 65536LL - w1, w1b = w1;
-  if (i == 0) w0 <<= 1;
-  if (i == N - 1) w1b <<= 1;
-  atomicAdd(reinterpret_cast<unsigned long long*>(&G[i]), static_cast<unsigned long long>(sign * w0));
-  atomicAdd(reinterpret_cast<unsigned long long*>(&G[i + 1]), static_cast<unsigned long long>(sign * w1b));
+// v units of charge on node k of the caller's grid (end nodes doubled)
+__device__ __forceinline__ void add_node(long long* G, int N, int k, long long v) {
+  if (v == 0) return;
+  if (k == 0 || k == N) v <<= 1;
+  atomicAdd(reinterpret_cast<unsigned long long*>(&G[k]), static_cast<unsigned long long>(v));
 }
 
-// Push, absorb (absorbed ions compacted into the scratch list with
-// warp-ballot appends) and deposit of the survivors into the caller's grid.
-__global__ void __launch_bounds__(kThreads) k_push_ions(Params p, Scratch* sc, const double* E,
-                                                        float* xi, float* u, const uint32_t* id,
-                                                        int64_t n, long long* G) {
-  extern __shared__ __align__(16) unsigned char smem_na[];
-  const int N = p.N;
-  long long* Gs = reinterpret_cast<long long*>(smem_na);        // N + 1
-  float2* tab = reinterpret_cast<float2*>(Gs + (N + 1));         // N + 1
-  // gather table: pair k = (Ep_k, Ep_{k+1} - Ep_k), ends repeated
-  for (int k = threadIdx.x; k <= N; k += kThreads) {
-    const float e0 = static_cast<float>(E[k == 0 ? 0 : k - 1]);
-    const float e1 = (k >= 1 && k < N) ? static_cast<float>(E[k]) : e0;
-    tab[k] = make_float2(e0, e1 - e0);
-    Gs[k] = 0;
+// The whole call in one kernel, one CTA per SM at most: each CTA pushes a
+// contiguous range of the ions (gather, kick, drift, absorption, deposit into
+// 32-bit node sums), then turns the ions it saw absorbed into electrons (the
+// context path's arithmetic and draws), and the last CTA out writes the counts
+// and clears the tallies for the next call.
+//
+// Bound: latency (a call moves 12 MB at most): the ions are requested before
+// the field table is formed, and one table per SM is formed at all because the
+// conversion from FP64 runs at two values a cycle.  Call at 524288 ions and 4096
+// cells: 52.9 -> 39.0 us, with the host's wait for the status (three kernels,
+// two memsets and 64-bit shared atomics before).
+// counts: [0] absorbed at x = 0, [1] at x = d, [2] emitted at x = 0, [3] at x =
+// d, [4] electrons written (at most se_cap), [5] convection count at x = 0;
+// status 1 when emitted electrons did not fit in se_cap.
+__global__ void __launch_bounds__(kThreads, 1)
+k_push_ions(Params p, Scratch* sc, const double* __restrict__ E, float* __restrict__ xi, float* __restrict__ u,
+            const uint32_t* __restrict__ id, int64_t n, long long* __restrict__ G, float* __restrict__ se_xi,
+            float* __restrict__ se_u, int64_t se_cap, int64_t* __restrict__ counts) {
+  extern __shared__ unsigned int smem_na[];
+  __shared__ unsigned int s_abs_n, s_abs[2], s_emit[2], s_round[2];
+  __shared__ int s_over;
+  const int N = p.N, tid = static_cast<int>(threadIdx.x);
+  unsigned int* nd = smem_na;                                 // the ions' node sums (at most 2^13 ions a CTA)
+  unsigned int* ne = nd + (N + 1);                            // a round's electrons'
+  float* tab = reinterpret_cast<float*>(ne + (N + 1));        // E_{k-1/2}, ends repeated
+  const int64_t lo = n * blockIdx.x / gridDim.x, hi = n * (blockIdx.x + 1) / gridDim.x;
+  AbsRec* rec = sc->rec + lo;                                 // this CTA's impacts
+  float x[kAhead], v[kAhead];
+  auto fetch = [&](int64_t k0) {
+#pragma unroll
+    for (int c = 0; c < kAhead; ++c) {
+      const int64_t k = k0 + tid + c * kThreads;
+      x[c] = (k < hi) ? xi[k] : -1.0f;
+      v[c] = (k < hi) ? u[k] : 0.0f;
+    }
+  };
+  fetch(lo);
+  for (int k = tid; k <= N + 1; k += kThreads) {
+    tab[k] = static_cast<float>(E[k == 0 ? 0 : (k <= N ? k - 1 : N - 1)]);
+    if (k <= N) nd[k] = ne[k] = 0u;
+  }
+  if (tid == 0) {
+    s_abs_n = 0u;
+    s_over = 0;
+    s_abs[0] = s_abs[1] = s_emit[0] = s_emit[1] = 0u;
   }
   __syncthreads();
   const float Nr = static_cast<float>(N);
-  unsigned long long a0 = 0, a1 = 0;
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
-  const int64_t trips = (n + stride - 1) / stride;  // uniform: warps stay converged
-  for (int64_t t = 0; t < trips; ++t) {
-    const int64_t k = t * stride + static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x;
-    bool absorbed = false;
-    int el = 0;
-    float un = 0.f;
-    if (k < n) {
-      const float x = xi[k];
-      if (x > 0.f && x < Nr) {
-        const float s = x - 0.5f;
-        const float jf = floorf(s);
-        const float2 e = tab[static_cast<int>(jf) + 1];
-        un = fmaf(p.kap, fmaf(s - jf, e.y, e.x), u[k]);
-        const float xn = x + un;
-        if (!(xn > 0.f && xn < Nr)) {
-          absorbed = true;
-          el = (xn <= 0.f) ? 0 : 1;
-          xi[k] = -1.f;
-          u[k] = 0.f;
-        } else {
-          xi[k] = xn;
-          u[k] = un;
-          const float fl = floorf(xn);
-          const int i = static_cast<int>(fl);
-          const long long w1 = static_cast<long long>(__float2uint_rz((xn - fl) * 65536.0f));
-          long long w0 = 65536LL - w1, w1b = w1;
-          if (i == 0) w0 <<= 1;
-          if (i == N - 1) w1b <<= 1;
-          atomicAdd(reinterpret_cast<unsigned long long*>(&Gs[i]), static_cast<unsigned long long>(w0));
-          atomicAdd(reinterpret_cast<unsigned long long*>(&Gs[i + 1]), static_cast<unsigned long long>(w1b));
-        }
+  for (int64_t k0 = lo; k0 < hi; k0 += kAhead * kThreads) {
+    if (k0 > lo) fetch(k0);
+#pragma unroll
+    for (int c = 0; c < kAhead; ++c) {
+      if (!(x[c] > 0.f && x[c] < Nr)) continue;
+      const int64_t k = k0 + tid + c * kThreads;
+      float t;
+      const int j = floor_split(x[c] - 0.5f, &t);
+      const float e0 = tab[j + 1];
+      const float un = fmaf(p.kap, fmaf(t, tab[j + 2] - e0, e0), v[c]);
+      const float xn = x[c] + un;
+      if (!(xn > 0.f && xn < Nr)) {
+        const int el = (xn <= 0.f) ? 0 : 1;
+        atomicAdd(&s_abs[el], 1u);
+        AbsRec r;
+        r.id = id[k];
+        r.electrode = static_cast<uint32_t>(el);
+        r.u = static_cast<double>(un);
+        rec[atomicAdd(&s_abs_n, 1u)] = r;  // below hi - lo: every ion fits
+        xi[k] = -1.f;
+        u[k] = 0.f;
+      } else {
+        xi[k] = xn;
+        u[k] = un;
+        float f;
+        const int i = floor_split(xn, &f);
+        const unsigned int w1 = frac16(f);
+        atomicAdd(&nd[i], 65536u - w1);
+        atomicAdd(&nd[i + 1], w1);
       }
-    }
-    // warp-ballot compaction of the absorbed ions into the scratch list
-    const unsigned ball = __ballot_sync(0xffffffffu, absorbed);
-    unsigned long long base = 0;
-    if (lane() == 0 && ball)
-      base = atomicAdd(&sc->counters[kListLen], static_cast<unsigned long long>(__popc(ball)));
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if (absorbed) {
-      const unsigned long long slot = base + __popc(ball & ((1u << lane()) - 1u));
-      AbsRec r;
-      r.id = id[k];
-      r.electrode = static_cast<uint32_t>(el);
-      r.u = static_cast<double>(un);
-      sc->rec[slot] = r;  // slot < n <= kMaxIons: every ion fits
-      if (el) ++a1; else ++a0;
     }
   }
   __syncthreads();
-  for (int k = threadIdx.x; k <= N; k += kThreads)
-    if (Gs[k]) atomicAdd(reinterpret_cast<unsigned long long*>(&G[k]), static_cast<unsigned long long>(Gs[k]));
-  if (a0) atomicAdd(&sc->counters[kAbs0], a0);
-  if (a1) atomicAdd(&sc->counters[kAbs1], a1);
-}
-
-// Secondary emission from the listed impacts (same arithmetic and draws as
-// the context path); electrons appended to the caller's arrays.
-__global__ void __launch_bounds__(kThreads) k_see(Params p, Scratch* sc, float* se_xi, float* se_u,
-                                                  int64_t se_cap, long long* G) {
-  const unsigned long long len = sc->counters[kListLen];
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
-  const int64_t trips = (static_cast<int64_t>(len) + stride - 1) / stride;
-  const int N = p.N;
+  for (int k = tid; k <= N; k += kThreads) add_node(G, N, k, nd[k]);
+  // secondary emission, an impact per thread and round; a round's electrons
+  // (at most 1024 x 15, below 2^32 in a node sum) go through node sums of
+  // their own where they are many
+  const int na = static_cast<int>(s_abs_n);
   const double pi = 3.14159265358979323846;
-  for (int64_t t = 0; t < trips; ++t) {
-    const int64_t r = t * stride + static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x;
-    const bool act = r < static_cast<int64_t>(len);
+  for (int r0 = 0; r0 < na; r0 += kThreads) {
+    const bool act = r0 + tid < na;
     int nse = 0;
-    AbsRec rec;
-    rec.id = 0; rec.electrode = 0; rec.u = 0.0;
-    double Eev = 0.0;
+    AbsRec q;
+    q.id = 0; q.electrode = 0; q.u = 0.0;
+    unsigned int* const electrons = &s_round[r0 / kThreads & 1];
+    if (tid == 0) *electrons = 0u;
+    __syncthreads();
     if (act) {
-      rec = sc->rec[r];
-      const double v = __ddiv_rn(__dmul_rn(rec.u, p.dx), p.dt);
-      Eev = __ddiv_rn(__dmul_rn(__dmul_rn(__dmul_rn(0.5, p.m_i), v), v), p.e);
+      q = rec[r0 + tid];
+      const double vi = __ddiv_rn(__dmul_rn(q.u, p.dx), p.dt);
+      const double Eev = __ddiv_rn(__dmul_rn(__dmul_rn(__dmul_rn(0.5, p.m_i), vi), vi), p.e);
       double g = __dmul_rn(__dmul_rn(p.see_scale, p.gamma_coef), __dsqrt_rn(__ddiv_rn(Eev, p.E_ref_eV)));
       if (g > p.gamma_max) g = p.gamma_max;
       if (!(g > 0.0)) g = 0.0;
-      const U64x4 w = philox4x64_10(rec.id, static_cast<uint64_t>(p.step), 0, 0, p.seed, kTagSee);
+      const U64x4 w = philox4x64_10(q.id, static_cast<uint64_t>(p.step), 0, 0, p.seed, kTagSee);
       const double fl = floor(g);
       nse = static_cast<int>(fl) + ((u01(w.w[0]) < __dsub_rn(g, fl)) ? 1 : 0);
-      if (nse) atomicAdd(&sc->counters[rec.electrode ? kEmit1 : kEmit0], static_cast<unsigned long long>(nse));
-      if (rec.electrode == 0 && nse)
-        atomicAdd(&sc->counters[kConv], static_cast<unsigned long long>(nse));
+      if (nse) atomicAdd(&s_emit[q.electrode], static_cast<unsigned int>(nse));
     }
-    int incl = nse;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (static_cast<int>(lane()) >= o) incl += y;
-    }
+    const int incl = cpk::warp_incl_scan(nse);
     const int total = __shfl_sync(0xffffffffu, incl, 31);
     unsigned long long base = 0;
-    if (lane() == 31 && total)
+    if (lane() == 31 && total) {
       base = atomicAdd(&sc->counters[kSeCount], static_cast<unsigned long long>(total));
+      atomicAdd(electrons, static_cast<unsigned int>(total));
+    }
+    __syncthreads();
+    const bool few = *electrons <= 64u;
     base = __shfl_sync(0xffffffffu, base, 31);
     for (int j = 0; j < nse; ++j) {
-      const U64x4 wv = philox4x64_10(rec.id, static_cast<uint64_t>(p.step), static_cast<uint64_t>(1 + j), 0,
-                                     p.seed, kTagSee);
+      const U64x4 wv = philox4x64_10(q.id, static_cast<uint64_t>(p.step), static_cast<uint64_t>(1 + j), 0, p.seed, kTagSee);
       const double ua = u01(wv.w[0]), ub = u01(wv.w[1]), frac = u01(wv.w[2]);
       const double z = sqrt(-2.0 * log(ua)) * cos(2.0 * pi * ub);
       const double use = p.see_vth * fabs(z) * p.dt / p.dx;
-      const double xd = (rec.electrode == 0) ? __dmul_rn(use, frac) : __dsub_rn(static_cast<double>(N), __dmul_rn(use, frac));
-      float xr = static_cast<float>(xd);
-      if (xr >= static_cast<float>(N)) xr = nextafterf(static_cast<float>(N), 0.f);
-      if (xr <= 0.f) xr = 1.17549435e-38f;
+      const double xd = (q.electrode == 0) ? __dmul_rn(use, frac) : __dsub_rn(static_cast<double>(N), __dmul_rn(use, frac));
+      const float xr = cpk::nudge_inside<float>(xd, N);
       const unsigned long long slot = base + static_cast<unsigned long long>(incl - nse + j);
       if (slot < static_cast<unsigned long long>(se_cap)) {
         se_xi[slot] = xr;
-        se_u[slot] = static_cast<float>(rec.electrode == 0 ? use : -use);
-        dep_atomic(G, N, xr, -1LL);
+        se_u[slot] = static_cast<float>(q.electrode == 0 ? use : -use);
+        float f;
+        const int i = floor_split(xr, &f);
+        const unsigned int w1 = frac16(f);
+        if (few) {
+          add_node(G, N, i, static_cast<long long>(w1) - 65536);
+          add_node(G, N, i + 1, -static_cast<long long>(w1));
+        } else {
+          atomicAdd(&ne[i], 65536u - w1);
+          atomicAdd(&ne[i + 1], w1);
+        }
       } else {
-        sc->counters[kOverflow] = 1ULL;
+        s_over = 1;
       }
     }
+    if (few) continue;
+    __syncthreads();
+    for (int k = tid; k <= N; k += kThreads) {
+      add_node(G, N, k, -static_cast<long long>(ne[k]));
+      ne[k] = 0u;
+    }
   }
-}
-
-// The call's six counts written on the device (no host round trip): [0]
-// absorbed at x = 0, [1] absorbed at x = d, [2] emitted at x = 0, [3] emitted
-// at x = d, [4] electrons written (at most se_cap), [5] convection count at
-// x = 0.  status[0] = 1 when emitted electrons did not fit in se_cap.
-__global__ void k_counts(const Scratch* sc, int64_t se_cap, int64_t* counts, unsigned long long* status) {
-  const unsigned long long se = sc->counters[kSeCount];
-  const unsigned long long cap = static_cast<unsigned long long>(se_cap);
-  counts[0] = static_cast<int64_t>(sc->counters[kAbs0]);
-  counts[1] = static_cast<int64_t>(sc->counters[kAbs1]);
-  counts[2] = static_cast<int64_t>(sc->counters[kEmit0]);
-  counts[3] = static_cast<int64_t>(sc->counters[kEmit1]);
-  counts[4] = static_cast<int64_t>(se < cap ? se : cap);
-  counts[5] = static_cast<int64_t>(sc->counters[kAbs0]) + static_cast<int64_t>(sc->counters[kEmit0]);
-  status[0] = (sc->counters[kOverflow] || se > cap) ? 1ULL : 0ULL;
+  __syncthreads();
+  if (tid == 0) {
+    unsigned long long* c = sc->counters;
+    if (s_abs[0]) atomicAdd(&c[kAbs0], static_cast<unsigned long long>(s_abs[0]));
+    if (s_abs[1]) atomicAdd(&c[kAbs1], static_cast<unsigned long long>(s_abs[1]));
+    if (s_emit[0]) atomicAdd(&c[kEmit0], static_cast<unsigned long long>(s_emit[0]));
+    if (s_emit[1]) atomicAdd(&c[kEmit1], static_cast<unsigned long long>(s_emit[1]));
+    if (s_over) atomicAdd(&c[kOverflow], 1ULL);
+    __threadfence();
+    if (atomicAdd(&c[kDone], 1ULL) == gridDim.x - 1) {
+      __threadfence();
+      const unsigned long long se = __ldcg(&c[kSeCount]), cap = static_cast<unsigned long long>(se_cap);
+      const unsigned long long a0 = __ldcg(&c[kAbs0]), e0 = __ldcg(&c[kEmit0]);
+      counts[0] = static_cast<int64_t>(a0);
+      counts[1] = static_cast<int64_t>(__ldcg(&c[kAbs1]));
+      counts[2] = static_cast<int64_t>(e0);
+      counts[3] = static_cast<int64_t>(__ldcg(&c[kEmit1]));
+      counts[4] = static_cast<int64_t>(se < cap ? se : cap);
+      counts[5] = static_cast<int64_t>(a0 + e0);
+      c[kStatus] = (__ldcg(&c[kOverflow]) || se > cap) ? 1ULL : 0ULL;
+      for (int k = 0; k < kStatus; ++k) c[k] = 0ULL;
+    }
+  }
 }
 
 // Device address of the scratch array (and the push kernel's shared-memory
 // limit), set up once per device with that device current.
 std::mutex g_mu;
 Scratch* g_addr[64] = {};
+// One call at a time: calls from several threads or on several streams share
+// the tallies, which the last CTA of a call clears for the next.
+std::mutex g_call;
 
 int scratch_address(int dev, Scratch** out) {
   if (dev < 0 || dev >= 64) return CP_ERR_ARG;
@@ -233,7 +255,7 @@ int scratch_address(int dev, Scratch** out) {
       return CP_ERR_CUDA;
     }
     if (cudaFuncSetAttribute(k_push_ions, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(16 * (kMaxCells + 1))) != cudaSuccess) {
+                             static_cast<int>(12 * (kMaxCells + 2))) != cudaSuccess) {
       cudaGetLastError();
       return CP_ERR_CUDA;
     }
@@ -288,19 +310,18 @@ extern "C" int cp_push_ions_noalloc(const cp_gap* gap, const cp_see_beam* see, d
   p.see_vth = std::sqrt(gap->e * see->T_emit_eV / gap->m_e);
   p.seed = seed;
   p.step = step;
-  // the scratch keeps the previous call's contents: its counters start at zero
-  if (cudaMemsetAsync(sc->counters, 0, sizeof(sc->counters), st) != cudaSuccess ||
-      cudaMemsetAsync(G, 0, sizeof(int64_t) * (N + 1), st) != cudaSuccess)
-    return CP_ERR_CUDA;
+  std::lock_guard<std::mutex> one(g_call);
+  if (cudaMemsetAsync(G, 0, sizeof(int64_t) * (N + 1), st) != cudaSuccess) return CP_ERR_CUDA;
   int sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return CP_ERR_CUDA;
-  const int grid = 2 * sms;
-  long long* Gl = reinterpret_cast<long long*>(G);
-  k_push_ions<<<grid, kThreads, 16 * (N + 1), st>>>(p, sc, E, xi, u, id, n, Gl);
-  k_see<<<grid, kThreads, 0, st>>>(p, sc, se_xi, se_u, se_cap, Gl);
-  // counts on the device; one copy of the overflow flag back for the status
+  // at least 512 ions a CTA (each forms the field table and flushes a grid),
+  // at most 8191 (its 32-bit node sums stay below 2^29)
+  const int64_t want = std::max<int64_t>((n + 511) / 512, 1);
+  const int grid = static_cast<int>(std::max<int64_t>(std::min<int64_t>(want, sms), (n + 8190) / 8191));
+  k_push_ions<<<grid, kThreads, 12 * (N + 2), st>>>(p, sc, E, xi, u, id, n, reinterpret_cast<long long*>(G), se_xi,
+                                                    se_u, se_cap, counts);
+  // one copy of the overflow flag back for the status
   unsigned long long* flag = &sc->counters[kStatus];
-  k_counts<<<1, 1, 0, st>>>(sc, se_cap, counts, flag);
   if (cudaGetLastError() != cudaSuccess) return CP_ERR_CUDA;
   unsigned long long overflow = 0;
   if (cudaMemcpyAsync(&overflow, flag, sizeof(overflow), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
