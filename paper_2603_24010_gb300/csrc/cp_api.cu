@@ -8,8 +8,10 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdint>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <utility>
 #include <vector>
@@ -64,6 +66,26 @@ cudaError_t samples_launch(const DevParams* P, const cp_diag* hist, int64_t firs
 
 using cpk::kSpecies;
 
+// Page-locked memory that small read-backs go through, so that the copies of
+// a call run without the driver's own staging and end in one wait.  An
+// ensemble's instances share one; the lock lets threads take turns.
+struct Readback {
+  static constexpr size_t kBytes = 256 << 10;
+  std::mutex mu;
+  void* p = nullptr;
+  Readback() {
+    if (cudaHostAlloc(&p, kBytes, cudaHostAllocDefault) != cudaSuccess) {
+      cudaGetLastError();
+      p = nullptr;  // copies then go straight to the caller's memory
+    }
+  }
+  ~Readback() {
+    if (p) cudaFreeHost(p);
+  }
+  Readback(const Readback&) = delete;
+  Readback& operator=(const Readback&) = delete;
+};
+
 struct cp_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
@@ -97,8 +119,11 @@ struct cp_ctx {
   bool initialized = false;
   int compact_every = 128;
   int since_compact = 0;
+  int64_t level = -1;     // the stored level where the host knows it (left by the last steps), else -1
   int64_t max_steps = 0;
   double sigma0 = 0.0;
+  Readback* io = nullptr;  // this context's own, or its ensemble's
+  bool own_io = false;
   bool ens_member = false;  // advanced by a cp_batch (its own absorbed-ion lists unused)
   // particles staged on the host until the first step
   std::vector<double> hx[kSpecies], hu[kSpecies];
@@ -116,6 +141,9 @@ struct cp_ctx {
   int64_t t_n[3] = {0, 0, 0};
   std::vector<cudaEvent_t> ev_pool;
   std::vector<double> last_step_ms;
+  ~cp_ctx() {
+    if (own_io) delete io;
+  }
 };
 
 namespace {
@@ -415,11 +443,71 @@ int initialize(cp_ctx* c, int mode, double tol) {
   return CP_OK;
 }
 
-int read_status(cp_ctx* c) {
-  int st = 0;
-  CP_CUDA(cudaMemcpyAsync(&st, &c->dS->status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+struct Part {
+  void* dst;
+  const void* src;
+  size_t bytes;
+};
+
+// The parts, read back with one wait.  With a check, the first part comes
+// first and the rest reaches the caller only if ok() then holds.
+template <typename Ok>
+int fetch(cp_ctx* c, const Part* parts, int n, bool check, Ok ok) {
+  size_t total = 0;
+  for (int k = 0; k < n; ++k) total += (parts[k].bytes + 15) & ~size_t(15);
+  if (!c->io || !c->io->p || total > Readback::kBytes) {
+    for (int k = 0; k < n; ++k) {
+      CP_CUDA(cudaMemcpyAsync(parts[k].dst, parts[k].src, parts[k].bytes, cudaMemcpyDeviceToHost, c->stream));
+      if (k == n - 1 || (k == 0 && check)) CP_CUDA(cudaStreamSynchronize(c->stream));
+      if (k == 0 && check && !ok()) return CP_ERR_ARG;
+    }
+    return CP_OK;
+  }
+  std::lock_guard<std::mutex> turn(c->io->mu);
+  char* q = static_cast<char*>(c->io->p);
+  for (int k = 0; k < n; ++k) {
+    CP_CUDA(cudaMemcpyAsync(q, parts[k].src, parts[k].bytes, cudaMemcpyDeviceToHost, c->stream));
+    q += (parts[k].bytes + 15) & ~size_t(15);
+  }
   CP_CUDA(cudaStreamSynchronize(c->stream));
-  return st;
+  q = static_cast<char*>(c->io->p);
+  for (int k = 0; k < n; ++k) {
+    std::memcpy(parts[k].dst, q, parts[k].bytes);
+    q += (parts[k].bytes + 15) & ~size_t(15);
+    if (k == 0 && check && !ok()) return CP_ERR_ARG;
+  }
+  return CP_OK;
+}
+
+int fetch(cp_ctx* c, const Part* parts, int n) {
+  return fetch(c, parts, n, false, [] { return true; });
+}
+
+// Status and level after steps (a step call's only wait).
+int read_status(cp_ctx* c) {
+  struct {
+    int64_t level;
+    int32_t pushed, status;
+  } h;
+  static_assert(offsetof(cpk::DevState, status) - offsetof(cpk::DevState, level) == 12, "one copy");
+  const Part part = {&h, &c->dS->level, sizeof(h)};
+  CP_TRY(fetch(c, &part, 1));
+  c->level = h.level;
+  return h.status;
+}
+
+// The level steps start from.  The host knows it from the steps before; it is
+// unknown again until the steps about to run have been read back.  (On a
+// stream under capture it is fetched, which fails before anything is captured.)
+int take_level(cp_ctx* c, int64_t* level) {
+  *level = c->level;
+  c->level = -1;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (*level >= 0 && cudaStreamIsCapturing(c->stream, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone)
+    return CP_OK;
+  CP_CUDA(cudaMemcpyAsync(level, &c->dS->level, sizeof(*level), cudaMemcpyDeviceToHost, c->stream));
+  CP_CUDA(cudaStreamSynchronize(c->stream));
+  return CP_OK;
 }
 
 // Capture compact_every step launches plus one removal launch into a graph.
@@ -502,8 +590,7 @@ int do_steps(cp_ctx* c, int mode, int32_t n_steps, double tol) {
   c->launches = 0;
   if (!c->initialized) CP_TRY(initialize(c, mode, tol));
   int64_t level = 0;
-  CP_CUDA(cudaMemcpyAsync(&level, &c->dS->level, sizeof(level), cudaMemcpyDeviceToHost, c->stream));
-  CP_CUDA(cudaStreamSynchronize(c->stream));
+  CP_TRY(take_level(c, &level));
   if (level + n_steps > c->max_steps) return CP_ERR_ARG;
   if (c->timing) {
     CP_TRY(do_steps_timed(c, mode, n_steps, tol));
@@ -536,8 +623,8 @@ int do_steps(cp_ctx* c, int mode, int32_t n_steps, double tol) {
 
 extern "C" {
 
-int cp_create(const cp_gap* gap, const cp_circuit* circ, const cp_see_beam* see, const cp_run* run,
-              void* stream, cp_ctx** out) {
+static int create_ctx(const cp_gap* gap, const cp_circuit* circ, const cp_see_beam* see, const cp_run* run,
+                      void* stream, cp_ctx** out) {
   if (!gap || !circ || !see || !run || !out) return CP_ERR_ARG;
   *out = nullptr;
   if (gap->n_cells < 2 || !(gap->d > 0) || !(run->dt > 0) || !(gap->weight > 0) ||
@@ -673,6 +760,14 @@ int cp_create(const cp_gap* gap, const cp_circuit* circ, const cp_see_beam* see,
   return CP_OK;
 }
 
+int cp_create(const cp_gap* gap, const cp_circuit* circ, const cp_see_beam* see, const cp_run* run,
+              void* stream, cp_ctx** out) {
+  CP_TRY(create_ctx(gap, circ, see, run, stream, out));
+  (*out)->io = new (std::nothrow) Readback();
+  (*out)->own_io = true;
+  return CP_OK;
+}
+
 int cp_set_particles(cp_ctx* c, int32_t species, const double* x, const double* v,
                      const uint32_t* id, int64_t n, int32_t units) {
   if (!c || species < 0 || species >= kSpecies || n < 0 || c->initialized ||
@@ -796,31 +891,27 @@ int cp_predictor_samples(cp_ctx* c, int64_t first_level, int64_t n, float* X, fl
 int cp_read_scalars(cp_ctx* c, cp_diag* out) {
   if (!c || !out) return CP_ERR_ARG;
   if (!c->initialized) return CP_ERR_ARG;
-  CP_CUDA(cudaMemcpyAsync(out, &c->dS->cur, sizeof(cp_diag), cudaMemcpyDeviceToHost, c->stream));
-  CP_CUDA(cudaStreamSynchronize(c->stream));
-  return CP_OK;
+  const Part part = {out, &c->dS->cur, sizeof(cp_diag)};
+  return fetch(c, &part, 1);
 }
 
 int cp_read_history(cp_ctx* c, int64_t first, int64_t n, cp_diag* out) {
   if (!c || !out || first < 0 || n < 0 || !c->initialized) return CP_ERR_ARG;
+  if (first > c->hist_rows || n > c->hist_rows - first) return CP_ERR_ARG;
   int64_t level = 0;
-  CP_CUDA(cudaMemcpyAsync(&level, &c->dS->level, sizeof(level), cudaMemcpyDeviceToHost, c->stream));
-  CP_CUDA(cudaStreamSynchronize(c->stream));
-  if (first + n > level + 1 || first + n > c->hist_rows) return CP_ERR_ARG;
-  if (n == 0) return CP_OK;
-  CP_CUDA(cudaMemcpyAsync(out, c->hist + first, sizeof(cp_diag) * n, cudaMemcpyDeviceToHost, c->stream));
-  CP_CUDA(cudaStreamSynchronize(c->stream));
-  return CP_OK;
+  const Part part[2] = {{&level, &c->dS->level, sizeof(level)}, {out, c->hist + first, sizeof(cp_diag) * n}};
+  return fetch(c, part, n > 0 ? 2 : 1, true, [&] { return first + n <= level + 1; });
 }
 
 int cp_read_grid(cp_ctx* c, double* phi, double* rho, double* E, int64_t* G, int32_t n_nodes) {
   if (!c || n_nodes != c->N + 1 || !c->initialized) return CP_ERR_ARG;
   const int N = c->N;
   std::vector<long long> g(N + 1);
-  if (phi) CP_CUDA(cudaMemcpyAsync(phi, c->phi, sizeof(double) * (N + 1), cudaMemcpyDeviceToHost, c->stream));
-  if (E) CP_CUDA(cudaMemcpyAsync(E, c->E64, sizeof(double) * N, cudaMemcpyDeviceToHost, c->stream));
-  CP_CUDA(cudaMemcpyAsync(g.data(), c->Glast, sizeof(long long) * (N + 1), cudaMemcpyDeviceToHost, c->stream));
-  CP_CUDA(cudaStreamSynchronize(c->stream));
+  Part part[3] = {{g.data(), c->Glast, sizeof(long long) * (N + 1)}};
+  int parts = 1;
+  if (phi) part[parts++] = {phi, c->phi, sizeof(double) * (N + 1)};
+  if (E) part[parts++] = {E, c->E64, sizeof(double) * N};
+  CP_TRY(fetch(c, part, parts));
   for (int i = 0; i <= N; ++i) {
     if (G) G[i] = g[i];
     if (rho) rho[i] = static_cast<double>(g[i]) * c->hp.scale;
@@ -883,9 +974,8 @@ int cp_get_level(cp_ctx* c, int64_t* level) {
     *level = 0;
     return CP_OK;
   }
-  CP_CUDA(cudaMemcpyAsync(level, &c->dS->level, sizeof(int64_t), cudaMemcpyDeviceToHost, c->stream));
-  CP_CUDA(cudaStreamSynchronize(c->stream));
-  return CP_OK;
+  const Part part = {level, &c->dS->level, sizeof(int64_t)};
+  return fetch(c, &part, 1);
 }
 
 // ---- checkpoint ---------------------------------------------------------------
@@ -971,6 +1061,7 @@ int cp_load_state(cp_ctx* c, const void* buf, size_t len) {
   for (int s = 0; s < kSpecies; ++s)
     if (h.slots[s] > c->cap[s]) return CP_ERR_CAPACITY;
   if (h.hist_n > c->hist_rows) return CP_ERR_CAPACITY;
+  c->level = -1;
   cpk::DevState saved, cur;
   std::memcpy(&saved, p, sizeof(saved));
   p += sizeof(saved);
@@ -1328,12 +1419,14 @@ int cp_batch_create(int32_t n, const cp_gap* gaps, const cp_circuit* circuits,
   b->inst.reserve(n);
   for (int i = 0; i < n; ++i) {
     cp_ctx* c = nullptr;
-    const int rc = cp_create(&gaps[i], &circuits[i], &sees[i], &runs[i], stream, &c);
+    const int rc = create_ctx(&gaps[i], &circuits[i], &sees[i], &runs[i], stream, &c);
     if (rc != CP_OK) {
       batch_free(b);
       delete b;
       return rc;
     }
+    c->own_io = (i == 0);
+    c->io = (i == 0) ? new (std::nothrow) Readback() : b->inst[0]->io;
     b->inst.push_back(c);
   }
   // an ensemble's small instances lose particles fast: its own default
@@ -1858,8 +1951,7 @@ int g2_steps(cp_gap2d* g, int mode, int32_t n_steps, double tol) {
   g->launches = 0;
   if (!g->initialized) CP_TRY(g2_init(g, mode, tol));
   int64_t level = 0;
-  CP_CUDA(cudaMemcpyAsync(&level, &c->dS->level, sizeof(level), cudaMemcpyDeviceToHost, c->stream));
-  CP_CUDA(cudaStreamSynchronize(c->stream));
+  CP_TRY(take_level(c, &level));
   if (level + n_steps > c->max_steps) return CP_ERR_ARG;
   std::vector<std::pair<int, size_t>> rec;
   auto mark_end = [&](void) -> int {
