@@ -35,6 +35,9 @@
 //   electrons go straight to the global grid (the tail of a CTA with impacts
 //   took 6-8 us; step at 3e5 particles 19.4 -> 18.3 us, at 3e7 with impacts
 //   in every CTA 102.1 -> 98.3).
+// * after the wait one warp of a CTA reads what the solve left (level, flags,
+//   slots in use): read by every warp of 304 CTAs, those few lines took longer
+//   than the field table (1 us of a step at 3e5 particles).
 //
 // FP64 particles: an SM issues 2 FP64 operations a cycle, so comparisons,
 // floors and conversions are done on the integer pipe (8 FP64 operations a
@@ -42,9 +45,11 @@
 // populations reach every SM.
 //
 // Graph-timed step before -> after (GB300): FP64, 256 cells, 1.4e5 particles
-// 38.6 -> 20.0 us; FP64 Tesla gap 40.9 -> 22.5; FP32, 4096 cells, 3.3e5
-// particles 22.9 -> 19.4, 1e6 (1531 cells) 17.5 -> 15.9, 1.5e7 59.3 -> 53.9,
-// 3.1e7 (impacts every step) 118 -> 113.7.
+// 38.6 -> 18.3 us; FP64 Tesla gap 40.9 -> 21.8; FP32, 4096 cells, 3.3e5
+// particles 22.9 -> 17.0, 1e6 (1531 cells) 17.5 -> 15.1, 1.5e7 59.3 -> 51.2,
+// 3.1e7 (impacts every step) 118 -> 109.
+
+#include <cstddef>
 
 #include "cp_common.cuh"
 #include "cp_mlp.cuh"
@@ -278,48 +283,61 @@ struct SeeConst {
 __device__ __forceinline__ double over_E_ref(const SeeConst* c, double E) { return div_by(E, c->E_ref_eV, c->r_E_ref); }
 
 constexpr unsigned int kFewElectrons = 32;  // emitted by a CTA straight into the global grid
-constexpr int kRecShared = 32;  // absorbed-ion records kept in shared memory (the others in global)
+constexpr int kRecShared = 28;  // absorbed-ion records kept in shared memory (the others in global)
 
-// PUSH: the step's push; else the deposit of the loaded particles (level 0).
-template <typename real, bool PUSH>
-__global__ void __launch_bounds__(kThreads, kCtasPerSm) k_push(Bufs B) {
+// Static shared memory of a push: a multiple of 128 bytes, since the dynamic
+// part follows it and the ring wants whole aligned sectors (behind 944 bytes,
+// which split every 32-byte sector of the copies in two, the step at 3e7
+// particles took 110 us instead of 97).
+template <typename real>
+struct alignas(128) PushShared {
+  int abs_n, over;
+  unsigned int cnt[2][kSpecies];
+  unsigned int emit[2];
+  long long conv, energy;
+  unsigned int cfl;
+  real* xi[kSpecies];
+  real* u[kSpecies];
+  long long n[kSpecies];     // slots in use
+  int tile[kSpecies + 1];    // first tile of each species in the flat list
+  int64_t step;
+  int stop, half, moved;
+  SeeConst see;
+  AbsRec rec[kRecShared];
+};
+
+// The push of one CTA.  PUSH: the step's push; else the deposit of the loaded
+// particles (level 0).  The list and the level are read before the wait, where
+// a CTA that starts late (other kernels on the device held its place) may find
+// them already moved on by CTAs of this very push that have finished.  What
+// the solve left is compared after the wait: on a difference nothing has been
+// done, the result is false, and the CTA begins again with LATE, from what
+// the solve left.
+template <typename real, bool PUSH, bool LATE>
+__device__ __forceinline__ bool push_cta(const Bufs& B, PushShared<real>& sh, unsigned char* smem, int G) {
   using V = Vec<real>;
   using real2 = typename Pair<real>::type;
   const DevParams* __restrict__ P = B.P;
   DevState* S = B.S;
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int s_abs_n, s_over;
-  __shared__ unsigned int s_cnt[2][kSpecies];
-  __shared__ unsigned int s_emit[2];
-  __shared__ long long s_conv, s_energy;
-  __shared__ unsigned int s_cfl;
-  __shared__ real* s_xi[kSpecies];
-  __shared__ real* s_u[kSpecies];
-  __shared__ long long s_n[kSpecies];     // slots in use
-  __shared__ int s_tile[kSpecies + 1];    // first tile of each species in the flat list
-  __shared__ SeeConst C;
-  __shared__ AbsRec s_rec[kRecShared];
+  int &s_abs_n = sh.abs_n, &s_over = sh.over;
+  auto& s_cnt = sh.cnt;
+  auto& s_emit = sh.emit;
+  long long &s_conv = sh.conv, &s_energy = sh.energy;
+  unsigned int& s_cfl = sh.cfl;
+  auto& s_xi = sh.xi;
+  auto& s_u = sh.u;
+  auto& s_n = sh.n;
+  auto& s_tile = sh.tile;
+  SeeConst& C = sh.see;
+  auto& s_rec = sh.rec;
 
+  if (LATE) __syncthreads();  // the first attempt's readings are done
   const int tid = static_cast<int>(threadIdx.x);
   const int N = P->N;
   long long* Gs = reinterpret_cast<long long*>(smem + kRingBytes);
   unsigned int* nd = reinterpret_cast<unsigned int*>(smem + kRingBytes + align16(sizeof(long long) * (N + 1)));
   real* Et = reinterpret_cast<real*>(reinterpret_cast<unsigned char*>(nd) + align16(sizeof(unsigned int) * (N + 1)));
-  // With a network installed the launch has one CTA more, which runs the
-  // learned predictor for the level the previous solve committed (levels
-  // >= 1).  Scheduled last, it takes the first slot a pushing CTA frees, so
-  // the network runs beside the other CTAs' ends.
-  const bool pred_cta = (B.net != nullptr && B.net_in_push);
-  const int G = static_cast<int>(gridDim.x) - (pred_cta ? 1 : 0);  // pushing CTAs
   const int cta = static_cast<int>(blockIdx.x);
-  if (cta == G) {
-    cudaGridDependencySynchronize();
-    cudaTriggerProgrammaticLaunchCompletion();
-    if (ldcg(&S->status) != 0) return;
-    if (PUSH && ldcg(&S->level) >= 1) predictor_in_push(S, B.net, P->C, reinterpret_cast<PredScratch*>(smem));
-    return;
-  }
-
   // --- before the previous solve has finished --------------------------------
   for (int k = tid; k <= N; k += kThreads) nd[k] = 0u;
   if (tid == 0) {
@@ -337,13 +355,15 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_push(Bufs B) {
       s_xi[tid] = static_cast<real*>(ldcg(&S->xi[tid]));
       s_u[tid] = static_cast<real*>(ldcg(&S->u[tid]));
       // the solve rounds n_alloc up to a multiple of 4, this reads it before or after
-      n = min(static_cast<long long>((ldcg(&S->n_alloc[tid]) + 3) & ~int64_t(3)), static_cast<long long>(P->cap[tid]));
+      n = LATE ? static_cast<long long>(ldcg(&S->n_proc[tid]))
+               : min(static_cast<long long>((ldcg(&S->n_alloc[tid]) + 3) & ~int64_t(3)), static_cast<long long>(P->cap[tid]));
       s_n[tid] = n;
     }
     int t = static_cast<int>((n + V::kTileN - 1) / V::kTileN);
     t = warp_incl_scan(t);
     if (tid < kSpecies) s_tile[tid + 1] = t;
     if (tid == 0) s_tile[0] = 0;
+    if (tid == kSpecies) sh.step = LATE ? ldcg(&S->level) : ldcg(B.next_step);
   }
   if (PUSH && tid == kThreads - 32) {
     C.see_scale = P->see_scale; C.gamma_coef = P->gamma_coef; C.gamma_max = P->gamma_max;
@@ -360,7 +380,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_push(Bufs B) {
   const int Bn = PUSH ? P->beam_per_step : 0;
   const int nbc = (Bn + G - 1) / G;
   const int kb0 = min(Bn, cta * nbc), kb1 = min(Bn, kb0 + nbc);
-  const int64_t step = ldcg(B.next_step);  // the level this push starts from
+  __syncthreads();
+  const int64_t step = sh.step;  // the level this push starts from (one thread's reading for the whole CTA)
   auto draw_beam = [&](int kk, real* x, real* u) {
     const U64x4 wv = philox4x64_10(static_cast<uint64_t>(kk), static_cast<uint64_t>(step), 0, 0, P->seed, kTagBeam);
     const double frac = u01(wv.w[0]);
@@ -368,9 +389,6 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_push(Bufs B) {
     *x = nudge_inside<real>(__dsub_rn(static_cast<double>(N), __dmul_rn(ub, frac)), N);
     *u = static_cast<real>(-ub);
   };
-  real bx = real(0), bu = real(0);
-  if (kb0 + tid < kb1) draw_beam(kb0 + tid, &bx, &bu);
-  __syncthreads();
   // This CTA's tiles cta, cta + G, ... of the flat list, species by species:
   // `left` tiles of species `s`, the next at x, u (this thread's particles);
   // the species' last four, at x_end, are not copied.
@@ -419,11 +437,31 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_push(Bufs B) {
   };
 #pragma unroll
   for (int j = 0; j < kStages - 1; ++j) issue();
+  // this thread's beam ion of the first round
+  real bx = real(0), bu = real(0);
+  if (kb0 + tid < kb1) draw_beam(kb0 + tid, &bx, &bu);
 
-  cudaGridDependencySynchronize();
-  cudaTriggerProgrammaticLaunchCompletion();
-  const int stop = ldcg(&S->status);
-  const bool half = (ldcg(&S->pushed) == 0);
+  if (!LATE) {
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();
+  }
+  // what the solve left, by one warp of the CTA (read by all, the line serves
+  // thousands of warps at once)
+  if (tid < 32) {
+    static_assert(offsetof(DevState, pushed) == offsetof(DevState, level) + 8 &&
+                      offsetof(DevState, status) == offsetof(DevState, level) + 12,
+                  "level | pushed, status");
+    long long w = 0;  // lane 0: level, 1: pushed and status, 2-4: slots in use
+    if (tid < 2) w = ldcg(reinterpret_cast<const long long*>(&S->level) + tid);
+    else if (tid < 2 + kSpecies) w = ldcg(&S->n_proc[tid - 2]);
+    const bool differs = !LATE && ((tid == 0 && w != step) || (tid >= 2 && tid < 2 + kSpecies && w != s_n[tid - 2]));
+    const unsigned int moved = __ballot_sync(0xffffffffu, differs);
+    if (tid == 1) {
+      sh.half = (static_cast<int>(w) == 0);
+      sh.stop = static_cast<int>(w >> 32);
+      sh.moved = (moved != 0u);
+    }
+  }
   // the field table of the solve just finished: eight loads per thread in
   // flight together (one L2 round trip for N <= 4095)
   if (PUSH && any) {
@@ -445,10 +483,12 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_push(Bufs B) {
       }
     }
   }
-  if (stop) {
+  __syncthreads();
+  if (sh.stop || sh.moved) {
     cp_async_wait<0>();
-    return;
+    return sh.stop != 0;
   }
+  const bool half = sh.half;
   // the beam: slots behind the ions in use (ions are appended by the beam
   // alone, so the slots are known without a shared counter)
   bool folded = false;
@@ -474,7 +514,6 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_push(Bufs B) {
       s_over = 1;
     }
   }
-  __syncthreads();
 
   const real Nr = static_cast<real>(N);
   const int cap = P->abs_cap;
@@ -697,6 +736,32 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_push(Bufs B) {
     }
     if (s_over) atomicCAS(&S->status, 0, CP_ERR_CAPACITY);
   }
+  return true;
+}
+
+template <typename real, bool PUSH>
+__device__ __noinline__ void push_cta_late(const Bufs& B, PushShared<real>& sh, unsigned char* smem, int G) {
+  push_cta<real, PUSH, true>(B, sh, smem, G);
+}
+
+template <typename real, bool PUSH>
+__global__ void __launch_bounds__(kThreads, kCtasPerSm) k_push(const __grid_constant__ Bufs B) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ PushShared<real> sh;
+  // With a network installed the launch has one CTA more, which runs the
+  // learned predictor for the level the previous solve committed (levels
+  // >= 1).  Scheduled last, it takes the first slot a pushing CTA frees, so
+  // the network runs beside the other CTAs' ends.
+  const bool pred_cta = (B.net != nullptr && B.net_in_push);
+  const int G = static_cast<int>(gridDim.x) - (pred_cta ? 1 : 0);  // pushing CTAs
+  if (static_cast<int>(blockIdx.x) == G) {
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();
+    if (ldcg(&B.S->status) != 0) return;
+    if (PUSH && ldcg(&B.S->level) >= 1) predictor_in_push(B.S, B.net, B.P->C, reinterpret_cast<PredScratch*>(smem));
+    return;
+  }
+  if (!push_cta<real, PUSH, false>(B, sh, smem, G)) push_cta_late<real, PUSH>(B, sh, smem, G);
 }
 
 // ---------------------------------------------------------------------------
