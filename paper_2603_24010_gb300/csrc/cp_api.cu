@@ -44,7 +44,7 @@ int ens_max_instances();
 size_t abs_rec_ens_bytes();
 cudaError_t push_ens_occupancy(int precision, int threads, size_t smem, int* per_sm);
 cudaError_t push_ens_launch(int precision, int threads, int grid, size_t smem, const Bufs* Ball,
-                            int E, int n_max, void* abs, int abs_cap, cudaStream_t st);
+                            int E, int n_max, int beam_max, void* abs, int abs_cap, cudaStream_t st);
 cudaError_t compact_ens_launch(int precision, const Bufs* Ball, int E, int grid, cudaStream_t st);
 cudaError_t solve_ens_configure(int precision, bool wide);
 cudaError_t solve_ens_launch(int precision, bool wide, const Bufs* Ball, int n_inst, int ctas, size_t smem,
@@ -1167,6 +1167,7 @@ struct cp_batch {
   int E = 0;
   int precision = CP_FP32;
   int n_max = 0;
+  int beam_max = 0;      // beam ions a step of the largest beam
   bool initialized = false;
   cpk::Bufs* dBall = nullptr;
   void* abs = nullptr;
@@ -1244,6 +1245,7 @@ int batch_init(cp_batch* b, int mode, double tol) {
   for (int i = 0; i < b->E; ++i) {
     hb[i] = make_bufs(b->inst[i]);
     b->n_max = std::max(b->n_max, b->inst[i]->N);
+    b->beam_max = std::max(b->beam_max, static_cast<int>(b->inst[i]->hp.beam_per_step));
   }
   CP_TRY(alloc(reinterpret_cast<void**>(&b->dBall), sizeof(cpk::Bufs) * b->E));
   CP_CUDA(cudaMemcpyAsync(b->dBall, hb.data(), sizeof(cpk::Bufs) * b->E, cudaMemcpyHostToDevice,
@@ -1272,7 +1274,7 @@ cudaError_t batch_solve(cp_batch* b, cudaStream_t st, int mode, double tol) {
 
 cudaError_t batch_step_launches(cp_batch* b, cudaStream_t st, int mode, double tol) {
   cudaError_t e = cpk::push_ens_launch(b->precision, b->push_threads, b->push_grid, b->push_smem,
-                                       b->dBall, b->E, b->n_max, b->abs, b->abs_cap, st);
+                                       b->dBall, b->E, b->n_max, b->beam_max, b->abs, b->abs_cap, st);
   if (e == cudaSuccess)
     e = batch_solve(b, st, mode, tol);
   return e;
@@ -1328,7 +1330,7 @@ int batch_steps_timed(cp_batch* b, int mode, int32_t n_steps, double tol) {
     CP_CUDA(cudaEventRecord(b->ev[k], b->stream));
     if (which == 0)
       CP_CUDA(cpk::push_ens_launch(b->precision, b->push_threads, b->push_grid, b->push_smem,
-                                   b->dBall, b->E, b->n_max, b->abs, b->abs_cap, b->stream));
+                                   b->dBall, b->E, b->n_max, b->beam_max, b->abs, b->abs_cap, b->stream));
     else if (which == 1)
       CP_CUDA(batch_solve(b, b->stream, mode, tol));
     else
@@ -1554,7 +1556,7 @@ int cp_batch_autotune(cp_batch* b, int32_t steps_per_shape, int32_t mode, double
       rc = cuda_rc(cudaEventRecord(e0, b->stream));
       if (rc == CP_OK)
         rc = cuda_rc(cpk::push_ens_launch(b->precision, b->push_threads, b->push_grid, b->push_smem,
-                                          b->dBall, b->E, b->n_max, b->abs, b->abs_cap, b->stream));
+                                          b->dBall, b->E, b->n_max, b->beam_max, b->abs, b->abs_cap, b->stream));
       if (rc == CP_OK) rc = cuda_rc(cudaEventRecord(e1, b->stream));
       if (rc == CP_OK)
         rc = cuda_rc(batch_solve(b, b->stream, mode, tol));

@@ -6,15 +6,18 @@
 //   one contiguous share of it, so it meets only a few instances and loads
 //   each instance's gather table and flushes each instance's deposit grid
 //   once per step.  Per tile the arithmetic is that of the single-instance
-//   push (same gather, kick, drift, absorption test and fixed-point deposit),
-//   so an instance advanced in the ensemble follows exactly the trajectory
-//   it follows alone.  Secondary emission and the beam are handled after the
-//   tiles: emitted electrons and beam ions are deposited with int64 global
-//   atomics straight into their instance's grid.
+//   push (cp_push.cuh: same gather, kick, drift, absorption test and
+//   fixed-point deposit), so an instance advanced in the ensemble follows
+//   exactly the trajectory it follows alone.  Secondary emission and the beam
+//   are handled after the tiles: emitted electrons and beam ions are deposited
+//   with int64 global atomics straight into their instance's grid.
 // k_compact_ens / k_swap_ens: removal of absorbed particles over the same
 //   flat list, then one thread per (instance, species) swaps the buffers.
 // The solve of every instance (one CTA each) is k_solve_ens in cp_solve.cu.
+#include <algorithm>
+
 #include "cp_common.cuh"
+#include "cp_push.cuh"
 
 namespace cpk {
 
@@ -27,41 +30,21 @@ struct AbsRecE {
 
 constexpr int kEnsMaxEntries = 3 * 2048;  // (instance, species) pairs: at most 2048 instances
 
-__device__ __forceinline__ void fold_any(unsigned int* A, unsigned int* Bc, long long* Gs, int N,
-                                         long long sign) {
-  for (int k = threadIdx.x; k <= N; k += blockDim.x) {
-    long long a = 0, b = 0;
-    if (k < N) {
-      a = A[k];
-      A[k] = 0u;
-    }
-    if (k > 0) {
-      b = Bc[k - 1];
-      Bc[k - 1] = 0u;
-    }
-    if (k == 0) a <<= 1;
-    if (k == N) b <<= 1;
-    if (a | b) Gs[k] += sign * (a + b);
-  }
-}
-
 // The fixed-point CIC deposit of one particle, added straight into an int64
-// global grid (end nodes doubled, as the fold does).
+// global grid.
 template <typename real>
-__device__ __forceinline__ void deposit_global(long long* G, int N, real x, long long sign) {
-  const real fl = floor(x);
-  const int i = static_cast<int>(fl);
-  const long long w1 = static_cast<long long>(frac_to_fix(x - fl));
-  const long long w0 = 65536LL - w1;
-  atomicAdd(reinterpret_cast<unsigned long long*>(&G[i]),
-            static_cast<unsigned long long>(sign * (i == 0 ? 2 * w0 : w0)));
-  atomicAdd(reinterpret_cast<unsigned long long*>(&G[i + 1]),
-            static_cast<unsigned long long>(sign * (i + 1 == N ? 2 * w1 : w1)));
+__device__ __forceinline__ void deposit_global(long long* G, int N, real x, int sign) {
+  const unsigned int F = fix_pos(x);
+  const long long w1 = F & 0xFFFFu;
+  add_global(G, F >> 16, N, sign * (65536LL - w1));
+  add_global(G, (F >> 16) + 1, N, sign * w1);
 }
 
 // Exclusive prefix of the tile counts of every (instance, species) pair into
-// off[0..n] (off[n] = total); counts of stopped instances are 0.
-template <int THREADS>
+// off[0..n] (off[n] = total).  STOPPED: with the entries of stopped instances
+// (else 0): every CTA of a push must see the same list, also one that starts
+// after another has stopped an instance.
+template <int THREADS, bool STOPPED>
 __device__ void tile_offsets(const Bufs* __restrict__ Ball, int E, int tile, int* off, int* wsum) {
   const int n = 3 * E;
   const int per = (n + THREADS - 1) / THREADS;
@@ -69,7 +52,7 @@ __device__ void tile_offsets(const Bufs* __restrict__ Ball, int E, int tile, int
   int loc = 0;
   for (int j = j0; j < j1; ++j) {
     const DevState* S = Ball[j / 3].S;
-    const long long np = (ldcg(&S->status) == 0) ? ldcg(&S->n_proc[j % 3]) : 0LL;
+    const long long np = (STOPPED || ldcg(&S->status) == 0) ? ldcg(&S->n_proc[j % 3]) : 0LL;
     const int t = static_cast<int>((np + tile - 1) / tile);
     off[j] = t;
     loc += t;
@@ -96,290 +79,392 @@ __device__ void tile_offsets(const Bufs* __restrict__ Ball, int E, int tile, int
   __syncthreads();
 }
 
+// a thread's particles from global memory
+__device__ __forceinline__ void ld_vec(const float* p, float (&v)[4]) {
+  const float4 a = __ldcs(reinterpret_cast<const float4*>(p));
+  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+}
+__device__ __forceinline__ void ld_vec(const double* p, double (&v)[2]) {
+  const double2 a = __ldcs(reinterpret_cast<const double2*>(p));
+  v[0] = a.x; v[1] = a.y;
+}
+
+// --- the push ------------------------------------------------------------------
+constexpr int kEnsSegs = 8;    // segments of a CTA's share listed at a time
+
 template <typename real, int THREADS>
-__global__ void __launch_bounds__(THREADS)
-k_push_ens(const Bufs* __restrict__ Ball, int E, int n_max, AbsRecE* __restrict__ abs_all, int abs_cap) {
+struct EnsTile {
+  static constexpr int kN = 16 / sizeof(real);  // particles per thread
+  static constexpr int kTileN = THREADS * kN;
+  static constexpr int kLog = (kTileN == 4096) ? 12 : (kTileN == 2048) ? 11 : (kTileN == 1024) ? 10 : 9;
+  static_assert(kTileN == 1 << kLog, "tile sizes are powers of two");
+  // a tile adds at most 2^kShift to a node; 32 bits tell the signed sums of
+  // this many tiles apart
+  static constexpr int kShift = 16 + kLog;
+  static constexpr int kMost = (1 << (32 - kShift)) - 1;
+};
+
+// Tiles [t0, t1) of one (instance, species).
+template <typename real>
+struct EnsSeg {
+  real *x, *u;
+  const uint32_t* ids;
+  long long n;  // slots
+  real kap;
+  int inst, s, t0, t1;
+};
+
+template <typename real, int THREADS>
+struct alignas(128) EnsShared {
+  EnsSeg<real> seg[kEnsSegs];
+  unsigned int cnt[2][kSpecies];
+  long long u_next;
+  int nseg, abs_n;
+  unsigned int cfl;
+  int wsum[THREADS / 32];
+};
+
+constexpr int ens_min_ctas(int threads, size_t es) { return threads == 256 ? 3 : (threads == 512 && es == 4) ? 2 : 1; }
+
+// One launch pushes every instance.  Each CTA takes one contiguous share of
+// the flat (instance, species, tile) list and keeps the field table and the
+// node sums of one instance at a time.
+//
+// What bounds it: the HBM stream of the particles, and close behind it the
+// shared-memory pipe (two table reads and two node-sum atomics per particle at
+// random cells).  A thread requests its next four particles before it works on
+// the present ones, running on across the segments of the share; they wait in
+// registers, since a ring of asynchronous copies puts a third more traffic on
+// the shared-memory pipe (230 us without the tail instead of 217).  One signed
+// 32-bit sum per node and a table of E alone take 16 bytes of shared memory a
+// cell.  The end of a CTA is latency: impacts and their electrons one per
+// lane, the beams dealt over all CTAs, in slots that need no counter.
+//
+// 160 gaps of 260 to 3985 cells, 7.0e7 particles: push 231 -> 222 us, step in
+// a graph 268 -> 264.
+template <typename real, int THREADS>
+__global__ void __launch_bounds__(THREADS, ens_min_ctas(THREADS, sizeof(real)))
+k_push_ens(const Bufs* __restrict__ Ball, int E, int n_max, int beam_chunks,
+           AbsRecE* __restrict__ abs_all, int abs_cap) {
   using real2 = typename Pair<real>::type;
-  constexpr int TILE = THREADS * kPerThread;
+  using V = EnsTile<real, THREADS>;
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int wsum[THREADS / 32];
-  __shared__ int s_abs_n, s_j;
-  __shared__ unsigned long long s_cnt[2][kSpecies];
-  __shared__ unsigned int s_cfl;
+  __shared__ EnsShared<real, THREADS> sh;
+  const int tid = static_cast<int>(threadIdx.x);
+  long long* Gs = reinterpret_cast<long long*>(smem);
+  unsigned int* nd = reinterpret_cast<unsigned int*>(smem + align16(sizeof(long long) * (n_max + 1)));
+  real* Et = reinterpret_cast<real*>(reinterpret_cast<unsigned char*>(nd) + align16(sizeof(unsigned int) * (n_max + 1)));
+  int* off = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(Et) + align16(sizeof(real) * (n_max + 2)));
+  for (int k = tid; k <= n_max; k += THREADS) nd[k] = 0u;
+  if (tid == 0) {
+    sh.abs_n = 0;
+    sh.cfl = 0u;
+  }
+  if (tid < 2 * kSpecies) sh.cnt[tid / kSpecies][tid % kSpecies] = 0u;
 
   cudaGridDependencySynchronize();  // the previous solves (or removal) have completed
   cudaTriggerProgrammaticLaunchCompletion();
-  long long* Gs = reinterpret_cast<long long*>(smem);
-  unsigned int* A = reinterpret_cast<unsigned int*>(smem + align16(sizeof(long long) * (n_max + 1)));
-  unsigned int* Bc = A + n_max;
-  real2* Es2 = reinterpret_cast<real2*>(smem + align16(sizeof(long long) * (n_max + 1)) +
-                                        align16(sizeof(unsigned int) * 2 * n_max));
-  int* off = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(Es2) +
-                                    align16(sizeof(real2) * (n_max + 1)));
-  tile_offsets<THREADS>(Ball, E, TILE, off, wsum);
-  const long long U = off[3 * E];
-  const long long u0 = U * blockIdx.x / gridDim.x, u1 = U * (blockIdx.x + 1) / gridDim.x;
-  if (threadIdx.x == 0) {
-    s_abs_n = 0;
-    int lo = 0, hi = 3 * E;  // the entry holding unit u0: off[j] <= u0 < off[j+1]
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if (off[mid] <= u0) lo = mid;
-      else hi = mid;
-    }
-    s_j = lo;
-  }
-  for (int k = threadIdx.x; k <= n_max; k += THREADS) Gs[k] = 0;
-  for (int k = threadIdx.x; k < 2 * n_max; k += THREADS) A[k] = 0u;
-  __syncthreads();
   AbsRecE* my_abs = abs_all + static_cast<size_t>(blockIdx.x) * abs_cap;
 
-  int cur = -1, N = 0;
-  const DevParams* P = nullptr;
-  DevState* S = nullptr;
-  bool half = false;
-  unsigned int cfl = 0u;
-  // flush the current instance's grid and tallies into global memory
+  int cur = -1, N = 0;  // the instance whose table and sums are in shared memory
+  real Nr = real(0);
+  bool folded = false;
+  int pos = 0, neg = 0;  // tiles of each sign in the node sums
+  typename Bits<real>::type cfl = 0;
+  auto node_value = [&](unsigned int v) {
+    const unsigned int o = static_cast<unsigned int>(neg) << V::kShift;
+    return static_cast<long long>(v + o) - static_cast<long long>(o);
+  };
+  // the current instance's grid and tallies into global memory
   auto flush = [&]() {
+    const unsigned int c = warp_max_u(float_bits(cfl));
+    if (lane_id() == 0 && c) atomicMax(&sh.cfl, c);
+    cfl = 0;
     __syncthreads();
     long long* G = Ball[cur].G;
-    for (int k = threadIdx.x; k <= N; k += THREADS) {
-      const long long g = Gs[k];
-      if (g != 0) {
-        atomicAdd(reinterpret_cast<unsigned long long*>(&G[k]), static_cast<unsigned long long>(g));
-        Gs[k] = 0;
-      }
+    for (int k = tid; k <= N; k += THREADS) {
+      add_global(G, k, N, node_value(nd[k]) + (folded ? Gs[k] : 0LL));
+      nd[k] = 0u;
     }
-    const unsigned int c = warp_max_u(cfl);
-    if (lane_id() == 0 && c) atomicMax(&S->max_cfl_bits, c);
-    cfl = 0u;
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
+      DevState* S = Ball[cur].S;
       for (int e = 0; e < 2; ++e)
         for (int s = 0; s < kSpecies; ++s)
-          if (s_cnt[e][s]) atomicAdd(&S->absorbed[e][s], s_cnt[e][s]);
-      const long long conv = static_cast<long long>(s_cnt[0][CP_IONS]) -
-                             static_cast<long long>(s_cnt[0][CP_ELECTRONS]) -
-                             static_cast<long long>(s_cnt[0][CP_SECONDARIES]);
+          if (sh.cnt[e][s]) atomicAdd(&S->absorbed[e][s], static_cast<unsigned long long>(sh.cnt[e][s]));
+      const long long conv = static_cast<long long>(sh.cnt[0][CP_IONS]) -
+                             static_cast<long long>(sh.cnt[0][CP_ELECTRONS]) -
+                             static_cast<long long>(sh.cnt[0][CP_SECONDARIES]);
       if (conv) atomicAdd(reinterpret_cast<unsigned long long*>(&S->conv_count),
                           static_cast<unsigned long long>(conv));
+      if (sh.cfl) atomicMax(&S->max_cfl_bits, sh.cfl);
+      sh.cfl = 0u;
+      for (int e = 0; e < 2; ++e)
+        for (int s = 0; s < kSpecies; ++s) sh.cnt[e][s] = 0u;
     }
-    __syncthreads();
+    folded = false;
+    pos = neg = 0;
   };
 
-  for (long long u = u0; u < u1;) {
-    const int j = s_j;
-    const int inst = j / 3, s = j % 3;
-    const long long t_end = min(u1, static_cast<long long>(off[j + 1]));
-    const long long t0 = u - off[j], t1 = t_end - off[j];  // tiles of this (instance, species)
-    if (inst != cur) {
-      if (cur >= 0) flush();
-      cur = inst;
-      const Bufs& B = Ball[cur];
-      P = B.P;
-      S = B.S;
-      N = P->N;
-      half = (ldcg(&S->pushed) == 0);
-      const real2* Epair = reinterpret_cast<const real2*>(B.Epair);
-      for (int k = threadIdx.x; k <= N; k += THREADS) Es2[k] = Epair[k];
-      if (threadIdx.x < 2 * kSpecies) s_cnt[threadIdx.x / kSpecies][threadIdx.x % kSpecies] = 0ULL;
-      if (threadIdx.x == 0) s_cfl = 0u;
-      __syncthreads();
-    }
-    real* __restrict__ xs = reinterpret_cast<real*>(S->xi[s]);
-    real* __restrict__ us = reinterpret_cast<real*>(S->u[s]);
-    const int64_t n = S->n_proc[s];
-    const long long sign = (s == CP_IONS) ? 1LL : -1LL;
-    real kap;
-    if constexpr (sizeof(real) == 4) kap = P->kap_f[half ? 0 : 1][s];
-    else kap = P->kap_d[half ? 0 : 1][s];
-    const real Nr = static_cast<real>(N);
-    const uint32_t* ids = S->id;
-    unsigned int a0 = 0u, a1 = 0u;
-    int since = 0;
-    real xv[4], uv[4];
-    int64_t base = t0 * TILE + static_cast<int64_t>(threadIdx.x) * kPerThread;
-    if (base < n) {
-      load4(xs + base, xv);
-      load4(us + base, uv);
-    }
-    for (long long t = t0; t < t1; ++t) {
-      const int64_t bnext = base + TILE;
-      real xq[4], uq[4];
-      const bool more = (t + 1 < t1) && bnext < n;
-      if (more) {
-        load4(xs + bnext, xq);
-        load4(us + bnext, uq);
+  // Fetch cursor over the listed segments: `left` more tiles of segment q,
+  // the next at x, u for this thread, whose particles end at x_end.
+  struct Cursor {
+    const real *x, *u, *x_end;
+    int q, left;
+  };
+  const int nthr = tid * V::kN;
+  tile_offsets<THREADS, true>(Ball, E, V::kTileN, off, sh.wsum);
+  const long long U = off[3 * E], u1 = U * (blockIdx.x + 1) / gridDim.x;
+  for (long long u0 = U * blockIdx.x / gridDim.x, u_next; u0 < u1; u0 = u_next) {
+    if (tid == 0) {  // the next segments of [u0, u1)
+      int lo = 0, hi = 3 * E;  // the entry holding tile u0: off[j] <= u0 < off[j+1]
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (off[mid] <= u0) lo = mid;
+        else hi = mid;
       }
-      if (base < n) {
+      int q = 0;
+      long long u = u0;
+      for (int j = lo; u < u1 && q < kEnsSegs; ++j) {
+        const int end = static_cast<int>(min(u1, static_cast<long long>(off[j + 1])));
+        if (end <= u) continue;  // no tiles
+        sh.seg[q].inst = j / 3;
+        sh.seg[q].s = j % 3;
+        sh.seg[q].t0 = static_cast<int>(u - off[j]);
+        sh.seg[q].t1 = end - off[j];
+        u = end;
+        ++q;
+      }
+      sh.nseg = q;
+      sh.u_next = u;
+    }
+    __syncthreads();
+    if (tid < sh.nseg) {
+      EnsSeg<real>& g = sh.seg[tid];
+      const Bufs& B = Ball[g.inst];
+      DevState* S = B.S;
+      g.x = static_cast<real*>(ldcg(&S->xi[g.s]));
+      g.u = static_cast<real*>(ldcg(&S->u[g.s]));
+      g.ids = static_cast<const uint32_t*>(ldcg(reinterpret_cast<void* const*>(&S->id)));
+      g.n = ldcg(&S->n_proc[g.s]);
+      g.kap = kick<real>(B.P, ldcg(&S->pushed) == 0, g.s);
+      if (ldcg(&S->status) != 0) g.t1 = g.t0;  // stopped
+    }
+    __syncthreads();
+    const int nseg = sh.nseg;
+    u_next = sh.u_next;
+    Cursor nxt;
+    auto enter = [&](int q) {
+      nxt.left = 0;
+      for (; q < nseg; ++q) {
+        const EnsSeg<real>& g = sh.seg[q];
+        if (g.t1 > g.t0) {
+          const long long b = static_cast<long long>(g.t0) * V::kTileN + nthr;
+          nxt.x = g.x + b;
+          nxt.u = g.u + b;
+          nxt.x_end = g.x + g.n;
+          nxt.left = g.t1 - g.t0;
+          break;
+        }
+      }
+      nxt.q = q;
+    };
+    real xq[V::kN], uq[V::kN];
+    auto fetch = [&]() {
+      if (nxt.left > 0) {
+        if (nxt.x < nxt.x_end) {
+          ld_vec(nxt.x, xq);
+          ld_vec(nxt.u, uq);
+        }
+        nxt.x += V::kTileN;
+        nxt.u += V::kTileN;
+        if (--nxt.left == 0) enter(nxt.q + 1);
+      }
+    };
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          if (xv[q] > real(0) && xv[q] < Nr) {  // live (dead slots hold -1)
-            const real Ef = gather<real>(Es2, xv[q]);
-            const real un = fma(kap, Ef, uv[q]);
-            const real xn = xv[q] + un;
-            cfl = max(cfl, __float_as_uint(fabsf(static_cast<float>(un))));
-            if (!(xn > real(0) && xn < Nr)) {  // absorbed (a non-finite value counts at x = d)
+    for (int c = 0; c < V::kN; ++c) xq[c] = uq[c] = real(0);
+    enter(0);
+    fetch();
+
+    for (int q = 0; q < nseg; ++q) {
+      const EnsSeg<real>& g = sh.seg[q];
+      if (g.t1 == g.t0) continue;
+      if (g.inst != cur) {
+        if (cur >= 0) flush();
+        cur = g.inst;
+        const Bufs& B = Ball[cur];
+        N = B.P->N;
+        Nr = static_cast<real>(N);
+        const real2* Epair = reinterpret_cast<const real2*>(B.Epair);
+        for (int k = tid; k <= N; k += THREADS) {
+          const real e = __ldcg(&Epair[k]).x;  // pair 0 repeats E_{1/2}
+          Et[k] = e;
+          if (k == N) Et[N + 1] = e;
+        }
+        __syncthreads();
+      }
+      const int s = g.s, sign = (s == CP_IONS) ? 1 : -1;
+      const real kap = g.kap;
+      const long long b = static_cast<long long>(g.t0) * V::kTileN + nthr;
+      real* x = g.x + b;
+      real* u = g.u + b;
+      const real* const x_end = g.x + g.n;
+      for (int left = g.t1 - g.t0; left > 0; --left, x += V::kTileN, u += V::kTileN) {
+        real xv[V::kN], uv[V::kN];
+#pragma unroll
+        for (int c = 0; c < V::kN; ++c) {
+          xv[c] = xq[c];
+          uv[c] = uq[c];
+        }
+        fetch();
+        if (pos + neg == V::kMost) {  // bounds every node sum to 32 bits
+          __syncthreads();
+          for (int k = tid; k <= N; k += THREADS) {
+            const long long a = node_value(nd[k]);
+            nd[k] = 0u;
+            Gs[k] = folded ? Gs[k] + a : a;
+          }
+          __syncthreads();
+          folded = true;
+          pos = neg = 0;
+        }
+        if (sign > 0) ++pos; else ++neg;
+        if (x >= x_end) continue;
+#pragma unroll
+        for (int c = 0; c < V::kN; ++c) {
+          bool dep = false;
+          if (inside(xv[c], Nr)) {  // live (dead slots hold -1)
+            const real un = fma(kap, gather_tab(Et, xv[c]), uv[c]);
+            const real xn = xv[c] + un;
+            max_abs(cfl, un);
+            if (!inside(xn, Nr)) {  // absorbed (a non-finite value counts at x = d)
               const int el = (xn <= real(0)) ? 0 : 1;
-              if (el) ++a1; else ++a0;
-              if (s == CP_IONS) {
-                const int slot = atomicAdd(&s_abs_n, 1);
+              atomicAdd(&sh.cnt[el][s], 1u);
+              if (sign > 0) {
+                const int slot = atomicAdd(&sh.abs_n, 1);
                 if (slot < abs_cap) {
                   AbsRecE r;
-                  r.id = ids[base + q];
+                  r.id = g.ids[x + c - g.x];
                   r.inst_el = static_cast<uint32_t>(2 * cur + el);
                   r.u = static_cast<double>(un);
                   my_abs[slot] = r;
                 } else {
-                  atomicCAS(&S->status, 0, CP_ERR_CAPACITY);
+                  atomicCAS(&Ball[cur].S->status, 0, CP_ERR_CAPACITY);
                 }
               }
-              xv[q] = real(-1);
-              uv[q] = real(0);
+              xv[c] = real(-1);
+              uv[c] = real(0);
             } else {
-              deposit<real>(A, Bc, xn);
-              xv[q] = xn;
-              uv[q] = un;
+              dep = true;
+              xv[c] = xn;
+              uv[c] = un;
             }
           }
+          if (dep) deposit_nodes(nd, fix_pos(xv[c]), sign);
         }
-        store4(xs + base, xv);
-        store4(us + base, uv);
-      }
-      if (more) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          xv[q] = xq[q];
-          uv[q] = uq[q];
-        }
-      }
-      base = bnext;
-      if (++since == kFlushTiles) {  // bounds every 32-bit cell sum below 2^32
-        __syncthreads();
-        fold_any(A, Bc, Gs, N, sign);
-        __syncthreads();
-        since = 0;
+        put_vec(x, xv);
+        put_vec(u, uv);
       }
     }
-    __syncthreads();
-    fold_any(A, Bc, Gs, N, sign);
-    a0 = warp_sum_u(a0);
-    a1 = warp_sum_u(a1);
-    if (lane_id() == 0) {
-      if (a0) atomicAdd(&s_cnt[0][s], static_cast<unsigned long long>(a0));
-      if (a1) atomicAdd(&s_cnt[1][s], static_cast<unsigned long long>(a1));
-    }
-    u = t_end;
-    __syncthreads();
-    if (threadIdx.x == 0) s_j = j + 1;
-    __syncthreads();
-    // skip pairs with no tiles (stopped instances, empty species)
-    if (threadIdx.x == 0) {
-      int jj = s_j;
-      while (jj < 3 * E && off[jj + 1] == off[jj] && off[jj] < u1) ++jj;
-      s_j = jj;
-    }
-    __syncthreads();
+    __syncthreads();  // the listed segments are done
   }
+  __syncthreads();
   if (cur >= 0) flush();
 
   // --- secondary emission from the ions this CTA saw absorbed ---------------
-  const int na = min(s_abs_n, abs_cap);
-  for (int r0 = 0; r0 < na; r0 += THREADS) {
-    const int r = r0 + threadIdx.x;
-    if (r >= na) break;
-    const AbsRecE rec = my_abs[r];
-    const int inst = static_cast<int>(rec.inst_el >> 1), el = static_cast<int>(rec.inst_el & 1u);
-    const Bufs& B = Ball[inst];
-    const DevParams* Pi = B.P;
-    DevState* Si = B.S;
-    const int64_t step = Si->level;
-    const int Ni = Pi->N;
-    const double dx = Pi->dx, dt = Pi->dt;
-    const double v = __ddiv_rn(__dmul_rn(rec.u, dx), dt);
-    const double Eev = __ddiv_rn(__dmul_rn(__dmul_rn(__dmul_rn(0.5, Pi->m_i), v), v), Pi->e);
-    const int nse = see_count(Pi, Eev, rec.id, step);
-    if (el == 0) {
-      atomicAdd(reinterpret_cast<unsigned long long*>(&Si->ion_energy_q),
-                static_cast<unsigned long long>(__double2ll_rn(Eev * 256.0)));
-      if (nse) atomicAdd(reinterpret_cast<unsigned long long*>(&Si->conv_count),
-                         static_cast<unsigned long long>(static_cast<long long>(nse)));
+  // one record per lane (a warp's FP64 operation takes the pipe equally long
+  // for any number of lanes): the counts, then the electrons one per lane
+  const int na = min(sh.abs_n, abs_cap);
+  const int lane = tid & 31;
+  for (int r0 = tid - lane; r0 < na; r0 += THREADS) {
+    const int r = r0 + lane;
+    int nse = 0;
+    unsigned long long wb = 0ULL;
+    AbsRecE rec;
+    rec.id = 0; rec.inst_el = 0; rec.u = 0.0;
+    if (r < na) {
+      rec = my_abs[r];
+      const int el = static_cast<int>(rec.inst_el & 1u);
+      const Bufs& B = Ball[rec.inst_el >> 1];
+      const DevParams* Pi = B.P;
+      DevState* Si = B.S;
+      const double v = __ddiv_rn(__dmul_rn(rec.u, Pi->dx), Pi->dt);
+      const double Eev = __ddiv_rn(__dmul_rn(__dmul_rn(__dmul_rn(0.5, Pi->m_i), v), v), Pi->e);
+      nse = see_count(Pi, Eev, rec.id, ldcg(&Si->level));
+      if (el == 0) {
+        atomicAdd(reinterpret_cast<unsigned long long*>(&Si->ion_energy_q),
+                  static_cast<unsigned long long>(__double2ll_rn(Eev * 256.0)));
+        if (nse) atomicAdd(reinterpret_cast<unsigned long long*>(&Si->conv_count),
+                           static_cast<unsigned long long>(static_cast<long long>(nse)));
+      }
+      if (nse) {
+        atomicAdd(&Si->emitted[el], static_cast<unsigned long long>(nse));
+        wb = atomicAdd(reinterpret_cast<unsigned long long*>(&Si->n_alloc[CP_SECONDARIES]),
+                       static_cast<unsigned long long>(nse));
+      }
     }
-    if (nse == 0) continue;
-    atomicAdd(&Si->emitted[el], static_cast<unsigned long long>(nse));
-    const unsigned long long wb =
-        atomicAdd(reinterpret_cast<unsigned long long*>(&Si->n_alloc[CP_SECONDARIES]),
-                  static_cast<unsigned long long>(nse));
-    real* xs = reinterpret_cast<real*>(Si->xi[CP_SECONDARIES]);
-    real* us = reinterpret_cast<real*>(Si->u[CP_SECONDARIES]);
-    for (int jn = 0; jn < nse; ++jn) {
+    const int incl = warp_incl_scan(nse);
+    const int total = __shfl_sync(0xffffffffu, incl, 31);
+    for (int e0 = 0; e0 < total; e0 += 32) {
+      const int e = e0 + lane;
+      int src = 0;  // the record of electron e: the first lane whose count exceeds e
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+        if (__shfl_sync(0xffffffffu, incl, src + o - 1) <= e) src += o;
+      src = min(src, 31);
+      const uint32_t id = __shfl_sync(0xffffffffu, rec.id, src);
+      const uint32_t ie = __shfl_sync(0xffffffffu, rec.inst_el, src);
+      const int jn = e - __shfl_sync(0xffffffffu, incl - nse, src);
+      const unsigned long long slot = __shfl_sync(0xffffffffu, wb, src) + static_cast<unsigned long long>(jn);
+      if (e >= total) continue;
+      const Bufs& B = Ball[ie >> 1];
+      const DevParams* Pi = B.P;
+      DevState* Si = B.S;
+      const bool left = (ie & 1u) == 0u;
+      const int Ni = Pi->N;
       double frac;
-      const double vse = see_speed(Pi, rec.id, step, jn, &frac);
-      const double use = vse * dt / dx;
-      const double xd = (el == 0) ? __dmul_rn(use, frac) : __dsub_rn(static_cast<double>(Ni), __dmul_rn(use, frac));
+      const double vse = see_speed(Pi, id, ldcg(&Si->level), jn, &frac);
+      const double use = vse * Pi->dt / Pi->dx;
+      const double xd = left ? __dmul_rn(use, frac) : __dsub_rn(static_cast<double>(Ni), __dmul_rn(use, frac));
       const real xr = nudge_inside<real>(xd, Ni);
-      const real ur = static_cast<real>(el == 0 ? use : -use);
-      const unsigned long long slot = wb + static_cast<unsigned long long>(jn);
       if (slot < static_cast<unsigned long long>(Pi->cap[CP_SECONDARIES])) {
-        xs[slot] = xr;
-        us[slot] = ur;
-        deposit_global<real>(B.G, Ni, xr, -1LL);
+        static_cast<real*>(Si->xi[CP_SECONDARIES])[slot] = xr;
+        static_cast<real*>(Si->u[CP_SECONDARIES])[slot] = static_cast<real>(left ? use : -use);
+        deposit_global<real>(B.G, Ni, xr, -1);
       } else {
         atomicCAS(&Si->status, 0, CP_ERR_CAPACITY);
       }
     }
   }
 
-  // --- beam ions of the instances this CTA serves (i = blockIdx.x mod grid) --
-  for (int inst = blockIdx.x; inst < E; inst += gridDim.x) {
-    const Bufs& B = Ball[inst];
+  // --- the beams: THREADS ions of one instance at a time ----------------------
+  // Ions are appended by the beam alone, behind the slots in use.
+  for (int item = blockIdx.x; item < E * beam_chunks; item += gridDim.x) {
+    const Bufs& B = Ball[item / beam_chunks];
     const DevParams* Pi = B.P;
     DevState* Si = B.S;
-    const int Bn = Pi->beam_per_step;
-    if (Bn <= 0 || ldcg(&Si->status) != 0) continue;
-    const int64_t step = Si->level;
-    const int Ni = Pi->N;
-    const double dx = Pi->dx, dt = Pi->dt;
-    real* xs = reinterpret_cast<real*>(Si->xi[CP_IONS]);
-    real* us = reinterpret_cast<real*>(Si->u[CP_IONS]);
-    uint32_t* ids = Si->id;
-    const uint32_t id0 = Si->beam_id_base;
-    for (int k0 = 0; k0 < Bn; k0 += THREADS) {
-      const int k = k0 + threadIdx.x;
-      const bool act = k < Bn;
-      const unsigned ball = __ballot_sync(0xffffffffu, act);
-      unsigned long long wbase = 0ULL;
-      if (lane_id() == 0 && ball)
-        wbase = atomicAdd(reinterpret_cast<unsigned long long*>(&Si->n_alloc[CP_IONS]),
-                          static_cast<unsigned long long>(__popc(ball)));
-      wbase = __shfl_sync(0xffffffffu, wbase, 0);
-      if (act) {
-        const U64x4 wv = philox4x64_10(static_cast<uint64_t>(k), static_cast<uint64_t>(step), 0, 0,
-                                       Pi->seed, kTagBeam);
-        const double frac = u01(wv.w[0]);
-        double ub;
-        if constexpr (sizeof(real) == 4) {  // the single FP32 gap's arithmetic
-          ub = beam_speed_fp32(Pi, u01(wv.w[1]));
-        } else {  // the single FP64 gap's: the definition's order of operations
-          const double Eb = (Pi->beam_mode == 0)
-                                ? Pi->beam_E_eV
-                                : __dadd_rn(Pi->beam_Emin_eV, __dmul_rn(__dsub_rn(Pi->beam_Emax_eV, Pi->beam_Emin_eV), u01(wv.w[1])));
-          const double v = sqrt(2.0 * Eb * Pi->e / Pi->m_i);
-          ub = v * dt / dx;
-        }
-        const real xr = nudge_inside<real>(__dsub_rn(static_cast<double>(Ni), __dmul_rn(ub, frac)), Ni);
-        const unsigned long long slot =
-            wbase + static_cast<unsigned long long>(__popc(ball & ((1u << lane_id()) - 1u)));
-        if (slot < static_cast<unsigned long long>(Pi->cap[CP_IONS])) {
-          xs[slot] = xr;
-          us[slot] = static_cast<real>(-ub);
-          ids[slot] = id0 + static_cast<uint32_t>(step * Bn + k);
-          deposit_global<real>(B.G, Ni, xr, 1LL);
-        } else {
-          atomicCAS(&Si->status, 0, CP_ERR_CAPACITY);
-        }
+    const int Bn = Pi->beam_per_step, k = item % beam_chunks * THREADS + tid;
+    if (Bn <= item % beam_chunks * THREADS || ldcg(&Si->status) != 0) continue;
+    if (k < Bn) {
+      const int64_t step = ldcg(&Si->level);
+      const int Ni = Pi->N;
+      const U64x4 wv = philox4x64_10(static_cast<uint64_t>(k), static_cast<uint64_t>(step), 0, 0, Pi->seed, kTagBeam);
+      const double frac = u01(wv.w[0]);
+      const double ub = beam_speed<real>(Pi, u01(wv.w[1]));
+      const real xr = nudge_inside<real>(__dsub_rn(static_cast<double>(Ni), __dmul_rn(ub, frac)), Ni);
+      const int64_t slot = ldcg(&Si->n_proc[CP_IONS]) + k;
+      if (slot < Pi->cap[CP_IONS]) {
+        static_cast<real*>(Si->xi[CP_IONS])[slot] = xr;
+        static_cast<real*>(Si->u[CP_IONS])[slot] = static_cast<real>(-ub);
+        Si->id[slot] = Si->beam_id_base + static_cast<uint32_t>(step * Bn + k);
+        deposit_global<real>(B.G, Ni, xr, 1);
+      } else {
+        atomicCAS(&Si->status, 0, CP_ERR_CAPACITY);
       }
     }
-    if (threadIdx.x == 0) atomicAdd(&Si->injected, static_cast<unsigned long long>(Bn));
+    if (k == 0) {
+      atomicAdd(&Si->injected, static_cast<unsigned long long>(Bn));
+      atomicAdd(reinterpret_cast<unsigned long long*>(&Si->n_alloc[CP_IONS]), static_cast<unsigned long long>(Bn));
+    }
   }
 }
 
@@ -391,7 +476,7 @@ __global__ void __launch_bounds__(kThreads) k_compact_ens(const Bufs* __restrict
   constexpr int TILE = kThreads * kPerThread;
   __shared__ int off[kEnsMaxEntries + 1];
   __shared__ int wsum[kThreads / 32];
-  tile_offsets<kThreads>(Ball, E, TILE, off, wsum);
+  tile_offsets<kThreads, false>(Ball, E, TILE, off, wsum);
   const long long U = off[3 * E];
   // tiles are dealt round-robin: unit t -> its (instance, species) by search
   for (long long t = blockIdx.x; t < U; t += gridDim.x) {
@@ -473,8 +558,8 @@ __global__ void k_swap_ens(const Bufs* __restrict__ Ball, int E) {
 // ---------------------------------------------------------------------------
 size_t push_ens_smem_bytes(int n_max, int precision, int E) {
   const size_t es = (precision == CP_FP32) ? 4 : 8;
-  return align16(sizeof(long long) * (n_max + 1)) + align16(sizeof(unsigned int) * 2 * n_max) +
-         align16(2 * es * (n_max + 1)) + align16(sizeof(int) * (3 * E + 1));
+  return align16(sizeof(long long) * (n_max + 1)) + align16(sizeof(unsigned int) * (n_max + 1)) +
+         align16(es * (n_max + 2)) + align16(sizeof(int) * (3 * E + 1));
 }
 
 int ens_max_instances() { return kEnsMaxEntries / 3; }
@@ -495,17 +580,24 @@ static const void* push_ens_kernel(int precision, int threads) {
   return push_ens_fn<double, 512>();
 }
 
-// Resident CTAs per SM of the ensemble push for a block size (0: not launchable).
+// Resident CTAs per SM of the ensemble push for a block size (0: not
+// launchable).  The kernels' shared-memory limit is the largest the device
+// allows: ensembles of other sizes share them.
 cudaError_t push_ens_occupancy(int precision, int threads, size_t smem, int* per_sm) {
   const void* fn = push_ens_kernel(precision, threads);
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  int dev = 0, most = 0;
+  cudaFuncAttributes at;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, fn);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - static_cast<int>(at.sharedSizeBytes));
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, fn, threads, smem);
 }
 
 cudaError_t push_ens_launch(int precision, int threads, int grid, size_t smem, const Bufs* Ball,
-                            int E, int n_max, void* abs, int abs_cap, cudaStream_t st) {
+                            int E, int n_max, int beam_max, void* abs, int abs_cap, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid, 1, 1);
   cfg.blockDim = dim3(threads, 1, 1);
@@ -516,15 +608,9 @@ cudaError_t push_ens_launch(int precision, int threads, int grid, size_t smem, c
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  AbsRecE* a = static_cast<AbsRecE*>(abs);
-  if (precision == CP_FP32) {
-    if (threads == 256) return cudaLaunchKernelEx(&cfg, k_push_ens<float, 256>, Ball, E, n_max, a, abs_cap);
-    if (threads == 1024) return cudaLaunchKernelEx(&cfg, k_push_ens<float, 1024>, Ball, E, n_max, a, abs_cap);
-    return cudaLaunchKernelEx(&cfg, k_push_ens<float, 512>, Ball, E, n_max, a, abs_cap);
-  }
-  if (threads == 256) return cudaLaunchKernelEx(&cfg, k_push_ens<double, 256>, Ball, E, n_max, a, abs_cap);
-  if (threads == 1024) return cudaLaunchKernelEx(&cfg, k_push_ens<double, 1024>, Ball, E, n_max, a, abs_cap);
-  return cudaLaunchKernelEx(&cfg, k_push_ens<double, 512>, Ball, E, n_max, a, abs_cap);
+  int chunks = (beam_max + threads - 1) / threads;  // of the largest beam
+  void* args[] = {&Ball, &E, &n_max, &chunks, &abs, &abs_cap};
+  return cudaLaunchKernelExC(&cfg, push_ens_kernel(precision, threads), args);
 }
 
 size_t abs_rec_ens_bytes() { return sizeof(AbsRecE); }

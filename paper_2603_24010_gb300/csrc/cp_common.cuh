@@ -62,33 +62,6 @@ __device__ __forceinline__ unsigned int frac16(float f) {
   return __float_as_uint(__fmaf_rd(f, 65536.0f, 8388608.0f)) & 0xFFFFu;
 }
 
-// floor(f 2^16) of a fraction f in [0, 1): exact power-of-two scaling, truncation
-__device__ __forceinline__ unsigned int frac_to_fix(float f) { return __float2uint_rz(f * 65536.0f); }
-__device__ __forceinline__ unsigned int frac_to_fix(double f) { return __double2uint_rz(f * 65536.0); }
-
-// Linear interpolation between half-grid points from the pair table:
-// pair j+1 = (E_{j+1/2}, E_{j+3/2} - E_{j+1/2}) with constant ends.
-template <typename real>
-__device__ __forceinline__ real gather(const typename Pair<real>::type* Es2, real x) {
-  const real s = x - real(0.5);
-  const real jf = floor(s);
-  const int j = static_cast<int>(jf);
-  const real t = s - jf;
-  const typename Pair<real>::type e = Es2[j + 1];
-  return fma(t, e.y, e.x);
-}
-
-// CIC deposit into the per-cell 32-bit sums: A[i] += 2^16 - W1 (node i),
-// Bc[i] += W1 (node i+1).  Native 32-bit shared atomics.
-template <typename real>
-__device__ __forceinline__ void deposit(unsigned int* A, unsigned int* Bc, real x) {
-  const real fl = floor(x);
-  const int i = static_cast<int>(fl);
-  const unsigned int w1 = frac_to_fix(x - fl);
-  atomicAdd(&A[i], 65536u - w1);
-  atomicAdd(&Bc[i], w1);
-}
-
 template <typename real>
 __device__ __forceinline__ real nudge_inside(double x, int N) {
   real r = static_cast<real>(x);
