@@ -45,6 +45,7 @@ size_t abs_rec_ens_bytes();
 cudaError_t push_ens_occupancy(int precision, int threads, size_t smem, int* per_sm);
 cudaError_t push_ens_launch(int precision, int threads, int grid, size_t smem, const Bufs* Ball,
                             int E, int n_max, int beam_max, void* abs, int abs_cap, cudaStream_t st);
+cudaError_t compact_ens_configure(int precision);
 cudaError_t compact_ens_launch(int precision, const Bufs* Ball, int E, int grid, cudaStream_t st);
 cudaError_t solve_ens_configure(int precision, bool wide);
 cudaError_t solve_ens_launch(int precision, bool wide, const Bufs* Ball, int n_inst, int ctas, size_t smem,
@@ -397,7 +398,7 @@ int initialize(cp_ctx* c, int mode, double tol) {
   CP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
   if (per_sm < 1) return CP_ERR_ARG;
   c->grid = per_sm * sms;
-  c->compact_grid = 2 * sms;
+  c->compact_grid = 3 * sms;
   c->hp.abs_cap = 4096;
   CP_TRY(alloc(reinterpret_cast<void**>(&c->abs),
                sizeof(cpk::AbsRec) * (c->ens_member ? size_t(1)
@@ -1257,10 +1258,11 @@ int batch_init(cp_batch* b, int mode, double tol) {
     b->any_net = b->any_net || c->net != nullptr;
   }
   CP_CUDA(cpk::solve_ens_configure(b->precision, b->solve_wide));
+  CP_CUDA(cpk::compact_ens_configure(b->precision));
   int sms = 0;
   CP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device));
   b->solve_ctas = cpk::solve_ens_cluster_size(b->n_max, b->E, sms);
-  b->compact_grid = 2 * sms;
+  b->compact_grid = 3 * sms;
   CP_TRY(batch_set_shape(b, 512, 0));
   CP_CUDA(cudaStreamSynchronize(b->stream));
   b->initialized = true;

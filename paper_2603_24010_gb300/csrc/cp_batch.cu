@@ -12,7 +12,7 @@
 //   are handled after the tiles: emitted electrons and beam ions are deposited
 //   with int64 global atomics straight into their instance's grid.
 // k_compact_ens / k_swap_ens: removal of absorbed particles over the same
-//   flat list, then one thread per (instance, species) swaps the buffers.
+//   flat list, then one thread per instance swaps the buffers.
 // The solve of every instance (one CTA each) is k_solve_ens in cp_solve.cu.
 #include <algorithm>
 
@@ -141,7 +141,7 @@ constexpr int ens_min_ctas(int threads, size_t es) { return threads == 256 ? 3 :
 // lane, the beams dealt over all CTAs, in slots that need no counter.
 //
 // 160 gaps of 260 to 3985 cells, 7.0e7 particles: push 231 -> 222 us, step in
-// a graph 268 -> 264.
+// a graph 268 -> 264 (with the removal's interleaving 209 and 242).
 template <typename real, int THREADS>
 __global__ void __launch_bounds__(THREADS, ens_min_ctas(THREADS, sizeof(real)))
 k_push_ens(const Bufs* __restrict__ Ball, int E, int n_max, int beam_chunks,
@@ -472,53 +472,38 @@ k_push_ens(const Bufs* __restrict__ Ball, int E, int n_max, int beam_chunks,
 // Removal of absorbed particles over the flat (instance, species, tile) list
 // ---------------------------------------------------------------------------
 template <typename real>
-__global__ void __launch_bounds__(kThreads) k_compact_ens(const Bufs* __restrict__ Ball, int E) {
+__global__ void __launch_bounds__(kThreads, sizeof(real) == 4 ? 3 : 1) k_compact_ens(const Bufs* __restrict__ Ball, int E) {
   constexpr int TILE = kThreads * kPerThread;
-  __shared__ int off[kEnsMaxEntries + 1];
+  extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int wsum[kThreads / 32];
+  PackShared<real>& sh = *reinterpret_cast<PackShared<real>*>(smem);
+  int* off = reinterpret_cast<int*>(smem + align16(sizeof(PackShared<real>)));
   tile_offsets<kThreads, false>(Ball, E, TILE, off, wsum);
   const long long U = off[3 * E];
-  // tiles are dealt round-robin: unit t -> its (instance, species) by search
-  for (long long t = blockIdx.x; t < U; t += gridDim.x) {
-    int lo = 0, hi = 3 * E;
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if (off[mid] <= t) lo = mid;
-      else hi = mid;
-    }
-    const int inst = lo / 3, s = lo % 3;
-    DevState* S = Ball[inst].S;
-    const real* xs = reinterpret_cast<const real*>(S->xi[s]);
-    const real* us = reinterpret_cast<const real*>(S->u[s]);
-    real* xd = reinterpret_cast<real*>(S->xi_alt[s]);
-    real* ud = reinterpret_cast<real*>(S->u_alt[s]);
-    const uint32_t* is = S->id;
+  // each CTA takes one contiguous share of the tiles
+  const long long u1 = U * (blockIdx.x + 1) / gridDim.x;
+  long long u = U * blockIdx.x / gridDim.x;
+  int j = 0, hi = 3 * E;  // the entry holding tile u: off[j] <= u < off[j+1]
+  while (hi - j > 1) {
+    const int mid = (j + hi) >> 1;
+    if (off[mid] <= u) j = mid;
+    else hi = mid;
+  }
+  for (; u < u1; ++j) {
+    const long long end = min(u1, static_cast<long long>(off[j + 1]));
+    if (end <= u) continue;  // no tiles
+    DevState* S = Ball[j / 3].S;
+    const int s = j % 3;
+    const real* xs = static_cast<const real*>(S->xi[s]);
+    const real* us = static_cast<const real*>(S->u[s]);
+    const uint32_t* is = s == CP_IONS ? S->id : nullptr;
+    real* xd = static_cast<real*>(S->xi_alt[s]);
+    real* ud = static_cast<real*>(S->u_alt[s]);
     uint32_t* id_d = S->id_alt;
-    const int64_t n = S->n_proc[s];
-    const int64_t base = (t - off[lo]) * TILE + static_cast<int64_t>(threadIdx.x) * kPerThread;
-    real xv[4] = {real(-1), real(-1), real(-1), real(-1)}, uv[4] = {0, 0, 0, 0};
-    if (base < n) {
-      load4(xs + base, xv);
-      load4(us + base, uv);
-    }
-    int c = 0;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) c += (xv[q] > real(0)) ? 1 : 0;
-    const int incl = warp_incl_scan(c);
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    unsigned long long wb = 0ULL;
-    if (lane_id() == 31 && total > 0) wb = atomicAdd(&S->compact_n[s], static_cast<unsigned long long>(total));
-    wb = __shfl_sync(0xffffffffu, wb, 31);
-    unsigned long long o = wb + static_cast<unsigned long long>(incl - c);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (xv[q] > real(0)) {
-        xd[o] = xv[q];
-        ud[o] = uv[q];
-        if (s == CP_IONS) id_d[o] = is[base + q];
-        ++o;
-      }
-    }
+    const int64_t n = S->n_proc[s], chunks = off[j + 1] - off[j];
+    for (int64_t t = u - off[j]; t < end - off[j]; ++t)
+      pack_block<real>(sh, xs, us, is, n, chunks, t, xd, ud, id_d, &S->compact_n[s]);
+    u = end;
   }
 }
 
@@ -625,13 +610,26 @@ cudaError_t status_ens_launch(const Bufs* Ball, int E, int* out, cudaStream_t st
   return cudaGetLastError();
 }
 
+static size_t compact_ens_smem(int precision, int E) {
+  return align16(precision == CP_FP32 ? sizeof(PackShared<float>) : sizeof(PackShared<double>)) + sizeof(int) * (3 * E + 1);
+}
+
+// The removal's shared-memory limit: the largest number of instances'.
+cudaError_t compact_ens_configure(int precision) {
+  const void* fn = precision == CP_FP32 ? reinterpret_cast<const void*>(k_compact_ens<float>)
+                                        : reinterpret_cast<const void*>(k_compact_ens<double>);
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(compact_ens_smem(precision, ens_max_instances())));
+}
+
 cudaError_t compact_ens_launch(int precision, const Bufs* Ball, int E, int grid, cudaStream_t st) {
+  const size_t smem = compact_ens_smem(precision, E);
   if (precision == CP_FP32) {
-    k_compact_ens<float><<<grid, kThreads, 0, st>>>(Ball, E);
+    k_compact_ens<float><<<grid, kThreads, smem, st>>>(Ball, E);
     if (cudaGetLastError() != cudaSuccess) return cudaGetLastError();
     k_swap_ens<float><<<(E + 127) / 128, 128, 0, st>>>(Ball, E);
   } else {
-    k_compact_ens<double><<<grid, kThreads, 0, st>>>(Ball, E);
+    k_compact_ens<double><<<grid, kThreads, smem, st>>>(Ball, E);
     if (cudaGetLastError() != cudaSuccess) return cudaGetLastError();
     k_swap_ens<double><<<(E + 127) / 128, 128, 0, st>>>(Ball, E);
   }

@@ -3,17 +3,18 @@
 //
 // k_compact packs the live particles of every species into the spare
 //   buffers every few steps (dead slots are skipped by the push until then).
-#include "cp_common.cuh"
+#include "cp_push.cuh"
 
 namespace cpk {
 // ---------------------------------------------------------------------------
-// Removal of absorbed particles: live slots are packed into the spare buffer
-// (warp-contiguous, order not kept) and the buffers are swapped by the last
-// CTA.  Physics does not depend on particle order.
+// Removal of absorbed particles: live slots are packed into the spare buffers
+// (interleaved, see pack_block) and the buffers are swapped by the last CTA.
+// Physics does not depend on particle order.
 // ---------------------------------------------------------------------------
 template <typename real>
 __global__ void __launch_bounds__(kThreads) k_compact(Bufs B) {
   DevState* S = B.S;
+  __shared__ PackShared<real> sh;
   __shared__ unsigned int s_ticket;
   __shared__ int s_stop;
   if (threadIdx.x == 0) s_stop = (ldcg(&S->status) != 0);
@@ -24,39 +25,9 @@ __global__ void __launch_bounds__(kThreads) k_compact(Bufs B) {
     const real* us = reinterpret_cast<const real*>(S->u[s]);
     real* xd = reinterpret_cast<real*>(S->xi_alt[s]);
     real* ud = reinterpret_cast<real*>(S->u_alt[s]);
-    const uint32_t* is = S->id;
-    uint32_t* id_d = S->id_alt;
-    const int64_t n = S->n_proc[s];
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads * kPerThread;
-    // uniform trip count so that every warp stays converged for the shuffles
-    const int64_t trips = (n + stride - 1) / stride;
-    for (int64_t t = 0; t < trips; ++t) {
-      const int64_t base =
-          t * stride + (static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x) * kPerThread;
-      real xv[4] = {real(-1), real(-1), real(-1), real(-1)}, uv[4] = {0, 0, 0, 0};
-      if (base < n) {
-        load4(xs + base, xv);
-        load4(us + base, uv);
-      }
-      int c = 0;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) c += (xv[q] > real(0)) ? 1 : 0;
-      const int incl = warp_incl_scan(c);
-      const int total = __shfl_sync(0xffffffffu, incl, 31);
-      unsigned long long wb = 0ULL;
-      if (lane_id() == 31 && total > 0) wb = atomicAdd(&S->compact_n[s], static_cast<unsigned long long>(total));
-      wb = __shfl_sync(0xffffffffu, wb, 31);
-      unsigned long long o = wb + static_cast<unsigned long long>(incl - c);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (xv[q] > real(0)) {
-          xd[o] = xv[q];
-          ud[o] = uv[q];
-          if (s == CP_IONS) id_d[o] = is[base + q];
-          ++o;
-        }
-      }
-    }
+    const int64_t n = S->n_proc[s], chunks = pack_chunks(n);
+    for (int64_t t = blockIdx.x; t < chunks; t += gridDim.x)
+      pack_block<real>(sh, xs, us, s == CP_IONS ? S->id : nullptr, n, chunks, t, xd, ud, S->id_alt, &S->compact_n[s]);
   }
   __threadfence();
   __syncthreads();

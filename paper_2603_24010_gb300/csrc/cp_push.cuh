@@ -145,4 +145,107 @@ __device__ __forceinline__ double beam_speed(const DevParams* P, double u) {
   }
 }
 
+// --- removal of absorbed particles ------------------------------------------------
+// A block packs up to 2048 slots of a store at a time into the spare buffers:
+// warp w takes chunk `t` of 128 slots of region w (the store cut in 16 regions of
+// `region` slots), and the live ones leave interleaved, one of each warp in turn.
+//
+// The interleaving is for the pushes that follow.  Ions of one step's beam lie in
+// consecutive slots and, with one energy, in the same one or two cells, where a
+// warp's node-sum atomics go to the same addresses; dealt out, neighbouring lanes
+// hold ions of 16 distant regions.  Impacts spread over the CTAs likewise.  The
+// outputs go through shared memory and leave as whole runs.
+// Bound: the HBM stream.  3.1e7 particles of one beam energy: removal 330 -> 155
+// us, step in a graph 109 -> 98.6; 1.5e7: 148 -> 77, 51.2 -> 47.3; an ensemble of
+// 7.0e7: 530 -> 370, 264 -> 242 (packed warp by warp in place before, with an
+// atomic per warp and four partial stores).
+constexpr int kPackWarps = kThreads / 32;
+constexpr int kPackChunk = 32 * kPerThread;
+template <typename real>
+struct PackShared {
+  static constexpr int kSlots = kThreads * kPerThread;
+  real x[kSlots + kSlots / 32], u[kSlots + kSlots / 32];
+  uint32_t id[kSlots + kSlots / 32];
+  int before[kPackChunk];         // live slots of all warps with a rank below r
+  unsigned int longer[kPackChunk];  // warps with more than r live slots
+  int count[kPackWarps];
+  unsigned long long base;
+};
+
+// slots per region of n, and chunks per region
+__host__ __device__ inline int64_t pack_chunks(int64_t n) {
+  return (n + static_cast<int64_t>(kPackWarps) * kPackChunk - 1) / (static_cast<int64_t>(kPackWarps) * kPackChunk);
+}
+
+template <typename real>
+__device__ __forceinline__ void pack_block(PackShared<real>& sh, const real* __restrict__ xs, const real* __restrict__ us,
+                                           const uint32_t* __restrict__ is, int64_t n, int64_t chunks, int64_t t,
+                                           real* __restrict__ xd, real* __restrict__ ud, uint32_t* __restrict__ id_d,
+                                           unsigned long long* packed) {
+  const int tid = static_cast<int>(threadIdx.x), w = tid >> 5;
+  const int64_t base = (w * chunks + t) * kPackChunk + static_cast<int64_t>(lane_id()) * kPerThread;
+  real xv[kPerThread], uv[kPerThread];
+  uint32_t iv[kPerThread] = {0u, 0u, 0u, 0u};
+#pragma unroll
+  for (int q = 0; q < kPerThread; ++q) {
+    xv[q] = real(-1);
+    uv[q] = real(0);
+  }
+  if (base < n) {
+    load4(xs + base, xv);
+    load4(us + base, uv);
+    if (is) {
+      const uint4 a = __ldcs(reinterpret_cast<const uint4*>(is + base));
+      iv[0] = a.x; iv[1] = a.y; iv[2] = a.z; iv[3] = a.w;
+    }
+  }
+  int c = 0;
+#pragma unroll
+  for (int q = 0; q < kPerThread; ++q) c += (xv[q] > real(0)) ? 1 : 0;
+  const int incl = warp_incl_scan(c);
+  if (lane_id() == 31) sh.count[w] = incl;
+  __syncthreads();  // also: the block before has left the buffers
+  if (tid < kPackChunk) {
+    int b = 0;
+    unsigned int m = 0u;
+#pragma unroll
+    for (int q = 0; q < kPackWarps; ++q) {
+      const int cq = sh.count[q];
+      b += min(cq, tid);
+      m |= (cq > tid ? 1u : 0u) << q;
+    }
+    sh.before[tid] = b;
+    sh.longer[tid] = m;
+  } else if (tid == kThreads - 1) {
+    int total = 0;
+#pragma unroll
+    for (int q = 0; q < kPackWarps; ++q) total += sh.count[q];
+    sh.base = total ? atomicAdd(packed, static_cast<unsigned long long>(total)) : 0ULL;
+  }
+  __syncthreads();
+  int r = incl - c;
+#pragma unroll
+  for (int q = 0; q < kPerThread; ++q) {
+    if (xv[q] > real(0)) {
+      const int o = sh.before[r] + __popc(sh.longer[r] & ((1u << w) - 1u));
+      ++r;
+      const int k = o + (o >> 5);
+      sh.x[k] = xv[q];
+      sh.u[k] = uv[q];
+      if (is) sh.id[k] = iv[q];
+    }
+  }
+  int total = 0;
+#pragma unroll
+  for (int q = 0; q < kPackWarps; ++q) total += sh.count[q];
+  const unsigned long long o0 = sh.base;
+  __syncthreads();
+  for (int o = tid; o < total; o += kThreads) {
+    const int k = o + (o >> 5);
+    xd[o0 + o] = sh.x[k];
+    ud[o0 + o] = sh.u[k];
+    if (is) id_d[o0 + o] = sh.id[k];
+  }
+}
+
 }  // namespace cpk
