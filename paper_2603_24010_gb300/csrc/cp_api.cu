@@ -104,7 +104,7 @@ struct cp_ctx {
   uint32_t* buf_id[2] = {nullptr, nullptr};
   long long* G = nullptr;
   long long* Glast = nullptr;
-  void* Epair = nullptr;
+  void* Etab = nullptr;
   double* phi = nullptr;
   double* E64 = nullptr;
   cpk::AbsRec* abs = nullptr;
@@ -159,6 +159,26 @@ int cuda_rc(cudaError_t e) { return e == cudaSuccess ? CP_OK : CP_ERR_CUDA; }
 #define CP_CUDA(expr) CP_TRY(cuda_rc(expr))
 
 int64_t round4(int64_t n) { return (n + 3) & ~int64_t(3); }
+
+// bytes of a field table: N + 2 values, whole 16-byte vectors
+size_t etab_bytes(const cp_ctx* c) { return (c->es * (c->N + 2) + 15) & ~size_t(15); }
+
+// A saved state holds the field as pairs (E_{k-1/2}, difference to the next);
+// pair 0 repeats E_{1/2} with slope 0, pair N has slope 0.
+template <typename real>
+void pairs_of_table(const unsigned char* tab, int N, unsigned char* pairs) {
+  for (int k = 0; k <= N; ++k) {
+    real e[2];
+    std::memcpy(e, tab + sizeof(real) * k, sizeof(e));
+    const real pr[2] = {e[0], (k == 0) ? real(0) : e[1] - e[0]};
+    std::memcpy(pairs + sizeof(pr) * k, pr, sizeof(pr));
+  }
+}
+
+template <typename real>
+void table_of_pairs(const unsigned char* pairs, int N, unsigned char* tab) {
+  for (int k = 0; k <= N + 1; ++k) std::memcpy(tab + sizeof(real) * k, pairs + 2 * sizeof(real) * std::min(k, N), sizeof(real));
+}
 
 // --- Tesla transformer (Sec. 2.1, App. A): BDF2 of the loop equations ----
 // Matrix of the level-n terms; coupled: loop 4 without its 1/C3 (the load
@@ -255,7 +275,7 @@ cpk::Bufs make_bufs(const cp_ctx* c) {
   B.S = c->dS;
   B.G = c->G;
   B.Glast = c->Glast;
-  B.Epair = c->Epair;
+  B.Etab = c->Etab;
   B.phi = c->phi;
   B.E64 = c->E64;
   B.abs = c->abs;
@@ -289,7 +309,7 @@ void free_all(cp_ctx* c) {
   }
   cudaFree(c->G);
   cudaFree(c->Glast);
-  cudaFree(c->Epair);
+  cudaFree(c->Etab);
   cudaFree(c->phi);
   cudaFree(c->E64);
   cudaFree(c->abs);
@@ -377,14 +397,14 @@ int initialize(cp_ctx* c, int mode, double tol) {
 
   CP_TRY(alloc(reinterpret_cast<void**>(&c->G), sizeof(long long) * (c->N + 1)));
   CP_TRY(alloc(reinterpret_cast<void**>(&c->Glast), sizeof(long long) * (c->N + 1)));
-  CP_TRY(alloc(&c->Epair, 2 * c->es * (c->N + 1)));
+  CP_TRY(alloc(&c->Etab, etab_bytes(c)));
   CP_TRY(alloc(reinterpret_cast<void**>(&c->phi), sizeof(double) * (c->N + 1)));
   CP_TRY(alloc(reinterpret_cast<void**>(&c->E64), sizeof(double) * c->N));
   c->hist_rows = c->max_steps + 1;
   CP_TRY(alloc(reinterpret_cast<void**>(&c->hist), sizeof(cp_diag) * c->hist_rows));
   CP_CUDA(cudaMemsetAsync(c->G, 0, sizeof(long long) * (c->N + 1), c->stream));
   CP_CUDA(cudaMemsetAsync(c->Glast, 0, sizeof(long long) * (c->N + 1), c->stream));
-  CP_CUDA(cudaMemsetAsync(c->Epair, 0, 2 * c->es * (c->N + 1), c->stream));
+  CP_CUDA(cudaMemsetAsync(c->Etab, 0, etab_bytes(c), c->stream));
   CP_CUDA(cudaMemsetAsync(c->hist, 0, sizeof(cp_diag) * c->hist_rows, c->stream));
 
   // launch shape: persistent grid of resident push CTAs, one solve cluster
@@ -1032,12 +1052,17 @@ int cp_save_state(cp_ctx* c, void* buf, size_t* len) {
     CP_TRY(d2h(S.u[s], c->es * h.slots[s]));
   }
   CP_TRY(d2h(S.id, 4 * h.slots[1]));
-  CP_TRY(d2h(c->Epair, 2 * c->es * (c->N + 1)));
+  unsigned char* const pairs = p;  // (E_{k-1/2}, difference to the next), k = 0..N, the ends repeated
+  std::vector<unsigned char> tab(etab_bytes(c));
+  CP_CUDA(cudaMemcpyAsync(tab.data(), c->Etab, tab.size(), cudaMemcpyDeviceToHost, c->stream));
+  p += 2 * c->es * (c->N + 1);
   CP_TRY(d2h(c->phi, sizeof(double) * (c->N + 1)));
   CP_TRY(d2h(c->E64, sizeof(double) * c->N));
   CP_TRY(d2h(c->Glast, sizeof(long long) * (c->N + 1)));
   CP_TRY(d2h(c->hist, sizeof(cp_diag) * h.hist_n));
   CP_CUDA(cudaStreamSynchronize(c->stream));
+  if (c->precision == CP_FP32) pairs_of_table<float>(tab.data(), c->N, pairs);
+  else pairs_of_table<double>(tab.data(), c->N, pairs);
   *len = need;
   return CP_OK;
 }
@@ -1089,7 +1114,11 @@ int cp_load_state(cp_ctx* c, const void* buf, size_t len) {
     CP_TRY(h2d(S.u[s], c->es * h.slots[s]));
   }
   CP_TRY(h2d(S.id, 4 * h.slots[1]));
-  CP_TRY(h2d(c->Epair, 2 * c->es * (c->N + 1)));
+  std::vector<unsigned char> tab(etab_bytes(c), 0);
+  if (c->precision == CP_FP32) table_of_pairs<float>(p, c->N, tab.data());
+  else table_of_pairs<double>(p, c->N, tab.data());
+  CP_CUDA(cudaMemcpyAsync(c->Etab, tab.data(), tab.size(), cudaMemcpyHostToDevice, c->stream));
+  p += 2 * c->es * (c->N + 1);
   CP_TRY(h2d(c->phi, sizeof(double) * (c->N + 1)));
   CP_TRY(h2d(c->E64, sizeof(double) * c->N));
   CP_TRY(h2d(c->Glast, sizeof(long long) * (c->N + 1)));
@@ -1806,14 +1835,14 @@ int g2_init(cp_gap2d* g, int mode, double tol) {
   const int N = c->N;
   CP_TRY(alloc(reinterpret_cast<void**>(&c->G), sizeof(long long) * (N + 1)));
   CP_TRY(alloc(reinterpret_cast<void**>(&c->Glast), sizeof(long long) * (N + 1)));
-  CP_TRY(alloc(&c->Epair, 2 * sizeof(float) * (N + 1)));
+  CP_TRY(alloc(&c->Etab, etab_bytes(c)));
   CP_TRY(alloc(reinterpret_cast<void**>(&c->phi), sizeof(double) * (N + 1)));
   CP_TRY(alloc(reinterpret_cast<void**>(&c->E64), sizeof(double) * N));
   c->hist_rows = c->max_steps + 1;
   CP_TRY(alloc(reinterpret_cast<void**>(&c->hist), sizeof(cp_diag) * c->hist_rows));
   CP_CUDA(cudaMemsetAsync(c->G, 0, sizeof(long long) * (N + 1), c->stream));
   CP_CUDA(cudaMemsetAsync(c->Glast, 0, sizeof(long long) * (N + 1), c->stream));
-  CP_CUDA(cudaMemsetAsync(c->Epair, 0, 2 * sizeof(float) * (N + 1), c->stream));
+  CP_CUDA(cudaMemsetAsync(c->Etab, 0, etab_bytes(c), c->stream));
   CP_CUDA(cudaMemsetAsync(c->hist, 0, sizeof(cp_diag) * c->hist_rows, c->stream));
   c->solve_wide = true;  // the mean's grid counts 2^32 per macroparticle
   CP_CUDA(cpk::solve_configure(c->precision, c->solve_wide));

@@ -146,7 +146,6 @@ template <typename real, int THREADS>
 __global__ void __launch_bounds__(THREADS, ens_min_ctas(THREADS, sizeof(real)))
 k_push_ens(const Bufs* __restrict__ Ball, int E, int n_max, int beam_chunks,
            AbsRecE* __restrict__ abs_all, int abs_cap) {
-  using real2 = typename Pair<real>::type;
   using V = EnsTile<real, THREADS>;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ EnsShared<real, THREADS> sh;
@@ -294,12 +293,8 @@ k_push_ens(const Bufs* __restrict__ Ball, int E, int n_max, int beam_chunks,
         const Bufs& B = Ball[cur];
         N = B.P->N;
         Nr = static_cast<real>(N);
-        const real2* Epair = reinterpret_cast<const real2*>(B.Epair);
-        for (int k = tid; k <= N; k += THREADS) {
-          const real e = __ldcg(&Epair[k]).x;  // pair 0 repeats E_{1/2}
-          Et[k] = e;
-          if (k == N) Et[N + 1] = e;
-        }
+        const real* Etab = static_cast<const real*>(B.Etab);
+        for (int k = tid; k < N + 2; k += THREADS) Et[k] = __ldcg(&Etab[k]);
         __syncthreads();
       }
       const int s = g.s, sign = (s == CP_IONS) ? 1 : -1;

@@ -15,17 +15,6 @@ namespace cpk {
 
 __host__ __device__ constexpr size_t align16(size_t b) { return (b + 15) & ~size_t(15); }
 
-template <typename real>
-struct Pair;
-template <>
-struct Pair<float> {
-  using type = float2;
-};
-template <>
-struct Pair<double> {
-  using type = double2;
-};
-
 // ---------------------------------------------------------------------------
 // 16-byte vector access to 4 consecutive particles (streaming cache hints:
 // the stores are larger than L2 and touched once per step)

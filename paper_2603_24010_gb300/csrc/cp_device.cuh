@@ -11,9 +11,9 @@
 //   G[N+1]        int64 charge grid being deposited for the next level
 //                 (2^16 units per macroparticle charge)
 //   Glast[N+1]    int64 charge grid of the current level (read-back copy)
-//   Epair[N+1]    gather table of the current level in particle precision:
-//                 pair k = (Ep_k, Ep_{k+1} - Ep_k) with Ep_0 = E_{1/2},
-//                 Ep_k = E_{k-1/2} (k = 1..N), Ep_{N+1} = E_{N-1/2}
+//   Etab[N+2]     gather table of the current level in particle precision:
+//                 Etab_0 = E_{1/2}, Etab_k = E_{k-1/2} (k = 1..N), Etab_{N+1} =
+//                 E_{N-1/2}
 //   phi[N+1], E64[N]  FP64 potential and field of the current level
 //   abs[grid*cap] per-CTA lists of ions absorbed in the current push
 //   hist[rows]    one cp_diag row per level
@@ -170,7 +170,7 @@ struct Bufs {
   DevState* S;
   long long* G;
   long long* Glast;
-  void* Epair;
+  void* Etab;
   double* phi;
   double* E64;
   AbsRec* abs;

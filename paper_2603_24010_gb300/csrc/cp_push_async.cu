@@ -181,7 +181,6 @@ struct alignas(128) PushShared {
 template <typename real, bool PUSH, bool LATE>
 __device__ __forceinline__ bool push_cta(const Bufs& B, PushShared<real>& sh, unsigned char* smem, int G) {
   using V = Vec<real>;
-  using real2 = typename Pair<real>::type;
   const DevParams* __restrict__ P = B.P;
   DevState* S = B.S;
   int &s_abs_n = sh.abs_n, &s_over = sh.over;
@@ -327,27 +326,7 @@ __device__ __forceinline__ bool push_cta(const Bufs& B, PushShared<real>& sh, un
       sh.moved = (moved != 0u);
     }
   }
-  // the field table of the solve just finished: eight loads per thread in
-  // flight together (one L2 round trip for N <= 4095)
-  if (PUSH && any) {
-    const real2* Epair = reinterpret_cast<const real2*>(B.Epair);
-    for (int k0 = tid; k0 <= N; k0 += 8 * kThreads) {
-      real e[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int k = k0 + q * kThreads;
-        e[q] = (k <= N) ? __ldcg(&Epair[k]).x : real(0);  // pair 0 repeats E_{1/2}
-      }
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int k = k0 + q * kThreads;
-        if (k <= N) {
-          Et[k] = e[q];
-          if (k == N) Et[N + 1] = e[q];
-        }
-      }
-    }
-  }
+  if (PUSH && any) load_table<real, kThreads>(Et, B.Etab, N);  // of the solve just finished
   __syncthreads();
   if (sh.stop || sh.moved) {
     cp_async_wait<0>();

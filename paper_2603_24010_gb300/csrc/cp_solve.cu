@@ -463,7 +463,7 @@ __device__ __noinline__ int commit_level(DevState* S, cp_diag* hist, int64_t his
 // Everything the refinement needs of the solve (rare path).
 struct Refine {
   double *ph, *Ee, *bb, *rr;
-  double *sc, *wd, *slotd, *edge;  // edge[3]: this rank's first and last potential, first field
+  double *sc, *wd, *slotd, *edge;  // edge[2]: this rank's first and last potential
   unsigned long long (*wu)[32];
   MaxSlot* slot;
   double* s_eta;
@@ -497,10 +497,9 @@ __device__ __forceinline__ double row_residual(const double* ph, double b, int k
 
 // At most three sweeps x -= A^{-1} r in FP64, until the backward error is
 // within tol; all threads of the cluster.  Returns the last backward error;
-// *phi0 and *nextE are the refined potential of node 0 and the next chunk's
-// first field.
+// *phi0 is the refined potential of node 0.
 __device__ __noinline__ double refine(const Refine& R, const DevParams* P, double prev_phi, double next_phi,
-                                      double* phi0, double* nextE) {
+                                      double* phi0) {
   cg::cluster_group cl = cg::this_cluster();
   const int rank = static_cast<int>(cl.block_rank()), nr = static_cast<int>(cl.num_blocks());
   const int m = R.m, lo = R.lo, hi = R.hi, N = R.N;
@@ -525,10 +524,6 @@ __device__ __noinline__ double refine(const Refine& R, const DevParams* P, doubl
     *phi0 = cl.map_shared_rank(R.edge, 0)[0];
     for (int k = threadIdx.x; k < m; k += kSolveThreads)
       R.Ee[k] = (R.ph[k] - ((k + 1 < m) ? R.ph[k + 1] : next_phi)) * R.inv_dx;
-    __syncthreads();
-    if (threadIdx.x == 0 && m > 0) R.edge[2] = R.Ee[0];
-    cl.sync();
-    *nextE = (hi < N) ? cl.map_shared_rank(R.edge, rank + 1)[2] : 0.0;
     // backward error over the cluster
     unsigned long long rm = 0ULL, xm = 0ULL, bm = 0ULL;
     for (int k = threadIdx.x; k < m; k += kSolveThreads) {
@@ -576,7 +571,6 @@ __device__ __noinline__ double refine(const Refine& R, const DevParams* P, doubl
 
 template <typename real, typename Acc>
 __device__ __forceinline__ void solve_body(const Bufs& B, int do_push, int mode, double tol) {
-  using real2 = typename Pair<real>::type;
   cg::cluster_group cl = cg::this_cluster();
   const int rank = static_cast<int>(cl.block_rank());
   const int nr = static_cast<int>(cl.num_blocks());
@@ -593,7 +587,7 @@ __device__ __forceinline__ void solve_body(const Bufs& B, int do_push, int mode,
   __shared__ unsigned long long wu[3][32];
   __shared__ double wd[32];
   __shared__ double sc[48];
-  __shared__ double s_edge[3];
+  __shared__ double s_edge[2];
   __shared__ double slotd, s_eta;
 
   const int tid = static_cast<int>(threadIdx.x), lane = tid & 31, warp = tid >> 5;
@@ -637,12 +631,11 @@ __device__ __forceinline__ void solve_body(const Bufs& B, int do_push, int mode,
   cudaGridDependencySynchronize();  // the push that deposited G has completed
   cudaTriggerProgrammaticLaunchCompletion();
   const int stop = ldcg(&S->status);
-  long long G0 = 0, Gnext = 0;
+  long long G0 = 0;
   if (warp < kRowWarps) {
     for (int k = tid; k < m; k += kRowThreads) Gv[k] = ldcg(&B.G[lo + k]);
   } else if (warp == kCircuitWarp) {
     G0 = ldcg(&B.G[0]);
-    if (hi < N) Gnext = ldcg(&B.G[hi]);
     const unsigned long long* src = reinterpret_cast<const unsigned long long*>(S);
     for (int k = lane; k < kStateWords; k += 32) s_st[kStateWord0 + k] = ldcg(&src[kStateWord0 + k]);
     __syncwarp();
@@ -880,7 +873,7 @@ __device__ __forceinline__ void solve_body(const Bufs& B, int do_push, int mode,
   } else if (warp == kCircuitWarp) {
     // The neighbouring chunks' edge values follow from the exact prefixes with
     // the same arithmetic their owners use, so no exchange is needed:
-    // x_{lo-1} needs P_{lo-1} = P_lo - S'_{lo-1}; x_hi needs P_hi; E_hi needs S'_hi.
+    // x_{lo-1} needs P_{lo-1} = P_lo - S'_{lo-1}; x_hi needs P_hi.
     Seg<Acc> no;  // everything up to and including this rank's rows
     if (lane == rank) slotA[rank] = mine;
     __syncwarp();
@@ -889,20 +882,17 @@ __device__ __forceinline__ void solve_body(const Bufs& B, int do_push, int mode,
     const int i = (lane == 0) ? lo - 1 : (lane == 1) ? hi : 0;  // lanes 0-2: x_{lo-1}, x_hi, x_0
     const Acc Pi = (lane == 0) ? ro.s2 - static_cast<Acc>(ro.s1) : (lane == 1) ? no.s2 : Acc(0);
     const double x = fma(static_cast<double>(N - i), D0, alpha * acc_to_double(U - Pi));
-    const double e = fma(Ea, static_cast<double>(no.s1 + Gnext), E0);
     if (lane == 0) sc[26] = (lo > 0) ? x : 0.0;
     if (lane == 1) sc[27] = (hi < N) ? x : 0.0;
-    if (lane == 1) sc[28] = (hi < N) ? e : 0.0;
     if (lane == 2) sc[29] = x;
   }
   __syncthreads();
   const double prev_phi = sc[26], next_phi = sc[27], phi0 = sc[29];
-  double nextE = sc[28];
   double phi0_fin = phi0;
   int status = 0;  // of the committed values (commit warp of rank 0)
-  real2* Epair = reinterpret_cast<real2*>(B.Epair);
+  real* Etab = static_cast<real*>(B.Etab);
   if (warp < kRowWarps) {
-    // outputs; the gather table pairs need the next row's field value
+    // outputs
     unsigned long long rm = 0ULL, xm = 0ULL;
     for (int k = tid; k < m; k += kRowThreads) {
       const int i = lo + k;
@@ -913,15 +903,9 @@ __device__ __forceinline__ void solve_body(const Bufs& B, int do_push, int mode,
       B.E64[i] = Ee[k];
       B.phi[i] = x;
       const real e0 = ef[k];
-      const real e1 = (i + 1 < N) ? ((k + 1 < m) ? ef[k + 1] : static_cast<real>(nextE)) : e0;
-      real2 pr;
-      pr.x = e0;
-      pr.y = e1 - e0;
-      Epair[i + 1] = pr;
-      if (i == 0) {
-        pr.y = real(0);
-        Epair[0] = pr;
-      }
+      Etab[i + 1] = e0;
+      if (i == 0) Etab[0] = e0;
+      if (i == N - 1) Etab[N + 1] = e0;
     }
     rm = warp_max_u64(rm);
     xm = warp_max_u64(xm);
@@ -973,21 +957,15 @@ __device__ __forceinline__ void solve_body(const Bufs& B, int do_push, int mode,
     R.lo = lo; R.hi = hi; R.m = m; R.N = N;
     R.gam = gam; R.inv_dx = inv_dx; R.tol = tol;
     R.strict_rlc = strict_rlc;
-    eta = refine(R, P, prev_phi, next_phi, &phi0_fin, &nextE);
+    eta = refine(R, P, prev_phi, next_phi, &phi0_fin);
     for (int k = tid; k < m; k += kSolveThreads) {
       const int i = lo + k;
       B.E64[i] = Ee[k];
       B.phi[i] = ph[k];
       const real e0 = static_cast<real>(Ee[k]);
-      const real e1 = (i + 1 < N) ? static_cast<real>((k + 1 < m) ? Ee[k + 1] : nextE) : e0;
-      real2 pr;
-      pr.x = e0;
-      pr.y = e1 - e0;
-      Epair[i + 1] = pr;
-      if (i == 0) {
-        pr.y = real(0);
-        Epair[0] = pr;
-      }
+      Etab[i + 1] = e0;
+      if (i == 0) Etab[0] = e0;
+      if (i == N - 1) Etab[N + 1] = e0;
     }
     if (rank == 0 && warp == kCommitWarp)
       status = commit_level(S, B.hist, B.hist_rows, B.vs, P, st, sc, do_push, mode, strict_c, phi0_fin, eta);
