@@ -61,9 +61,9 @@ def workload(name, seed, pairs=None):
     return cfg
 
 
-PUSH_PROFILE = os.path.join(ROOT, "profiles", "k_push_async_gap_1d_fp32_large.md")
+PUSH_PROFILE = os.path.join(ROOT, "profiles", "k_push_gap_1d_fp32_large.md")
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_2603_24010_gb300", "csrc", f)
-                  for f in ("cp_push_async.cu", "cp_push.cu", "cp_common.cuh", "cp_device.cuh")]
+                  for f in ("cp_push_async.cu", "cp_push.cuh", "cp_push.cu", "cp_common.cuh", "cp_device.cuh")]
 
 
 def kernel_source_hash():

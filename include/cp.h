@@ -321,7 +321,7 @@ int cp_read_launch_times(cp_ctx* ctx, double* ms, int64_t cap, int64_t* n);
    electrons written (at most se_cap), and the convection count at x = 0.  The first call on a device looks up the
    scratch array's address; make that first call before any stream capture.
    The call synchronises `stream`.  Every call shares the one scratch array:
-   calls that overlap on the GPU (other streams, other host threads) race.
+   calls from several host threads take turns.
    Errors: CP_ERR_ARG (null buffer, n_cells outside 2..4096, bad sizes, a
    SEE law cp_create would refuse: gamma_max outside 0..14, a negative or
    non-finite scale, gamma_coef, E_ref_eV or T_emit_eV; a count or energy

@@ -46,8 +46,8 @@
 //
 // Graph-timed step before -> after (GB300): FP64, 256 cells, 1.4e5 particles
 // 38.6 -> 18.3 us; FP64 Tesla gap 40.9 -> 21.8; FP32, 4096 cells, 3.3e5
-// particles 22.9 -> 16.7, 1e6 (1531 cells) 17.5 -> 15.1, 1.5e7 59.3 -> 47.3,
-// 3.1e7 (impacts every step) 118 -> 98.6.
+// particles 22.9 -> 16.3, 1e6 (1531 cells) 17.5 -> 14.8, 1.5e7 59.3 -> 46.6,
+// 3.1e7 (impacts every step) 118 -> 98.3.
 
 #include <cstddef>
 
