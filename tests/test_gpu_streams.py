@@ -67,3 +67,52 @@ def test_threads_on_their_own_streams(env, calls):
             np.testing.assert_array_equal(got[k], h[k], err_msg=k)
         np.testing.assert_array_equal(g.grid()["G"], G)
         g.close()
+
+
+def make_any(native, what, stream):
+    if what == "2d":
+        cfg = W.scaled(W.gap_2d(4, 128, 128, 150_000, beam_per_step=400), see_scale=8.0)
+        g = native.Gap2D(cfg, max_steps=200, stream=stream)
+        xi, eta, ue, we, ui, wi = W.load_pairs_2d(cfg)
+        g.set_particles(native.ELECTRONS, xi, eta, ue, we)
+        g.set_particles(native.IONS, xi, eta, ui, wi)
+        return g
+    if what == "ensemble":
+        cfgs = W.ensemble(24, seed=3, steps=200, thin=20, n_cells_max=2048)
+        b = native.Batch(cfgs, max_steps=200, stream=stream)
+        for i, cfg in enumerate(cfgs):
+            xi, ue, ui = W.load_pairs(cfg)
+            b.set_particles(i, native.ELECTRONS, xi, ue)
+            b.set_particles(i, native.IONS, xi, ui)
+        return b
+    return make(native, configs()[0], stream)
+
+
+def outcome(what, g):
+    if what == "2d":
+        return [g.history()["V_gap"], g.history()["n_live"], g.fields()["G"]]
+    if what == "ensemble":
+        return [x for i in range(0, 24, 5) for x in (g.history(i)["V_gap"], g.history(i)["n_live"], g.grid(i)["G"])]
+    return [g.history()["V_gap"], g.history()["n_live"], g.grid()["G"]]
+
+
+def test_all_paths_beside_one_another(env):
+    torch, native = env
+    paths = ["2d", "ensemble", "1d", "2d"]
+    want = {}
+    for what in set(paths):
+        g = make_any(native, what, None)
+        advance(native, g, [130, 1, 1, 60])
+        want[what] = outcome(what, g)
+        g.close()
+    streams = [torch.cuda.Stream() for _ in paths]
+    gaps = [make_any(native, what, st.cuda_stream) for what, st in zip(paths, streams)]
+    ts = [threading.Thread(target=advance, args=(native, g, [130, 1, 1, 60])) for g in gaps]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    for what, g in zip(paths, gaps):
+        for a, b in zip(outcome(what, g), want[what]):
+            np.testing.assert_array_equal(a, b, err_msg=what)
+        g.close()
