@@ -29,8 +29,8 @@ int solve_ens_cluster_size(int n_max, int E, int sms);
 cudaError_t push_configure(int precision);
 cudaError_t solve_configure(int precision, bool wide);
 cudaError_t push_occupancy(int precision, size_t smem, int* blocks_per_sm);
-cudaError_t push_launch(int precision, const Bufs& B, int grid, size_t smem, cudaStream_t st,
-                        int do_push);
+cudaError_t push_launch(int precision, const Bufs& B, int grid, size_t smem, cudaStream_t st, int do_push,
+                        bool behind_solve);
 cudaError_t solve_launch(int precision, bool wide, const Bufs& B, int ctas, size_t smem, cudaStream_t st,
                          int do_push, int mode, double tol);
 cudaError_t compact_launch(int precision, const Bufs& B, int grid, cudaStream_t st);
@@ -458,7 +458,7 @@ int initialize(cp_ctx* c, int mode, double tol) {
   c->initialized = true;
   // deposit rho^0 and solve level 0
   const cpk::Bufs B0 = make_bufs(c);
-  CP_CUDA(cpk::push_launch(c->precision, B0, c->grid, c->smem, c->stream, 0));
+  CP_CUDA(cpk::push_launch(c->precision, B0, c->grid, c->smem, c->stream, 0, false));
   CP_CUDA(solve(c, B0, c->stream, 0, mode, tol));
   c->launches += 2;
   return CP_OK;
@@ -543,7 +543,7 @@ int build_graph(cp_ctx* c, int mode, double tol) {
   CP_CUDA(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
   cudaError_t e = cudaSuccess;
   for (int k = 0; k < c->compact_every && e == cudaSuccess; ++k) {
-    e = cpk::push_launch(c->precision, B, c->grid, c->smem, c->cap_stream, 1);
+    e = cpk::push_launch(c->precision, B, c->grid, c->smem, c->cap_stream, 1, k > 0);
     if (e == cudaSuccess) e = solve(c, B, c->cap_stream, 1, mode, tol);
   }
   if (e == cudaSuccess) e = cpk::compact_launch(c->precision, B, c->compact_grid, c->cap_stream);
@@ -570,7 +570,7 @@ int timed_launch(cp_ctx* c, int which, int mode, double tol, std::vector<std::pa
   CP_CUDA(cudaEventRecord(c->ev_pool[k], c->stream));
   const cpk::Bufs B = make_bufs(c);
   if (which == 0)
-    CP_CUDA(cpk::push_launch(c->precision, B, c->grid, c->smem, c->stream, 1));
+    CP_CUDA(cpk::push_launch(c->precision, B, c->grid, c->smem, c->stream, 1, c->since_compact > 0));
   else if (which == 1)
     CP_CUDA(solve(c, B, c->stream, 1, mode, tol));
   else
@@ -627,7 +627,7 @@ int do_steps(cp_ctx* c, int mode, int32_t n_steps, double tol) {
       left -= c->compact_every;
       continue;
     }
-    CP_CUDA(cpk::push_launch(c->precision, B, c->grid, c->smem, c->stream, 1));
+    CP_CUDA(cpk::push_launch(c->precision, B, c->grid, c->smem, c->stream, 1, c->since_compact > 0));
     CP_CUDA(solve(c, B, c->stream, 1, mode, tol));
     c->launches += 2;
     --left;

@@ -20,7 +20,8 @@
 //   their way while one is processed, without registers held for them and
 //   without block-wide waits.  The first tiles are requested before the wait
 //   (the solve changes no particle but the up to three padding slots behind
-//   a species' last one, and the last vector is read directly);
+//   a species' last one, and the last vector is read directly; a push behind
+//   anything else than a solve starts when that has completed, push_launch);
 // * the beam ions are drawn before the wait (their draws need the level
 //   alone, which the previous push left in B.next_step);
 // * one flat list of tiles over the three species, so that small species
@@ -653,8 +654,14 @@ cudaError_t push_occupancy(int precision, size_t smem, int* blocks_per_sm) {
 
 // Push and solve are launched with programmatic dependent launch: each may
 // be scheduled while its predecessor finishes and waits in
-// cudaGridDependencySynchronize() until that grid has completed.
-cudaError_t push_launch(int precision, const Bufs& B, int grid, size_t smem, cudaStream_t st, int do_push) {
+// cudaGridDependencySynchronize() until that grid has completed.  A push reads
+// particles, store pointers and slot counts ahead of that wait, which is sound
+// behind a solve alone: the solve let it start only after its own wait for the
+// push that wrote them.  behind_solve = false (behind a removal, a graph or
+// nothing) leaves the attribute out, and the push starts when everything
+// before it has completed.
+cudaError_t push_launch(int precision, const Bufs& B, int grid, size_t smem, cudaStream_t st, int do_push,
+                        bool behind_solve) {
   cudaLaunchConfig_t cfg = {};
   // one CTA more runs the learned predictor when the push carries it
   cfg.gridDim = dim3(grid + ((B.net != nullptr && B.net_in_push) ? 1 : 0), 1, 1);
@@ -665,7 +672,7 @@ cudaError_t push_launch(int precision, const Bufs& B, int grid, size_t smem, cud
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = behind_solve ? 1 : 0;
   void* args[] = {const_cast<Bufs*>(&B)};
   return cudaLaunchKernelExC(&cfg, push_fn(precision, do_push), args);
 }
