@@ -1747,7 +1747,9 @@ int g2_push(cp_gap2d* g, cudaStream_t st) {
   return CP_OK;
 }
 
-// Capture sort_every steps and the re-sort that follows them.
+// Capture sort_every steps.  (The re-sort is not among them: its padding may
+// need more slots than the particles do, and then only a step that follows is
+// refused.)
 int g2_build_graph(cp_gap2d* g, int mode, double tol) {
   cp_ctx* c = g->c;
   if (c->gexec[mode] && c->gtol[mode] == tol) return CP_OK;
@@ -1768,7 +1770,6 @@ int g2_build_graph(cp_gap2d* g, int mode, double tol) {
     rc = g2_push(g, c->cap_stream);
     if (rc == CP_OK) rc = g2_solve(g, c->cap_stream, true, 1, mode, tol);
   }
-  if (rc == CP_OK) rc = g2_sort(g, c->cap_stream);
   const cudaError_t e = cudaStreamEndCapture(c->cap_stream, &gr);
   g->launches = launches;
   if (rc != CP_OK || e != cudaSuccess) {
@@ -2002,7 +2003,8 @@ int g2_steps(cp_gap2d* g, int mode, int32_t n_steps, double tol) {
     if (!g->timing && g->since_sort == 0 && n_steps - k >= g->sort_every) {
       CP_TRY(g2_build_graph(g, mode, tol));
       CP_CUDA(cudaGraphLaunch(c->gexec[mode], c->stream));
-      g->launches += 5 * g->sort_every + 5;
+      g->launches += 5 * g->sort_every;
+      g->since_sort = g->sort_every;
       k += g->sort_every;
       continue;
     }
