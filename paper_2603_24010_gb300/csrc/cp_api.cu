@@ -1747,7 +1747,13 @@ int g2_push(cp_gap2d* g, cudaStream_t st) {
   return CP_OK;
 }
 
-// Capture sort_every steps.  (The re-sort is not among them: its padding may
+// Steps of a graph: sort_every, at most 16, so that its memory and the time to
+// capture it stay small whatever the sort's period (32 x 32 cells, a period of
+// 20000: one graph of them all took 0.8 GB of host and 0.2 GB of device memory
+// and the first call 50.1 us a step; 16 a graph 30.7, as every later call).
+int g2_graph_steps(const cp_gap2d* g) { return std::min(g->sort_every, 16); }
+
+// Capture a graph of steps.  (The re-sort is not among them: its padding may
 // need more slots than the particles do, and then only a step that follows is
 // refused.)
 int g2_build_graph(cp_gap2d* g, int mode, double tol) {
@@ -1766,7 +1772,7 @@ int g2_build_graph(cp_gap2d* g, int mode, double tol) {
   cudaGraph_t gr = nullptr;
   CP_CUDA(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
   int rc = CP_OK;
-  for (int k = 0; k < g->sort_every && rc == CP_OK; ++k) {
+  for (int k = 0; k < g2_graph_steps(g) && rc == CP_OK; ++k) {
     rc = g2_push(g, c->cap_stream);
     if (rc == CP_OK) rc = g2_solve(g, c->cap_stream, true, 1, mode, tol);
   }
@@ -2000,12 +2006,13 @@ int g2_steps(cp_gap2d* g, int mode, int32_t n_steps, double tol) {
       if (g->timing) CP_TRY(mark_end());
       g->since_sort = 0;
     }
-    if (!g->timing && g->since_sort == 0 && n_steps - k >= g->sort_every) {
+    const int whole = g2_graph_steps(g);
+    if (!g->timing && std::min(n_steps - k, g->sort_every - g->since_sort) >= whole) {
       CP_TRY(g2_build_graph(g, mode, tol));
       CP_CUDA(cudaGraphLaunch(c->gexec[mode], c->stream));
-      g->launches += 5 * g->sort_every;
-      g->since_sort = g->sort_every;
-      k += g->sort_every;
+      g->launches += 5 * whole;
+      g->since_sort += whole;
+      k += whole;
       continue;
     }
     if (g->timing) CP_TRY(g2_timed(g, 0, &rec));

@@ -47,3 +47,46 @@ def test_a_call_that_ends_at_a_resort_keeps_its_particles(native):
         g.step(native.WEAK, 1)
     assert e.value.status == native.ERR_CAPACITY
     g.close()
+
+
+@pytest.mark.parametrize("sort_every", [5, 16, 17, 40, 1000])
+def test_any_period_gives_the_same_steps(native, sort_every):
+    """Graphs, single steps and re-sorts in every mixture against one step a call."""
+    cfg = W.gap_2d(3, Nx=64, Ny=64, n_pairs=20_000, steps=80, beam_per_step=32)
+    p = W.load_pairs_2d(cfg)
+
+    def run(calls, every):
+        g = native.Gap2D(cfg, max_steps=80, sort_every=every)
+        g.set_particles(native.ELECTRONS, *p[:4])
+        g.set_particles(native.IONS, p[0], p[1], p[4], p[5])
+        for n in calls:
+            g.step(native.WEAK, n)
+        h, G = g.history(), g.fields()["G"]
+        g.close()
+        return h, G
+
+    want, G0 = run([1] * 80, 16)
+    for calls in ([80], [7, 33, 40], [20, 60]):
+        h, G = run(calls, sort_every)
+        for k in ("absorbed", "emitted", "injected", "n_live", "conv_count", "V_gap"):
+            np.testing.assert_array_equal(h[k], want[k], err_msg=k)
+        np.testing.assert_array_equal(G, G0)
+
+
+def test_a_long_period_makes_no_long_graph(native):
+    """The device memory of a call's graph does not grow with the period."""
+    import torch
+    steps = 20_000
+    cfg = W.gap_2d(0, Nx=32, Ny=32, n_pairs=100, steps=steps, beam_per_step=0)
+    p = W.load_pairs_2d(cfg)
+    g = native.Gap2D(cfg, max_steps=steps, sort_every=steps)
+    g.set_particles(native.ELECTRONS, *p[:4])
+    g.set_particles(native.IONS, p[0], p[1], p[4], p[5])
+    g.step(native.WEAK, 0)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    g.step(native.WEAK, steps)
+    # a graph of 16 steps takes 2 MB, one of 20000 takes 200
+    assert free - torch.cuda.mem_get_info()[0] < 32 << 20
+    assert g.level == steps
+    g.close()
