@@ -305,10 +305,8 @@ int cp_read_launch_times(cp_ctx* ctx, double* ms, int64_t cap, int64_t* n);
 /* Allocation-free push of one FP32 ion population through one step (the
    paper has no counterpart; this serves callers that cannot call cudaMalloc,
    e.g. a step inside a real-time loop or a process that must not grow
-   device memory after start-up).  It needs no context: every input and
-   output is a caller-owned device buffer, and the scratch it needs (the
-   list of ions absorbed in the push) is a static device array of 8 MiB that
-   every GPU loading this library holds until the process exits.
+   device memory after start-up).  It needs no context and no device memory
+   but the caller's: every input and output is a caller-owned device buffer.
    Computes what one cp_step call does for ions alone: gather of the field E
    (N FP64 edge values E_{k+1/2}, device), kick (half kick if half_kick != 0)
    and drift of xi/u (device, FP32 cell units, updated in place; absorbed
@@ -318,15 +316,15 @@ int cp_read_launch_times(cp_ctx* ctx, double* ms, int64_t cap, int64_t* n);
    macroparticle).  Emitted electrons are written to se_xi/se_u (device,
    capacity se_cap).  counts (device, 6 int64, written on the device): ions
    absorbed at x = 0 and x = d, electrons emitted at x = 0 and x = d,
-   electrons written (at most se_cap), and the convection count at x = 0.  The first call on a device looks up the
-   scratch array's address; make that first call before any stream capture.
-   The call synchronises `stream`.  Every call shares the one scratch array:
-   calls from several host threads take turns.
+   electrons written (at most se_cap), and the convection count at x = 0.
+   The first call on a device sets up the kernel; make that first call before
+   any stream capture.  The call synchronises `stream` and waits for nothing
+   else: calls from several host threads on several streams are independent.
    Errors: CP_ERR_ARG (null buffer, n_cells outside 2..4096, bad sizes, a
    SEE law cp_create would refuse: gamma_max outside 0..14, a negative or
    non-finite scale, gamma_coef, E_ref_eV or T_emit_eV; a count or energy
    law other than floor + Bernoulli and the half-Maxwellian),
-   CP_ERR_CAPACITY (n > 524288 ions, the scratch's limit; or more emitted
+   CP_ERR_CAPACITY (n > 524288 ions; or more emitted
    electrons than se_cap), CP_ERR_CUDA. */
 int cp_push_ions_noalloc(const cp_gap* gap, const cp_see_beam* see, double dt, uint64_t seed,
                          int64_t step, int32_t half_kick, const double* E, float* xi, float* u,

@@ -5,10 +5,11 @@
 // memory after start-up, or code that runs while another component owns the
 // allocator.  For them cp_push_ions_noalloc pushes one FP32 ion population
 // through one step (gather, kick, drift, absorption, ion-induced secondary
-// emission, deposit) using only buffers the caller passes in.  The scratch
-// it needs -- the list of ions absorbed in the push, which the context path
-// keeps in memory it allocates -- lives in the file-scope array below, which
-// every GPU that loads this library holds until the process exits.
+// emission, deposit) using only buffers the caller passes in.  What the
+// context path keeps in memory of its own stays in those too: the impacts of
+// a CTA are listed in its shared memory, their velocities in the ions' u
+// until their electrons are drawn, and the tallies are the caller's counts.
+// So calls share nothing: each waits for its own stream alone.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -20,7 +21,6 @@
 
 namespace cpk_na {
 
-using cpk::AbsRec;
 using cpk::floor_split;
 using cpk::frac16;
 using cpk::kTagSee;
@@ -30,20 +30,13 @@ using cpk::U64x4;
 
 constexpr int kThreads = 1024;
 constexpr int kMaxCells = 4096;          // shared-memory grid limit
-constexpr int64_t kMaxIons = 1 << 19;    // absorbed-ion records the scratch can hold
-constexpr int kCounters = 16;            // tallies, see the enum
+constexpr int64_t kMaxIons = 1 << 19;    // ions of one call
+constexpr int kMostCta = 8191;           // ions of one CTA (13-bit places in its list of impacts)
 constexpr int kAhead = 4;                // ions per thread requested together
 
-// Scratch: counters, then one record per ion that may be absorbed (8 MiB + 128 B).
-struct Scratch {
-  unsigned long long counters[kCounters];
-  AbsRec rec[kMaxIons];
-};
-static __device__ __align__(256) Scratch g_scratch;
-
-// Tally slots in Scratch::counters; all but the status are zero between calls
-enum { kSeCount = 0, kOverflow = 1, kAbs0 = 2, kAbs1 = 3, kEmit0 = 4, kEmit1 = 5, kDone = 6,
-       kStatus = kCounters - 1 };
+// The caller's six counts while the kernel runs: the first four as they are
+// returned, then the electrons asked for so far and the CTAs that are done.
+enum { kAbs0 = 0, kAbs1 = 1, kEmit0 = 2, kEmit1 = 3, kSeCount = 4, kDone = 5, kCounts = 6 };
 
 struct Params {
   int N;
@@ -63,33 +56,39 @@ __device__ __forceinline__ void add_node(long long* G, int N, int k, long long v
   atomicAdd(reinterpret_cast<unsigned long long*>(&G[k]), static_cast<unsigned long long>(v));
 }
 
-// The whole call in one kernel, one CTA per SM at most: each CTA pushes a
-// contiguous range of the ions (gather, kick, drift, absorption, deposit into
-// 32-bit node sums), then turns the ions it saw absorbed into electrons (the
-// context path's arithmetic and draws), and the last CTA out writes the counts
-// and clears the tallies for the next call.
+// The grid and the counts start at zero.
+__global__ void __launch_bounds__(256) k_clear(long long* __restrict__ G, int nodes, unsigned long long* __restrict__ counts) {
+  const int k = blockIdx.x * 256 + threadIdx.x;
+  if (k < nodes) G[k] = 0;
+  if (k < kCounts) counts[k] = 0ULL;
+}
+
+// The whole call in one kernel (and a clear), one CTA per SM at most: each CTA
+// pushes a contiguous range of the ions (gather, kick, drift, absorption,
+// deposit into 32-bit node sums), then turns the ions it saw absorbed into
+// electrons (the context path's arithmetic and draws), and the last CTA out
+// completes the counts.
 //
 // Bound: latency (a call moves 12 MB at most): the ions are requested before
 // the field table is formed, and one table per SM is formed at all because the
 // conversion from FP64 runs at two values a cycle.  Call at 524288 ions and 4096
-// cells: 52.9 -> 39.0 us, with the host's wait for the status (three kernels,
-// two memsets and 64-bit shared atomics before).
+// cells: 52.9 -> 39.6 us, with the host's wait for the counts (three kernels,
+// two memsets and 64-bit shared atomics before; 39.0 with a list of impacts in
+// memory that all calls share and take turns for).
 // counts: [0] absorbed at x = 0, [1] at x = d, [2] emitted at x = 0, [3] at x =
-// d, [4] electrons written (at most se_cap), [5] convection count at x = 0;
-// status 1 when emitted electrons did not fit in se_cap.
+// d, [4] electrons written (at most se_cap), [5] convection count at x = 0.
 __global__ void __launch_bounds__(kThreads, 1)
-k_push_ions(Params p, Scratch* sc, const double* __restrict__ E, float* __restrict__ xi, float* __restrict__ u,
+k_push_ions(Params p, const double* __restrict__ E, float* __restrict__ xi, float* __restrict__ u,
             const uint32_t* __restrict__ id, int64_t n, long long* __restrict__ G, float* __restrict__ se_xi,
-            float* __restrict__ se_u, int64_t se_cap, int64_t* __restrict__ counts) {
+            float* __restrict__ se_u, int64_t se_cap, unsigned long long* __restrict__ counts) {
   extern __shared__ unsigned int smem_na[];
   __shared__ unsigned int s_abs_n, s_abs[2], s_emit[2], s_round[2];
-  __shared__ int s_over;
   const int N = p.N, tid = static_cast<int>(threadIdx.x);
   unsigned int* nd = smem_na;                                 // the ions' node sums (at most 2^13 ions a CTA)
   unsigned int* ne = nd + (N + 1);                            // a round's electrons'
   float* tab = reinterpret_cast<float*>(ne + (N + 1));        // E_{k-1/2}, ends repeated
   const int64_t lo = n * blockIdx.x / gridDim.x, hi = n * (blockIdx.x + 1) / gridDim.x;
-  AbsRec* rec = sc->rec + lo;                                 // this CTA's impacts
+  uint16_t* hit = reinterpret_cast<uint16_t*>(tab + (N + 2));  // this CTA's impacts: place from lo on | electrode << 13
   float x[kAhead], v[kAhead];
   auto fetch = [&](int64_t k0) {
 #pragma unroll
@@ -106,7 +105,6 @@ k_push_ions(Params p, Scratch* sc, const double* __restrict__ E, float* __restri
   }
   if (tid == 0) {
     s_abs_n = 0u;
-    s_over = 0;
     s_abs[0] = s_abs[1] = s_emit[0] = s_emit[1] = 0u;
   }
   __syncthreads();
@@ -125,13 +123,9 @@ k_push_ions(Params p, Scratch* sc, const double* __restrict__ E, float* __restri
       if (!(xn > 0.f && xn < Nr)) {
         const int el = (xn <= 0.f) ? 0 : 1;
         atomicAdd(&s_abs[el], 1u);
-        AbsRec r;
-        r.id = id[k];
-        r.electrode = static_cast<uint32_t>(el);
-        r.u = static_cast<double>(un);
-        rec[atomicAdd(&s_abs_n, 1u)] = r;  // below hi - lo: every ion fits
+        hit[atomicAdd(&s_abs_n, 1u)] = static_cast<uint16_t>(static_cast<int>(k - lo) | el << 13);  // every ion fits
         xi[k] = -1.f;
-        u[k] = 0.f;
+        u[k] = un;  // until its electrons are drawn
       } else {
         xi[k] = xn;
         u[k] = un;
@@ -153,44 +147,48 @@ k_push_ions(Params p, Scratch* sc, const double* __restrict__ E, float* __restri
   for (int r0 = 0; r0 < na; r0 += kThreads) {
     const bool act = r0 + tid < na;
     int nse = 0;
-    AbsRec q;
-    q.id = 0; q.electrode = 0; q.u = 0.0;
+    uint32_t ion = 0;
+    int el = 0;
     unsigned int* const electrons = &s_round[r0 / kThreads & 1];
     if (tid == 0) *electrons = 0u;
     __syncthreads();
     if (act) {
-      q = rec[r0 + tid];
-      const double vi = __ddiv_rn(__dmul_rn(q.u, p.dx), p.dt);
+      const int h = hit[r0 + tid];
+      const int64_t k = lo + (h & 0x1FFF);
+      el = h >> 13;
+      ion = id[k];
+      const double vi = __ddiv_rn(__dmul_rn(static_cast<double>(u[k]), p.dx), p.dt);
+      u[k] = 0.f;
       const double Eev = __ddiv_rn(__dmul_rn(__dmul_rn(__dmul_rn(0.5, p.m_i), vi), vi), p.e);
       double g = __dmul_rn(__dmul_rn(p.see_scale, p.gamma_coef), __dsqrt_rn(__ddiv_rn(Eev, p.E_ref_eV)));
       if (g > p.gamma_max) g = p.gamma_max;
       if (!(g > 0.0)) g = 0.0;
-      const U64x4 w = philox4x64_10(q.id, static_cast<uint64_t>(p.step), 0, 0, p.seed, kTagSee);
+      const U64x4 w = philox4x64_10(ion, static_cast<uint64_t>(p.step), 0, 0, p.seed, kTagSee);
       const double fl = floor(g);
       nse = static_cast<int>(fl) + ((u01(w.w[0]) < __dsub_rn(g, fl)) ? 1 : 0);
-      if (nse) atomicAdd(&s_emit[q.electrode], static_cast<unsigned int>(nse));
+      if (nse) atomicAdd(&s_emit[el], static_cast<unsigned int>(nse));
     }
     const int incl = cpk::warp_incl_scan(nse);
     const int total = __shfl_sync(0xffffffffu, incl, 31);
     unsigned long long base = 0;
     if (lane() == 31 && total) {
-      base = atomicAdd(&sc->counters[kSeCount], static_cast<unsigned long long>(total));
+      base = atomicAdd(&counts[kSeCount], static_cast<unsigned long long>(total));
       atomicAdd(electrons, static_cast<unsigned int>(total));
     }
     __syncthreads();
     const bool few = *electrons <= 64u;
     base = __shfl_sync(0xffffffffu, base, 31);
     for (int j = 0; j < nse; ++j) {
-      const U64x4 wv = philox4x64_10(q.id, static_cast<uint64_t>(p.step), static_cast<uint64_t>(1 + j), 0, p.seed, kTagSee);
+      const U64x4 wv = philox4x64_10(ion, static_cast<uint64_t>(p.step), static_cast<uint64_t>(1 + j), 0, p.seed, kTagSee);
       const double ua = u01(wv.w[0]), ub = u01(wv.w[1]), frac = u01(wv.w[2]);
       const double z = sqrt(-2.0 * log(ua)) * cos(2.0 * pi * ub);
       const double use = p.see_vth * fabs(z) * p.dt / p.dx;
-      const double xd = (q.electrode == 0) ? __dmul_rn(use, frac) : __dsub_rn(static_cast<double>(N), __dmul_rn(use, frac));
+      const double xd = (el == 0) ? __dmul_rn(use, frac) : __dsub_rn(static_cast<double>(N), __dmul_rn(use, frac));
       const float xr = cpk::nudge_inside<float>(xd, N);
       const unsigned long long slot = base + static_cast<unsigned long long>(incl - nse + j);
       if (slot < static_cast<unsigned long long>(se_cap)) {
         se_xi[slot] = xr;
-        se_u[slot] = static_cast<float>(q.electrode == 0 ? use : -use);
+        se_u[slot] = static_cast<float>(el == 0 ? use : -use);
         float f;
         const int i = floor_split(xr, &f);
         const unsigned int w1 = frac16(f);
@@ -201,8 +199,6 @@ k_push_ions(Params p, Scratch* sc, const double* __restrict__ E, float* __restri
           atomicAdd(&ne[i], 65536u - w1);
           atomicAdd(&ne[i + 1], w1);
         }
-      } else {
-        s_over = 1;
       }
     }
     if (few) continue;
@@ -214,54 +210,37 @@ k_push_ions(Params p, Scratch* sc, const double* __restrict__ E, float* __restri
   }
   __syncthreads();
   if (tid == 0) {
-    unsigned long long* c = sc->counters;
-    if (s_abs[0]) atomicAdd(&c[kAbs0], static_cast<unsigned long long>(s_abs[0]));
-    if (s_abs[1]) atomicAdd(&c[kAbs1], static_cast<unsigned long long>(s_abs[1]));
-    if (s_emit[0]) atomicAdd(&c[kEmit0], static_cast<unsigned long long>(s_emit[0]));
-    if (s_emit[1]) atomicAdd(&c[kEmit1], static_cast<unsigned long long>(s_emit[1]));
-    if (s_over) atomicAdd(&c[kOverflow], 1ULL);
+    if (s_abs[0]) atomicAdd(&counts[kAbs0], static_cast<unsigned long long>(s_abs[0]));
+    if (s_abs[1]) atomicAdd(&counts[kAbs1], static_cast<unsigned long long>(s_abs[1]));
+    if (s_emit[0]) atomicAdd(&counts[kEmit0], static_cast<unsigned long long>(s_emit[0]));
+    if (s_emit[1]) atomicAdd(&counts[kEmit1], static_cast<unsigned long long>(s_emit[1]));
     __threadfence();
-    if (atomicAdd(&c[kDone], 1ULL) == gridDim.x - 1) {
+    if (atomicAdd(&counts[kDone], 1ULL) == gridDim.x - 1) {
       __threadfence();
-      const unsigned long long se = __ldcg(&c[kSeCount]), cap = static_cast<unsigned long long>(se_cap);
-      const unsigned long long a0 = __ldcg(&c[kAbs0]), e0 = __ldcg(&c[kEmit0]);
-      counts[0] = static_cast<int64_t>(a0);
-      counts[1] = static_cast<int64_t>(__ldcg(&c[kAbs1]));
-      counts[2] = static_cast<int64_t>(e0);
-      counts[3] = static_cast<int64_t>(__ldcg(&c[kEmit1]));
-      counts[4] = static_cast<int64_t>(se < cap ? se : cap);
-      counts[5] = static_cast<int64_t>(a0 + e0);
-      c[kStatus] = (__ldcg(&c[kOverflow]) || se > cap) ? 1ULL : 0ULL;
-      for (int k = 0; k < kStatus; ++k) c[k] = 0ULL;
+      const unsigned long long se = __ldcg(&counts[kSeCount]), cap = static_cast<unsigned long long>(se_cap);
+      counts[4] = se < cap ? se : cap;
+      counts[5] = __ldcg(&counts[kAbs0]) + __ldcg(&counts[kEmit0]);
     }
   }
 }
 
-// Device address of the scratch array (and the push kernel's shared-memory
-// limit), set up once per device with that device current.
-std::mutex g_mu;
-Scratch* g_addr[64] = {};
-// One call at a time: calls from several threads or on several streams share
-// the tallies, which the last CTA of a call clears for the next.
-std::mutex g_call;
+constexpr size_t push_smem(int N) { return 12 * static_cast<size_t>(N + 2) + sizeof(uint16_t) * (kMostCta + 1); }
 
-int scratch_address(int dev, Scratch** out) {
+// The push kernel's shared-memory limit, set once per device.
+std::mutex g_mu;
+bool g_ready[64] = {};
+
+int configure(int dev) {
   if (dev < 0 || dev >= 64) return CP_ERR_ARG;
   std::lock_guard<std::mutex> lock(g_mu);
-  if (!g_addr[dev]) {
-    void* ptr = nullptr;
-    if (cudaGetSymbolAddress(&ptr, g_scratch) != cudaSuccess || !ptr) {
-      cudaGetLastError();
-      return CP_ERR_CUDA;
-    }
+  if (!g_ready[dev]) {
     if (cudaFuncSetAttribute(k_push_ions, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(12 * (kMaxCells + 2))) != cudaSuccess) {
+                             static_cast<int>(push_smem(kMaxCells))) != cudaSuccess) {
       cudaGetLastError();
       return CP_ERR_CUDA;
     }
-    g_addr[dev] = static_cast<Scratch*>(ptr);
+    g_ready[dev] = true;
   }
-  *out = g_addr[dev];
   return CP_OK;
 }
 
@@ -286,11 +265,10 @@ extern "C" int cp_push_ions_noalloc(const cp_gap* gap, const cp_see_beam* see, d
       see->energy_law != CP_SEE_ENERGY_MAXWELL)
     return CP_ERR_ARG;
   if (gap->n_cells < 2 || gap->n_cells > kMaxCells) return CP_ERR_ARG;  // shared-memory grid limit
-  if (n > kMaxIons) return CP_ERR_CAPACITY;  // beyond the scratch array: every ion might be absorbed
+  if (n > kMaxIons) return CP_ERR_CAPACITY;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return CP_ERR_CUDA;
-  Scratch* sc = nullptr;
-  const int rc = scratch_address(dev, &sc);
+  const int rc = configure(dev);
   if (rc != CP_OK) return rc;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int N = gap->n_cells;
@@ -310,23 +288,21 @@ extern "C" int cp_push_ions_noalloc(const cp_gap* gap, const cp_see_beam* see, d
   p.see_vth = std::sqrt(gap->e * see->T_emit_eV / gap->m_e);
   p.seed = seed;
   p.step = step;
-  std::lock_guard<std::mutex> one(g_call);
-  if (cudaMemsetAsync(G, 0, sizeof(int64_t) * (N + 1), st) != cudaSuccess) return CP_ERR_CUDA;
   int sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return CP_ERR_CUDA;
   // at least 512 ions a CTA (each forms the field table and flushes a grid),
   // at most 8191 (its 32-bit node sums stay below 2^29)
   const int64_t want = std::max<int64_t>((n + 511) / 512, 1);
-  const int grid = static_cast<int>(std::max<int64_t>(std::min<int64_t>(want, sms), (n + 8190) / 8191));
-  k_push_ions<<<grid, kThreads, 12 * (N + 2), st>>>(p, sc, E, xi, u, id, n, reinterpret_cast<long long*>(G), se_xi,
-                                                    se_u, se_cap, counts);
-  // one copy of the overflow flag back for the status
-  unsigned long long* flag = &sc->counters[kStatus];
+  const int grid = static_cast<int>(std::max<int64_t>(std::min<int64_t>(want, sms), (n + kMostCta - 1) / kMostCta));
+  long long* Gl = reinterpret_cast<long long*>(G);
+  unsigned long long* tally = reinterpret_cast<unsigned long long*>(counts);
+  k_clear<<<(N + 256) / 256, 256, 0, st>>>(Gl, N + 1, tally);
+  k_push_ions<<<grid, kThreads, push_smem(N), st>>>(p, E, xi, u, id, n, Gl, se_xi, se_u, se_cap, tally);
   if (cudaGetLastError() != cudaSuccess) return CP_ERR_CUDA;
-  unsigned long long overflow = 0;
-  if (cudaMemcpyAsync(&overflow, flag, sizeof(overflow), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+  // the counts back for the status: the electrons asked for may exceed se_cap
+  int64_t c[kCounts];
+  if (cudaMemcpyAsync(c, counts, sizeof(c), cudaMemcpyDefault, st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess)
     return CP_ERR_CUDA;
-  if (overflow) return CP_ERR_CAPACITY;
-  return CP_OK;
+  return c[kEmit0] + c[kEmit1] > se_cap ? CP_ERR_CAPACITY : CP_OK;
 }
