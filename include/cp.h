@@ -51,7 +51,7 @@ extern "C" {
 #define CP_ERR_CAPACITY (-4)  /* a particle store or scratch list overflowed */
 #define CP_ERR_RESIDUAL (-5)  /* strict solve missed the requested residual */
 #define CP_ERR_NONFINITE (-6) /* NaN/Inf in the field or circuit state */
-#define CP_ERR_TIMEOUT (-7)   /* reserved: a bounded device wait gave up */
+#define CP_ERR_TIMEOUT (-7)   /* a bounded device wait gave up */
 
 #define CP_ELECTRONS 0
 #define CP_IONS 1

@@ -253,7 +253,8 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v)
 }
 
 struct alignas(16) MaxSlot {
-  unsigned long long rmax, xmax, bmax, pad;  // bit patterns of non-negative doubles (bmax: integer)
+  unsigned long long rmax, xmax, bmax;  // bit patterns of non-negative doubles (bmax: integer)
+  unsigned long long lost;              // the rank's wait for the totals ran out
 };
 
 // Dynamic shared memory of one rank's rows: G, phi, E, b and r.
@@ -283,10 +284,16 @@ __device__ __forceinline__ void push16(uint32_t dst, unsigned long long a, unsig
                "l"(a), "l"(b), "r"(bar)
                : "memory");
 }
+// Polls of an exchange's barrier before a rank gives up (which: 0 the totals,
+// 1 the maxima).  A test builds the library with limits that run out.
+constexpr int kMostPolls = 1 << 20;
+#ifndef CP_EXCHANGE_POLLS
+#define CP_EXCHANGE_POLLS(which) kMostPolls
+#endif
 // Wait for the barrier's first phase; false when the limit of polls is
 // reached (a rank that never sent: cannot happen unless one failed).
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar) {
-  for (int i = 0; i < (1 << 20); ++i) {
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, int limit) {
+  for (int i = 0; i < limit; ++i) {
     uint32_t done;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -460,6 +467,32 @@ __device__ __noinline__ int commit_level(DevState* S, cp_diag* hist, int64_t his
   return status;
 }
 
+// A rank is lost when one of its waits ran out, or when another rank says with
+// its maxima that its first did.  It commits and refines nothing (the status is
+// CP_ERR_TIMEOUT) and leaves behind two cluster barriers: at the first every
+// rank has sent all it sends or has left, at the second those about to refine
+// have read the flags, and have left as well.  What is addressed to it must
+// have arrived before it may leave.
+__device__ __noinline__ void leave_lost(uint64_t* bars) {
+  cg::cluster_group cl = cg::this_cluster();
+  cl.sync();
+  cl.sync();
+  mbar_wait(&bars[0], kMostPolls);
+  mbar_wait(&bars[1], kMostPolls);
+  asm volatile("cp.async.wait_all;" ::: "memory");  // the network's copies
+}
+
+// Before a refinement: whether any rank is lost (all ranks that are not call
+// this: they have the same backward error).
+__device__ __noinline__ bool any_lost(int* lost) {
+  cg::cluster_group cl = cg::this_cluster();
+  cl.sync();
+  int n = 0;
+  for (unsigned r = 0; r < cl.num_blocks(); ++r) n += *cl.map_shared_rank(lost, r);
+  cl.sync();
+  return n != 0;
+}
+
 // Everything the refinement needs of the solve (rare path).
 struct Refine {
   double *ph, *Ee, *bb, *rr;
@@ -589,6 +622,7 @@ __device__ __forceinline__ void solve_body(const Bufs& B, int do_push, int mode,
   __shared__ double sc[48];
   __shared__ double s_edge[2];
   __shared__ double slotd, s_eta;
+  __shared__ int s_lost;                                    // an exchange of this rank was not completed
 
   const int tid = static_cast<int>(threadIdx.x), lane = tid & 31, warp = tid >> 5;
   const DevParams* P = &sP;
@@ -600,6 +634,7 @@ __device__ __forceinline__ void solve_body(const Bufs& B, int do_push, int mode,
     unsigned long long* dst = reinterpret_cast<unsigned long long*>(&sP);
     for (int k = tid; k < static_cast<int>(sizeof(DevParams) / 8); k += kSolveThreads) dst[k] = src[k];
   }
+  if (tid == 0) s_lost = 0;
   if (nr > 1) {
     if (tid == 0) {
       mbar_init(&bars[0]);
@@ -805,7 +840,10 @@ __device__ __forceinline__ void solve_body(const Bufs& B, int do_push, int mode,
           push16(dst + 16, static_cast<unsigned long long>(tot.s1), 0ULL, bar);
         }
       }
-      if (!mbar_wait(&bars[0]) && lane == 0) atomicCAS(&S->status, 0, CP_ERR_TIMEOUT);
+      if (__any_sync(0xffffffffu, !mbar_wait(&bars[0], CP_EXCHANGE_POLLS(0))) && lane == 0) {
+        s_lost = 1;
+        atomicCAS(&S->status, 0, CP_ERR_TIMEOUT);
+      }
       v.s1 = 0;
       v.s2 = 0;
       if (lane < nr) v = slotA[lane];
@@ -894,7 +932,7 @@ __device__ __forceinline__ void solve_body(const Bufs& B, int do_push, int mode,
   if (warp < kRowWarps) {
     // outputs
     unsigned long long rm = 0ULL, xm = 0ULL;
-    for (int k = tid; k < m; k += kRowThreads) {
+    for (int k = tid; k < (s_lost ? 0 : m); k += kRowThreads) {
       const int i = lo + k;
       const double x = ph[k];
       const double ri = row_residual(ph, bb[k], k, i, m, gam, prev_phi, next_phi);
@@ -917,7 +955,7 @@ __device__ __forceinline__ void solve_body(const Bufs& B, int do_push, int mode,
     }
   } else if (warp == kCommitWarp) {
     if (last_rows && lane == 31) B.phi[N] = 0.0;
-    if (rank == 0)
+    if (rank == 0 && !s_lost)
       status = commit_level(S, B.hist, B.hist_rows, B.vs, P, st, sc, do_push, mode, strict_c, phi0, 0.0);
   }
   if (warp != kCommitWarp)  // the commit goes on beside the error's exchange
@@ -932,9 +970,12 @@ __device__ __forceinline__ void solve_body(const Bufs& B, int do_push, int mode,
       if (lane < nr) {
         const uint32_t dst = remote_addr(&slotC[rank], lane), bar = remote_addr(&bars[1], lane);
         push16(dst, q.rmax, q.xmax, bar);
-        push16(dst + 16, q.bmax, 0ULL, bar);
+        push16(dst + 16, q.bmax, s_lost ? 1ULL : 0ULL, bar);
       }
-      if (!mbar_wait(&bars[1]) && lane == 0) atomicCAS(&S->status, 0, CP_ERR_TIMEOUT);
+      const bool out = __any_sync(0xffffffffu, !mbar_wait(&bars[1], CP_EXCHANGE_POLLS(1)));
+      const bool told = __any_sync(0xffffffffu, lane < nr && slotC[lane].lost != 0ULL);
+      if (lane == 0 && (out || told)) s_lost = 1;
+      if (lane == 0 && out) atomicCAS(&S->status, 0, CP_ERR_TIMEOUT);
       q.rmax = warp_max_u64(lane < nr ? slotC[lane].rmax : 0ULL);
       q.xmax = warp_max_u64(lane < nr ? slotC[lane].xmax : 0ULL);
       q.bmax = warp_max_u64(lane < nr ? slotC[lane].bmax : 0ULL);
@@ -948,8 +989,13 @@ __device__ __forceinline__ void solve_body(const Bufs& B, int do_push, int mode,
     }
   }
   __syncthreads();
+  if (s_lost) {
+    leave_lost(bars);
+    return;
+  }
   double eta = s_eta;
-  if (eta > tol) {  // the same on every rank
+  if (eta > tol) {  // the same on every rank that is not lost
+    if (nr > 1 && any_lost(&s_lost)) return;
     Refine R;
     R.ph = ph; R.Ee = Ee; R.bb = bb; R.rr = rr;
     R.sc = sc; R.wd = wd; R.slotd = &slotd; R.edge = s_edge;
