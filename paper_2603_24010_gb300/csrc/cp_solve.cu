@@ -1026,14 +1026,19 @@ __device__ __forceinline__ void solve_body(const Bufs& B, int do_push, int mode,
   if (runs_net) predictor_update(P, S, st, s_net, sc, strict_c, phi0_fin);
 }
 
+// Registers: one CTA per SM here, 168 a thread without spills (96 is the
+// compiler's own choice: graph step at 1531 cells and 1e6 particles 15.24 us
+// instead of 15.09, at 4096 cells and 3.3e5 16.2 instead of 15.95); the
+// ensemble's clusters share the SMs, two CTAs each (step of 160 instances 238.5
+// us, 247.6 with one CTA per SM).
 template <typename real, typename Acc>
-__global__ void __launch_bounds__(kSolveThreads) k_solve(Bufs B, int do_push, int mode, double tol) {
+__global__ void __launch_bounds__(kSolveThreads, 1) k_solve(Bufs B, int do_push, int mode, double tol) {
   solve_body<real, Acc>(B, do_push, mode, tol);
 }
 
 // Ensemble: cluster i solves instance i.
 template <typename real, typename Acc>
-__global__ void __launch_bounds__(kSolveThreads)
+__global__ void __launch_bounds__(kSolveThreads, 2)
 k_solve_ens(const Bufs* __restrict__ Ball, int do_push, int mode, double tol) {
   const Bufs B = Ball[blockIdx.x / cg::this_cluster().num_blocks()];
   solve_body<real, Acc>(B, do_push, mode, tol);
