@@ -1197,7 +1197,7 @@ struct cp_batch {
   int E = 0;
   int precision = CP_FP32;
   int n_max = 0;
-  int beam_max = 0;      // beam ions a step of the largest beam
+  int beam_max = 0;      // beam ions a step of the largest beam, as far as a store may hold them
   bool initialized = false;
   cpk::Bufs* dBall = nullptr;
   void* abs = nullptr;
@@ -1275,7 +1275,9 @@ int batch_init(cp_batch* b, int mode, double tol) {
   for (int i = 0; i < b->E; ++i) {
     hb[i] = make_bufs(b->inst[i]);
     b->n_max = std::max(b->n_max, b->inst[i]->N);
-    b->beam_max = std::max(b->beam_max, static_cast<int>(b->inst[i]->hp.beam_per_step));
+    // (the first ion beyond the store stops the instance with CP_ERR_CAPACITY)
+    const int64_t beam = std::min<int64_t>(b->inst[i]->hp.beam_per_step, b->inst[i]->cap[CP_IONS] + 1);
+    b->beam_max = std::max(b->beam_max, static_cast<int>(beam));
   }
   CP_TRY(alloc(reinterpret_cast<void**>(&b->dBall), sizeof(cpk::Bufs) * b->E));
   CP_CUDA(cudaMemcpyAsync(b->dBall, hb.data(), sizeof(cpk::Bufs) * b->E, cudaMemcpyHostToDevice,

@@ -433,12 +433,14 @@ k_push_ens(const Bufs* __restrict__ Ball, int E, int n_max, int beam_chunks,
 
   // --- the beams: THREADS ions of one instance at a time ----------------------
   // Ions are appended by the beam alone, behind the slots in use.
-  for (int item = blockIdx.x; item < E * beam_chunks; item += gridDim.x) {
-    const Bufs& B = Ball[item / beam_chunks];
+  for (long long item = blockIdx.x; item < static_cast<long long>(E) * beam_chunks; item += gridDim.x) {
+    const int inst = static_cast<int>(item / beam_chunks);
+    const int k0 = static_cast<int>(item - static_cast<long long>(inst) * beam_chunks) * THREADS;  // below the largest beam
+    const Bufs& B = Ball[inst];
     const DevParams* Pi = B.P;
     DevState* Si = B.S;
-    const int Bn = Pi->beam_per_step, k = item % beam_chunks * THREADS + tid;
-    if (Bn <= item % beam_chunks * THREADS || ldcg(&Si->status) != 0) continue;
+    const int Bn = Pi->beam_per_step, k = k0 + tid;
+    if (Bn <= k0 || ldcg(&Si->status) != 0) continue;
     if (k < Bn) {
       const int64_t step = ldcg(&Si->level);
       const int Ni = Pi->N;
@@ -588,7 +590,7 @@ cudaError_t push_ens_launch(int precision, int threads, int grid, size_t smem, c
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  int chunks = (beam_max + threads - 1) / threads;  // of the largest beam
+  int chunks = beam_max / threads + (beam_max % threads != 0 ? 1 : 0);  // of the largest beam
   void* args[] = {&Ball, &E, &n_max, &chunks, &abs, &abs_cap};
   return cudaLaunchKernelExC(&cfg, push_ens_kernel(precision, threads), args);
 }
