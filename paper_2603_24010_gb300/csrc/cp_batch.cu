@@ -621,15 +621,12 @@ cudaError_t compact_ens_configure(int precision) {
 
 cudaError_t compact_ens_launch(int precision, const Bufs* Ball, int E, int grid, cudaStream_t st) {
   const size_t smem = compact_ens_smem(precision, E);
-  if (precision == CP_FP32) {
-    k_compact_ens<float><<<grid, kThreads, smem, st>>>(Ball, E);
-    if (cudaGetLastError() != cudaSuccess) return cudaGetLastError();
-    k_swap_ens<float><<<(E + 127) / 128, 128, 0, st>>>(Ball, E);
-  } else {
-    k_compact_ens<double><<<grid, kThreads, smem, st>>>(Ball, E);
-    if (cudaGetLastError() != cudaSuccess) return cudaGetLastError();
-    k_swap_ens<double><<<(E + 127) / 128, 128, 0, st>>>(Ball, E);
-  }
+  if (precision == CP_FP32) k_compact_ens<float><<<grid, kThreads, smem, st>>>(Ball, E);
+  else k_compact_ens<double><<<grid, kThreads, smem, st>>>(Ball, E);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  if (precision == CP_FP32) k_swap_ens<float><<<(E + 127) / 128, 128, 0, st>>>(Ball, E);
+  else k_swap_ens<double><<<(E + 127) / 128, 128, 0, st>>>(Ball, E);
   return cudaGetLastError();
 }
 
