@@ -440,10 +440,10 @@ int cp_mlp_adam(float* params, const float* grad, float* m, float* v, int64_t t,
  * Ensemble of independent gap instances (uneven cells and particle counts,
  * their own circuits, SEE scales and beams) advanced together: per step one
  * persistent push launch over the particle tiles of every instance and one
- * solve launch with one CTA per instance, replayed from a CUDA graph.  An
- * instance advanced in the ensemble gives bit for bit the results it gives
- * as a context of its own (same per-particle arithmetic, integer charge,
- * counter-based draws, exact integer solve).
+ * solve launch with a small cluster of CTAs per instance, replayed from a
+ * CUDA graph.  An instance advanced in the ensemble gives bit for bit the
+ * results it gives as a context of its own (same per-particle arithmetic,
+ * integer charge, counter-based draws, exact integer solve).
  * ------------------------------------------------------------------------ */
 typedef struct cp_batch cp_batch;
 
@@ -470,8 +470,8 @@ int cp_batch_step_weak(cp_batch* b, int32_t n_steps);
    arguments and errors as cp_set_predictor, any time; each instance has its
    own network and window), and advance every instance with the learned
    weak scheme.  An instance without a network runs the plain weak scheme,
-   as cp_step_weak.  The ensemble's solve runs the network in the same CTA
-   after the commit; results are those of the instance's own context. */
+   as cp_step_weak.  The ensemble's solve runs the network after the commit;
+   results are those of the instance's own context. */
 int cp_batch_set_predictor(cp_batch* b, int32_t i, const float* params, const cp_predictor* norm);
 int cp_batch_step_weak_learned(cp_batch* b, int32_t n_steps);
 

@@ -13,7 +13,8 @@
 //   with int64 global atomics straight into their instance's grid.
 // k_compact_ens / k_swap_ens: removal of absorbed particles over the same
 //   flat list, then one thread per instance swaps the buffers.
-// The solve of every instance (one CTA each) is k_solve_ens in cp_solve.cu.
+// The solve of every instance (a cluster of 1, 2 or 4 CTAs) is
+// k_solve_ens in cp_solve.cu.
 #include <algorithm>
 
 #include "cp_common.cuh"

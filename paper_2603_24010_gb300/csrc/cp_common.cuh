@@ -139,12 +139,6 @@ __device__ __forceinline__ int warp_incl_scan(int v) {
   return v;
 }
 
-__device__ __forceinline__ unsigned int warp_sum_u(unsigned int v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 __device__ __forceinline__ unsigned int warp_max_u(unsigned int v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));

@@ -31,8 +31,7 @@ namespace cpk {
 constexpr int kSpecies = 3;
 constexpr int kThreads = 512;          // threads per CTA of the push kernel
 constexpr int kCtasPerSm = 2;          // resident push CTAs per SM
-constexpr int kPerThread = 4;          // particles per thread per tile (one 16 B vector for FP32)
-constexpr int kTile = kThreads * kPerThread;  // particles per CTA tile
+constexpr int kPerThread = 4;          // slots per thread of a removal's block (one 16 B vector for FP32)
 constexpr int kFlushTiles = 31;        // tiles between flushes of the 32-bit cell sums
 constexpr int kSolveCtas = 8;          // CTAs (one cluster) of the coupled solve (portable)
 constexpr int kSolveCtasMax = 16;      // non-portable cluster size used where the GPU allows it

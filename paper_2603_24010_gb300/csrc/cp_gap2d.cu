@@ -27,7 +27,6 @@
 
 #include <algorithm>
 
-
 #include "cp_common.cuh"
 #include "cp_gap2d.cuh"
 
@@ -45,7 +44,6 @@ struct Stencil2 {
 };
 
 __device__ __forceinline__ int wrapi(int j, int N) { return j < 0 ? j + N : (j >= N ? j - N : j); }
-__device__ __forceinline__ int modp(int j, int N) { const int r = j % N; return r < 0 ? r + N : r; }
 
 __device__ __forceinline__ Stencil2 stencil2(const Dev2D& D, float x, float y) {
   Stencil2 st;
@@ -94,16 +92,6 @@ __device__ __forceinline__ int win_rel(int gx, int gy, int ox, int oy, int Ny) {
   if (static_cast<unsigned>(lx) > static_cast<unsigned>(kW2 - 2) ||
       static_cast<unsigned>(ly) > static_cast<unsigned>(kW2 - 2))
     return -1;
-  return lx * kW2 + ly;
-}
-
-// window coordinates of a global node (x index gx, y index gy); -1 if outside
-__device__ __forceinline__ int win_index(int gx, int gy, int ox, int oy, int Ny) {
-  const int lx = gx - ox;
-  int ly = gy - oy;
-  if (ly < 0) ly += Ny;
-  if (ly >= Ny) ly -= Ny;
-  if (lx < 0 || lx >= kW2 || ly < 0 || ly >= kW2) return -1;
   return lx * kW2 + ly;
 }
 
@@ -1236,10 +1224,6 @@ __global__ void k2_tables(Dev2D* Dp, double r2) {
 // ---------------------------------------------------------------------------
 // Host-side launchers
 // ---------------------------------------------------------------------------
-size_t dev2d_bytes() { return sizeof(Dev2D); }
-size_t absrec2_bytes() { return sizeof(AbsRec2); }
-int tile2() { return kT2; }
-
 constexpr size_t kCwinBytes = sizeof(Window2);
 
 cudaError_t push2_occupancy(int* per_sm) {
