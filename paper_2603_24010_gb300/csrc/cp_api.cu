@@ -1682,6 +1682,8 @@ struct cp_gap2d {
   double t_ms[3] = {0.0, 0.0, 0.0};  // push, solve (all kernels), sort
   int64_t t_n[3] = {0, 0, 0};
   std::vector<cudaEvent_t> ev;
+  cudaGraphExec_t gexec[2][3] = {};      // steps, and a re-sort followed by steps, by coupling mode
+  double gtol[2][3] = {};
   cudaStream_t side = nullptr;           // captured beside the main stream: the mean's solve
   cudaEvent_t fork = nullptr, join = nullptr;
 };
@@ -1694,7 +1696,16 @@ int g2_alloc(cp_gap2d* g, void** p, size_t bytes) {
   return CP_OK;
 }
 
+void g2_drop_graphs(cp_gap2d* g) {
+  for (auto& kind : g->gexec)
+    for (cudaGraphExec_t& e : kind) {
+      if (e) cudaGraphExecDestroy(e);
+      e = nullptr;
+    }
+}
+
 void g2_free(cp_gap2d* g) {
+  g2_drop_graphs(g);
   for (void* p : g->owned) cudaFree(p);
   g->owned.clear();
   for (cudaEvent_t e : g->ev) cudaEventDestroy(e);
@@ -1755,15 +1766,16 @@ int g2_push(cp_gap2d* g, cudaStream_t st) {
 // and the first call 50.1 us a step; 16 a graph 30.7, as every later call).
 int g2_graph_steps(const cp_gap2d* g) { return std::min(g->sort_every, 16); }
 
-// Capture a graph of steps.  (The re-sort is not among them: its padding may
-// need more slots than the particles do, and then only a step that follows is
-// refused.)
-int g2_build_graph(cp_gap2d* g, int mode, double tol) {
+// Capture a graph of steps, or of the re-sort that is due and the steps behind
+// it.  (A re-sort never ends a graph: its padding may need more slots than the
+// particles do, and then only a step that follows is refused.)
+int g2_build_graph(cp_gap2d* g, bool sort, int mode, double tol) {
   cp_ctx* c = g->c;
-  if (c->gexec[mode] && c->gtol[mode] == tol) return CP_OK;
-  if (c->gexec[mode]) {
-    cudaGraphExecDestroy(c->gexec[mode]);
-    c->gexec[mode] = nullptr;
+  cudaGraphExec_t& exec = g->gexec[sort][mode];
+  if (exec && g->gtol[sort][mode] == tol) return CP_OK;
+  if (exec) {
+    cudaGraphExecDestroy(exec);
+    exec = nullptr;
   }
   if (!g->side) {
     CP_CUDA(cudaStreamCreateWithFlags(&g->side, cudaStreamNonBlocking));
@@ -1773,7 +1785,7 @@ int g2_build_graph(cp_gap2d* g, int mode, double tol) {
   const int64_t launches = g->launches;
   cudaGraph_t gr = nullptr;
   CP_CUDA(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
-  int rc = CP_OK;
+  int rc = sort ? g2_sort(g, c->cap_stream) : CP_OK;
   for (int k = 0; k < g2_graph_steps(g) && rc == CP_OK; ++k) {
     rc = g2_push(g, c->cap_stream);
     if (rc == CP_OK) rc = g2_solve(g, c->cap_stream, true, 1, mode, tol);
@@ -1784,10 +1796,10 @@ int g2_build_graph(cp_gap2d* g, int mode, double tol) {
     if (gr) cudaGraphDestroy(gr);
     return CP_ERR_CUDA;
   }
-  const cudaError_t e2 = cudaGraphInstantiate(&c->gexec[mode], gr, 0);
+  const cudaError_t e2 = cudaGraphInstantiate(&exec, gr, 0);
   cudaGraphDestroy(gr);
   CP_CUDA(e2);
-  c->gtol[mode] = tol;
+  g->gtol[sort][mode] = tol;
   return CP_OK;
 }
 
@@ -2002,20 +2014,24 @@ int g2_steps(cp_gap2d* g, int mode, int32_t n_steps, double tol) {
     return CP_OK;
   };
   for (int k = 0; k < n_steps;) {
-    if (g->since_sort == g->sort_every) {  // periodic re-sort (also drops absorbed slots)
+    // periodic re-sort (also drops absorbed slots), due ahead of this step; the
+    // steps up to the next one from graphs, unless a graph would serve once (a
+    // first period of a single graph, not behind a re-sort)
+    const bool due = g->since_sort == g->sort_every;
+    const int whole = g2_graph_steps(g), room = due ? g->sort_every : g->sort_every - g->since_sort;
+    if (!g->timing && std::min(n_steps - k, room) >= whole && (due || g->sort_every >= 2 * whole)) {
+      CP_TRY(g2_build_graph(g, due, mode, tol));
+      CP_CUDA(cudaGraphLaunch(g->gexec[due][mode], c->stream));
+      g->launches += 5 * whole + (due ? 5 : 0);
+      g->since_sort = (due ? 0 : g->since_sort) + whole;
+      k += whole;
+      continue;
+    }
+    if (due) {
       if (g->timing) CP_TRY(g2_timed(g, 2, &rec));
       CP_TRY(g2_sort(g, c->stream));
       if (g->timing) CP_TRY(mark_end());
       g->since_sort = 0;
-    }
-    const int whole = g2_graph_steps(g);
-    if (!g->timing && std::min(n_steps - k, g->sort_every - g->since_sort) >= whole) {
-      CP_TRY(g2_build_graph(g, mode, tol));
-      CP_CUDA(cudaGraphLaunch(c->gexec[mode], c->stream));
-      g->launches += 5 * whole;
-      g->since_sort += whole;
-      k += whole;
-      continue;
     }
     if (g->timing) CP_TRY(g2_timed(g, 0, &rec));
     CP_TRY(g2_push(g, c->stream));
@@ -2114,6 +2130,7 @@ int cp2d_step_weak(cp_gap2d* g, int32_t n_steps) { return g2_steps(g, 1, n_steps
 
 int cp2d_set_predictor(cp_gap2d* g, const float* params, const cp_predictor* norm) {
   if (!g) return CP_ERR_ARG;
+  g2_drop_graphs(g);  // they carry the old buffer set
   return cp_set_predictor(g->c, params, norm);  // the mean problem's context
 }
 
