@@ -142,7 +142,7 @@ constexpr int ens_min_ctas(int threads, size_t es) { return threads == 256 ? 3 :
 // lane, the beams dealt over all CTAs, in slots that need no counter.
 //
 // 160 gaps of 260 to 3985 cells, 7.0e7 particles: push 231 -> 222 us, step in
-// a graph 268 -> 264 (with the removal's interleaving 209 and 242).
+// a graph 268 -> 264 (with the removal's interleaving 209 and 239).
 template <typename real, int THREADS>
 __global__ void __launch_bounds__(THREADS, ens_min_ctas(THREADS, sizeof(real)))
 k_push_ens(const Bufs* __restrict__ Ball, int E, int n_max, int beam_chunks,

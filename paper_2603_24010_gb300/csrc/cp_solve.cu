@@ -176,8 +176,8 @@ __device__ void cluster_tri_solve_f64(double* v, int lo, int m, int N, double b0
 // Rows per thread: chunk / 256, and the cluster has one CTA per 256 rows up
 // to 16.  FP64 is what a row costs (about a dozen operations at 2 per cycle
 // and SM), so more rows per SM cost more than the exchange saves.
-// Measured (GB300, event-bracketed launch; an empty kernel reads 4-5 us): 11.2
-// us at 256 cells and 12.7 us at 4096, against 18.4 us for one 16-CTA cluster
+// Measured (GB300, event-bracketed launch; an empty kernel reads 4-5 us): 11.6
+// us at 256 cells and 12.4 us at 4096, against 18.4 us for one 16-CTA cluster
 // of 512 threads with cluster barriers, remote loads and a commit at the end.
 // Graph-timed step: 22.9 against 30.4 us (4096 cells, 3.3e5 FP32 particles),
 // 17.5 against 24.5 us (1531 cells, 1e6), 118 against 125 us (4096, 3.1e7).
